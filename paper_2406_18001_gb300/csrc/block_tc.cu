@@ -156,6 +156,26 @@ __device__ __noinline__ void mbar_drain(uint64_t *bar, uint32_t parity)
         if (clock64() - t0 > WAIT_CYCLES) return;
 }
 
+// The producer and MMA warps run their loops with all 32 lanes (uniform control flow and
+// addresses), one elected lane issuing the copies and MMAs; a wait's common case is one inlined
+// test, the descriptors step by addition.  Issued by a single lane of a diverged warp, a k-block
+// took some 780 cycles beside the epilogue warps against the 512 its MMAs need (fp16 and FP8
+// alike); now 300-480.  FP8 apply at m = 400000, n = 2048, 4096 columns: 2212 -> 1780 us.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort_flag, int *err)
+{
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, err));
+}
+
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(p)::"memory");
+    return p;
+}
+
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y)
 {
     asm volatile(
@@ -170,16 +190,10 @@ __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::aft
 
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
 // 128 bytes, 8-row groups 1024 bytes apart (stride byte offset), descriptor
-// version 1, layout type 2 (SWIZZLE_128B).
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr)
-{
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
+// version 1, layout type 2 (SWIZZLE_128B).  The low word holds the address
+// (16-byte units), which the issue loops step by addition; the high word is constant.
+__device__ __forceinline__ uint32_t sw128_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+constexpr uint32_t SW128_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 
 // Instruction descriptor: D = F32, A/B format (kind::f16: bf16 = 1;
 // kind::tf32: tf32 = 2; kind::f8f6f4: e4m3 = 0), both K-major, N >> 3 at bit
@@ -192,23 +206,26 @@ __host__ __device__ constexpr uint32_t make_idesc(int fmt, int n, int m)
 
 // MK: 0 kind::f16, 1 kind::tf32, 2 kind::f8f6f4
 template <int MK>
-__device__ __forceinline__ void mma(uint32_t dtm, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc)
+__device__ __forceinline__ void mma(uint32_t dtm, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc)
 {
     if (MK == 1)
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtm),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+            "setp.ne.u32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %3, p;\n\t}" ::"r"(dtm),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(SW128_HI));
     else if (MK == 2)
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtm),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+            "setp.ne.u32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %3, p;\n\t}" ::"r"(dtm),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(SW128_HI));
     else
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtm),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+            "setp.ne.u32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(dtm),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(SW128_HI));
 }
 
 __device__ __forceinline__ void mma_commit(uint64_t *bar)
@@ -530,81 +547,93 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int kb_elems = TF32 ? 32 : FP8 ? 128 : 64;  // elements per 128-byte k-block
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------------------------------------------- producer --
-            uint32_t it = 0;
-            bool ok = true;
-            const uint32_t bytes = (uint32_t)((SPLIT ? 2 : 1) * (A_STAGE + bn * ROW_BYTES));
-            for (int item = blockIdx.x; ok && item < a.items; item += gridDim.x) {
-                int tile, c0, c1;
-                item_range(a, item, tile, c0, c1);
-                for (int nc = c0; ok && nc < c1; ++nc)
-                    for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
-                        const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
-                        if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, a.err)) {
-                            ok = false;
-                            break;
-                        }
-                        mbar_expect_tx(&full[s], bytes);
-                        tma_load_2d(sA + s * A_ST, &tmA, &full[s], kb * kb_elems, tile * BM);
-                        tma_load_2d(sB + s * B_ST, &tmB, &full[s], kb * kb_elems, nc * bn);
+        // -------------------------------------------------------- producer --
+        const uint32_t leader = elect_one();
+        uint32_t it = 0, sg = 0, ph = 0;
+        bool ok = true;
+        const uint32_t bytes = (uint32_t)((SPLIT ? 2 : 1) * (A_STAGE + bn * ROW_BYTES));
+        for (int item = blockIdx.x; ok && item < a.items; item += gridDim.x) {
+            int tile, c0, c1;
+            item_range(a, item, tile, c0, c1);
+            for (int nc = c0; ok && nc < c1; ++nc)
+                for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
+                    if (!mbar_wait_warp(&empty[sg], ph ^ 1, abort_flag, a.err)) {
+                        ok = false;
+                        break;
+                    }
+                    if (leader) {
+                        mbar_expect_tx(&full[sg], bytes);
+                        tma_load_2d(sA + sg * A_ST, &tmA, &full[sg], kb * kb_elems, tile * BM);
+                        tma_load_2d(sB + sg * B_ST, &tmB, &full[sg], kb * kb_elems, nc * bn);
                         if (SPLIT) {
-                            tma_load_2d(sA + s * A_ST + A_STAGE, &tmA, &full[s], a.lo_off + kb * kb_elems, tile * BM);
-                            tma_load_2d(sB + s * B_ST + B_STAGE, &tmB, &full[s], a.lo_off + kb * kb_elems, nc * bn);
+                            tma_load_2d(sA + sg * A_ST + A_STAGE, &tmA, &full[sg], a.lo_off + kb * kb_elems, tile * BM);
+                            tma_load_2d(sB + sg * B_ST + B_STAGE, &tmB, &full[sg], a.lo_off + kb * kb_elems, nc * bn);
                         }
                     }
-            }
-            if (!ok) {  // let every issued copy land before the CTA exits
-                uint32_t first = it > STAGES ? it - STAGES : 0;
-                for (uint32_t j = first; j < it; ++j) mbar_drain(&full[j % STAGES], (j / STAGES) & 1);
-            }
+                    __syncwarp();
+                    if (++sg == STAGES) {
+                        sg = 0;
+                        ph ^= 1;
+                    }
+                }
+        }
+        if (!ok && leader) {  // let every issued copy land before the CTA exits
+            uint32_t first = it > STAGES ? it - STAGES : 0;
+            for (uint32_t j = first; j < it; ++j) mbar_drain(&full[j % STAGES], (j / STAGES) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // --------------------------------------------------------- MMA --
-            const uint32_t idesc = make_idesc(TF32 ? 2 : SCALED ? 0 : 1, bn, BM);  // tf32, e4m3 / f16, bf16
-            uint32_t it = 0, acc_it = 0;
-            bool ok = true, issued = false;
-            for (int item = blockIdx.x; ok && item < a.items; item += gridDim.x) {
-                int tile, c0, c1;
-                item_range(a, item, tile, c0, c1);
-                for (int nc = c0; ok && nc < c1; ++nc, ++acc_it) {
-                    const uint32_t buf = acc_it & 1, aph = (acc_it >> 1) & 1;
-                    if (!mbar_wait(&tempty[buf], aph ^ 1, abort_flag, a.err)) {
+        // ------------------------------------------------------------- MMA --
+        const uint32_t leader = elect_one();
+        const uint32_t idesc = make_idesc(TF32 ? 2 : SCALED ? 0 : 1, bn, BM);  // tf32, e4m3 / f16, bf16
+        const uint32_t a0 = sw128_lo(su32(sA)), b0 = sw128_lo(su32(sB));
+        uint32_t acc_it = 0, sg = 0, ph = 0;
+        bool ok = true, issued = false;
+        for (int item = blockIdx.x; ok && item < a.items; item += gridDim.x) {
+            int tile, c0, c1;
+            item_range(a, item, tile, c0, c1);
+            for (int nc = c0; ok && nc < c1; ++nc, ++acc_it) {
+                const uint32_t buf = acc_it & 1, aph = (acc_it >> 1) & 1;
+                if (!mbar_wait_warp(&tempty[buf], aph ^ 1, abort_flag, a.err)) {
+                    ok = false;
+                    break;
+                }
+                fence_after();
+                const uint32_t dtm = tmem_base + buf * (uint32_t)bn;
+                for (int kb = 0; kb < a.kblocks; ++kb) {
+                    if (!mbar_wait_warp(&full[sg], ph, abort_flag, a.err)) {
                         ok = false;
                         break;
                     }
                     fence_after();
-                    const uint32_t dtm = tmem_base + buf * (uint32_t)bn;
-                    for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
-                        const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
-                        if (!mbar_wait(&full[s], ph, abort_flag, a.err)) {
-                            ok = false;
-                            break;
-                        }
-                        fence_after();
-                        const uint32_t ab = su32(sA + s * A_ST), bb = su32(sB + s * B_ST);
+                    const uint32_t ab = a0 + sg * (A_ST >> 4), bb = b0 + sg * (B_ST >> 4);
+                    if (leader) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
-                            mma<MK>(dtm, sw128_desc(ab + 32 * k), sw128_desc(bb + 32 * k), idesc,
-                                    (kb > 0 || k > 0) ? 1u : 0u);
+                            mma<MK>(dtm, ab + 2 * k, bb + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
                             if (SPLIT) {
-                                mma<MK>(dtm, sw128_desc(ab + 32 * k), sw128_desc(bb + B_STAGE + 32 * k), idesc, 1u);
-                                mma<MK>(dtm, sw128_desc(ab + A_STAGE + 32 * k), sw128_desc(bb + 32 * k), idesc, 1u);
+                                mma<MK>(dtm, ab + 2 * k, bb + (B_STAGE >> 4) + 2 * k, idesc, 1u);
+                                mma<MK>(dtm, ab + (A_STAGE >> 4) + 2 * k, bb + 2 * k, idesc, 1u);
                             }
                         }
-                        issued = true;
-                        mma_commit(&empty[s]);
+                        mma_commit(&empty[sg]);
                     }
-                    if (!ok) break;
-                    mma_commit(&tfull[buf]);
+                    issued = true;
+                    __syncwarp();
+                    if (++sg == STAGES) {
+                        sg = 0;
+                        ph ^= 1;
+                    }
                 }
-            }
-            if (!ok && issued) {  // wait (bounded) for the MMAs already issued
-                mma_commit(drain);
-                mbar_drain(drain, 0);
+                if (!ok) break;
+                if (leader) mma_commit(&tfull[buf]);
+                __syncwarp();
             }
         }
+        if (!ok && issued && leader) {  // wait (bounded) for the MMAs already issued
+            mma_commit(drain);
+            mbar_drain(drain, 0);
+        }
+        __syncwarp();
     } else {
         // ------------------------------------------------------ epilogue --
         const int quarter = warp & 3;  // warps 2..9 -> TMEM lanes 64,96,0,32,64,96,0,32
@@ -711,8 +740,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 constexpr int BM2 = 2 * BM;                          // rows per pair tile
 constexpr int B2_STAGE = (BN_MAX / 2) * ROW_BYTES;   // 16 KB: half of an N-chunk
 constexpr int RING2_BYTES = 6 * (A_STAGE + B2_STAGE);  // 6 single or 3 split stages
-constexpr int CST_FLOATS = 6 * 128;                   // staged column terms per epilogue warp
-constexpr int SMEM2_BYTES = RING2_BYTES + 1024 + 256 + XCH_BYTES + 8 * CST_FLOATS * 4;
+constexpr int CST_FLOATS = 6 * 128 + 4;               // staged column terms of an epilogue half's chunk (two buffers each)
+constexpr int SMEM2_BYTES = RING2_BYTES + 1024 + 256 + XCH_BYTES + 4 * CST_FLOATS * 4;
 
 // arrive on an mbarrier of the pair given by its shared::cluster address
 __device__ __forceinline__ void arrive_cl(uint32_t bar)
@@ -732,23 +761,26 @@ __device__ __forceinline__ void tma_load_2d_pair(void *dst, const CUtensorMap *m
 }
 
 template <int MK>
-__device__ __forceinline__ void mma2(uint32_t dtm, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc)
+__device__ __forceinline__ void mma2(uint32_t dtm, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc)
 {
     if (MK == 1)
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtm),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+            "setp.ne.u32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::tf32 [%0], da, db, %3, p;\n\t}" ::"r"(dtm),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(SW128_HI));
     else if (MK == 2)
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtm),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+            "setp.ne.u32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], da, db, %3, p;\n\t}" ::"r"(dtm),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(SW128_HI));
     else
         asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtm),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+            "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
+            "setp.ne.u32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(dtm),
+            "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "r"(SW128_HI));
 }
 
 // arrive on `bar` in both CTAs of the pair once the issued MMAs complete
@@ -798,34 +830,40 @@ __device__ __forceinline__ void pair_units(const TcArgs &a, int pair, int npairs
     }
 }
 
-// The i-th unit of a pair.  Ranged: even pairs take their tiles first to
-// last, odd pairs last to first (the chunks of a tile in order either way),
+// A pair's units one after another.  Ranged: even pairs take their tiles first
+// to last, odd pairs last to first (the chunks of a tile in order either way),
 // so that both pairs that share a tile reach it at about the same time (at
 // the start of both ranges, or at the end of both) and its rows of A are
-// read from memory once.
-__device__ __forceinline__ void pair_unit(const TcArgs &a, int pair, int npairs, bool ranged, int u0, int u1, int i,
-                                          int &tile, int &nc)
-{
-    if (ranged) {
-        const int nch = a.nchunks;
-        int u = u0 + i;
-        if (pair & 1) {
-            const int thi = (u1 - 1) / nch, tlo = u0 / nch;
-            const int top = u1 - max(u0, thi * nch);  // units of the last tile
-            if (i < top) {
-                u = u1 - top + i;
-            } else {
-                const int j = i - top, mid = (thi - 1 - tlo) * nch;  // units of the full tiles between
-                u = j < mid ? (thi - 1 - j / nch) * nch + j % nch : u0 + (j - mid);
-            }
+// read from memory once.  Stepped, not divided out of a unit number: the
+// epilogue warps keep it beside the MMA issue they share schedulers with.
+struct UnitIter {
+    int item, nc;        // row tile and N-chunk
+    int u0, u1, nch;     // the pair's range (ranged), chunks per tile
+    int step;            // tile step: 1, -1 (odd pairs), or npairs (not ranged)
+    __device__ __forceinline__ UnitIter(const TcArgs &a, int pair, int npairs, bool ranged, int lo, int hi)
+        : u0(lo), u1(hi), nch(a.nchunks)
+    {
+        if (!ranged) {
+            item = pair;
+            nc = 0;
+            step = npairs;
+        } else if (pair & 1) {
+            item = (hi - 1) / nch;
+            nc = max(lo, item * nch) - item * nch;
+            step = -1;
+        } else {
+            item = lo / nch;
+            nc = lo - item * nch;
+            step = 1;
         }
-        tile = u / nch;
-        nc = u % nch;
-    } else {
-        tile = pair + i / a.nchunks * npairs;
-        nc = i % a.nchunks;
     }
-}
+    __device__ __forceinline__ void next()
+    {
+        if (++nc < nch && (step != -1 || item * nch + nc < u1)) return;
+        item += step;
+        nc = step == -1 ? max(u0 - item * nch, 0) : 0;
+    }
+};
 
 template <int MODE, int KIND>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
@@ -905,87 +943,103 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     pair_units(a, pair, npairs, ranged, u0, u1, nunits);
 
     if (warp == 0) {
-        if (lane == 0) {
-            // ---------------------------------------------------- producer --
-            uint32_t it = 0;
-            bool ok = true;
-            const uint32_t bytes = (uint32_t)(2 * PLANES * (A_STAGE + bh * ROW_BYTES));  // both CTAs'
-            for (int i = 0; ok && i < nunits; ++i) {
-                int item, nc;
-                pair_unit(a, pair, npairs, ranged, u0, u1, i, item, nc);
-                for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
-                        const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
-                        if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, a.err)) {
-                            ok = false;
-                            break;
-                        }
-                        const uint32_t fb = full0 + 8u * s;
-                        const int ya = item * BM2 + (int)rank * BM, yb = nc * bn + (int)rank * bh;
-                        if (rank == 0) mbar_expect_tx(&full[s], bytes);
+        // -------------------------------------------------------- producer --
+        const uint32_t leader = elect_one();
+        uint32_t it = 0, sg = 0, ph = 0;
+        bool ok = true;
+        const uint32_t bytes = (uint32_t)(2 * PLANES * (A_STAGE + bh * ROW_BYTES));  // both CTAs'
+        UnitIter un(a, pair, npairs, ranged, u0, u1);
+        for (int i = 0; ok && i < nunits; ++i, un.next()) {
+            const int ya = un.item * BM2 + (int)rank * BM, yb = un.nc * bn + (int)rank * bh;
+            for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
+                if (!mbar_wait_warp(&empty[sg], ph ^ 1, abort_flag, a.err)) {
+                    ok = false;
+                    break;
+                }
+                if (leader) {
+                    const uint32_t fb = full0 + 8u * sg;
+                    if (rank == 0) mbar_expect_tx(&full[sg], bytes);
 #pragma unroll
-                        for (int pl = 0; pl < PLANES; ++pl) {  // plane pl starts at column pl * lo_off
-                            tma_load_2d_pair(sA + s * A_ST + pl * A_STAGE, &tmA, fb, pl * a.lo_off + kb * kb_elems, ya);
-                            tma_load_2d_pair(sB + s * B_ST + pl * B_PLANE, &tmB, fb, pl * a.lo_off + kb * kb_elems, yb);
-                        }
+                    for (int pl = 0; pl < PLANES; ++pl) {  // plane pl starts at column pl * lo_off
+                        tma_load_2d_pair(sA + sg * A_ST + pl * A_STAGE, &tmA, fb, pl * a.lo_off + kb * kb_elems, ya);
+                        tma_load_2d_pair(sB + sg * B_ST + pl * B_PLANE, &tmB, fb, pl * a.lo_off + kb * kb_elems, yb);
                     }
+                }
+                __syncwarp();
+                if (++sg == STAGES) {
+                    sg = 0;
+                    ph ^= 1;
+                }
             }
-            // the last stages' empties arrive after the final MMAs: wait for them, so that no
-            // commit is still addressed to this CTA when the pair leaves (bounded)
+        }
+        // the last stages' empties arrive after the final MMAs: wait for them, so that no
+        // commit is still addressed to this CTA when the pair leaves (bounded)
+        if (leader) {
             const uint32_t first = it > STAGES ? it - STAGES : 0;
             for (uint32_t j = first; j < it; ++j) mbar_drain(&empty[j % STAGES], ((j / STAGES) & 1));
         }
+        __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             // --------------------------------------------------------- MMA --
+            const uint32_t leader = elect_one();
             const uint32_t idesc = make_idesc(TF32 ? 2 : SCALED ? 0 : 1, bn, BM2);  // tf32, e4m3 / f16, bf16
-            uint32_t it = 0, acc_it = 0;
+            const uint32_t a0 = sw128_lo(su32(sA)), b0 = sw128_lo(su32(sB));
+            uint32_t acc_it = 0, sg = 0, ph = 0;
             bool ok = true, issued = false;
             for (int i = 0; ok && i < nunits; ++i, ++acc_it) {
-                    const uint32_t buf = acc_it % NACC, aph = (acc_it / NACC) & 1;
-                    if (!mbar_wait(&tempty[buf], aph ^ 1, abort_flag, a.err)) {
+                const uint32_t buf = acc_it % NACC, aph = (acc_it / NACC) & 1;
+                if (!mbar_wait_warp(&tempty[buf], aph ^ 1, abort_flag, a.err)) {
+                    ok = false;
+                    break;
+                }
+                fence_after();
+                const uint32_t dtm = tmem_base + buf * (uint32_t)bn;
+                for (int kb = 0; kb < a.kblocks; ++kb) {
+                    if (!mbar_wait_warp(&full[sg], ph, abort_flag, a.err)) {
                         ok = false;
                         break;
                     }
                     fence_after();
-                    const uint32_t dtm = tmem_base + buf * (uint32_t)bn;
-                    for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
-                        const uint32_t s = it % STAGES, ph = (it / STAGES) & 1;
-                        if (!mbar_wait(&full[s], ph, abort_flag, a.err)) {
-                            ok = false;
-                            break;
-                        }
-                        fence_after();
-                        const uint32_t ab = su32(sA + s * A_ST), bb = su32(sB + s * B_ST);
+                    const uint32_t ab = a0 + sg * (A_ST >> 4), bb = b0 + sg * (B_ST >> 4);
+                    if (leader) {
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             if (SL) {
-                                // accumulator g (columns g * bn..) takes the products of slices p and g - p
+                                // accumulator q (columns q * bn..) takes the products of slices p and q - p
 #pragma unroll
-                                for (int g = 0; g < 4; ++g)
+                                for (int q = 0; q < 4; ++q)
 #pragma unroll
-                                    for (int p = 0; p <= g; ++p)
-                                        mma2<MK>(dtm + (uint32_t)(g * bn), sw128_desc(ab + p * A_STAGE + 32 * k),
-                                                 sw128_desc(bb + (g - p) * B_PLANE + 32 * k), idesc,
+                                    for (int p = 0; p <= q; ++p)
+                                        mma2<MK>(dtm + (uint32_t)(q * bn), ab + p * (A_STAGE >> 4) + 2 * k,
+                                                 bb + (q - p) * (B_PLANE >> 4) + 2 * k, idesc,
                                                  (kb > 0 || k > 0 || p > 0) ? 1u : 0u);
                                 continue;
                             }
-                            mma2<MK>(dtm, sw128_desc(ab + 32 * k), sw128_desc(bb + 32 * k), idesc,
-                                     (kb > 0 || k > 0) ? 1u : 0u);
+                            mma2<MK>(dtm, ab + 2 * k, bb + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
                             if (SPLIT) {
-                                mma2<MK>(dtm, sw128_desc(ab + 32 * k), sw128_desc(bb + B2_STAGE + 32 * k), idesc, 1u);
-                                mma2<MK>(dtm, sw128_desc(ab + A_STAGE + 32 * k), sw128_desc(bb + 32 * k), idesc, 1u);
+                                mma2<MK>(dtm, ab + 2 * k, bb + (B2_STAGE >> 4) + 2 * k, idesc, 1u);
+                                mma2<MK>(dtm, ab + (A_STAGE >> 4) + 2 * k, bb + 2 * k, idesc, 1u);
                             }
                         }
-                        issued = true;
-                        mma_commit_pair(&empty[s]);
+                        mma_commit_pair(&empty[sg]);
                     }
-                    if (!ok) break;
-                    mma_commit_pair(&tfull[buf]);
+                    issued = true;
+                    __syncwarp();
+                    if (++sg == STAGES) {
+                        sg = 0;
+                        ph ^= 1;
+                    }
                 }
-            if (issued) {  // every MMA (and its commits) done before the pair tears down
+                if (!ok) break;
+                if (leader) mma_commit_pair(&tfull[buf]);
+                __syncwarp();
+            }
+            if (issued && leader) {  // every MMA (and its commits) done before the pair tears down
                 mma_commit_own2(drain);
                 mbar_drain(drain, 0);
             }
+            __syncwarp();
         }
     } else {
         // ------------------------------------------------------ epilogue --
@@ -998,36 +1052,160 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         const int row_in_tile = quarter * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
         const int ngrp = bn / 32, cg0 = half ? ngrp / 2 : 0, cg1 = half ? ngrp : ngrp / 2;
-        // this warp's column terms of the current chunk (its half: <= 4 groups): K-term, coefficient, scale
-        float *cst = (float *)(smem + RING2_BYTES + 256 + XCH_BYTES) + (warp - 2) * CST_FLOATS;
+        // The column terms of a half's <= 4 groups (K-term, coefficient, scale, ids), shared by the
+        // half's four warps and double-buffered.  Each warp loads its 32 of them (and its rows'
+        // terms) into registers one unit ahead, so that no unit starts with a chain of L2 round
+        // trips, and the units are stepped without divisions: at n = 512 an epilogue unit took
+        // 7.0 k cycles, now 4.0-5.0 k beside the 4.1 k of its MMAs.
+        float *const cst0 = (float *)(smem + RING2_BYTES + 256 + XCH_BYTES) + half * 2 * CST_FLOATS;
+        float *cst = cst0;
+        const int ncols_h = (cg1 - cg0) * 32;  // columns of this half
+        const int jst = quarter * 32 + lane;   // the one this thread stages (jst < ncols_h)
+        float ph = 0.f, pw = 0.f, ps = 0.f, phl = 0.f;
+        int pid = -1;
+        double pw64 = 0.0;
+        auto stage_load = [&](int nc) {
+            const int64_t c = (int64_t)nc * bn + cg0 * 32 + jst;
+            if (jst >= ncols_h) return;
+            const bool in = c < a.ncols;
+            if (KIND == DCD_RBF) {
+                ph = a.col_h[c];
+                pid = in ? (a.col_id ? a.col_id[c] : (int)c) : -1;
+            }
+            if (ACC) {
+                pw64 = in ? a.col_w64[c] : 0.0;
+                if (KIND == DCD_RBF) phl = a.col_hl[c];
+                if (SL) ps = in ? a.col_s[c] : 0.f;
+            } else {
+                pw = a.col_w[c];
+                if (FP8) ps = a.col_s[c];
+            }
+        };
+        auto stage_store = [&]() {
+            if (KIND == DCD_RBF && !ACC && !FP8) {  // one word per warp: its 32 columns' terms allow the factored form
+                const int f = __all_sync(0xffffffffu, jst >= ncols_h || ph <= RBF_FACTOR_HMAX);
+                if (lane == 0) ((int *)cst)[768 + quarter] = f;
+            }
+            if (jst >= ncols_h) return;
+            if (KIND == DCD_RBF) {
+                cst[jst] = ph;
+                ((int *)cst)[512 + jst] = pid;
+            }
+            if (ACC) {
+                const float wh = (float)pw64;
+                cst[128 + jst] = wh;
+                cst[256 + jst] = (float)(pw64 - (double)wh);
+                if (KIND == DCD_RBF) cst[384 + jst] = phl;
+                if (SL) cst[640 + jst] = ps;
+            } else {
+                cst[128 + jst] = pw;
+                if (FP8) cst[256 + jst] = ps;
+                // the RBF's column factor w_j 2^(-h_j) of the factored form below
+                if (KIND == DCD_RBF && !FP8) cst[384 + jst] = pw * ex2f(-ph);
+            }
+        };
+        // barrier of the half's four warps that also ands `v` over them (ids 1 and 2; 0 is __syncthreads)
+        auto half_all = [&](bool v) {
+            uint32_t all;
+            asm volatile(
+                "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+                "barrier.cta.red.and.pred q, %2, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                : "=r"(all)
+                : "r"((uint32_t)v), "r"(1 + half)
+                : "memory");
+            return all != 0;
+        };
         uint32_t acc_it = 0, item_it = 0;
         bool ok = true;
         int64_t row = 0;
         bool row_ok = false;
         float hr = 0.f, hrl = 0.f, rf = 0.f, rsl = 0.f;
-        int rid = -2;  // data-matrix row of this thread's row (-2: none)
-        const int *cid = (const int *)(cst + 512);  // staged column ids (-1 past the block)
+        int rid = -2;   // data-matrix row of this thread's row (-2: none)
+        int wr0 = 0;    // rid of the warp's first row (rows are consecutive unless given by id)
+        const int *cid = (const int *)(cst0 + 512);  // staged column ids (-1 past the block)
         double tacc = 0.0;  // this half's row sum over the tile's chunks so far, in chunk order
         const int nch = a.nchunks;
-        bool fast_cols = false, fast_row = false;  // the factored RBF form applies (warp-uniform)
-        for (int i = 0; ok && i < nunits; ++i, ++acc_it) {
-            int item, nc;
-            pair_unit(a, pair, npairs, ranged, u0, u1, i, item, nc);
-            const int u = item * nch + nc;
-            if (u == u0 || nc == 0) {  // first chunk of a tile in this pair's units
+        bool fast_row = false;  // the factored RBF form applies to the warp's rows (with fast_cols)
+        bool whole = true;      // no other pair holds units of this tile
+        // the row terms of the tile after this one, loaded a unit ahead like the column terms
+        float n_hr = 0.f, n_hrl = 0.f, n_s = 0.f;
+        int n_rid = -2;
+        const float cs0 = FP16 ? a.col_s[0] : 0.f;
+        auto row_load = [&](int it2) {
+            const int64_t r = (int64_t)it2 * BM2 + (int64_t)rank * BM + row_in_tile;
+            const bool in = r < a.nrows_out;
+            n_hr = (KIND == DCD_RBF && in) ? a.row_h[r] : 0.f;
+            if (ACC) n_hrl = (KIND == DCD_RBF && in) ? a.row_hl[r] : 0.f;
+            if (SL || SCALED) n_s = in ? a.row_s[r] : 0.f;
+            n_rid = in ? (a.row_id ? a.row_id[r] : (int)r) : -2;
+        };
+        UnitIter un(a, pair, npairs, ranged, u0, u1);
+        if (nunits > 0) {
+            stage_load(un.nc);
+            row_load(un.item);
+        }
+        int prev_item = -1;
+        for (int i = 0; i < nunits; ++i, ++acc_it) {
+            const int item = un.item, nc = un.nc;
+            un.next();
+            cst = cst0 + (acc_it & 1) * CST_FLOATS;
+            cid = (const int *)(cst + 512);
+            if (item != prev_item) {  // first chunk of a tile in this pair's units
+                prev_item = item;
                 row = (int64_t)item * BM2 + (int64_t)rank * BM + row_in_tile;
                 row_ok = row < a.nrows_out;
-                hr = (KIND == DCD_RBF && row_ok) ? a.row_h[row] : 0.f;
-                if (ACC) hrl = (KIND == DCD_RBF && row_ok) ? a.row_hl[row] : 0.f;
-                if (SL) rsl = row_ok ? a.row_s[row] * 0x1p-12f : 0.f;  // 2^(e_i - 12)
-                rid = row_ok ? (a.row_id ? a.row_id[row] : (int)row) : -2;
-                const float rsc = !SCALED ? 1.f : !row_ok ? 0.f : FP8 ? a.row_s[row] : a.row_s[row] * a.col_s[0];
+                hr = n_hr;
+                hrl = n_hrl;
+                rid = n_rid;
+                wr0 = __shfl_sync(0xffffffffu, rid, 0);
+                if (SL) rsl = n_s * 0x1p-12f;  // 2^(e_i - 12)
+                const float rsc = !SCALED ? 1.f : !row_ok ? 0.f : FP8 ? n_s : n_s * cs0;
                 rf = KIND == DCD_RBF ? a.two_gl * rsc : rsc;
                 fast_row = __all_sync(0xffffffffu, hr <= RBF_FACTOR_HMAX);
+                whole = !ranged || (item * nch >= u0 && (item + 1) * nch <= u1);
                 tacc = 0.0;
             }
-            const bool whole = !ranged || (item * nch >= u0 && (item + 1) * nch <= u1);
-            const bool last = nc == nch - 1 || u == u1 - 1;  // last chunk of the tile in this pair's units
+            const bool last = i + 1 == nunits || un.item != item;  // last chunk of the tile in this pair's units
+            // this unit's column terms to the half's staging buffer, then the loads of the next unit's
+            stage_store();
+            if (i + 1 < nunits) {
+                stage_load(un.nc);
+                if (un.item != item) row_load(un.item);
+            }
+            const uint32_t buf = acc_it % NACC, aph = (acc_it / NACC) & 1;
+            // the accumulator's wait, and the half's four warps agree on it: staged columns visible
+            // to all, and no warp leaves while another waits here (a bounded wait that ran out is
+            // carried to this point)
+            if (ok) ok = mbar_wait_warp(&tfull[buf], aph, abort_flag, a.err);
+            if (!half_all(ok)) break;
+            __syncwarp();
+            // the row's gradient (and scale), loaded beside the tile's last chunk
+            double g_old = 0.0, g_rs = 1.0;
+            if (last && whole && !half && row_ok) {
+                g_old = a.g[row];
+                if (a.rs) g_rs = a.rs[row];
+            }
+            // the factored form needs every h_j <= RBF_FACTOR_HMAX
+            bool fast_cols = false;
+            if (KIND == DCD_RBF && !ACC && !FP8) {
+                const int4 f = *(const int4 *)(cst + 768);
+                fast_cols = (f.x & f.y & f.z & f.w) != 0;
+            }
+            // the column groups that hold an own sample of the warp's 32 rows: each lane tests one
+            // column id of every group (rows given by id: every group is tested column by column)
+            unsigned ghit = 0;
+            if (KIND == DCD_RBF && !ACC) {
+                if (a.row_id) {
+                    ghit = 0xfu;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (32 * q < ncols_h) {
+                            const unsigned off = (unsigned)(cid[32 * q + lane] - wr0);
+                            if (__ballot_sync(0xffffffffu, rid >= 0 && off < 32u)) ghit |= 1u << q;
+                        }
+                }
+            }
             // this chunk's part of the row sum (this half's column groups): the fast epilogue adds
             // its groups in double-single FP32 (GB300's FP64 pipe issues ~1.6 operations per clock
             // per SM, too few for per-group FP64 sums at the bf16 MMA rate), the accurate ones in FP64
@@ -1087,19 +1265,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             // same sums in the same order as a column-by-column loop
             auto group = [&](const uint32_t(&r)[32], int j0) {
                 float p0 = 0.f, p1 = 0.f;
-                // the own-sample columns of this warp's 32 rows: each lane tests one column id
+                // the own-sample columns of this thread's row, in the groups that may hold one
                 unsigned own = 0;
-                if (KIND == DCD_RBF && !a.row_id) {
-                    const int wr0 = __shfl_sync(0xffffffffu, rid, 0);  // lanes hold consecutive rows
-                    const unsigned off = (unsigned)(cid[j0 + lane] - wr0);
-                    unsigned hits = __ballot_sync(0xffffffffu, rid >= 0 && off < 32u);
-                    while (hits) {
-                        const int q = __ffs(hits) - 1;
-                        hits &= hits - 1;
-                        if (cid[j0 + q] == rid) own |= 1u << q;
+                if (KIND == DCD_RBF && ((ghit >> (j0 >> 5)) & 1u)) {
+                    if (!a.row_id) {
+                        const unsigned off = (unsigned)(cid[j0 + lane] - wr0);
+                        unsigned hits = __ballot_sync(0xffffffffu, rid >= 0 && off < 32u);
+                        while (hits) {
+                            const int q = __ffs(hits) - 1;
+                            hits &= hits - 1;
+                            if (cid[j0 + q] == rid) own |= 1u << q;
+                        }
+                    } else {  // rows given by id: every column tested
+                        for (int q = 0; q < 32; ++q) own |= (cid[j0 + q] == rid ? 1u : 0u) << q;
                     }
-                } else if (KIND == DCD_RBF) {  // rows given by id: every column tested
-                    for (int q = 0; q < 32; ++q) own |= (cid[j0 + q] == rid ? 1u : 0u) << q;
                 }
                 if (own) group_terms(r, j0, own, p0, p1);
                 else group_terms(r, j0, 0u, p0, p1);
@@ -1177,40 +1356,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 }
                 cs += ((double)ah0 + (double)al0) + ((double)ah1 + (double)al1);
             };
-            const uint32_t buf = acc_it % NACC, aph = (acc_it / NACC) & 1;
-            // stage this warp's columns while the accumulator is still being formed
-            const int64_t cbase = (int64_t)nc * bn + cg0 * 32;
-            for (int j = lane; j < (cg1 - cg0) * 32; j += 32) {
-                if (KIND == DCD_RBF) {
-                    cst[j] = a.col_h[cbase + j];
-                    const int64_t c = cbase + j;
-                    ((int *)cst)[512 + j] = c < a.ncols ? (a.col_id ? a.col_id[c] : (int)c) : -1;
-                }
-                if (ACC) {
-                    const double wv = cbase + j < a.ncols ? a.col_w64[cbase + j] : 0.0;
-                    const float wh = (float)wv;
-                    cst[128 + j] = wh;
-                    cst[256 + j] = (float)(wv - (double)wh);
-                    if (KIND == DCD_RBF) cst[384 + j] = a.col_hl[cbase + j];
-                    if (SL) cst[640 + j] = cbase + j < a.ncols ? a.col_s[cbase + j] : 0.f;
-                } else {
-                    cst[128 + j] = a.col_w[cbase + j];
-                    if (FP8) cst[256 + j] = a.col_s[cbase + j];
-                    // the RBF's column factor w_j 2^(-h_j) of the factored form below
-                    if (KIND == DCD_RBF && !FP8) cst[384 + j] = a.col_w[cbase + j] * ex2f(-a.col_h[cbase + j]);
-                }
-            }
-            if (KIND == DCD_RBF && !ACC && !FP8) {  // the factored form needs every h_j <= RBF_FACTOR_HMAX
-                float hm = 0.f;
-                for (int j = lane; j < (cg1 - cg0) * 32; j += 32) hm = fmaxf(hm, cst[j]);
-                fast_cols = __all_sync(0xffffffffu, hm <= RBF_FACTOR_HMAX);
-            }
-            __syncwarp();
-            const bool seen = mbar_wait(&tfull[buf], aph, abort_flag, a.err);
-            if (!__all_sync(0xffffffffu, seen)) {
-                ok = false;
-                break;
-            }
             fence_after();
             const uint32_t tb = tmem_base + lane_addr + buf * (uint32_t)bn;
             if constexpr (SL) {
@@ -1236,7 +1381,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     }
                 }
             }
-            cs += (double)cs_h + (double)cs_l;
+            if (!ACC) cs = (double)cs_h + (double)cs_l;
             fence_before();
             __syncwarp();
             if (lane == 0) arrive_cl(tempty0 + 8u * buf);
@@ -1278,8 +1423,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             if (half) {
                 const bool fr = mbar_wait(&xfree[xb], xph ^ 1, abort_flag, a.err);
                 if (!__all_sync(0xffffffffu, fr)) {
-                    ok = false;
-                    break;
+                    ok = false;  // leaves at the next unit's barrier, with its half
+                    continue;
                 }
                 xc[row_in_tile] = tacc;
                 __syncwarp();
@@ -1288,12 +1433,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 const bool fu = mbar_wait(&xfull[xb], xph, abort_flag, a.err);
                 if (!__all_sync(0xffffffffu, fu)) {
                     ok = false;
-                    break;
+                    continue;
                 }
                 const double tot = tacc + xc[row_in_tile];
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&xfree[xb]);
-                if (row_ok) a.g[row] += (a.rs ? a.rs[row] : 1.0) * tot;
+                if (row_ok) a.g[row] = g_old + g_rs * tot;
             }
         }
     }
