@@ -102,6 +102,34 @@ cudaError_t launch_block_simt_f64(const double *A, int64_t lda, int64_t m, int64
                                   int *err, cudaStream_t st, const double *B = nullptr, int64_t ldb = 0,
                                   int64_t mb = 0);
 
+// The FP64 form's kernel block from exact slice products on the tensor cores (block_f64.cu).
+constexpr int64_t F64S_N_MAX = 512;     // exact slice-product sums up to this many features
+constexpr double F64S_HMAX = 8.0;       // RBF: largest gamma |a|^2 the expansion is used for
+struct F64Sliced {
+    const void *packed = nullptr;       // m rows of f64s_row_bytes(n): eight bf16 planes
+    const int32_t *ex = nullptr;        // per row: exponent
+    const double *h = nullptr;          // per row: gamma |a|^2 (RBF)
+    int64_t m = 0, n = 0;
+    double *part = nullptr;             // apply: f64s_part_bytes(m, ncols)
+    unsigned *cnt = nullptr;            // apply: f64s_tiles(m) counters, zero before the first launch (left at zero)
+};
+int64_t f64s_row_bytes(int64_t n);
+size_t f64s_part_bytes(int64_t m, int64_t ncols);
+int64_t f64s_tiles(int64_t m);
+// stat: two words (zeroed here): whether a value rules the form out, and the largest gamma |a|^2
+cudaError_t launch_pack_f64s(const double *A, int64_t lda, int64_t m, int64_t n, const KernelParams &kp, void *packed,
+                             int32_t *ex, double *h, unsigned long long *stat, cudaStream_t st);
+// rows, cols: packed rows (all of f.packed, or gathered ones with the data rows they hold in
+// row_id / col_id).  apply (out == nullptr): g[i] += rs[i] * sum_c K(i, c) w[c], over rows 0..nrows-1
+// of f; store: out[r*ldo + c] = K(r, c).
+cudaError_t launch_block_f64s(const F64Sliced &f, const void *rows, int64_t nrows, const int32_t *row_id,
+                              const void *cols, int64_t ncols, const int32_t *col_id, const KernelParams &kp,
+                              const double *w, const double *rs, double *g, double *out, int64_t ldo, int *err,
+                              cudaStream_t st);
+// 2-D tensor map over a row-major bf16 matrix of nrows x cols elements, box of box_rows x 64,
+// 128-byte swizzle, out-of-range rows read as zero (block_tc.cu)
+bool make_map_bf16_2d(CUtensorMap *map, const void *base, int64_t cols, int64_t nrows, int box_rows);
+
 // tcgen05 kernel block over the packed, padded operand copy (bf16 or fp32
 // rows of n_pad elements, zero padded).
 // Packed operand modes (also the pack kernel's dst_kind):

@@ -253,6 +253,11 @@ struct Solver {
     // the accurate epilogue of the recomputed gradient: low parts of the RBF terms, and the
     // gathered columns' power-of-two scales of the sliced operand
     float *row_hlr = nullptr, *col_hlr = nullptr, *col_sr = nullptr;
+    // FP64 form of a dense matrix on the tensor cores (exact slice products): the sliced rows,
+    // the gathered sampled rows in sbuf[].As
+    bool f64s = false;
+    F64Sliced fs;
+    void *ws_f64s = nullptr;
     // CSR data matrix: the CUDA-core SpMM block (FP32, or FP64 in the FP64 mode)
     bool csr = false;
     CsrOperand ca;
@@ -317,6 +322,7 @@ struct Solver {
         if (csr_join) cudaEventDestroy(csr_join);
         if (ws_csc) cudaFreeAsync(ws_csc, st);
         if (ws_cstep) cudaFreeAsync(ws_cstep, st);
+        if (ws_f64s) cudaFreeAsync(ws_f64s, st);
         if (ws) cudaFreeAsync(ws, st);
     }
 
@@ -750,6 +756,10 @@ struct Solver {
             op.a64 = (const double *)vals;
             op.lda = A->ld;
         }
+        if (!csr && !tc && !literal) {
+            const dcd_status fst = setup_f64s(set3 ? 3 : set2 ? 2 : 1);
+            if (fst != DCD_OK) return fst;
+        }
 
         // labels
         if (problem == 0) {
@@ -777,6 +787,68 @@ struct Solver {
                 dcd_status s2 = full_pass();
                 if (s2 != DCD_OK) return s2;
             }
+        }
+        return DCD_OK;
+    }
+
+    // The FP64 form's block through exact slices (block_f64.cu) where it is the faster one and as
+    // exact: n within the exact sums, every value finite with a moderate exponent, and for the RBF
+    // gamma |a|^2 <= F64S_HMAX (the expansion's error).  The line is on the products m sb n of the
+    // block, by measured time of sample + Gram + block a step (direct / slices, us): blocks of at
+    // most 32 columns, whose direct form is spread over every SM, 2000 x 64 x 16 (2.0 M) 36 / 56,
+    // 6000 x 64 x 8 (3.1 M) 39 / 44, 2000 x 200 x 8 (3.2 M) 58 / 53, 6000 x 200 x 8 (9.6 M)
+    // 74 / 52, 6000 x 512 x 32 511 / 93: from 6 M; wider ones, in tiles of 64 rows, 2000 x 64 x 64
+    // (8.2 M) 351 / 71, 6000 x 512 x 256 9510 / 148: from 1 M.  No memory for the slices (16 bytes
+    // a value): the direct form.
+    dcd_status setup_f64s(int sets)
+    {
+        const double work = (double)m * (double)sb * (double)n;
+        if (n > F64S_N_MAX || work < (sb > 32 ? 1e6 : 6e6) || !tc_available()) return DCD_OK;
+        const size_t rb = (size_t)f64s_row_bytes(n);
+        Arena ar;
+        for (int pass = 0; pass < 2; ++pass) {
+            ar.used = 0;
+            void *pk = ar.take((size_t)m * rb, 1024);
+            void *rows[3];
+            for (int q = 0; q < 3; ++q) rows[q] = ar.take(q < sets ? (size_t)sb * rb : 0, 1024);
+            int32_t *ex = (int32_t *)ar.take(sizeof(int32_t) * m);
+            double *h = (double *)ar.take(sizeof(double) * m);
+            double *part = (double *)ar.take(f64s_part_bytes(m, sb));
+            unsigned *cnt = (unsigned *)ar.take(sizeof(unsigned) * f64s_tiles(m));
+            unsigned long long *stat = (unsigned long long *)ar.take(2 * sizeof(unsigned long long));
+            if (pass == 0) {
+                const cudaError_t e = malloc_async(&ws_f64s, ar.used + 1024, st);
+                if (e == cudaErrorMemoryAllocation) {
+                    cudaGetLastError();
+                    ws_f64s = nullptr;
+                    return DCD_OK;
+                }
+                if (e != cudaSuccess) return cuda_status(e);
+                ar.base = (char *)ws_f64s;
+                continue;
+            }
+            DCD_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned) * f64s_tiles(m), st));
+            DCD_TRY(launch_pack_f64s(op.a64, op.lda, m, n, kp, pk, ex, h, stat, st));
+            unsigned long long hs[2] = {1, 0};
+            DCD_TRY(cudaMemcpyAsync(hs, stat, sizeof(hs), cudaMemcpyDeviceToHost, st));
+            DCD_TRY(cudaStreamSynchronize(st));
+            double hmax;
+            memcpy(&hmax, &hs[1], sizeof(hmax));
+            if (hs[0] || !(hmax <= F64S_HMAX)) {
+                DCD_TRY(cudaFreeAsync(ws_f64s, st));
+                ws_f64s = nullptr;
+                return DCD_OK;
+            }
+            fs.packed = pk;
+            fs.ex = ex;
+            fs.h = h;
+            fs.m = m;
+            fs.n = n;
+            fs.part = part;
+            fs.cnt = cnt;
+            for (int q = 0; q < 3; ++q) sbuf[q].As = rows[q];
+            As = sbuf[0].As;
+            f64s = true;
         }
         return DCD_OK;
     }
@@ -856,6 +928,7 @@ struct Solver {
     cudaError_t gather(int64_t ncols)
     {
         if (csr) return launch_csr_colmap(ca, S, ncols, cm, err, st);
+        if (f64s) return launch_gather_rows(fs.packed, f64s_row_bytes(n), S, ncols, m, As, err, st);
         return gather_op(ncols, op, As, col_h);
     }
     cudaError_t gather_op(int64_t ncols, const Operand &x, void *Asx, float *chx)
@@ -878,8 +951,19 @@ struct Solver {
             return launch_block_tc(B, B, kp, col_h, col_h, nullptr, nullptr, nullptr, (float *)Kss, ldk, ncols, ncols,
                                    err, st, lower);
         }
+        if (f64s)
+            return launch_block_f64s(fs, As, ncols, S, As, ncols, S, kp, nullptr, nullptr, nullptr, (double *)Kss, ldk,
+                                     err, st);
         return launch_block_simt_f64(op.a64, op.lda, m, n, kp, S, ncols, S, ncols, nullptr, nullptr, nullptr,
                                      (double *)Kss, ldk, err, st);
+    }
+
+    // the FP64 form's block and gradient update of a step whose rows are gathered
+    cudaError_t block_f64_apply(int64_t ncols, const double *rs)
+    {
+        if (f64s)
+            return launch_block_f64s(fs, fs.packed, m, nullptr, As, ncols, S, kp, w64, rs, g, nullptr, 0, err, st);
+        return launch_block_simt_f64(op.a64, op.lda, m, n, kp, nullptr, m, S, ncols, w64, rs, g, nullptr, 0, err, st);
     }
 
     // g += rs * K(A, A_S) w64 with the step operand, or (ref) with the
@@ -925,8 +1009,8 @@ struct Solver {
             return cuda_status(
                 launch_block_tc(Aop, Bop, kp, x.row_h, chx, col_w, rs, g, nullptr, 0, m, ncols, err, st, false, &tsplit));
         }
-        return cuda_status(launch_block_simt_f64(op.a64, op.lda, m, n, kp, nullptr, m, S, ncols, w64, rs, g, nullptr,
-                                                 0, err, st));
+        if (f64s) DCD_TRY(gather(ncols));
+        return cuda_status(block_f64_apply(ncols, rs));
     }
 
     // Columns past ncols of the FP32 coefficient buffer must be zero: the
@@ -1464,6 +1548,9 @@ struct Solver {
             return launch_block_tc(Ro, Co, kp, R.col_h, Cq.col_h, nullptr, nullptr, nullptr, (float *)dfs_kx, cnt, cnt,
                                    cnt, err, s2);
         }
+        if (f64s)
+            return launch_block_f64s(fs, sbuf[q2].As, cnt, sbuf[q2].S, sbuf[q].As, cnt, sbuf[q].S, kp, nullptr, nullptr,
+                                     nullptr, (double *)dfs_kx, cnt, err, s2);
         return launch_block_simt_f64(op.a64, op.lda, m, n, kp, sbuf[q2].S, cnt, sbuf[q].S, cnt, nullptr, nullptr,
                                      nullptr, (double *)dfs_kx, cnt, err, s2);
     }
@@ -1523,8 +1610,7 @@ struct Solver {
         else if (tc)
             DCD_TRY(block_tc_apply(ncols, rs));  // (every set's coefficients past sb stay zero)
         else
-            DCD_TRY(launch_block_simt_f64(op.a64, op.lda, m, n, kp, nullptr, m, S, ncols, w64, rs, g, nullptr, 0,
-                                          err, st));
+            DCD_TRY(block_f64_apply(ncols, rs));
         DCD_TRY(launch_update(S, delta, ncols, diag, alpha, g, ctr, (uint64_t)cnt, m, err, st));
         if (has2) DCD_TRY(cudaStreamWaitEvent(st, la_join, 0));
         if (has1) DCD_TRY(cudaStreamWaitEvent(st, df_side, 0));
@@ -1607,7 +1693,7 @@ struct Solver {
         const int64_t ncols = cnt * o.b;
         cudaError_t e =
             launch_sample(problem, o.seed, ctr_la + q, 0, m, o.b, cnt, S, err, st, ctr_la + (qnext < 0 ? 1 - q : qnext));
-        const bool rows_gathered = tc && !csr;  // the cross product reads the gathered rows
+        const bool rows_gathered = (tc && !csr) || f64s;  // the cross product reads the gathered rows
         if (e == cudaSuccess && sampled && !rows_gathered) e = cudaEventRecord(sampled, st);
         if (e == cudaSuccess) e = gather(ncols);
         if (e == cudaSuccess && sampled && rows_gathered) e = cudaEventRecord(sampled, st);
@@ -1658,8 +1744,7 @@ struct Solver {
         else if (tc)
             DCD_TRY(block_tc_apply(ncols, rs));
         else
-            DCD_TRY(launch_block_simt_f64(op.a64, op.lda, m, n, kp, nullptr, m, S, ncols, w64, rs, g, nullptr, 0,
-                                          err, st));
+            DCD_TRY(block_f64_apply(ncols, rs));
         if (!fu.done) DCD_TRY(launch_update(S, delta, ncols, diag, alpha, g, ctr, (uint64_t)cnt, m, err, st));
         if (next) DCD_TRY(cudaStreamWaitEvent(st, la_join, 0));
         return DCD_OK;
@@ -1869,8 +1954,7 @@ struct Solver {
         else if (tc)
             DCD_TRY(block_tc_apply(ncols, rs));
         else
-            DCD_TRY(launch_block_simt_f64(op.a64, op.lda, m, n, kp, nullptr, m, S, ncols, w64, rs, g, nullptr, 0, err,
-                                          st));
+            DCD_TRY(block_f64_apply(ncols, rs));
         tm.stop(stats.ms_block);
         tm.start();
         if (!fu.done) DCD_TRY(launch_update(S, delta, ncols, diag, alpha, g, ctr, (uint64_t)cnt, m, err, st));
