@@ -783,120 +783,174 @@ cudaError_t refined_bdcd_b(const KT *Kss, int64_t ldk, const int32_t *S, int nbl
 
 }  // namespace
 
-// The same chain for cnt <= DCD_FAST_MAX with its state in registers: the
-// whole CTA first forms the coupling coefficients C[j][t] = y_t y_j K_tj
-// (+ omega when S_t = S_j, the repeat term of the unrolled update) in shared
-// memory; then one warp runs the chain with lane l holding, for t = l, l+32,
-// ..., alpha_t, g_t, 1/eta_t and the pending corrections of g_t and rho_t in
-// registers (the gradient correction starts at g_t, so the step's gradient
-// is read, not formed).  A step is the owner lane's clipped Newton step
-// (Algorithm 2, the arithmetic of recur_dcd_kernel), a broadcast, and one FMA
-// per later coordinate.  GB300's FP64 compare-and-select costs ~110 cycles
-// of latency against 25 for min/max and 65 for add/FMA (measured), so the
-// zero tests on the chain are integer tests of the bit patterns.
+// The same chain for cnt <= DCD_FAST_MAX with its state in registers.  The whole CTA forms the
+// coupling coefficients C[j][t] = y_t y_j K_tj (+ omega when S_t = S_j, the repeat term of the
+// unrolled update; zero for t <= j) in shared memory, y's signs by integer operations; then warp k
+// runs the coordinates 32 k .. 32 k + 31 with lane l holding alpha_t, g_t and 1/eta_t of t = 32 k + l
+// in registers.
+//
+// What bounds it is the latency of dependent FP64 instructions in one warp (about 64 cycles each,
+// and some 80 of throughput per scheduler), so a round is cut to four: every lane forms its
+// coordinate's candidate step (Algorithm 2, the arithmetic of recur_dcd_kernel: rho - g and
+// rho - g / eta, clipped by integer comparisons of the bit patterns, less rho), a ballot finds the
+// next coordinate whose step is not zero -- those before it take a zero step, which changes
+// nothing -- and one FMA moves its step into every later gradient.  A round is one nonzero step, so
+// coordinates at a bound cost nothing.  The later groups' warps, each on its own scheduler, apply
+// the steps as they are published (shared memory, release / acquire) and take over when the groups
+// before them are done.  One warp in lockstep over all coordinates took 1.2 k cycles per
+// coordinate.  Measured per step: s = 64 (split bf16, m = 2000, n = 64) 38 -> 10.7 us over a whole
+// solve; s = 8 (FP64) 7.6 -> 2.7; s = 32 on CSR data from alpha = 0, every step nonzero, 26 -> 18.
 constexpr int DCD_FAST_MAX = 128;
 constexpr int DCD_FAST_K = DCD_FAST_MAX / 32;
 
-template <typename KT>
+__device__ __forceinline__ int ld_acquire_shared(const int *p)
+{
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(ptx::su32(p)) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_release_shared(int *p, int v)
+{
+    asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(ptx::su32(p)), "r"(v) : "memory");
+}
+
+// clip(x, 0, nu) by the bit patterns (nub: those of nu, +infinity for no upper bound); a NaN gives 0,
+// as fmin(fmax(x, 0), nu) does
+__device__ __forceinline__ double clip_bits(double x, long long nub)
+{
+    const long long b = __double_as_longlong(x);
+    if (b <= 0 || b > 0x7ff0000000000000LL) return 0.0;
+    return __longlong_as_double(b > nub ? nub : b);
+}
+
 // pend (optional): alpha and g at the step's coordinates are pend[0][t] + pend[1][t] and
 // pend[2][t] + pend[3][t] (a snapshot and the parts not yet in it) instead of alpha[S[t]], g[S[t]]
+template <typename KT>
 __global__ void __launch_bounds__(DCD_THREADS) recur_dcd_fast_kernel(const KT *Kss, int64_t ldk, const int32_t *S,
                                                                      int cnt, const double *y, const double *alpha,
                                                                      const double *g, double omega, double nu,
                                                                      double *delta, double *w64, float *w32,
-                                                                     DcdPending pend)
+                                                                     DcdPending pend, int *err)
 {
     extern __shared__ double fsm[];
-    double *C = fsm;                                   // C[j * cnt + t]
-    double *yS = C + (size_t)cnt * cnt;
-    int32_t *sI = (int32_t *)(yS + cnt);
-    for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+    const int ldc = cnt | 1;                            // odd: no bank conflicts down a column
+    double *C = fsm;                                    // C[j * ldc + t]
+    double *list_t = C + (size_t)cnt * ldc;             // the nonzero steps so far, and their coordinates
+    int *list_j = (int *)(list_t + cnt);
+    int32_t *sI = list_j + cnt;
+    uint32_t *sy = (uint32_t *)(sI + cnt);              // sign bit of y
+    uint32_t *rep = sy + cnt;                           // rep[j * 4 + q]: later t = 32 q + bit with S_t = S_j
+    int *pub = (int *)(rep + DCD_FAST_K * cnt);         // steps published, groups done
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int t = threadIdx.x;  // warps 0..3: this thread's coordinate, if t < cnt
+    const bool mine = t < cnt;
+    double a0 = 0.0, a1 = 0.0, g0 = 0.0, g1 = 0.0;
+    if (mine) {
         const int32_t i = S[t];
         sI[t] = i;
-        yS[t] = y[i];
+        sy[t] = (uint32_t)__double2hiint(y[i]) & 0x80000000u;
+        if (pend.alpha_snap) {
+            a0 = pend.alpha_snap[t];
+            a1 = pend.alpha_add[t];
+            g0 = pend.g_snap[t];
+            g1 = pend.g_add[t];
+        } else {
+            a0 = alpha[i];
+            g0 = g[i];
+        }
+    }
+    if (threadIdx.x == 0) pub[0] = pub[1] = 0;
+    __syncthreads();
+    double ie = 0.0;
+    if (mine) {
+        const double eta = kval(Kss, ldk, t, t) + omega;  // G_k = V^T U_k + omega I, y_t^2 = 1
+        ie = eta > 0.0 ? 1.0 / eta : 0.0;
+    }
+    // C and the repeat masks, a warp per row t (lanes: columns j)
+    for (int r = warp; r < cnt; r += DCD_THREADS / 32) {
+        const int32_t ir = sI[r];
+        const uint32_t yr = sy[r];
+        for (int q = 0; 32 * q < cnt; ++q) {
+            const int j = 32 * q + lane;
+            const bool in = j < cnt;
+            const bool same = in && sI[in ? j : 0] == ir;
+            if (in) {
+                double v = 0.0;
+                if (r > j) {
+                    v = kval(Kss, ldk, r, j);
+                    v = __hiloint2double((int)((uint32_t)__double2hiint(v) ^ yr ^ sy[j]), __double2loint(v));
+                    if (same) v += omega;
+                }
+                C[j * ldc + r] = v;
+            }
+            const uint32_t mask = __ballot_sync(0xffffffffu, same && j > r);  // positions after r with r's index
+            if (lane == 0) rep[r * DCD_FAST_K + q] = mask;
+        }
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    double a[DCD_FAST_K], gg[DCD_FAST_K], ie[DCD_FAST_K], corr[DCD_FAST_K], rc[DCD_FAST_K], th[DCD_FAST_K];
-    auto nonzero = [](double x) { return (__double_as_longlong(x) << 1) != 0; };  // x != 0 (+-0 are zero)
-    int32_t id[DCD_FAST_K];
-    if (threadIdx.x < 32) {  // the chain warp's state (loads in flight while C is formed)
-#pragma unroll
-        for (int k = 0; k < DCD_FAST_K; ++k) {
-            const int t = 32 * k + lane;
-            const bool v = t < cnt;
-            const int32_t i = v ? sI[t] : -1;
-            id[k] = i;
-            if (pend.alpha_snap) {
-                a[k] = v ? pend.alpha_snap[t] + pend.alpha_add[t] : 0.0;
-                gg[k] = v ? pend.g_snap[t] + pend.g_add[t] : 0.0;
-            } else {
-                a[k] = v ? alpha[i] : 0.0;
-                gg[k] = v ? g[i] : 0.0;
-            }
-            const double eta = v ? kval(Kss, ldk, t, t) + omega : 0.0;  // G_k = V^T U_k + omega I, y_t^2 = 1
-            ie[k] = eta > 0.0 ? 1.0 / eta : 0.0;
-            corr[k] = gg[k];  // the gradient of coordinate t as the corrections arrive
-            rc[k] = 0.0;
-            th[k] = 0.0;
-        }
+    if (32 * warp >= cnt) return;
+    double rho = a0, gj = g0;  // alpha_t (and the steps of earlier repeats), the gradient as corrections arrive
+    if (pend.alpha_snap) {
+        rho += a1;
+        gj += g1;
     }
-    for (int e = threadIdx.x; e < cnt * cnt; e += blockDim.x) {
-        const int j = e / cnt, t = e - j * cnt;
-        C[e] = yS[t] * yS[j] * kval(Kss, ldk, t, j) + (sI[t] == sI[j] ? omega : 0.0);
-    }
-    __syncthreads();
-    if (threadIdx.x >= 32) return;
-    double rh[DCD_FAST_K];  // rho_t = alpha_t plus the steps of earlier repeats of its index
-#pragma unroll
-    for (int k = 0; k < DCD_FAST_K; ++k) rh[k] = a[k] + rc[k];
-    const bool clipnu = nu <= 1.7976931348623157e308;  // L1: the box's upper bound; L2: none
-#pragma unroll
-    for (int k = 0; k < DCD_FAST_K; ++k) {
-        if (32 * k >= cnt) break;
-        for (int jj = 0; jj < 32 && 32 * k + jj < cnt; ++jj) {
-            const int j = 32 * k + jj;
-            // every lane forms its coordinate's candidate step (convergent code: GB300's FP64 pipe
-            // charges a warp instruction the same with one lane or 32); lane jj's is the step
-            double t_j;
-            {
-                const double rho = rh[k], gj = corr[k];
-                double c1 = fmax(rho - gj, 0.0), c2 = fmax(rho - gj * ie[k], 0.0);
-                if (clipnu) {
-                    c1 = fmin(c1, nu);
-                    c2 = fmin(c2, nu);
-                }
-                // the projected gradient clip(rho - g) - rho is nonzero iff the clip moved rho
-                const long long b1 = __double_as_longlong(c1), b0 = __double_as_longlong(rho);
-                const bool moved = b1 != b0 && ((b1 | b0) << 1) != 0;  // +0 and -0 are the same value
-                t_j = moved && nonzero(ie[k]) ? c2 - rho : 0.0;
-                if (lane == jj) th[k] = t_j;
-            }
-            t_j = __shfl_sync(0xffffffffu, t_j, jj);
-            if (nonzero(t_j)) {
-                const int32_t ij = __shfl_sync(0xffffffffu, id[k], jj);
-                const double *Cj = C + (size_t)j * cnt;
-#pragma unroll
-                for (int kk = k; kk < DCD_FAST_K; ++kk) {
-                    if (32 * kk >= cnt) break;  // warp-uniform
-                    const int t = 32 * kk + lane;
-                    const bool later = t > j && t < cnt;
-                    corr[kk] = fma(later ? Cj[t] : 0.0, t_j, corr[kk]);
-                    const bool rep = later && id[kk] == ij;
-                    if (__any_sync(0xffffffffu, rep) && rep) rh[kk] += t_j;  // repeats are rare
-                }
+    const int tc = mine ? t : cnt - 1;  // a valid column for lanes past the end
+    auto apply = [&](int j, double tj) {
+        gj = fma(C[j * ldc + tc], tj, gj);
+        const uint32_t m = rep[j * DCD_FAST_K + warp];
+        if (m) rho += (m >> lane) & 1u ? tj : 0.0;  // repeats are rare (warp-uniform)
+    };
+    int n = 0;  // published steps applied (or, in the chain below, published)
+    if (warp > 0) {
+        const long long t0 = clock64();
+        for (;;) {
+            const int dn = ld_acquire_shared(pub + 1);
+            const int np = ld_acquire_shared(pub);
+            for (; n < np; ++n) apply(list_j[n], list_t[n]);
+            if (dn >= warp) break;
+            if (clock64() - t0 > 4200000000LL) {  // about 2 s
+                set_error(err, DEV_TIMEOUT);
+                break;
             }
         }
+        __syncwarp();
     }
-#pragma unroll
-    for (int k = 0; k < DCD_FAST_K; ++k) {
-        const int t = 32 * k + lane;
-        if (t < cnt) {
-            delta[t] = th[k];
-            const double wv = yS[t] * th[k];
-            if (w64) w64[t] = wv;
-            if (w32) w32[t] = (float)wv;
+    const bool more = 32 * (warp + 1) < cnt;
+    const long long nub = __double_as_longlong(nu);
+    double th = 0.0;
+    uint32_t left = __ballot_sync(0xffffffffu, mine);  // coordinates not yet decided
+    const bool solvable = (__double_as_longlong(ie) << 1) != 0;
+    for (;;) {
+        const double c1 = clip_bits(rho - gj, nub), c2 = clip_bits(fma(-gj, ie, rho), nub);
+        // the projected gradient clip(rho - g) - rho is nonzero iff the clip moved rho
+        const long long b1 = __double_as_longlong(c1), b0 = __double_as_longlong(rho);
+        const bool moved = b1 != b0 && ((b1 | b0) << 1) != 0;  // +0 and -0 are the same value
+        const double st = moved && solvable ? c2 - rho : 0.0;
+        const uint32_t nz = __ballot_sync(0xffffffffu, (__double_as_longlong(st) << 1) != 0) & left;
+        if (!nz) break;
+        const int l = __ffs(nz) - 1, j = 32 * warp + l;
+        const double tj = __shfl_sync(0xffffffffu, st, l);
+        if (lane == l) {
+            th = tj;
+            if (more) {
+                list_j[n] = j;
+                list_t[n] = tj;
+                st_release_shared(pub, n + 1);
+            }
         }
+        ++n;
+        left &= ~((2u << l) - 1u);
+        apply(j, tj);
+    }
+    __syncwarp();
+    if (more && lane == 0) st_release_shared(pub + 1, warp + 1);
+    if (mine) {
+        delta[t] = th;
+        // y_t th
+        const double wv = __hiloint2double((int)((uint32_t)__double2hiint(th) ^ sy[t]), __double2loint(th));
+        if (w64) w64[t] = wv;
+        if (w32) w32[t] = (float)wv;
     }
 }
 
@@ -909,7 +963,7 @@ cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const in
     const DcdPending pd = pend ? *pend : DcdPending{};
     if (pend && cnt > DCD_FAST_MAX) return cudaErrorInvalidValue;
     if (cnt <= DCD_FAST_MAX) {
-        const size_t fsm = sizeof(double) * (size_t)(cnt * cnt + cnt) + sizeof(int32_t) * cnt;
+        const size_t fsm = sizeof(double) * (size_t)(cnt * (cnt | 1) + cnt) + sizeof(int32_t) * ((3 + DCD_FAST_K) * cnt + 2);
         static bool fattr[2] = {false, false};
         if (kss_f64) {
             if (!fattr[1]) {
@@ -919,7 +973,7 @@ cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const in
                 fattr[1] = true;
             }
             recur_dcd_fast_kernel<double><<<1, DCD_THREADS, fsm, st>>>((const double *)Kss, ldk, S, (int)cnt, y, alpha,
-                                                                       g, omega, nu, delta, w64, w32, pd);
+                                                                       g, omega, nu, delta, w64, w32, pd, err);
         } else {
             if (!fattr[0]) {
                 cudaError_t e = cudaFuncSetAttribute(recur_dcd_fast_kernel<float>,
@@ -928,7 +982,7 @@ cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const in
                 fattr[0] = true;
             }
             recur_dcd_fast_kernel<float><<<1, DCD_THREADS, fsm, st>>>((const float *)Kss, ldk, S, (int)cnt, y, alpha,
-                                                                      g, omega, nu, delta, w64, w32, pd);
+                                                                      g, omega, nu, delta, w64, w32, pd, err);
         }
         return cudaGetLastError();
     }
