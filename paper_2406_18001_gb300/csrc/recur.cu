@@ -616,6 +616,154 @@ __global__ void __launch_bounds__(256) bdcd_residual_kernel(const KT *Kss, int64
     if (lane == 0) rho[p] = rhs64[p] - (acc * inv_lambda + mdiag * dm);
 }
 
+// ------------------------------------- BDCD, FP64 forward substitution ---
+// The FP64 form up to FWD64_SB rows and b <= 32.  The inverses W_j = G_jj^-1 come first, a CTA per
+// block (they need only the Gram); one CTA then walks the blocks: a warp forms Delta_j = W_j r_j,
+// several lanes a row, and every thread subtracts G_pj Delta_j from the right-hand side of its
+// later row p.  The Gram entries are read as Kss[tb+q][p] (K is symmetric; consecutive threads,
+// consecutive addresses), those of the next block's step in flight while this one's Delta is formed.
+//
+// The FP64 pipe bounds it (a warp instruction per scheduler every ~80 cycles): sb^2 / 2 FMAs and
+// nblk dependent products.  One pass replaces three FP32 passes with FP64 residuals, whose rounds
+// each waited on the single CTA's chain: sb = 256, b = 16: 215 us of recurrence a step -> 45 us
+// (the inverses, 16 us, beside the block before).  Beyond FWD64_SB rows the square overtakes the
+// refined chain.
+constexpr int FWD64_SB = 1024;
+constexpr int INV64_NT = 256;
+
+// W_j by Gauss-Jordan on [G_jj | I], only the columns that can change at pivot k touched; the owner of
+// the next pivot forms its reciprocal.  W: nblk blocks of b x b, row-major.
+template <typename KT>
+__global__ void __launch_bounds__(INV64_NT) bdcd_inverse64_kernel(const KT *Kss, int64_t ldk, int b, double lambda,
+                                                                  double mdiag, double *W, int *err)
+{
+    __shared__ double a[2][32][65];
+    __shared__ double ip_s[2];
+    const int j = blockIdx.x, tid = threadIdx.x;
+    const int64_t o = (int64_t)j * b;
+    const int wd = 2 * b;
+    for (int e = tid; e < b * wd; e += INV64_NT) {
+        const int p = e / wd, q = e - p * wd;
+        a[0][p][q] = q >= b ? (q - b == p ? 1.0 : 0.0) : kval(Kss, ldk, o + p, o + q) / lambda + (p == q ? mdiag : 0.0);
+        if (p == 0 && q == 0) ip_s[0] = 1.0 / a[0][0][0];
+    }
+    __syncthreads();
+    int cur = 0;
+    bool bad = false;
+    for (int k = 0; k < b; ++k) {
+        const double piv = a[cur][k][k];
+        if (!(piv > 0.0)) {  // the same value in every thread
+            bad = true;
+            break;
+        }
+        const double ip = ip_s[k & 1];
+        // columns k .. b + k: the left half before k is done, the right half past b + k still zero
+        for (int e = tid; e < b * (b + 1); e += INV64_NT) {
+            const int p = e / (b + 1), q = k + (e - p * (b + 1));
+            const double pk = a[cur][k][q] * ip;
+            const double v = p == k ? pk : fma(-a[cur][p][k], pk, a[cur][p][q]);
+            a[cur ^ 1][p][q] = v;
+            if (p == k + 1 && q == k + 1 && k + 1 < b) ip_s[(k + 1) & 1] = 1.0 / v;
+        }
+        // the next right-half column is still the identity's
+        for (int p = tid; p < b; p += INV64_NT)
+            if (k + 1 < b) a[cur ^ 1][p][b + k + 1] = p == k + 1 ? 1.0 : 0.0;
+        cur ^= 1;
+        __syncthreads();
+    }
+    if (bad) {
+        if (tid == 0) set_error(err, DEV_NOT_SPD);
+        return;
+    }
+    double *w = W + o * b;
+    for (int e = tid; e < b * b; e += INV64_NT) w[e] = a[cur][e / b][b + e % b];
+}
+
+template <typename KT, int BT, int FWD64_NT>
+__global__ void __launch_bounds__(FWD64_NT) bdcd_forward64_kernel(const KT *Kss, int64_t ldk, const int32_t *S,
+                                                                  int nblk, int b, double lambda, double mdiag,
+                                                                  const double *g, const double *W, double *delta,
+                                                                  double *w64, float *w32)
+{
+    __shared__ double r[FWD64_SB], ds[BT];
+    __shared__ int32_t sI[FWD64_SB];
+    const int sb = nblk * b, tid = threadIdx.x, lane = tid & 31;
+    const double inv_lam = 1.0 / lambda;
+    for (int p = tid; p < sb; p += FWD64_NT) {
+        const int32_t i = S[p];
+        sI[p] = i;
+        r[p] = -g[i];
+    }
+    // warp 0: its block's inverse, LPR lanes a row (lane: row lane / LPR, every LPR-th column)
+    constexpr int LPR = BT <= 8 ? 4 : BT <= 16 ? 2 : 1, QL = BT / LPR;
+    const int wp = lane / LPR, wq = lane % LPR;
+    double wv[QL];
+    auto load_w = [&](int j) {
+#pragma unroll
+        for (int i = 0; i < QL; ++i) {
+            const int q = wq + LPR * i;
+            wv[i] = wp < b && q < b ? W[((int64_t)j * b + wp) * b + q] : 0.0;
+        }
+    };
+    if (tid < 32) load_w(0);
+    // this thread's first later row: its Gram entries of the coming step
+    double kr[BT];
+    auto load_k = [&](int j, int p) {
+#pragma unroll
+        for (int q = 0; q < BT; ++q) kr[q] = q < b && p < sb ? kval(Kss, ldk, (int64_t)j * b + q, p) : 0.0;
+    };
+    auto update = [&](int tb, int p) {  // r_p -= G_pj Delta_j
+        double s0 = 0.0, s1 = 0.0, dm = 0.0;
+        const int32_t ip = sI[p];
+        bool rep = false;
+#pragma unroll
+        for (int q = 0; q < BT; q += 2) {
+            if (q < b) s0 = fma(kr[q], ds[q], s0);
+            if (q + 1 < b) s1 = fma(kr[q + 1], ds[q + 1], s1);
+        }
+        for (int q = 0; q < b; ++q) rep |= sI[tb + q] == ip;
+        if (rep)
+            for (int q = 0; q < b; ++q) dm += sI[tb + q] == ip ? ds[q] : 0.0;
+        r[p] -= (s0 + s1) * inv_lam + (rep ? mdiag * dm : 0.0);
+    };
+    load_k(0, b + tid);
+    __syncthreads();
+    for (int j = 0; j < nblk; ++j) {
+        const int tb = j * b;
+        if (tid < 32) {
+            double d0 = 0.0, d1 = 0.0;
+#pragma unroll
+            for (int i = 0; i < QL; i += 2) {
+                const int q = wq + LPR * i;
+                if (q < b) d0 = fma(wv[i], r[tb + q], d0);
+                if (i + 1 < QL && q + LPR < b) d1 = fma(wv[i + 1], r[tb + q + LPR], d1);
+            }
+            double d = d0 + d1;
+#pragma unroll
+            for (int o = LPR / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (wp < b && wq == 0) {
+                ds[wp] = d;
+                delta[tb + wp] = d;
+            }
+            if (j + 1 < nblk) load_w(j + 1);
+        }
+        __syncthreads();
+        const int p0 = tb + b + tid;
+        if (p0 < sb) update(tb, p0);
+        for (int p = p0 + FWD64_NT; p < sb; p += FWD64_NT) {
+            load_k(j, p);
+            update(tb, p);
+        }
+        if (j + 1 < nblk) load_k(j + 1, p0 + b);
+        __syncthreads();
+    }
+    for (int p = tid; p < sb; p += FWD64_NT) {
+        const double w = delta[p] / lambda;
+        if (w64) w64[p] = w;
+        if (w32) w32[p] = (float)w;
+    }
+}
+
 // Chains longer than one cluster launch takes: blocked forward substitution.
 // The chain is cut into diagonal panels of pb blocks; each panel is solved by
 // the cluster recurrence (with its own refinement rounds) from right-hand
@@ -1013,6 +1161,18 @@ cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const in
     return cudaGetLastError();
 }
 
+bool recur_bdcd_forward64(int64_t nblk, int b)
+{
+    return b <= 32 && nblk >= 1 && nblk * b <= FWD64_SB;
+}
+
+cudaError_t launch_bdcd_inverse64(const double *Kss, int64_t ldk, int64_t nblk, int b, double lambda, double mdiag,
+                                  double *W, int *err, cudaStream_t st)
+{
+    bdcd_inverse64_kernel<double><<<(unsigned)nblk, INV64_NT, 0, st>>>(Kss, ldk, b, lambda, mdiag, W, err);
+    return cudaGetLastError();
+}
+
 size_t recur_bdcd_scratch_bytes(int64_t nblk, int b)
 {
     const size_t sb = (size_t)nblk * b;
@@ -1040,10 +1200,25 @@ bool recur_bdcd_lower_gram(int64_t nblk, int b, int refinements, int64_t ldk)
 
 cudaError_t launch_recur_bdcd(const void *Kss, int kss_f64, int64_t ldk, const int32_t *S, int64_t nblk, int b,
                               double lambda, double mdiag, const double *g, int refinements, void *scratch,
-                              double *delta, double *w64, float *w32, FusedUpdate *upd, int *err, cudaStream_t st)
+                              double *delta, double *w64, float *w32, FusedUpdate *upd, int *err, cudaStream_t st,
+                              const double *W64)
 {
     if (upd) upd->done = false;
     if (nblk <= 0) return cudaSuccess;
+    if (kss_f64 && recur_bdcd_forward64(nblk, b)) {
+        const double *K = (const double *)Kss;
+        if (!W64) {  // nblk b (b + 1) doubles of scratch hold the inverses
+            const cudaError_t e = launch_bdcd_inverse64(K, ldk, nblk, b, lambda, mdiag, (double *)scratch, err, st);
+            if (e != cudaSuccess) return e;
+            W64 = (const double *)scratch;
+        }
+        // (threads: as many as the block's Gram entries a thread leave registers for)
+        auto kfn = b <= 8    ? bdcd_forward64_kernel<double, 8, 512>
+                   : b <= 16 ? bdcd_forward64_kernel<double, 16, 512>
+                             : bdcd_forward64_kernel<double, 32, 256>;
+        kfn<<<1, b <= 16 ? 512 : 256, 0, st>>>(K, ldk, S, (int)nblk, b, lambda, mdiag, g, W64, delta, w64, w32);
+        return cudaGetLastError();
+    }
     if (b <= 32 && nblk * b <= 8192 && refinements >= 0 &&
         chain_layout((int)(nblk * b), b, kss_f64 ? 8 : 4, ldk).total <= CHAIN_SMEM_MAX) {
         if (kss_f64)

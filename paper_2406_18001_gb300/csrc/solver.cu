@@ -442,6 +442,11 @@ struct Solver {
             double *dl = (double *)ar.take(sizeof(double) * col_pad);
             double *wv = (double *)ar.take(sizeof(double) * col_pad);
             double *lb = (double *)ar.take(problem == 1 ? recur_bdcd_scratch_bytes(o.s, o.b) : 0);
+            // the FP64 recurrence's block inverses of each buffer set
+            const bool fwd64 = problem == 1 && !tc && recur_bdcd_forward64(o.s, o.b);
+            double *w64i[3];
+            for (int q = 0; q < 3; ++q)
+                w64i[q] = (double *)ar.take(fwd64 && (q == 0 || (q == 1 && set2)) ? sizeof(double) * sb * o.b : 0);
             uint64_t *cr = (uint64_t *)ar.take(sizeof(uint64_t));
             // the second set of step buffers and the look-ahead counter
             int32_t *sidx_b = (int32_t *)ar.take(set2 ? sizeof(int32_t) * col_pad : 0);
@@ -556,6 +561,7 @@ struct Solver {
             sbuf[2].col_s = cs_c;
             sbuf[2].Kss = kss_c;
             sbuf[2].Lbuf = lb_c;
+            for (int q = 0; q < 3; ++q) sbuf[q].W64 = fwd64 ? w64i[q] : nullptr;
             sbuf[0].delta = dl;
             sbuf[0].w64 = wv;
             sbuf[0].col_w = cw;
@@ -1154,6 +1160,7 @@ struct Solver {
         float *col_h = nullptr, *col_s = nullptr;
         void *Kss = nullptr;
         double *Lbuf = nullptr;
+        double *W64 = nullptr;  // the FP64 recurrence's block inverses (null: it forms them itself)
         // the chain's outputs (per set with the deferred gradient; shared otherwise)
         double *delta = nullptr, *w64 = nullptr;
         float *col_w = nullptr;
@@ -1698,6 +1705,8 @@ struct Solver {
         if (e == cudaSuccess) e = gather(ncols);
         if (e == cudaSuccess && sampled && rows_gathered) e = cudaEventRecord(sampled, st);
         if (e == cudaSuccess) e = gram(ncols);
+        if (e == cudaSuccess && sbuf[q].W64)
+            e = launch_bdcd_inverse64((const double *)Kss, ldk, cnt, o.b, lambda, (double)m, sbuf[q].W64, err, st);
         st = keep;
         return cuda_status(e);
     }
@@ -1724,7 +1733,7 @@ struct Solver {
                                      tc ? col_w : nullptr, err, st));
         else
             DCD_TRY(launch_recur_bdcd(Kss, tc ? 0 : 1, ldk, S, cnt, o.b, lambda, (double)m, g, tc ? 1 : 2, Lbuf,
-                                      delta, w64, tc ? col_w : nullptr, &fu, err, st));
+                                      delta, w64, tc ? col_w : nullptr, &fu, err, st, sbuf[p].W64));
         if (next) {
             DCD_TRY(cudaStreamWaitEvent(st2, la_fork, 0));
             dcd_status r = lag_side(1 - p, next, st2);
