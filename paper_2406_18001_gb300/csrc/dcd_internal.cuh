@@ -230,10 +230,37 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
 // kernel before it writes, started once that kernel has started.  prio: the launch's scheduling
 // priority (0: the stream's), so that its CTAs take SMs before those of kernels beside it)
 
+// Value of an e4m3 code (OCP FP8: sign, 4 exponent bits with bias 7, 3
+// mantissa bits; exponent field 0 holds the subnormals f * 2^-9; 0x7f / 0xff
+// are NaN).  Exact in FP32: the float's bits are assembled directly.
+__device__ __forceinline__ float e4m3_value(uint32_t c)
+{
+    const uint32_t e = (c >> 3) & 15u, f = c & 7u;
+    float v;
+    if ((c & 0x7Fu) == 0x7Fu) v = __int_as_float(0x7fc00000);
+    else if (e) v = __uint_as_float(((e + 120u) << 23) | (f << 20));  // (1 + f/8) * 2^(e-7)
+    else v = (float)f * 0.001953125f;                                 // f * 2^-9
+    return (c & 0x80u) ? -v : v;
+}
+
+// Packed operands with their RBF row terms (pack.cu): rows `rows` (or the first count) of a dense
+// source in the operand kind `kind` (PACK_BF16, _TF32, _BF16X3, _TF32X3, _FP16, _SLICED) and h[r] =
+// gamma log2(e) ||x_r||^2 of the packed row (0 for the other kernels).  src_scale: the per-row scales
+// of an FP8 source.  sc: the scales of the rows (FP16, all the one that gbits from
+// launch_absmax_rows fixes; SLICED).  h_lo (TF32X3, SLICED): the term as a pair h + h_lo.
+cudaError_t launch_pack_terms(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
+                              void *dst, int kind, int64_t n_pad, int64_t count, const KernelParams &kp, float *h,
+                              int *err, cudaStream_t st, const float *src_scale = nullptr, float *sc = nullptr,
+                              const unsigned *gbits = nullptr, float *h_lo = nullptr);
+// The largest magnitude over the first count rows of a dense source, folded by atomicMax into *bits
+// (FP32 bits; zero it first); a value that is not finite sets DEV_BAD_VALUE.
+cudaError_t launch_absmax_rows(const void *src, int dtype, int64_t ld, int64_t n, int64_t count, unsigned *bits,
+                               int *err, cudaStream_t st, const float *src_scale = nullptr);
+
 // setup / per-step helpers (sample_update.cu)
-// src_scale: the per-row scales of an FP8 source (dtype DCD_FP8E4M3), else unused
+// FP64 rows (n_pad doubles each, zero padded) of rows `rows` (or the first count) of a dense source
 cudaError_t launch_pack_rows(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                             void *dst, int dst_kind, int64_t n_pad, int64_t count, int *err, cudaStream_t st,
+                             double *dst, int64_t n_pad, int64_t count, int *err, cudaStream_t st,
                              const float *src_scale = nullptr);
 // Per-row e4m3 codes and scales of rows `rows` (or the first count) of a
 // dense source: quantised from F64/F32/BF16, copied from an FP8 source.
@@ -243,34 +270,15 @@ cudaError_t launch_quantize_rows(const void *src, int dtype, int64_t ld, int64_t
                                  int *err, cudaStream_t st);
 cudaError_t launch_label_check(const double *y, int64_t m, int *bad, cudaStream_t st);
 cudaError_t launch_f64_to_f32(const double *src, int64_t count, float *dst, cudaStream_t st);
-// h_lo (PACK_TF32X3, PACK_SLICED): the term as a pair of floats h + h_lo (FP64 sums), for the accurate
-// epilogue; PACK_SLICED takes its per-row scales in `scale`
-cudaError_t launch_row_terms(const void *packed, int kind, int64_t n_pad, int64_t m, const KernelParams &kp,
-                             float *h, cudaStream_t st, const float *scale = nullptr, float *h_lo = nullptr);
+// the RBF terms of FP8 rows with their scales
+cudaError_t launch_row_terms_fp8(const void *packed, int64_t n_pad, int64_t m, const KernelParams &kp, float *h,
+                                 cudaStream_t st, const float *rscale);
 // with the rows, optionally the per-row values f0 (and f1) of the same
 // indices: d0[j] = f0[idx[j]] (0 for an index outside [0, m))
 cudaError_t launch_gather_rows(const void *src, int64_t row_bytes, const int32_t *idx, int64_t count, int64_t m,
                                void *dst, int *err, cudaStream_t st, const float *f0 = nullptr, float *d0 = nullptr,
                                const float *f1 = nullptr, float *d1 = nullptr, const float *f2 = nullptr,
                                float *d2 = nullptr);
-// The largest magnitude over rows `rows` (or the first count) of a dense
-// source, folded by atomicMax into *bits (FP32 bits; zero it first).
-cudaError_t launch_absmax_rows(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                               int64_t count, unsigned *bits, int *err, cudaStream_t st,
-                               const float *src_scale = nullptr);
-// fp16 rows (PACK_FP16) of rows `rows` (or the first count) of a dense
-// source, all scaled by the power of two that *gbits (launch_absmax_rows over
-// every row that shares the scale) fixes, written to sc[r] for each row; an
-// FP8 source is dequantised first.  dst rows are n_pad fp16 values (zero padded).
-cudaError_t launch_pack_fp16(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                             void *dst, int64_t n_pad, int64_t count, float *sc, const unsigned *gbits, int *err,
-                             cudaStream_t st, const float *src_scale = nullptr);
-// Sliced rows (PACK_SLICED) of rows `rows` (or the first count) of a dense
-// source, with their power-of-two scales in sc (count floats); an FP8
-// source is dequantised first.  dst rows are 4 planes of n_pad bf16.
-cudaError_t launch_pack_sliced(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                               void *dst, int64_t n_pad, int64_t count, float *sc, int *err, cudaStream_t st,
-                               const float *src_scale = nullptr);
 cudaError_t launch_fill_f64(double *p, double v, int64_t count, cudaStream_t st);
 // out[i] = start + i, i < count (shard.cu)
 cudaError_t launch_iota(int32_t *out, int64_t count, int64_t start, cudaStream_t st);

@@ -67,19 +67,6 @@ cudaError_t launch_sample(int method, uint64_t seed, const uint64_t *ctr_dev, ui
 }
 
 // ------------------------------------------------------------ packing -----
-// Value of an e4m3 code (OCP FP8: sign, 4 exponent bits with bias 7, 3
-// mantissa bits; exponent field 0 holds the subnormals f * 2^-9; 0x7f / 0xff
-// are NaN).  Exact in FP32: the float's bits are assembled directly.
-__device__ __forceinline__ float e4m3_value(uint32_t c)
-{
-    const uint32_t e = (c >> 3) & 15u, f = c & 7u;
-    float v;
-    if ((c & 0x7Fu) == 0x7Fu) v = __int_as_float(0x7fc00000);
-    else if (e) v = __uint_as_float(((e + 120u) << 23) | (f << 20));  // (1 + f/8) * 2^(e-7)
-    else v = (float)f * 0.001953125f;                                 // f * 2^-9
-    return (c & 0x80u) ? -v : v;
-}
-
 // Nearest e4m3 code of x (ties to even), saturating at +-448.
 __device__ __forceinline__ uint32_t e4m3_code(float x)
 {
@@ -101,14 +88,11 @@ __device__ __forceinline__ float load_as_f32(const void *src, int dtype, int64_t
     }
 }
 
-// dst row r (n_pad elements, zero padded) = src row rows[r] (or r),
-// converted to bf16 (round to nearest even, dst_kind 0), fp32 (1, the tf32
-// path reads fp32 storage) or fp64 (2).  An FP8 source is dequantised with
-// its row scales (exactly, for fp64).
-// Row indices outside [0, m) produce a zero row and set DEV_BAD_INDEX.
+// dst row r (n_pad doubles, zero padded) = src row rows[r] (or r) in FP64; an FP8 source is
+// dequantised with its row scales (exactly).  Row indices outside [0, m) produce a zero row and
+// set DEV_BAD_INDEX.
 __global__ void pack_rows_kernel(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                                 void *dst, int dst_kind, int64_t n_pad, int64_t count, int *err,
-                                 const float *src_scale)
+                                 double *dst, int64_t n_pad, int64_t count, int *err, const float *src_scale)
 {
     const int64_t total = count * n_pad;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -117,54 +101,25 @@ __global__ void pack_rows_kernel(const void *src, int dtype, int64_t ld, int64_t
         const bool inb = sr >= 0 && sr < m;
         if (!inb && c == 0) set_error(err, DEV_BAD_INDEX);
         const float rsc = (dtype == DCD_FP8E4M3 && inb) ? src_scale[sr] : 0.f;
-        if (dst_kind == 2) {
-            double v = 0.0;
-            if (c < n && inb)
-                v = (dtype == DCD_F64)       ? ((const double *)src)[sr * ld + c]
-                    : (dtype == DCD_FP8E4M3) ? (double)rsc * (double)e4m3_value(((const uint8_t *)src)[sr * ld + c])
-                                             : (double)load_as_f32(src, dtype, sr * ld + c);
-            ((double *)dst)[e] = v;
-            continue;
-        }
-        float v = (c < n && inb) ? load_as_f32(src, dtype, sr * ld + c, rsc) : 0.f;
-        if (dst_kind == PACK_BF16X3) {
-            // hi = bf16(v), lo = bf16(v - hi); v - hi is exact in fp32
-            __nv_bfloat16 hi = __float2bfloat16_rn(v);
-            __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-            __nv_bfloat16 *d = (__nv_bfloat16 *)dst + r * 2 * n_pad;
-            d[c] = hi;
-            d[n_pad + c] = lo;
-        } else if (dst_kind == PACK_TF32X3) {
-            // hi = tf32(v), lo = tf32(v - hi) (v - hi exact in fp32), both on the tf32 grid
-            uint32_t th, tl;
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(th) : "f"(v));
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(tl) : "f"(v - __uint_as_float(th)));
-            float *d = (float *)dst + r * 2 * n_pad;
-            d[c] = __uint_as_float(th);
-            d[n_pad + c] = __uint_as_float(tl);
-        } else if (dst_kind == 1) {
-            // round to the tf32 grid (10-bit mantissa, nearest, ties away) so the
-            // tensor core sees exactly the stored value and the row norms match
-            uint32_t t;
-            asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(t) : "f"(v));
-            ((float *)dst)[e] = __uint_as_float(t);
-        } else {
-            ((__nv_bfloat16 *)dst)[e] = __float2bfloat16_rn(v);
-        }
+        double v = 0.0;
+        if (c < n && inb)
+            v = (dtype == DCD_F64)       ? ((const double *)src)[sr * ld + c]
+                : (dtype == DCD_FP8E4M3) ? (double)rsc * (double)e4m3_value(((const uint8_t *)src)[sr * ld + c])
+                                         : (double)load_as_f32(src, dtype, sr * ld + c);
+        dst[e] = v;
     }
 }
 
 cudaError_t launch_pack_rows(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                             void *dst, int dst_kind, int64_t n_pad, int64_t count, int *err, cudaStream_t st,
+                             double *dst, int64_t n_pad, int64_t count, int *err, cudaStream_t st,
                              const float *src_scale)
 {
-    if (dst_kind == PACK_FP8 || (dtype == DCD_FP8E4M3 && !src_scale)) return cudaErrorInvalidValue;
+    if (dtype == DCD_FP8E4M3 && !src_scale) return cudaErrorInvalidValue;
     if (count <= 0) return cudaSuccess;
     int64_t total = count * n_pad;
     int64_t blocks = (total + 255) / 256;
     if (blocks > 152 * 32) blocks = 152 * 32;
-    pack_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dtype, ld, m, n, rows, dst, dst_kind, n_pad, count, err,
-                                                        src_scale);
+    pack_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dtype, ld, m, n, rows, dst, n_pad, count, err, src_scale);
     return cudaGetLastError();
 }
 
@@ -172,145 +127,6 @@ cudaError_t launch_pack_rows(const void *src, int dtype, int64_t ld, int64_t m, 
 // scale = fl32(max|a| / 448), code = e4m3(fl32(a / scale)) with IEEE FP32
 // division; a row of zeros gets scale 0 and zero codes.  An FP8 source is
 // copied with its scale.  Columns n..ldq-1 of the destination are zero.
-// One warp per row: the row's largest magnitude fixes sc = 2^e with
-// max |a| in [2^(e-1), 2^e) (1 for a zero row); u = a / sc in (-1, 1) is cut
-// by round-to-nearest into s0 = rint(64 u) and, from the remainder r in
-// [-1/2, 1/2], s_p = rint(128 r) for p = 1..3 -- integers in [-64, 64], exact
-// in bf16, with u = s0 2^-6 + s1 2^-13 + s2 2^-20 + s3 2^-27 to within 2^-28.
-// Every step is exact in FP64 (power-of-two scalings and differences of
-// numbers within a factor two).  Columns n..n_pad-1 are zero.
-__global__ void pack_sliced_kernel(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                                   __nv_bfloat16 *dst, int64_t n_pad, int64_t count, float *sc, int *err,
-                                   const float *src_scale)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (r >= count) return;
-    const int64_t sr = rows ? (int64_t)rows[r] : r;
-    const bool inb = sr >= 0 && sr < m;
-    if (!inb && lane == 0) set_error(err, DEV_BAD_INDEX);
-    const float rsc = (dtype == DCD_FP8E4M3 && inb) ? src_scale[sr] : 0.f;
-    auto val = [&](int64_t c) -> double {
-        if (c >= n || !inb) return 0.0;
-        if (dtype == DCD_F64) return ((const double *)src)[sr * ld + c];
-        if (dtype == DCD_FP8E4M3) return (double)rsc * (double)e4m3_value(((const uint8_t *)src)[sr * ld + c]);
-        return (double)load_as_f32(src, dtype, sr * ld + c);
-    };
-    double mx = 0.0;
-    for (int64_t c = lane; c < n; c += 32) mx = fmax(mx, fabs(val(c)));
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    int e = 0;
-    if (mx > 0.0 && isfinite(mx)) frexp(mx, &e);
-    else if (!(mx == 0.0) && lane == 0) set_error(err, DEV_BAD_VALUE);
-    if (lane == 0) sc[r] = (float)ldexp(1.0, e);
-    __nv_bfloat16 *d = dst + r * 4 * n_pad;
-    for (int64_t c = lane; c < n_pad; c += 32) {
-        double v = ldexp(val(c), 6 - e);
-        const double s0 = rint(v);
-        v = (v - s0) * 128.0;
-        const double s1 = rint(v);
-        v = (v - s1) * 128.0;
-        const double s2 = rint(v);
-        v = (v - s2) * 128.0;
-        const double s3 = rint(v);
-        d[c] = __double2bfloat16(s0);
-        d[n_pad + c] = __double2bfloat16(s1);
-        d[2 * n_pad + c] = __double2bfloat16(s2);
-        d[3 * n_pad + c] = __double2bfloat16(s3);
-    }
-}
-
-// The largest magnitude over rows `rows` (or the first count) of a dense
-// source, folded into *bits (the FP32 bit pattern, which orders like the value
-// for non-negative floats) by atomicMax; a non-finite value sets
-// DEV_BAD_VALUE.  One warp per row.
-__global__ void absmax_rows_kernel(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                                   int64_t count, unsigned *bits, int *err, const float *src_scale)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (r >= count) return;
-    const int64_t sr = rows ? (int64_t)rows[r] : r;
-    if (sr < 0 || sr >= m) return;  // the pack reports bad indices
-    const float rsc = dtype == DCD_FP8E4M3 ? src_scale[sr] : 0.f;
-    float mx = 0.f;
-    bool bad = false;
-    for (int64_t c = lane; c < n; c += 32) {
-        const float v = load_as_f32(src, dtype, sr * ld + c, rsc);
-        bad |= !isfinite(v);
-        mx = fmaxf(mx, fabsf(v));
-    }
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (__any_sync(0xffffffffu, bad)) {
-        if (lane == 0) set_error(err, DEV_BAD_VALUE);
-        return;
-    }
-    if (lane == 0) atomicMax(bits, __float_as_uint(mx));
-}
-
-// One warp per row.  The scale is one power of two for every row, sc = 2^(e -
-// 15) with the largest magnitude over the matrix in [2^(e-1), 2^e) (from
-// *gbits), so that |a| / sc < 2^15 (fp16's largest finite value is 65504);
-// q = fp16(a / sc) rounds to nearest even (the division by a power of two is
-// exact).  fp16's exponent range keeps every value down to 2^-29 of the
-// largest at full precision.  A zero matrix gets sc = 2^-15.  sc[r] = sc for
-// every row; columns n..n_pad-1 are zero.
-__global__ void pack_fp16_kernel(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                                 __half *dst, int64_t n_pad, int64_t count, float *sc, const unsigned *gbits,
-                                 int *err, const float *src_scale)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    if (r >= count) return;
-    const int64_t sr = rows ? (int64_t)rows[r] : r;
-    const bool inb = sr >= 0 && sr < m;
-    if (!inb && lane == 0) set_error(err, DEV_BAD_INDEX);
-    const float rsc = (dtype == DCD_FP8E4M3 && inb) ? src_scale[sr] : 0.f;
-    const float mx = __uint_as_float(*gbits);
-    int e = 0;
-    if (mx > 0.f && isfinite(mx)) frexpf(mx, &e);
-    e = max(e, -110);  // the scale 2^(e - 15) stays a normal FP32 number
-    if (lane == 0) sc[r] = ldexpf(1.f, e - 15);
-    __half *d = dst + r * n_pad;
-    for (int64_t c = lane; c < n_pad; c += 32)
-        d[c] = __float2half_rn((c < n && inb) ? ldexpf(load_as_f32(src, dtype, sr * ld + c, rsc), 15 - e) : 0.f);
-}
-
-cudaError_t launch_absmax_rows(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                               int64_t count, unsigned *bits, int *err, cudaStream_t st, const float *src_scale)
-{
-    if (count <= 0) return cudaSuccess;
-    if (dtype == DCD_FP8E4M3 && !src_scale) return cudaErrorInvalidValue;
-    const int64_t blocks = (count * 32 + 255) / 256;
-    absmax_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dtype, ld, m, n, rows, count, bits, err, src_scale);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pack_fp16(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                             void *dst, int64_t n_pad, int64_t count, float *sc, const unsigned *gbits, int *err,
-                             cudaStream_t st, const float *src_scale)
-{
-    if (count <= 0) return cudaSuccess;
-    if (!sc || !gbits || n_pad < n || n_pad % 64 || (dtype == DCD_FP8E4M3 && !src_scale))
-        return cudaErrorInvalidValue;
-    const int64_t blocks = (count * 32 + 255) / 256;
-    pack_fp16_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dtype, ld, m, n, rows, (__half *)dst, n_pad, count, sc,
-                                                       gbits, err, src_scale);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pack_sliced(const void *src, int dtype, int64_t ld, int64_t m, int64_t n, const int32_t *rows,
-                               void *dst, int64_t n_pad, int64_t count, float *sc, int *err, cudaStream_t st,
-                               const float *src_scale)
-{
-    if (count <= 0) return cudaSuccess;
-    if (!sc || n_pad < n || n_pad % 64 || (dtype == DCD_FP8E4M3 && !src_scale)) return cudaErrorInvalidValue;
-    const int64_t blocks = (count * 32 + 255) / 256;
-    pack_sliced_kernel<<<(unsigned)blocks, 256, 0, st>>>(src, dtype, ld, m, n, rows, (__nv_bfloat16 *)dst, n_pad,
-                                                         count, sc, err, src_scale);
-    return cudaGetLastError();
-}
-
 // ------------------------------------------------ literal-order step --
 // The paper's printed order (Algorithms 2 and 4) keeps the m x sb block U_k /
 // Q_k in memory and forms U_j^T alpha_sk from it.  literal_partial_kernel:
@@ -480,110 +296,35 @@ cudaError_t launch_f64_to_f32(const double *src, int64_t count, float *dst, cuda
     return cudaGetLastError();
 }
 
-// h[r] = gamma * log2(e) * ||x_r||^2 of the packed (already rounded) row, for
-// the RBF expansion ||a||^2 + ||b||^2 - 2 a.b (Section 5.2); 0 for the other
-// kernels.  For split rows the norm is the one the three MMAs reproduce,
-// sum(hi^2 + 2 hi lo), so that a row's distance to itself stays ~0; FP8 and
-// FP16 rows take the dequantised norm rscale[r]^2 * sum value(q)^2.  One warp
-// per row, FP64 partial sums, fixed order.
-__global__ void row_terms_kernel(const void *packed, int kind, int64_t n_pad, int64_t m, double scale, float *h,
-                                 const float *rscale, float *h_lo)
+// h[r] = gamma * log2(e) * ||x_r||^2 of an FP8 row, the dequantised norm rscale[r]^2 * sum
+// value(q)^2, for the RBF expansion ||a||^2 + ||b||^2 - 2 a.b (Section 5.2); 0 for the other
+// kernels.  One warp per row: FP32 sums of a lane's columns, combined in FP64, fixed order.
+// (pack.cu forms the other operands' terms as it packs them.)
+__global__ void row_terms_fp8_kernel(const uint8_t *packed, int64_t n_pad, int64_t m, double scale, float *h,
+                                     const float *rscale)
 {
     const int lane = threadIdx.x & 31;
     const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (r >= m) return;
-    if (kind == PACK_SLICED) {
-        // the slices' own product sums, truncated as the apply truncates them (groups p + q <= 3),
-        // exact in FP64: a.a = sc^2 2^-12 (S0 + 2^-7 S1 + 2^-14 S2 + 2^-21 S3)
-        const __nv_bfloat16 *row = (const __nv_bfloat16 *)packed + r * 4 * n_pad;
-        double S0 = 0.0, S1 = 0.0, S2 = 0.0, S3 = 0.0;
-        for (int64_t c = lane; c < n_pad; c += 32) {
-            const double a0 = __bfloat162float(row[c]), a1 = __bfloat162float(row[n_pad + c]);
-            const double a2 = __bfloat162float(row[2 * n_pad + c]), a3 = __bfloat162float(row[3 * n_pad + c]);
-            S0 += a0 * a0;
-            S1 += 2.0 * a0 * a1;
-            S2 += 2.0 * a0 * a2 + a1 * a1;
-            S3 += 2.0 * (a0 * a3 + a1 * a2);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            S0 += __shfl_xor_sync(0xffffffffu, S0, o);
-            S1 += __shfl_xor_sync(0xffffffffu, S1, o);
-            S2 += __shfl_xor_sync(0xffffffffu, S2, o);
-            S3 += __shfl_xor_sync(0xffffffffu, S3, o);
-        }
-        if (lane == 0) {
-            const double sc = rscale[r];
-            const double v = scale * (sc * sc) * 0x1p-12 * (S0 + 0x1p-7 * S1 + 0x1p-14 * S2 + 0x1p-21 * S3);
-            const float vh = (float)v;
-            h[r] = vh;
-            if (h_lo) h_lo[r] = (float)(v - (double)vh);
-        }
-        return;
-    }
-    if (kind == PACK_FP16) {
-        // fp16 values: their squares are exact in FP64 and summed in FP64; times the row scale^2
-        const __half *row = (const __half *)packed + r * n_pad;
-        double sd = 0.0;
-        for (int64_t c = lane; c < n_pad; c += 32) {
-            const double v = __half2float(row[c]);
-            sd = fma(v, v, sd);
-        }
-        for (int o = 16; o > 0; o >>= 1) sd += __shfl_xor_sync(0xffffffffu, sd, o);
-        if (lane == 0) h[r] = (float)(scale * sd * (double)rscale[r] * (double)rscale[r]);
-        return;
-    }
-    if (kind == PACK_TF32X3) {
-        // split tf32: the products the three MMAs form, hi.hi + 2 hi.lo, each exact in FP64 (24-bit
-        // factors) and summed in FP64; the term is stored as a pair of floats hi + lo (h_lo given) for
-        // the accurate epilogue, or rounded to one float
-        const float *row = (const float *)packed + r * 2 * n_pad;
-        double sd = 0.0;
-        for (int64_t c = lane; c < n_pad; c += 32) {
-            const double hi = row[c], lo = row[n_pad + c];
-            sd = fma(hi, hi + 2.0 * lo, sd);
-        }
-        for (int o = 16; o > 0; o >>= 1) sd += __shfl_xor_sync(0xffffffffu, sd, o);
-        if (lane == 0) {
-            const double v = scale * sd;
-            const float vh = (float)v;
-            h[r] = vh;
-            if (h_lo) h_lo[r] = (float)(v - (double)vh);
-        }
-        return;
-    }
-    // per-lane FP32 sums (each lane adds n_pad/32 squares), combined in FP64
     float sf = 0.f;
     for (int64_t c = lane; c < n_pad; c += 32) {
-        if (kind == PACK_TF32) {
-            const float v = ((const float *)packed)[r * n_pad + c];
-            sf = fmaf(v, v, sf);
-        } else if (kind == PACK_BF16X3) {
-            const __nv_bfloat16 *row = (const __nv_bfloat16 *)packed + r * 2 * n_pad;
-            const float hi = __bfloat162float(row[c]), lo = __bfloat162float(row[n_pad + c]);
-            sf = fmaf(hi, hi + 2.f * lo, sf);
-        } else if (kind == PACK_FP8) {  // sum of value(q)^2; the row scale comes in below
-            const float v = e4m3_value(((const uint8_t *)packed)[r * n_pad + c]);
-            sf = fmaf(v, v, sf);
-        } else {
-            const float v = __bfloat162float(((const __nv_bfloat16 *)packed)[r * n_pad + c]);
-            sf = fmaf(v, v, sf);
-        }
+        const float v = e4m3_value(packed[r * n_pad + c]);
+        sf = fmaf(v, v, sf);
     }
     double s = sf;
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (kind == PACK_FP8) s *= (double)rscale[r] * (double)rscale[r];
+    s *= (double)rscale[r] * (double)rscale[r];
     if (lane == 0) h[r] = (float)(scale * s);
 }
 
-cudaError_t launch_row_terms(const void *packed, int kind, int64_t n_pad, int64_t m, const KernelParams &kp,
-                             float *h, cudaStream_t st, const float *rscale, float *h_lo)
+cudaError_t launch_row_terms_fp8(const void *packed, int64_t n_pad, int64_t m, const KernelParams &kp, float *h,
+                                 cudaStream_t st, const float *rscale)
 {
-    if ((kind == PACK_FP8 || kind == PACK_SLICED || kind == PACK_FP16) && !rscale) return cudaErrorInvalidValue;
-    if (h_lo && kind != PACK_TF32X3 && kind != PACK_SLICED) return cudaErrorInvalidValue;
+    if (!rscale) return cudaErrorInvalidValue;
     if (m <= 0) return cudaSuccess;
-    double scale = (kp.kind == DCD_RBF) ? kp.gamma * 1.4426950408889634 : 0.0;
-    int64_t blocks = (m * 32 + 255) / 256;
-    row_terms_kernel<<<(unsigned)blocks, 256, 0, st>>>(packed, kind, n_pad, m, scale, h, rscale, h_lo);
+    const double scale = (kp.kind == DCD_RBF) ? kp.gamma * 1.4426950408889634 : 0.0;
+    const int64_t blocks = (m * 32 + 255) / 256;
+    row_terms_fp8_kernel<<<(unsigned)blocks, 256, 0, st>>>((const uint8_t *)packed, n_pad, m, scale, h, rscale);
     return cudaGetLastError();
 }
 

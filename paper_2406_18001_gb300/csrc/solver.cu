@@ -670,8 +670,7 @@ struct Solver {
             const void *v = host ? (const void *)h_vals : A->values;
             if (conv32) DCD_TRY(launch_f64_to_f32((const double *)v, nnz, (float *)ca.vals32, st));
             if (conv64)
-                DCD_TRY(launch_pack_rows(v, A->dtype, nnz, 1, nnz, nullptr, (double *)ca.vals64, PACK_F64, nnz, 1,
-                                         err, st));
+                DCD_TRY(launch_pack_rows(v, A->dtype, nnz, 1, nnz, nullptr, (double *)ca.vals64, nnz, 1, err, st));
             // CSR checks, squared row norms and the longest row (err[2] = bad entries, err[3] = max length)
             int *bad = err + 2, *maxlen = err + 3;
             CsrOperand chk = ca;
@@ -720,28 +719,25 @@ struct Solver {
             } else if (fp16) {
                 // one power-of-two scale for the matrix, from its largest magnitude (err[5], zeroed above)
                 unsigned *gbits = (unsigned *)(err + 5);
-                DCD_TRY(launch_absmax_rows(vals, A->dtype, A->ld, m, n, nullptr, m, gbits, err, st, src_scale));
-                DCD_TRY(launch_pack_fp16(vals, A->dtype, A->ld, m, n, nullptr, op.packed, n_pad, m, op.row_s, gbits, err,
-                                         st, src_scale));
+                DCD_TRY(launch_absmax_rows(vals, A->dtype, A->ld, n, m, gbits, err, st, src_scale));
+                DCD_TRY(launch_pack_terms(vals, A->dtype, A->ld, m, n, nullptr, op.packed, op.kind, n_pad, m, kp,
+                                          op.row_h, err, st, src_scale, op.row_s, gbits));
                 dcd_status qs = check_device_error();  // non-finite values: EINVAL
                 if (qs != DCD_OK) return qs;
             } else {
-                DCD_TRY(launch_pack_rows(vals, A->dtype, A->ld, m, n, nullptr, op.packed, op.kind, n_pad, m, err, st,
-                                         src_scale));
+                DCD_TRY(launch_pack_terms(vals, A->dtype, A->ld, m, n, nullptr, op.packed, op.kind, n_pad, m, kp,
+                                          op.row_h, err, st, src_scale, nullptr, nullptr,
+                                          acc_ref && !ref_op ? row_hlr : nullptr));
             }
-            DCD_TRY(launch_row_terms(op.packed, op.kind, n_pad, m, kp, op.row_h, st, op.row_s));
+            if (fp8) DCD_TRY(launch_row_terms_fp8(op.packed, n_pad, m, kp, op.row_h, st, op.row_s));
             if (ref_op) {
                 opr.n_pad = n_pad_r;
                 opr.kind = kind_r;
-                if (sliced_ref) {
-                    DCD_TRY(launch_pack_sliced(vals, A->dtype, A->ld, m, n, nullptr, opr.packed, n_pad_r, m, opr.row_s,
-                                               err, st, src_scale));
-                    DCD_TRY(cudaMemsetAsync(col_sr, 0, sizeof(float) * col_pad, st));
-                } else {
-                    opr.row_s = nullptr;
-                    DCD_TRY(launch_pack_rows(vals, A->dtype, A->ld, m, n, nullptr, opr.packed, opr.kind, n_pad_r, m,
-                                             err, st, src_scale));
-                }
+                if (!sliced_ref) opr.row_s = nullptr;
+                // with the RBF terms as hi + lo pairs
+                DCD_TRY(launch_pack_terms(vals, A->dtype, A->ld, m, n, nullptr, opr.packed, opr.kind, n_pad_r, m, kp,
+                                          opr.row_h, err, st, src_scale, opr.row_s, nullptr, row_hlr));
+                if (sliced_ref) DCD_TRY(cudaMemsetAsync(col_sr, 0, sizeof(float) * col_pad, st));
                 DCD_TRY(cudaMemsetAsync(col_hr, 0, sizeof(float) * col_pad, st));
             } else {
                 opr = op;
@@ -749,13 +745,10 @@ struct Solver {
                 col_hr = col_h;
                 ref_shared = true;
             }
-            if (acc_ref) {  // the RBF terms of the recomputed gradient's operand, as hi + lo pairs
-                DCD_TRY(launch_row_terms(opr.packed, opr.kind, opr.n_pad, m, kp, opr.row_h, st,
-                                         opr.kind == PACK_SLICED ? opr.row_s : nullptr, row_hlr));
-                DCD_TRY(cudaMemsetAsync(col_hlr, 0, sizeof(float) * col_pad, st));
-            }
+            if (acc_ref) DCD_TRY(cudaMemsetAsync(col_hlr, 0, sizeof(float) * col_pad, st));
         } else if (need_pack) {
-            DCD_TRY(launch_pack_rows(vals, A->dtype, A->ld, m, n, nullptr, op.packed, 2, n, m, err, st, src_scale));
+            DCD_TRY(launch_pack_rows(vals, A->dtype, A->ld, m, n, nullptr, (double *)op.packed, n, m, err, st,
+                                     src_scale));
             op.a64 = (const double *)op.packed;
             op.lda = n;
         } else {
@@ -2330,7 +2323,7 @@ dcd_status component_block_csr(const dcd_matrix *A, const KernelParams &kp, int3
     if (fp64) {
         ca.vals64 = conv64 ? (const double *)(base + ov) : (const double *)A->values;
         if (conv64)
-            DCD_TRY(launch_pack_rows(A->values, A->dtype, nnz, 1, nnz, nullptr, base + ov, PACK_F64, nnz, 1, err, st));
+            DCD_TRY(launch_pack_rows(A->values, A->dtype, nnz, 1, nnz, nullptr, (double *)(base + ov), nnz, 1, err, st));
     } else {
         ca.vals32 = conv32 ? (const float *)(base + ov) : (const float *)A->values;
         if (conv32) DCD_TRY(launch_f64_to_f32((const double *)A->values, nnz, (float *)(base + ov), st));
@@ -2405,7 +2398,7 @@ dcd_status component_block(const dcd_matrix *A, const dcd_kernel *k, int32_t pre
         int64_t lda = A->ld;
         if (pack) {
             double *p = (double *)(base + op64);
-            DCD_TRY(launch_pack_rows(A->values, A->dtype, A->ld, A->m, A->n, nullptr, p, 2, A->n, A->m, err, st,
+            DCD_TRY(launch_pack_rows(A->values, A->dtype, A->ld, A->m, A->n, nullptr, p, A->n, A->m, err, st,
                                      A->row_scale));
             a64 = p;
             lda = A->n;
@@ -2417,7 +2410,7 @@ dcd_status component_block(const dcd_matrix *A, const dcd_kernel *k, int32_t pre
             ldp = P->ld;
             if (packp) {
                 double *p = (double *)(base + opp);
-                DCD_TRY(launch_pack_rows(P->values, P->dtype, P->ld, P->m, P->n, nullptr, p, 2, P->n, P->m, err, st,
+                DCD_TRY(launch_pack_rows(P->values, P->dtype, P->ld, P->m, P->n, nullptr, p, P->n, P->m, err, st,
                                          P->row_scale));
                 p64 = p;
                 ldp = P->n;
@@ -2434,22 +2427,16 @@ dcd_status component_block(const dcd_matrix *A, const dcd_kernel *k, int32_t pre
     const int64_t n_pad = (A->n + kb - 1) / kb * kb;
     const size_t rb = (size_t)packed_row_bytes(pk, n_pad);
     const int64_t cpad = (ncols + 255) / 256 * 256;
+    const bool fp8 = pk == PACK_FP8, fp16 = pk == PACK_FP16, scaled = fp8 || fp16 || sliced;
+    // columns among the packed rows (every row of A packed): gathered, else packed themselves
+    const bool from_rows = !pts && !rows && nrows == A->m;
     size_t cur = 0;
+    // first what has to start at zero
     size_t oe = place(cur, 256);
-    size_t oa = place(cur, (size_t)nrows * rb);
-    size_t ob = place(cur, (size_t)ncols * rb);
-    size_t orh = place(cur, sizeof(float) * nrows);
     size_t och = place(cur, sizeof(float) * cpad);
     size_t ocw = place(cur, sizeof(float) * cpad);
-    const bool fp8 = pk == PACK_FP8, fp16 = pk == PACK_FP16;
-    size_t ors = place(cur, (fp8 || fp16 || sliced) ? sizeof(float) * nrows : 0);
-    size_t ocs = place(cur, (fp8 || fp16 || sliced) ? sizeof(float) * cpad : 0);
-    size_t orl = place(cur, accurate ? sizeof(float) * nrows : 0);
+    size_t ocs = place(cur, scaled ? sizeof(float) * cpad : 0);
     size_t ocl = place(cur, accurate ? sizeof(float) * cpad : 0);
-    // points form: global row ids (when offset) and column ids (-1 without col_ids)
-    const bool rid = pts && pts->row_id0 != 0, cid = pts && !pts->col_ids;
-    size_t ori = place(cur, rid ? sizeof(int32_t) * nrows : 0);
-    size_t oci = place(cur, cid ? sizeof(int32_t) * ncols : 0);
     // the apply form's balanced split over CTA pairs
     TcSplit sp;
     if (!out) {
@@ -2459,61 +2446,57 @@ dcd_status component_block(const dcd_matrix *A, const dcd_kernel *k, int32_t pre
         sp.pairs = std::max(sms / 2, 1);
         sp.chunks = tc_split_chunks(ncols);
     }
-    size_t osp = place(cur, sizeof(double) * tc_split_part_elems(sp.pairs, sp.chunks));
     size_t osc = place(cur, sizeof(unsigned) * 2 * sp.pairs);
+    const size_t zeroed = cur;
+    size_t oa = place(cur, (size_t)nrows * rb);
+    size_t ob = place(cur, (size_t)ncols * rb);
+    size_t orh = place(cur, sizeof(float) * nrows);
+    size_t ors = place(cur, scaled ? sizeof(float) * nrows : 0);
+    size_t orl = place(cur, accurate ? sizeof(float) * nrows : 0);
+    // points form: global row ids (when offset) and column ids (-1 without col_ids)
+    const bool rid = pts && pts->row_id0 != 0, cid = pts && !pts->col_ids;
+    size_t ori = place(cur, rid ? sizeof(int32_t) * nrows : 0);
+    size_t oci = place(cur, cid ? sizeof(int32_t) * ncols : 0);
+    size_t osp = place(cur, sizeof(double) * tc_split_part_elems(sp.pairs, sp.chunks));
     DCD_TRY(malloc_async(&cb.mem, cur + 1024, st));
     char *base = (char *)cb.mem;
     int *err = (int *)(base + oe);
     void *pa = base + oa, *pb = base + ob;
     float *rh = (float *)(base + orh), *ch = (float *)(base + och), *cw = (float *)(base + ocw);
-    float *rsa = (fp8 || fp16 || sliced) ? (float *)(base + ors) : nullptr;
-    float *rsb = (fp8 || fp16 || sliced) ? (float *)(base + ocs) : nullptr;
-    DCD_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
-    DCD_TRY(cudaMemsetAsync(ch, 0, sizeof(float) * cpad, st));
-    DCD_TRY(cudaMemsetAsync(cw, 0, sizeof(float) * cpad, st));
+    float *rsa = scaled ? (float *)(base + ors) : nullptr;
+    float *rsb = scaled ? (float *)(base + ocs) : nullptr;
+    float *rl = accurate ? (float *)(base + orl) : nullptr, *cl = accurate ? (float *)(base + ocl) : nullptr;
+    DCD_TRY(cudaMemsetAsync(base, 0, zeroed, st));
     if (!out) {
         sp.part = (double *)(base + osp);
         sp.cnt = (unsigned *)(base + osc);
-        DCD_TRY(cudaMemsetAsync(sp.cnt, 0, sizeof(unsigned) * 2 * sp.pairs, st));
     }
     const int32_t *pcols = pts ? nullptr : cols;  // rows of P: the first ncols
-    if (sliced) {
-        DCD_TRY(cudaMemsetAsync(rsb, 0, sizeof(float) * cpad, st));
-        DCD_TRY(launch_pack_sliced(A->values, A->dtype, A->ld, A->m, A->n, rows, pa, n_pad, nrows, rsa, err, st,
-                                   A->row_scale));
-        DCD_TRY(launch_pack_sliced(P->values, P->dtype, P->ld, P->m, P->n, pcols, pb, n_pad, ncols, rsb, err, st,
-                                   P->row_scale));
-    } else if (fp8) {
-        DCD_TRY(cudaMemsetAsync(rsb, 0, sizeof(float) * cpad, st));
+    unsigned *gbits = (unsigned *)(err + 2);
+    if (fp16) {
+        // one power-of-two scale for both operands: the largest magnitude over every row of A (the
+        // scale the solver's operand takes) and of the points
+        DCD_TRY(launch_absmax_rows(A->values, A->dtype, A->ld, A->n, A->m, gbits, err, st, A->row_scale));
+        if (pts) DCD_TRY(launch_absmax_rows(P->values, P->dtype, P->ld, P->n, P->m, gbits, err, st, P->row_scale));
+    }
+    if (fp8) {
         DCD_TRY(launch_quantize_rows(A->values, A->dtype, A->ld, A->m, A->n, rows, A->row_scale, (uint8_t *)pa, n_pad,
                                      rsa, nrows, err, st));
+        DCD_TRY(launch_row_terms_fp8(pa, n_pad, nrows, kp, rh, st, rsa));
+    } else {
+        DCD_TRY(launch_pack_terms(A->values, A->dtype, A->ld, A->m, A->n, rows, pa, pk, n_pad, nrows, kp, rh, err, st,
+                                  A->row_scale, rsa, gbits, rl));
+    }
+    if (from_rows) {
+        DCD_TRY(launch_gather_rows(pa, (int64_t)rb, cols, ncols, A->m, pb, err, st, rh, ch, rsa, rsb, rl, cl));
+    } else if (fp8) {
         DCD_TRY(launch_quantize_rows(P->values, P->dtype, P->ld, P->m, P->n, pcols, P->row_scale, (uint8_t *)pb,
                                      n_pad, rsb, ncols, err, st));
-    } else if (fp16) {
-        // one power-of-two scale for both operands: the largest magnitude over every row of A (the
-        // scale the solver's operand takes) and of the points (err[2])
-        unsigned *gbits = (unsigned *)(err + 2);
-        DCD_TRY(cudaMemsetAsync(gbits, 0, sizeof(unsigned), st));
-        DCD_TRY(cudaMemsetAsync(rsb, 0, sizeof(float) * cpad, st));
-        DCD_TRY(launch_absmax_rows(A->values, A->dtype, A->ld, A->m, A->n, nullptr, A->m, gbits, err, st,
-                                   A->row_scale));
-        if (pts)
-            DCD_TRY(launch_absmax_rows(P->values, P->dtype, P->ld, P->m, P->n, nullptr, P->m, gbits, err, st,
-                                       P->row_scale));
-        DCD_TRY(launch_pack_fp16(A->values, A->dtype, A->ld, A->m, A->n, rows, pa, n_pad, nrows, rsa, gbits, err, st,
-                                 A->row_scale));
-        DCD_TRY(launch_pack_fp16(P->values, P->dtype, P->ld, P->m, P->n, pcols, pb, n_pad, ncols, rsb, gbits, err,
-                                 st, P->row_scale));
+        DCD_TRY(launch_row_terms_fp8(pb, n_pad, ncols, kp, ch, st, rsb));
     } else {
-        DCD_TRY(launch_pack_rows(A->values, A->dtype, A->ld, A->m, A->n, rows, pa, pk, n_pad, nrows, err, st,
-                                 A->row_scale));
-        DCD_TRY(launch_pack_rows(P->values, P->dtype, P->ld, P->m, P->n, pcols, pb, pk, n_pad, ncols, err, st,
-                                 P->row_scale));
+        DCD_TRY(launch_pack_terms(P->values, P->dtype, P->ld, P->m, P->n, pcols, pb, pk, n_pad, ncols, kp, ch, err, st,
+                                  P->row_scale, rsb, gbits, cl));
     }
-    float *rl = accurate ? (float *)(base + orl) : nullptr, *cl = accurate ? (float *)(base + ocl) : nullptr;
-    if (cl) DCD_TRY(cudaMemsetAsync(cl, 0, sizeof(float) * cpad, st));
-    DCD_TRY(launch_row_terms(pa, pk, n_pad, nrows, kp, rh, st, rsa, rl));
-    DCD_TRY(launch_row_terms(pb, pk, n_pad, ncols, kp, ch, st, rsb, cl));
     if (w) DCD_TRY(launch_f64_to_f32(w, ncols, cw, st));
     const int32_t *aids = rows, *bids = cols;
     if (pts) {

@@ -136,8 +136,7 @@ extern "C" dcd_status dcd_kernel_block_static(const dcd_matrix *A, const dcd_ker
         int64_t lda = A->ld;
         if (A->dtype != DCD_F64) {
             double *p = (double *)(base + off_a);
-            STATIC_TRY(launch_pack_rows(A->values, A->dtype, A->ld, A->m, A->n, nullptr, p, PACK_F64, A->n, A->m, err,
-                                        st));
+            STATIC_TRY(launch_pack_rows(A->values, A->dtype, A->ld, A->m, A->n, nullptr, p, A->n, A->m, err, st));
             a64 = p;
             lda = A->n;
         }
@@ -147,10 +146,10 @@ extern "C" dcd_status dcd_kernel_block_static(const dcd_matrix *A, const dcd_ker
         void *pa = base + off_a, *pb = base + off_b;
         float *rh = (float *)(base + off_rh), *ch = (float *)(base + off_ch);
         STATIC_TRY(cudaMemsetAsync(ch, 0, sizeof(float) * (size_t)cpad, st));  // column terms past ncols read as 0
-        STATIC_TRY(launch_pack_rows(A->values, A->dtype, A->ld, A->m, A->n, rows, pa, pk, n_pad, nrows, err, st));
-        STATIC_TRY(launch_pack_rows(A->values, A->dtype, A->ld, A->m, A->n, cols, pb, pk, n_pad, ncols, err, st));
-        STATIC_TRY(launch_row_terms(pa, pk, n_pad, nrows, kp, rh, st));
-        STATIC_TRY(launch_row_terms(pb, pk, n_pad, ncols, kp, ch, st));
+        STATIC_TRY(launch_pack_terms(A->values, A->dtype, A->ld, A->m, A->n, rows, pa, pk, n_pad, nrows, kp, rh, err,
+                                     st));
+        STATIC_TRY(launch_pack_terms(A->values, A->dtype, A->ld, A->m, A->n, cols, pb, pk, n_pad, ncols, kp, ch, err,
+                                     st));
         TcOperand Aop{pa, nrows, n_pad, pk, nullptr, rows}, Bop{pb, ncols, n_pad, pk, nullptr, cols};
         STATIC_TRY(launch_block_tc(Aop, Bop, kp, rh, ch, nullptr, nullptr, nullptr, (float *)out, ldo, nrows, ncols,
                                    err, st));
