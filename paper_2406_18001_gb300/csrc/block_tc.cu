@@ -137,6 +137,14 @@ struct TcArgs {
     const int32_t *row_id;
     const int32_t *col_id;
     int dep_wait;         // apply: the epilogue waits for the grid before this one (griddepcontrol.wait)
+    // apply on pairs, per chunk (or null): every (row tile, N-chunk) unit is an item of its own and its
+    // row sums are written, not added to g: xout[chunk * ldx + row]
+    double *xout;
+    int64_t ldx;
+    // rows given by id (row_id): the first block column that holds row r's own sample, or -1, and
+    // the next column after column c that holds the same row (or null: the ids are compared)
+    const int32_t *row_link;
+    const int32_t *col_next;
 };
 
 // ------------------------------------------------- double-single helpers --
@@ -194,10 +202,15 @@ __device__ __forceinline__ void exp2_ds(float xh, float xl, float &kh, float &kl
     kl = sl * sc;
 }
 
+// an integer as a type (a compile-time argument of a generic lambda)
+template <int V> struct IntC { static constexpr int value = V; };
+
 // K(a_i, b_j) from the accumulator c; rf is the per-row factor: 2 gamma
 // log2(e) (RBF) or 1 (poly, linear), times the row scale in the fp8 and fp16
 // modes (where c already carries the column scale).
-template <int KIND>
+// DEG: the polynomial's degree where it is known (2, 3; the same products in the same order, without
+// a loop per value), else 0.
+template <int KIND, int DEG = 0>
 __device__ __forceinline__ float kf32(float c, float hr, float hc, float rf, const TcArgs &a)
 {
     if (KIND == DCD_RBF) {
@@ -207,6 +220,8 @@ __device__ __forceinline__ float kf32(float c, float hr, float hc, float rf, con
         return c * rf;
     } else {
         float t = fmaf(c, rf, a.coef0), r = t;
+        if (DEG == 2) return t * t;
+        if (DEG == 3) return t * t * t;
         for (int e = 1; e < a.degree; ++e) r *= t;
         return r;
     }
@@ -477,12 +492,23 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     tmem_ld32(tmem_base + lane_addr + buf * (uint32_t)bn + (uint32_t)(cg * 32), v);
                     const int j0 = (cg - cg0) * 32;
                     const int64_t colbase = (int64_t)nc * bn + cg * 32;
+                    // K with the own-sample rule of the RBF (d^2 = 0 where the row and the column are the
+                    // same data row)
+                    auto values = [&](auto deg) {
 #pragma unroll
-                    for (int q = 0; q < 32; ++q) {
-                        const float c = FP8 ? v[q] * ssc[j0 + q] : v[q];
-                        // K with the own-sample rule of the RBF (d^2 = 0 where the row and the column
-                        // are the same data row)
-                        v[q] = KIND == DCD_RBF && rid == sid[j0 + q] ? 1.f : kf32<KIND>(c, hr, sh[j0 + q], rf, a);
+                        for (int q = 0; q < 32; ++q) {
+                            const float c = FP8 ? v[q] * ssc[j0 + q] : v[q];
+                            v[q] = KIND == DCD_RBF && rid == sid[j0 + q]
+                                       ? 1.f
+                                       : kf32<KIND, decltype(deg)::value>(c, hr, sh[j0 + q], rf, a);
+                        }
+                    };
+                    if constexpr (KIND == DCD_POLY) {
+                        if (a.degree == 2) values(IntC<2>());
+                        else if (a.degree == 3) values(IntC<3>());
+                        else values(IntC<0>());
+                    } else {
+                        values(IntC<0>());
                     }
                     // the 32 x 32 group to memory in two 16-column halves through the transpose tile:
                     // lanes 0..15 write columns 0..15 of one row, lanes 16..31 of the next
@@ -734,6 +760,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const int bn = a.bn, bh = bn / 2;
     const int kb_elems = TF32 ? 32 : FP8 ? 128 : 64;
     const uint32_t full0 = ptx::mapa(su32(full), 0), tempty0 = ptx::mapa(su32(tempty), 0);
+    // per-chunk form: item i is chunk i % nxc of tile i / nxc, with one chunk each
+    const int nxc = a.xout ? (int)((a.ncols + bn - 1) / bn) : 1;
+    auto tile_of = [&](int item) { return nxc == 1 ? item : item / nxc; };
+    auto chunk_of = [&](int item) { return nxc == 1 ? 0 : item % nxc; };
     bool ranged;
     int u0, u1, nunits;
     pair_units(a, pair, npairs, ranged, u0, u1, nunits);
@@ -746,7 +776,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         const uint32_t bytes = (uint32_t)(2 * PLANES * (A_STAGE + bh * ROW_BYTES));  // both CTAs'
         UnitIter un(a, pair, npairs, ranged, u0, u1);
         for (int i = 0; ok && i < nunits; ++i, un.next()) {
-            const int ya = un.item * BM2 + (int)rank * BM, yb = un.nc * bn + (int)rank * bh;
+            const int ya = tile_of(un.item) * BM2 + (int)rank * BM, yb = (un.nc + chunk_of(un.item)) * bn + (int)rank * bh;
             for (int kb = 0; kb < a.kblocks; ++kb, ++it) {
                 if (!mbar_wait_warp(&empty[sg], ph ^ 1, abort_flag, a.err)) {
                     ok = false;
@@ -860,8 +890,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         float ph = 0.f, pw = 0.f, ps = 0.f, phl = 0.f;
         int pid = -1;
         double pw64 = 0.0;
-        auto stage_load = [&](int nc) {
-            const int64_t c = (int64_t)nc * bn + cg0 * 32 + jst;
+        auto stage_load = [&](int item, int nc) {
+            const int64_t c = (int64_t)(nc + chunk_of(item)) * bn + cg0 * 32 + jst;
             if (jst >= ncols_h) return;
             const bool in = c < a.ncols;
             if (KIND == DCD_RBF) {
@@ -925,19 +955,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         bool whole = true;      // no other pair holds units of this tile
         // the row terms of the tile after this one, loaded a unit ahead like the column terms
         float n_hr = 0.f, n_hrl = 0.f, n_s = 0.f;
-        int n_rid = -2;
+        int n_rid = -2, n_link = -1, link = -1;
         const float cs0 = FP16 ? a.col_s[0] : 0.f;
         auto row_load = [&](int it2) {
-            const int64_t r = (int64_t)it2 * BM2 + (int64_t)rank * BM + row_in_tile;
+            const int64_t r = (int64_t)tile_of(it2) * BM2 + (int64_t)rank * BM + row_in_tile;
             const bool in = r < a.nrows_out;
             n_hr = (KIND == DCD_RBF && in) ? a.row_h[r] : 0.f;
             if (ACC) n_hrl = (KIND == DCD_RBF && in) ? a.row_hl[r] : 0.f;
             if (SL || SCALED) n_s = in ? a.row_s[r] : 0.f;
             n_rid = in ? (a.row_id ? a.row_id[r] : (int)r) : -2;
+            if (KIND == DCD_RBF && !ACC) n_link = a.row_link && in ? a.row_link[r] : -1;
         };
         UnitIter un(a, pair, npairs, ranged, u0, u1);
         if (nunits > 0) {
-            stage_load(un.nc);
+            stage_load(un.item, un.nc);
             row_load(un.item);
         }
         int prev_item = -1;
@@ -948,11 +979,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             cid = (const int *)(cst + 512);
             if (item != prev_item) {  // first chunk of a tile in this pair's units
                 prev_item = item;
-                row = (int64_t)item * BM2 + (int64_t)rank * BM + row_in_tile;
+                row = (int64_t)tile_of(item) * BM2 + (int64_t)rank * BM + row_in_tile;
                 row_ok = row < a.nrows_out;
                 hr = n_hr;
                 hrl = n_hrl;
                 rid = n_rid;
+                link = n_link;
                 wr0 = __shfl_sync(0xffffffffu, rid, 0);
                 if (SL) rsl = n_s * 0x1p-12f;  // 2^(e_i - 12)
                 const float rsc = !SCALED ? 1.f : !row_ok ? 0.f : FP8 ? n_s : n_s * cs0;
@@ -965,7 +997,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             // this unit's column terms to the half's staging buffer, then the loads of the next unit's
             stage_store();
             if (i + 1 < nunits) {
-                stage_load(un.nc);
+                stage_load(un.item, un.nc);
                 if (un.item != item) row_load(un.item);
             }
             const uint32_t buf = acc_it % NACC, aph = (acc_it / NACC) & 1;
@@ -977,7 +1009,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             __syncwarp();
             // the row's gradient (and scale), loaded beside the tile's last chunk
             double g_old = 0.0, g_rs = 1.0;
-            if (last && whole && !half && row_ok) {
+            if (last && whole && !half && row_ok && !a.xout) {
                 g_old = a.g[row];
                 if (a.rs) g_rs = a.rs[row];
             }
@@ -990,8 +1022,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             // the column groups that hold an own sample of the warp's 32 rows: each lane tests one
             // column id of every group (rows given by id: every group is tested column by column)
             unsigned ghit = 0;
+            unsigned ownw[4] = {0u, 0u, 0u, 0u};  // rows with links: the own columns of the half's groups
             if (KIND == DCD_RBF && !ACC) {
-                if (a.row_id) {
+                if (a.row_link) {
+                    const int cb = (nc + chunk_of(item)) * bn + cg0 * 32;
+                    for (int q = link; q >= 0; q = a.col_next[q]) {  // rarely one, hardly ever two
+                        const int j = q - cb;
+#pragma unroll
+                        for (int w = 0; w < 4; ++w)
+                            if ((j >> 5) == w && j < ncols_h) ownw[w] |= 1u << (j & 31);
+                    }
+#pragma unroll
+                    for (int w = 0; w < 4; ++w)
+                        if (__any_sync(0xffffffffu, ownw[w] != 0u)) ghit |= 1u << w;
+                } else if (a.row_id) {
                     ghit = 0xfu;
                 } else {
 #pragma unroll
@@ -1011,7 +1055,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             // same sums in the same order as a column-by-column loop
             // the 32 columns' kernel values (`own`: bit q set where column q is this row's own
             // sample, d^2 = 0 there; the checked form runs only for the rare groups that hold one)
-            auto group_terms = [&](const uint32_t(&r)[32], int j0, unsigned own, float &p0, float &p1) {
+            auto group_terms = [&](const uint32_t(&r)[32], int j0, unsigned own, float &p0, float &p1, auto deg) {
+                constexpr int DEG = decltype(deg)::value;
                 if (KIND == DCD_RBF && !FP8 && !ACC && !own && fast_cols && fast_row) {
                     // K_ij w_j = 2^(rf c - h_i) (w_j 2^(-h_j)): the exponent's row and column terms split
                     // apart (both <= RBF_FACTOR_HMAX, so neither factor leaves the FP32 range); rf c <=
@@ -1043,8 +1088,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         c2 *= ss.z;
                         c3 *= ss.w;
                     }
-                    float k0 = kf32<KIND>(c0, hr, hh.x, rf, a), k1 = kf32<KIND>(c1, hr, hh.y, rf, a);
-                    float k2 = kf32<KIND>(c2, hr, hh.z, rf, a), k3 = kf32<KIND>(c3, hr, hh.w, rf, a);
+                    float k0 = kf32<KIND, DEG>(c0, hr, hh.x, rf, a), k1 = kf32<KIND, DEG>(c1, hr, hh.y, rf, a);
+                    float k2 = kf32<KIND, DEG>(c2, hr, hh.z, rf, a), k3 = kf32<KIND, DEG>(c3, hr, hh.w, rf, a);
                     if (own) {
                         k0 = (own >> (4 * q4)) & 1u ? 1.f : k0;
                         k1 = (own >> (4 * q4 + 1)) & 1u ? 1.f : k1;
@@ -1064,7 +1109,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 // the own-sample columns of this thread's row, in the groups that may hold one
                 unsigned own = 0;
                 if (KIND == DCD_RBF && ((ghit >> (j0 >> 5)) & 1u)) {
-                    if (!a.row_id) {
+                    if (a.row_link) {
+                        own = j0 == 0 ? ownw[0] : j0 == 32 ? ownw[1] : j0 == 64 ? ownw[2] : ownw[3];
+                    } else if (!a.row_id) {
                         const unsigned off = (unsigned)(cid[j0 + lane] - wr0);
                         unsigned hits = __ballot_sync(0xffffffffu, rid >= 0 && off < 32u);
                         while (hits) {
@@ -1076,8 +1123,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         for (int q = 0; q < 32; ++q) own |= (cid[j0 + q] == rid ? 1u : 0u) << q;
                     }
                 }
-                if (own) group_terms(r, j0, own, p0, p1);
-                else group_terms(r, j0, 0u, p0, p1);
+                if constexpr (KIND == DCD_POLY) {
+                    if (a.degree == 2) group_terms(r, j0, 0u, p0, p1, IntC<2>());
+                    else if (a.degree == 3) group_terms(r, j0, 0u, p0, p1, IntC<3>());
+                    else group_terms(r, j0, 0u, p0, p1, IntC<0>());
+                } else {
+                    if (own) group_terms(r, j0, own, p0, p1, IntC<0>());
+                    else group_terms(r, j0, 0u, p0, p1, IntC<0>());
+                }
                 float a0, b0, e0;
                 two_sum(p0, p1, a0, b0);
                 two_sum(cs_h, a0, cs_h, e0);
@@ -1234,7 +1287,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 const double tot = tacc + xc[row_in_tile];
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&xfree[xb]);
-                if (row_ok) a.g[row] = g_old + g_rs * tot;
+                if (row_ok) {
+                    if (a.xout) a.xout[chunk_of(item) * a.ldx + row] = tot;
+                    else a.g[row] = g_old + g_rs * tot;
+                }
             }
         }
     }
@@ -1363,6 +1419,15 @@ cudaError_t launch_mode2(int npairs, const CUtensorMap &mA, const CUtensorMap &m
 
 }  // namespace
 
+int tc_store_items(int64_t nrows, int64_t ncols, int bn, bool lower)
+{
+    const int tiles = (int)((nrows + BM - 1) / BM), chunks = (int)((ncols + bn - 1) / bn);
+    if (!lower) return tiles * chunks;
+    int items = 0;
+    for (int t = 0; t < tiles; ++t) items += lower_chunks(t, bn, chunks);
+    return items;
+}
+
 bool tc_available()
 {
     int dev = 0, major = 0, minor = 0;
@@ -1405,7 +1470,7 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
                             const float *col_h, const float *col_w, const double *rs, double *g, float *out,
                             int64_t ldo, int64_t nrows_out, int64_t ncols, int *err, cudaStream_t st, bool lower,
                             const TcSplit *split, bool pdl, int max_pairs, const TcAccurate *acc, bool pdl_wait,
-                            int prio)
+                            int prio, const TcCross *cross)
 {
     if (nrows_out <= 0 || ncols <= 0) return cudaSuccess;
     // the accurate apply epilogue: split-tf32 or sliced operands, FP64 coefficients, RBF terms as hi + lo
@@ -1423,10 +1488,14 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
     if (Aop.n_pad % kb_elems) return cudaErrorInvalidValue;
     int bn = (int)((ncols + 31) / 32) * 32;
     if (bn > (sliced ? SLICED_BN : BN_MAX)) bn = sliced ? SLICED_BN : BN_MAX;
-    // store mode (the sampled Gram) has few rows: narrower N-chunks give
-    // more work items and spread them over more SMs -- unless it is held to a
-    // few CTAs (max_pairs), where wide chunks mean fewer, longer items
-    if (out != nullptr && max_pairs <= 0) bn = bn > 64 ? 64 : bn;
+    // store mode (the sampled Gram) has few rows: narrower N-chunks give more work items and spread
+    // them over more SMs; held to a few CTAs (max_pairs), the narrowest chunks that still give each
+    // CTA one item
+    if (out != nullptr) {
+        const int bn0 = bn;
+        for (bn = bn0 < 64 ? bn0 : 64; max_pairs > 0 && bn < bn0 && tc_store_items(nrows_out, ncols, bn, lower) > max_pairs;)
+            bn = 2 * bn < bn0 ? 2 * bn : bn0;
+    }
     // the apply form runs on CTA pairs (each CTA stages half of an N-chunk of B)
     const bool pair = out == nullptr;
     CUtensorMap mA, mB;
@@ -1450,11 +1519,7 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
     a.bn = bn;
     a.store = out != nullptr;
     a.lower = a.store && lower;
-    a.items = a.store ? a.num_tiles * a.nchunks : a.num_tiles;
-    if (a.lower) {
-        a.items = 0;
-        for (int t = 0; t < a.num_tiles; ++t) a.items += lower_chunks(t, a.bn, a.nchunks);
-    }
+    a.items = a.store ? tc_store_items(nrows_out, ncols, bn, a.lower) : a.num_tiles;
     a.degree = kp.degree;
     a.two_gl = (float)(2.0 * kp.gamma * 1.4426950408889634);
     a.coef0 = (float)kp.coef0;
@@ -1466,6 +1531,15 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
     a.row_id = Aop.ids;
     a.col_id = Bop.ids;
     a.dep_wait = pdl_wait ? 1 : 0;
+    a.xout = cross ? cross->out : nullptr;
+    a.ldx = cross ? cross->ld : 0;
+    a.row_link = cross ? cross->row_link : nullptr;
+    a.col_next = cross ? cross->col_next : nullptr;
+    if (cross) {  // per chunk: the units are the items
+        if (!pair || acc || !cross->out || (cross->row_link && !cross->col_next)) return cudaErrorInvalidValue;
+        a.items = a.num_tiles * a.nchunks;
+        a.nchunks = 1;
+    }
     a.row_hl = acc ? acc->row_hl : nullptr;
     a.col_hl = acc ? acc->col_hl : nullptr;
     a.col_w64 = acc ? acc->w64 : nullptr;
@@ -1483,7 +1557,7 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
         if ((int64_t)a.num_tiles * a.nchunks >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
         int npairs = a.items < sms / 2 ? a.items : sms / 2;
         if (max_pairs > 0 && npairs > max_pairs) npairs = max_pairs;
-        if (split && split->part && split->cnt && split->pairs >= npairs && split->chunks >= a.nchunks) {
+        if (!cross && split && split->part && split->cnt && split->pairs >= npairs && split->chunks >= a.nchunks) {
             a.part = split->part;
             a.cnt = split->cnt;
             a.late_pairs = split->late_pairs;

@@ -179,6 +179,8 @@ __host__ __device__ inline int64_t packed_row_bytes(int kind, int64_t n_pad)
                                                         : 2 * n_pad;
 }
 bool tc_available();
+// the store form's work items with N-chunks of bn columns (128-row tiles; lower: those that reach the diagonal)
+int tc_store_items(int64_t nrows, int64_t ncols, int bn, bool lower);
 // lower (store form only): write only the N-chunks that reach the diagonal
 // (column chunk start <= last row of the tile); the rest of out is left as is
 //
@@ -214,6 +216,16 @@ inline int tc_split_chunks(int64_t ncols) { return ncols <= 128 ? 1 : (int)((nco
 // low parts of the RBF terms from launch_row_terms(..., h_lo) (RBF only).
 // Columns past ncols read as zero coefficients.  On sliced operands the dot
 // products come from the slices' exact integer sums (4 group accumulators).
+// The apply form of few rows against a step's columns (cross): the row sums of each N-chunk of 256
+// columns are written apart, out[chunk * ld + row], instead of added to g, and each (row tile, chunk)
+// is a unit of its own, so that the block spreads over as many CTA pairs.  row_link, col_next
+// (optional, rows given by ids): row r's own sample among the columns -- its first column or -1,
+// and the column after column c that holds the same row or -1 -- instead of comparing the ids.
+struct TcCross {
+    double *out = nullptr;
+    int64_t ld = 0;
+    const int32_t *row_link = nullptr, *col_next = nullptr;
+};
 struct TcAccurate {
     const double *w64 = nullptr;
     const float *row_hl = nullptr;
@@ -224,7 +236,7 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
                             double *g, float *out, int64_t ldo, int64_t nrows_out, int64_t ncols,
                             int *err, cudaStream_t st, bool lower = false, const TcSplit *split = nullptr,
                             bool pdl = false, int max_pairs = 0, const TcAccurate *acc = nullptr,
-                            bool pdl_wait = true, int prio = 0);
+                            bool pdl_wait = true, int prio = 0, const TcCross *cross = nullptr);
 // (pdl: launched as the programmatic dependent of the kernel before it in the stream, whose
 // results the epilogue waits for unless pdl_wait is false: a block that reads nothing the
 // kernel before it writes, started once that kernel has started.  prio: the launch's scheduling
@@ -284,9 +296,10 @@ cudaError_t launch_fill_f64(double *p, double v, int64_t count, cudaStream_t st)
 cudaError_t launch_iota(int32_t *out, int64_t count, int64_t start, cudaStream_t st);
 cudaError_t launch_init_grad(int problem, const double *y, const double *alpha, double diag, int64_t m, double *g,
                              cudaStream_t st);
-// the deferred gradient (solver.cu): acc[p] += add[p] (add may be NULL) + diag * (the sum of dprev
-// over the previous step's positions q holding row S[p], in position order) where any does -- the
-// update's part of the gradient at the next step's rows.  cprev <= 8192.
+// the deferred gradient (solver.cu): link[p] = the first position q of the previous step with Sprev[q]
+// == S[p], or -1.  cprev <= 8192.
+cudaError_t launch_defer_links(const int32_t *S, int64_t cnt, const int32_t *Sprev, int64_t cprev, int32_t *link,
+                               cudaStream_t st);
 // the deferred K-SVM step (sample_update.cu): alpha and g at S (before they change), and the
 // pending parts of the next step's alpha and g from this step's Kx = K(A_S, A_Sc) (row-major,
 // leading dimension ldx), theta and w = y theta
@@ -295,8 +308,6 @@ cudaError_t launch_dcd_snapshot(const int32_t *S, int64_t cnt, int64_t m, const 
 cudaError_t launch_dcd_pending(const int32_t *S, int64_t cnt, const double *y, const void *Kx, bool kx_f64,
                                int64_t ldx, const int32_t *Sc, const double *theta, const double *w, int64_t cc,
                                double diag, double *alpha_add, double *g_add, cudaStream_t st);
-cudaError_t launch_defer_repeat(const int32_t *S, int64_t cnt, const int32_t *Sprev, const double *dprev,
-                                int64_t cprev, double diag, const double *add, double *acc, cudaStream_t st);
 // (pdl: launched as the programmatic dependent of the kernel before it, whose results it does not
 // read; it signals its own dependent at once)
 cudaError_t launch_update(const int32_t *S, const double *delta, int64_t cnt, double diag, double *alpha,
@@ -423,6 +434,15 @@ struct FusedUpdate {
 // scratch of recur_cluster_scratch_bytes (super-block inverses, repeat masks and links)
 int recur_cluster_size(int nblk, int b, int rounds);
 size_t recur_cluster_scratch_bytes(int64_t nblk, int b);
+// The deferred gradient's right-hand side -(g[S_p] + sum_h x[h ldx + p] + mdiag (the sum of delta over the
+// previous step's positions that hold the row: link[p] the first or -1, next[q] the one after q)).
+struct ClusterRhs {
+    const double *x = nullptr;
+    int nx = 0;
+    int64_t ldx = 0;
+    const int32_t *link = nullptr, *next = nullptr;
+    const double *delta = nullptr;
+};
 // rhs: the right-hand sides by position (default -g[S]), for a diagonal panel of a longer chain
 cudaError_t launch_recur_cluster(const float *Kss, int64_t ldk, const int32_t *S, int nblk, int b, int P,
                                  double lambda, double mdiag, double *g, int rounds, void *scratch, double *delta,
@@ -437,11 +457,12 @@ cudaError_t launch_recur_cluster_chain(const float *Kss, int64_t ldk, const int3
                                        double lambda, double mdiag, double *g, int rounds, void *scratch,
                                        double *delta, double *w64, float *w32, const FusedUpdate *upd, int *err,
                                        cudaStream_t st, const double *rhs = nullptr, int trig_sup = -1,
-                                       bool rhs_add_g = false, int prio = 0);
+                                       const ClusterRhs *x = nullptr, int prio = 0);
 // (trig_sup: the super-block of 32 rows after whose first-round result a
 // kernel launched as this one's programmatic dependent may start; -1: at once.
-// rhs_add_g: the right-hand side is -(g[S] + rhs), rhs holding a part of the
-// gradient not yet added to g)
+// x: the part of the gradient at the rows that is not yet in g)
+// the links between a super-block scratch's positions that hold the same row (next position, or -1)
+const int32_t *recur_cluster_next(const void *scratch, int nblk, int b);
 // 2-D tensor map over a row-major fp32 matrix (rows x cols, leading dimension
 // ld elements, ld * 4 a multiple of 16), box of box_rows x box_cols, no
 // swizzle, out-of-range elements read as zero (block_tc.cu)

@@ -352,8 +352,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
     bdcd_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const int32_t *S, const float *X,
                         const float *Ng, const uint32_t *Mg, const int32_t *nextg, int nblk, int b, double lambda,
                         double mdiag, double *g, int rounds, double *delta, double *w64, float *w32, double *alpha,
-                        uint64_t *ctr, uint64_t ctr_advance, const double *rhs_in, int rhs_add_g, int trig_sup,
-                        int *err)
+                        uint64_t *ctr, uint64_t ctr_advance, const double *rhs_in, ClusterRhs x, int trig_sup, int *err)
 {
     extern __shared__ __align__(16) unsigned char sm[];
     const int P = (int)gridDim.x;  // the grid is one cluster
@@ -383,12 +382,24 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
     // gradient.  The CTA owning super-block trig_sup signals when its round-0 Delta is out (the
     // kernels forked beside the chain have the other SMs until then); every other CTA at once.
     const bool trig_own = trig_sup >= 0 && (trig_sup == cl_own(0, c, P) || (nown > 1 && trig_sup == cl_own(1, c, P)));
-    // -(g_S + rhs_in) is read before this CTA signals: a dependent may write g once every CTA has
+    // -(g_S + the part of the gradient not yet in g) is read before this CTA signals: a dependent may
+    // write g once every CTA has
     __shared__ double rhs_pre[CL_SLOTS * 32];
-    if (rhs_in && rhs_add_g) {
+    if (x.x) {
         for (int e = tid; e < nown * 32; e += CL_THREADS) {
             const int k = e >> 5, i = e & 31, J = cl_own(k, c, P);
-            if (i < cl_rows(J, Bs, sb)) rhs_pre[e] = -(g[S[J * Bs + i]] + rhs_in[J * Bs + i]);
+            if (i >= cl_rows(J, Bs, sb)) continue;
+            const int p = J * Bs + i;
+            const int32_t row = S[p];
+            int q = x.link[p];
+            double v = 0.0;
+            for (int h = 0; h < x.nx; ++h) v += x.x[(int64_t)h * x.ldx + p];
+            if (q >= 0) {  // rare: the previous step's positions that hold this row, in order
+                double sum = 0.0;
+                for (; q >= 0; q = x.next[q]) sum += x.delta[q];
+                v += mdiag * sum;
+            }
+            rhs_pre[e] = -(g[row] + v);
         }
         __syncthreads();
     }
@@ -468,12 +479,12 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
         // ---- the chain of round r ----
         // r'_J: all updates but the one from J-1, which N_J = X_J L_{J,J-1} applies after the product:
         // Delta_J = X_J r'_J - N_J Delta_{J-1}.  X_J r'_J is formed while Delta_{J-1} is on its way.
-        // the right-hand side: -g_S; or given (rhs_in); or -(g_S + rhs_in), a part of the gradient
-        // not yet in g added first (rhs_add_g; read at the start)
+        // the right-hand side: -g_S; or given (rhs_in); or with a part of the gradient not yet in g
+        // added first (x; read at the start)
         const double rhs = lane >= rows ? 0.0
-                           : !rhs_in    ? -g[S[row]]
-                           : rhs_add_g  ? rhs_pre[slot * 32 + lane]
-                                        : rhs_in[row];
+                           : x.x        ? rhs_pre[slot * 32 + lane]
+                           : rhs_in     ? rhs_in[row]
+                                        : -g[S[row]];
         float rr = r == 0 ? (float)rhs : 0.f;  // round 0: -g_S minus updates; round 1: sum of updates
         float hi = 0.f, lo = 0.f;              // round 0: double-single sum of L_{row, T<J} Delta0_T
         bool alive = J == 0 || wait_local(pbar, abort_flag, err);
@@ -686,10 +697,16 @@ cudaError_t launch_recur_cluster_prep(const float *Kss, int64_t ldk, const int32
     return cudaGetLastError();
 }
 
+const int32_t *recur_cluster_next(const void *scratch, int nblk, int b)
+{
+    const ClGeom G = cl_geom(nblk, b);
+    return (const int32_t *)((const float *)scratch + 2 * (size_t)G.nsup * 1024 + (size_t)G.nsup * CL_NSUP_MAX * 32);
+}
+
 cudaError_t launch_recur_cluster_chain(const float *Kss, int64_t ldk, const int32_t *S, int nblk, int b, int P,
                                        double lambda, double mdiag, double *g, int rounds, void *scratch,
                                        double *delta, double *w64, float *w32, const FusedUpdate *upd, int *err,
-                                       cudaStream_t st, const double *rhs, int trig_sup, bool rhs_add_g, int prio)
+                                       cudaStream_t st, const double *rhs, int trig_sup, const ClusterRhs *x, int prio)
 {
     const ClGeom G = cl_geom(nblk, b);
     const int sb = nblk * b;
@@ -728,7 +745,7 @@ cudaError_t launch_recur_cluster_chain(const float *Kss, int64_t ldk, const int3
     return cudaLaunchKernelEx(&cfg, kfn, kmap, S, (const float *)X, (const float *)N, (const uint32_t *)M,
                               (const int32_t *)next, nblk, b, lambda, mdiag, g, rounds, delta, w64, w32,
                               upd ? upd->alpha : (double *)nullptr, upd ? upd->ctr : (uint64_t *)nullptr,
-                              upd ? upd->ctr_advance : (uint64_t)0, rhs, rhs_add_g ? 1 : 0, trig_sup, err);
+                              upd ? upd->ctr_advance : (uint64_t)0, rhs, x ? *x : ClusterRhs{}, trig_sup, err);
 }
 
 cudaError_t launch_recur_cluster(const float *Kss, int64_t ldk, const int32_t *S, int nblk, int b, int P,

@@ -593,50 +593,39 @@ cudaError_t launch_dcd_pending(const int32_t *S, int64_t cnt, const double *y, c
     return cudaGetLastError();
 }
 
-// acc[p] += add[p] (add: optional) + diag * sum of dprev[q] over q with
-// Sprev[q] == S[p] (in position order, the update's own sum), where any q
-// matches: the update's part of the gradient at a row the next step samples.
-// One warp per position p, Sprev staged in shared memory, 32 positions q per
-// ballot.
+// link[p] = the first position q of the previous step with Sprev[q] == S[p], or -1: where the
+// update's part of the gradient at a row the next step samples is found.  One warp per position p,
+// Sprev staged in shared memory, 32 positions q per ballot.  It needs the samples only, so it runs
+// beside the recurrence; the recurrence after it adds the sums (the sums formed here, after the
+// recurrence they come from, were 5 us of the loop of steps).
 constexpr int REP_WARPS = 8;
 
 __global__ void __launch_bounds__(REP_WARPS * 32)
-    defer_repeat_kernel(const int32_t *S, int64_t cnt, const int32_t *Sprev, const double *dprev, int cprev,
-                        double diag, const double *add, double *acc)
+    defer_links_kernel(const int32_t *S, int64_t cnt, const int32_t *Sprev, int cprev, int32_t *link)
 {
-    __shared__ int32_t sp[UPD_MAX];
+    extern __shared__ int32_t sp[];  // as much as the step needs, so that the CTAs fit beside the block's
     for (int q = threadIdx.x; q < cprev; q += blockDim.x) sp[q] = Sprev[q];
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t p = (int64_t)blockIdx.x * REP_WARPS + (threadIdx.x >> 5);
     if (p >= cnt) return;  // warp-uniform
     const int32_t key = S[p];
-    double sum = 0.0;
-    bool any = false;
-    for (int q0 = 0; q0 < cprev; q0 += 32) {
+    int first = -1;
+    for (int q0 = 0; q0 < cprev && first < 0; q0 += 32) {
         const int q = q0 + lane;
-        unsigned hit = __ballot_sync(0xffffffffu, q < cprev && sp[q] == key);
-        any = any || hit != 0u;
-        while (hit) {  // rare: the matches in position order (every lane the same sum)
-            sum += dprev[q0 + __ffs(hit) - 1];
-            hit &= hit - 1u;
-        }
+        const unsigned hit = __ballot_sync(0xffffffffu, q < cprev && sp[q] == key);
+        if (hit) first = q0 + __ffs(hit) - 1;
     }
-    if (lane == 0) {
-        double v = acc[p];
-        if (add) v += add[p];
-        if (any) v += diag * sum;
-        acc[p] = v;
-    }
+    if (lane == 0) link[p] = first;
 }
 
-cudaError_t launch_defer_repeat(const int32_t *S, int64_t cnt, const int32_t *Sprev, const double *dprev,
-                                int64_t cprev, double diag, const double *add, double *acc, cudaStream_t st)
+cudaError_t launch_defer_links(const int32_t *S, int64_t cnt, const int32_t *Sprev, int64_t cprev, int32_t *link,
+                               cudaStream_t st)
 {
     if (cnt <= 0) return cudaSuccess;
     if (cprev > UPD_MAX) return cudaErrorInvalidValue;
-    defer_repeat_kernel<<<(unsigned)((cnt + REP_WARPS - 1) / REP_WARPS), REP_WARPS * 32, 0, st>>>(
-        S, cnt, Sprev, dprev, (int)cprev, diag, add, acc);
+    defer_links_kernel<<<(unsigned)((cnt + REP_WARPS - 1) / REP_WARPS), REP_WARPS * 32, sizeof(int32_t) * cprev, st>>>(
+        S, cnt, Sprev, (int)cprev, link);
     return cudaGetLastError();
 }
 

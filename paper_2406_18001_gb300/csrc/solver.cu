@@ -74,8 +74,8 @@ dcd_status csc_choose(const CsrOperand &ca, bool fp64, int64_t cnt, int maxrow, 
 
 constexpr int64_t SB_MAX = 8192;   // s*b per outer step
 constexpr int B_MAX = 128;         // block size
-constexpr int DF_XPAIRS = 8;       // CTA pairs (at most) of the deferred gradient's cross product
-constexpr int DF_GRAM_CTAS = 8;    // CTAs of the Gram computed beside the deferred step's block
+constexpr int DF_XPAIRS = 16;      // CTA pairs (at most) of the deferred gradient's cross product
+constexpr int DF_GRAM_CTAS = 24;   // CTAs (at most) of the Gram computed beside the deferred step's block
 
 // Set while the batched driver and the autotuner build their plans: those
 // capture many plans' steps into one graph and run without the look-ahead.
@@ -294,22 +294,21 @@ struct Solver {
     ~Solver()
     {
         if (graph_exec) cudaGraphExecDestroy(graph_exec);
-        for (auto &ge : graph_la)
-            if (ge) cudaGraphExecDestroy(ge);
+        for (auto &row : graph_steps)
+            for (auto &ge : row)
+                if (ge) cudaGraphExecDestroy(ge);
         if (st2) {
             cudaStreamSynchronize(st2);
             cudaStreamDestroy(st2);
         }
         if (la_fork) cudaEventDestroy(la_fork);
         if (la_join) cudaEventDestroy(la_join);
-        for (auto &ge : graph_df)
-            if (ge) cudaGraphExecDestroy(ge);
         for (cudaStream_t sx : {st3, st4})
             if (sx) {
                 cudaStreamSynchronize(sx);
                 cudaStreamDestroy(sx);
             }
-        for (cudaEvent_t ev : {df_fork, df_chained, df_rows, df_gram, df_side, df_xfork, df_xjoin, df_kx})
+        for (cudaEvent_t ev : {df_fork, df_chained, df_rows, df_gram, df_side, df_kx})
             if (ev) cudaEventDestroy(ev);
         if (ws_csr) cudaFreeAsync(ws_csr, st);
         for (void *w : ws_csr2)
@@ -470,10 +469,10 @@ struct Solver {
             // the kernel values of the step after next's rows against the next step's
             double *dsn = (double *)ar.take(dfs_pos ? 12 * sizeof(double) * col_pad : 0);
             void *dkx = ar.take(dfs_pos ? (size_t)sb * sb * (tc ? 4 : 8) : 0);
-            double *dfx = (double *)ar.take(df_pos ? 4 * sizeof(double) * col_pad : 0);  // x of sets 0-2, x2
-            double *xsp =
-                (double *)ar.take(df_pos ? 2 * sizeof(double) * tc_split_part_elems(DF_XPAIRS, split_chunks) : 0);
-            unsigned *xsc = (unsigned *)ar.take(df_pos ? 2 * sizeof(unsigned) * 2 * DF_XPAIRS : 0);
+            // x of sets 0-2, a part per chunk of 256 columns, and the links to the step before
+            const int64_t xparts = (sb + 255) / 256;
+            double *dfx = (double *)ar.take(df_pos ? 3 * sizeof(double) * xparts * col_pad : 0);
+            int32_t *dfl = (int32_t *)ar.take(df_pos ? 3 * sizeof(int32_t) * col_pad : 0);
             // the balanced split of the tensor-core apply over CTA pairs
             double *tsp = (double *)ar.take(tcd ? sizeof(double) * tc_split_part_elems(split_pairs, split_chunks) : 0);
             unsigned *tsc = (unsigned *)ar.take(tcd ? sizeof(unsigned) * 2 * split_pairs : 0);
@@ -571,19 +570,13 @@ struct Solver {
                     sbuf[q].w64 = dfd + (size_t)(2 * q - 1) * col_pad;
                     sbuf[q].col_w = dfw + (size_t)(q - 1) * col_pad;
                 }
-            for (int q = 0; q < 3; ++q) df_x[q] = df_pos ? dfx + (size_t)q * col_pad : nullptr;
+            for (int q = 0; q < 3; ++q) {
+                df_x[q] = df_pos ? dfx + (size_t)q * xparts * col_pad : nullptr;
+                df_link[q] = df_pos ? dfl + (size_t)q * col_pad : nullptr;
+            }
             for (int q = 0; q < 3; ++q)
                 for (int k = 0; k < 4; ++k) dfs_v[q][k] = dfs_pos ? dsn + (size_t)(4 * q + k) * col_pad : nullptr;
             dfs_kx = dkx;
-            df_x2 = df_pos ? dfx + 3 * (size_t)col_pad : nullptr;
-            xsplit2.part = df_pos ? xsp + tc_split_part_elems(DF_XPAIRS, split_chunks) : nullptr;
-            xsplit2.cnt = df_pos ? xsc + 2 * DF_XPAIRS : nullptr;
-            xsplit2.pairs = df_pos ? DF_XPAIRS : 0;
-            xsplit.part = xsp;
-            xsplit.cnt = xsc;
-            xsplit.pairs = df_pos ? DF_XPAIRS : 0;
-            xsplit.chunks = df_pos ? split_chunks : 0;
-            xsplit2.chunks = df_pos ? split_chunks : 0;
             ctr_la = crl;
             if (tcd) {
                 tsplit.part = tsp;
@@ -629,20 +622,19 @@ struct Solver {
             DCD_TRY(cudaMemsetAsync(sbuf[2].col_h, 0, sizeof(float) * col_pad, st));
             DCD_TRY(cudaMemsetAsync(sbuf[2].As, 0, (size_t)sb * row_bytes, st));
             if (scaled) DCD_TRY(cudaMemsetAsync(sbuf[2].col_s, 0, sizeof(float) * col_pad, st));
-            DCD_TRY(cudaMemsetAsync(xsplit.cnt, 0, 2 * sizeof(unsigned) * 2 * DF_XPAIRS, st));
             DCD_TRY(cudaEventCreateWithFlags(&df_fork, cudaEventDisableTiming));
             DCD_TRY(cudaEventCreateWithFlags(&df_chained, cudaEventDisableTiming));
             DCD_TRY(cudaEventCreateWithFlags(&df_side, cudaEventDisableTiming));
             DCD_TRY(cudaEventCreateWithFlags(&df_rows, cudaEventDisableTiming));
             DCD_TRY(cudaEventCreateWithFlags(&df_gram, cudaEventDisableTiming));
             DCD_TRY(cudaStreamCreateWithFlags(&st3, cudaStreamNonBlocking));
-            DCD_TRY(cudaStreamCreateWithFlags(&st4, cudaStreamNonBlocking));
-            DCD_TRY(cudaEventCreateWithFlags(&df_xfork, cudaEventDisableTiming));
-            DCD_TRY(cudaEventCreateWithFlags(&df_xjoin, cudaEventDisableTiming));
-            // the block leaves SMs for the recurrence ahead (one cluster) and the next step's Gram
-            // (measured at config 2: 64 of 76 pairs 88.0 us per step, 66 90.0, 68 100.5, 60 88.8)
+            // the block leaves SMs for the recurrence ahead (one cluster) and the next step's Gram (an
+            // item a CTA; its chunks are 256 columns at most)
             const int P = recur_cluster_size((int)o.s, o.b, 2);
-            df_pairs = std::max(split_pairs - (P + 1) / 2 - DF_GRAM_CTAS / 2, 1);
+            int gi = tc_store_items(sb, sb, 64, true);
+            for (int w = 128; gi > DF_GRAM_CTAS && w <= 256; w *= 2) gi = tc_store_items(sb, sb, w, true);
+            df_gram_ctas = std::min(gi, DF_GRAM_CTAS);
+            df_pairs = std::max(split_pairs - (P + 1) / 2 - (df_gram_ctas + 1) / 2, 1);
             int p_least = 0, p_greatest = 0;
             DCD_TRY(cudaDeviceGetStreamPriorityRange(&p_least, &p_greatest));
             df_prio = p_greatest;
@@ -1167,8 +1159,57 @@ struct Solver {
     int la_par = 0;        // the buffer set holding the next step's products
     int64_t la_cnt = 0;    // their step size (0: none pending)
     bool ref_shared = false;  // the recomputed gradient uses the step operand's buffers
-    cudaGraphExec_t graph_la[2] = {nullptr, nullptr};
-    int la_direct[2] = {0, 0};
+
+    // ---- replayed steps of the look-ahead bodies ----
+    // Graphs of 1, 3, 7 and 15 consecutive steady bodies, by the buffer set they start with; body(q) enqueues one on set q, the next on set q + 1 mod nsets.  Between two
+    // launches the GPU stands still for 5-7 us, within a graph a body follows in about one, so the
+    // longest graph that fits the steps to run is taken -- but one body where the stream is idle, as its
+    // kernels are submitted soonest and the long graph's while it runs (K-SVM FP64 at m = 2000, s = 8:
+    // 18.2 -> 15.0 us a step; K-RR fp16 at m = 50000, s = 64: GRAPH_KRR).  A graph is captured once every set has run a body
+    // directly (attributes and occupancy queries are then cached) and, the long ones, once the plan's
+    // steps so far and at hand pay for the capture (about 25 us a body against 5 us a step saved).
+    static constexpr int GRAPH_LENS = 4;
+    cudaGraphExec_t graph_steps[GRAPH_LENS][3] = {};
+    int body_direct[3] = {0, 0, 0};
+    bool idle = true;  // nothing of this plan is running or queued on the stream
+
+    template <class Body>
+    dcd_status replay_steps(int q, int nsets, int64_t avail, Body body, int64_t *ran)
+    {
+        const int lens[GRAPH_LENS] = {1, 3, 7, 15};
+        const int64_t worth[GRAPH_LENS] = {0, 32, 64, 128};
+        bool warm = true;
+        for (int i = 0; i < nsets; ++i) warm = warm && body_direct[i] > 0;
+        *ran = 1;
+        for (int k = GRAPH_LENS - 1; k >= 0 && !graph_failed; --k) {
+            const int len = lens[k];
+            if (avail < len || (len > 1 ? !warm || idle : body_direct[q] < 1)) continue;
+            cudaGraphExec_t &ge = graph_steps[k][q];
+            if (!ge) {
+                if (steps + avail < worth[k]) continue;
+                DCD_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+                dcd_status sc = DCD_OK;
+                for (int i = 0; i < len && sc == DCD_OK; ++i) sc = body((q + i) % nsets);
+                cudaGraph_t graph = nullptr;
+                const cudaError_t ec = cudaStreamEndCapture(st, &graph);
+                const bool ok = sc == DCD_OK && ec == cudaSuccess && graph != nullptr &&
+                                cudaGraphInstantiate(&ge, graph, 0) == cudaSuccess;
+                if (ok) stats.gpu_launches_per_step = count_kernel_nodes(graph) / len;
+                if (graph) cudaGraphDestroy(graph);
+                if (!ok) {
+                    cudaGetLastError();
+                    ge = nullptr;
+                    graph_failed = true;
+                    break;
+                }
+            }
+            DCD_TRY(cudaGraphLaunch(ge, st));
+            *ran = len;
+            return DCD_OK;
+        }
+        ++body_direct[q];
+        return body(q);
+    }
 
     // the step members point at buffer set p
     void use_bufs(int p)
@@ -1269,7 +1310,7 @@ struct Solver {
         return DCD_OK;
     }
 
-    dcd_status la_step(int64_t cnt)
+    dcd_status la_step(int64_t cnt, int64_t avail, int64_t *ran)
     {
         if (la_cnt != cnt) {  // nothing pending: this step's products first, on st
             DCD_TRY(cudaMemcpyAsync(ctr_la + la_par, ctr, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
@@ -1277,41 +1318,20 @@ struct Solver {
             if (r != DCD_OK) return r;
             la_cnt = cnt;
         }
-        const int p = la_par;
-        const int64_t next = (o.max_iters - done - cnt) >= o.s ? o.s : 0;  // only full steps are prepared ahead
-        if (next && cnt == o.s && !graph_failed) {
-            if (graph_la[p]) {
-                DCD_TRY(cudaGraphLaunch(graph_la[p], st));
-            } else if (la_direct[p] >= 1) {
-                DCD_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-                const dcd_status sc = la_body(p, cnt, next);
-                cudaGraph_t graph = nullptr;
-                const cudaError_t ec = cudaStreamEndCapture(st, &graph);
-                const bool ok = sc == DCD_OK && ec == cudaSuccess && graph != nullptr &&
-                                cudaGraphInstantiate(&graph_la[p], graph, 0) == cudaSuccess;
-                if (ok) stats.gpu_launches_per_step = count_kernel_nodes(graph);
-                if (graph) cudaGraphDestroy(graph);
-                if (!ok) {
-                    cudaGetLastError();
-                    graph_la[p] = nullptr;
-                    graph_failed = true;
-                    dcd_status r = la_body(p, cnt, next);
-                    if (r != DCD_OK) return r;
-                } else {
-                    DCD_TRY(cudaGraphLaunch(graph_la[p], st));
-                }
-            } else {
-                dcd_status r = la_body(p, cnt, next);
-                if (r != DCD_OK) return r;
-                ++la_direct[p];
-            }
-        } else {
-            dcd_status r = la_body(p, cnt, next);
-            if (r != DCD_OK) return r;
-        }
+        const int64_t left = o.max_iters - done;
+        const int64_t next = left - cnt >= o.s ? o.s : 0;  // only full steps are prepared ahead
+        dcd_status r = DCD_OK;
+        *ran = 1;
+        if (next && cnt == o.s)
+            r = replay_steps(la_par, 2, std::min<int64_t>(avail, left / o.s - 1),
+                             [&](int p) { return la_body(p, o.s, o.s); }, ran);
+        else
+            r = la_body(la_par, cnt, next);
+        if (r != DCD_OK) return r;
+        const int p = (la_par + (int)(*ran - 1)) & 1;  // the set of the last step run
         la_par = 1 - p;
         la_cnt = next;
-        use_bufs(p);  // the set just used is free (for a gradient recomputation) while the other holds products
+        use_bufs(p);  // free (for a gradient recomputation) while the other holds products
         return DCD_OK;
     }
 
@@ -1328,66 +1348,68 @@ struct Solver {
     //        on the SMs the others leave (its epilogue does not wait: it reads nothing the
     //        recurrence writes), update k;
     //   st2: step k+2's sample and gathers, then its Gram (a few CTAs) and prep, into nn;
-    //   st3, st4: after the gathers and recurrence k+1, x(k+2) into nn (two column halves).
+    //   st3: after the gathers, the links to step k+1's rows, and after recurrence k+1, x(k+2) into nn.
     // The association of the gradient's sums differs from the in-order step's; results agree to
     // rounding.  A gradient recomputation invalidates the recurrence and x computed ahead.
     bool df = false;
     int df_cur = 0;            // the set of the next step to run
     bool df_chain = false;     // its recurrence outputs (and x of the step after it) are in place
     int64_t df_prod = 0;       // step size of the products in (df_cur + 1) % 3 (0: none)
-    double *df_x[3] = {nullptr, nullptr, nullptr};  // per set: x of its step (col_pad doubles)
+    double *df_x[3] = {nullptr, nullptr, nullptr};  // per set: x of its step (a part per 256 columns)
     cudaStream_t st3 = nullptr, st4 = nullptr;  // x of the step after next, beside its Gram and prep
-    cudaEvent_t df_fork = nullptr, df_chained = nullptr, df_rows = nullptr, df_gram = nullptr, df_side = nullptr,
-                df_xfork = nullptr, df_xjoin = nullptr;
-    double *df_x2 = nullptr;   // the second column half's part of x
-    TcSplit xsplit, xsplit2;   // the cross product's halves' splits (they run beside the block)
+    cudaEvent_t df_fork = nullptr, df_chained = nullptr, df_rows = nullptr, df_gram = nullptr, df_side = nullptr;
+    int32_t *df_link[3] = {nullptr, nullptr, nullptr};  // per set: where its rows are in the step before
     int df_pairs = 0;          // CTA pairs of the block
+    int df_gram_ctas = 0;      // CTAs of the Gram beside it
     int df_prio = 0;           // launch priority of the recurrence and the block
-    cudaGraphExec_t graph_df[3] = {nullptr, nullptr, nullptr};
-    int df_direct[3] = {0, 0, 0};
 
-    // the recurrence of the step in set q on stream s, right-hand side -(g[S] + x) (x: nullptr for
-    // -g[S]), no fused update
-    dcd_status df_chain_of(int q, int64_t cnt, const double *x, cudaStream_t s, int prio = 0)
+    // the recurrence of the step in set q on stream s: right-hand side -(g[S] + x), x the part that
+    // step `prev`'s set holds (-1: none, -g[S]); no fused update
+    dcd_status df_chain_of(int q, int64_t cnt, int prev, cudaStream_t s, int prio = 0)
     {
         const StepBufs &Bq = sbuf[q];
         const int P = recur_cluster_size((int)cnt, o.b, 2);
         if (P <= 0) return DCD_EINTERNAL;
+        ClusterRhs x;
+        if (prev >= 0) {
+            x.x = df_x[q];
+            x.nx = (int)((sb + 255) / 256);
+            x.ldx = col_pad;
+            x.link = df_link[q];
+            x.next = recur_cluster_next(sbuf[prev].Lbuf, (int)o.s, o.b);
+            x.delta = sbuf[prev].delta;
+        }
         DCD_TRY(launch_recur_cluster_chain((const float *)Bq.Kss, ldk, Bq.S, (int)cnt, o.b, P, lambda, (double)m, g,
-                                           2, Bq.Lbuf, Bq.delta, Bq.w64, Bq.col_w, nullptr, err, s, x, -1, x != nullptr,
-                                           prio));
+                                           2, Bq.Lbuf, Bq.delta, Bq.w64, Bq.col_w, nullptr, err, s, nullptr, -1,
+                                           prev >= 0 ? &x : nullptr, prio));
         return DCD_OK;
     }
 
-    // x of the step in set r (full) from the step in set c (full, its recurrence done), on stream
-    // s; the product's columns in two launches (the second on sb, joined back), each on as many
-    // CTA pairs as row tiles, and the halves added in the repeat kernel
-    dcd_status df_cross(int r, int c, cudaStream_t s, cudaStream_t sb2)
+    // where the rows of the step in set r (full) are in the step before, in set c
+    dcd_status df_links_of(int r, int c, cudaStream_t s)
+    {
+        const int64_t nc = o.s * o.b;
+        return cuda_status(launch_defer_links(sbuf[r].S, nc, sbuf[c].S, nc, df_link[r], s));
+    }
+
+    // x of the step in set r (full) from the step in set c (full, its recurrence done), on stream s:
+    // a part per 256 columns, every (256-row tile, part) on a CTA pair of its own; the recurrence adds
+    // the parts and the update's (the links).  (Two column halves on four pairs each took 15 us, and
+    // a kernel that added them and the update's part 5 us more, both on the loop from one recurrence
+    // to the next.)
+    dcd_status df_cross(int r, int c, cudaStream_t s)
     {
         const StepBufs &Br = sbuf[r], &Bc = sbuf[c];
         const int64_t nc = o.s * o.b;
-        // split at a multiple of the 256-column chunk, so that neither launch reads the other's columns
-        const int64_t h = nc >= 512 ? nc / 2 / 256 * 256 : nc;
         TcOperand Ax{Br.As, nc, op.n_pad, op.kind, Br.col_s, Br.S};
-        if (h < nc) {
-            if (sb2 != s) {
-                DCD_TRY(cudaEventRecord(df_xfork, s));
-                DCD_TRY(cudaStreamWaitEvent(sb2, df_xfork, 0));
-            }
-            const size_t rb = (size_t)packed_row_bytes(op.kind, op.n_pad);
-            DCD_TRY(cudaMemsetAsync(df_x2, 0, sizeof(double) * nc, sb2));
-            TcOperand Bx{(const char *)Bc.As + h * rb, nc - h, op.n_pad, op.kind, Bc.col_s ? Bc.col_s + h : nullptr,
-                         Bc.S + h};
-            DCD_TRY(launch_block_tc(Ax, Bx, kp, Br.col_h, Bc.col_h + h, Bc.col_w + h, nullptr, df_x2, nullptr, 0, nc,
-                                    nc - h, err, sb2, false, &xsplit2, false, DF_XPAIRS));
-            if (sb2 != s) DCD_TRY(cudaEventRecord(df_xjoin, sb2));
-        }
-        DCD_TRY(cudaMemsetAsync(df_x[r], 0, sizeof(double) * nc, s));
-        TcOperand Bx{Bc.As, h, op.n_pad, op.kind, Bc.col_s, Bc.S};
-        DCD_TRY(launch_block_tc(Ax, Bx, kp, Br.col_h, Bc.col_h, Bc.col_w, nullptr, df_x[r], nullptr, 0, nc, h, err, s,
-                                false, &xsplit, false, DF_XPAIRS));
-        if (h < nc && sb2 != s) DCD_TRY(cudaStreamWaitEvent(s, df_xjoin, 0));
-        DCD_TRY(launch_defer_repeat(Br.S, nc, Bc.S, Bc.delta, nc, diag, h < nc ? df_x2 : nullptr, df_x[r], s));
+        TcOperand Bx{Bc.As, nc, op.n_pad, op.kind, Bc.col_s, Bc.S};
+        TcCross cr;
+        cr.out = df_x[r];
+        cr.ld = col_pad;
+        cr.row_link = df_link[r];
+        cr.col_next = recur_cluster_next(Bc.Lbuf, (int)o.s, o.b);
+        DCD_TRY(launch_block_tc(Ax, Bx, kp, Br.col_h, Bc.col_h, Bc.col_w, nullptr, nullptr, nullptr, 0, nc, nc, err, s,
+                                false, nullptr, false, DF_XPAIRS, nullptr, true, 0, &cr));
         return DCD_OK;
     }
 
@@ -1400,7 +1422,7 @@ struct Solver {
         // so that its cluster takes SMs first
         if (has2) DCD_TRY(cudaEventRecord(df_fork, st));
         if (has1) {
-            dcd_status r = df_chain_of(nxt, o.s, df_x[nxt], st, df_prio);
+            dcd_status r = df_chain_of(nxt, o.s, cur, st, df_prio);
             if (r != DCD_OK) return r;
         }
         if (has2) {
@@ -1409,7 +1431,9 @@ struct Solver {
             if (r != DCD_OK) return r;
             DCD_TRY(cudaEventRecord(df_rows, st2));
             DCD_TRY(cudaStreamWaitEvent(st3, df_rows, 0));
-            r = la_gram(nn, o.s, st2, DF_GRAM_CTAS);
+            r = df_links_of(nn, nxt, st3);
+            if (r != DCD_OK) return r;
+            r = la_gram(nn, o.s, st2, df_gram_ctas);
             if (r != DCD_OK) return r;
             DCD_TRY(cudaEventRecord(df_gram, st2));
         }
@@ -1430,7 +1454,7 @@ struct Solver {
                 DCD_TRY(cudaEventRecord(df_chained, st));
                 DCD_TRY(cudaStreamWaitEvent(st3, df_chained, 0));
             }
-            const dcd_status r = df_cross(nn, nxt, st3, st4);
+            const dcd_status r = df_cross(nn, nxt, st3);
             if (r != DCD_OK) return r;
             DCD_TRY(cudaEventRecord(df_side, st3));
         }
@@ -1453,7 +1477,7 @@ struct Solver {
     }
 
     // one full step through the deferred bodies
-    dcd_status df_step(int64_t cnt)
+    dcd_status df_step(int64_t cnt, int64_t avail, int64_t *ran)
     {
         const int cur = df_cur, nxt = (cur + 1) % 3, nn = (cur + 2) % 3;
         const int64_t rem1 = o.max_iters - done - cnt, rem2 = rem1 - o.s;
@@ -1466,7 +1490,7 @@ struct Solver {
                 la_cnt = cnt;
                 df_prod = 0;  // the position after this step is in ctr_la[nxt]; nothing sampled there
             }
-            dcd_status r = df_chain_of(cur, cnt, nullptr, st);
+            dcd_status r = df_chain_of(cur, cnt, -1, st);
             if (r != DCD_OK) return r;
             if (has1) {  // step k+1's products and x
                 if (df_prod != o.s) {
@@ -1474,42 +1498,26 @@ struct Solver {
                     if (r != DCD_OK) return r;
                     df_prod = o.s;
                 }
-                r = df_cross(nxt, cur, st, st);
+                r = df_links_of(nxt, cur, st);
+                if (r == DCD_OK) r = df_cross(nxt, cur, st);
                 if (r != DCD_OK) return r;
             }
             df_chain = true;
         }
-        const bool graphable = !graph_failed && has1 && has2;  // the steady state replays three graphs
-        if (graphable && graph_df[cur]) {
-            DCD_TRY(cudaGraphLaunch(graph_df[cur], st));
-        } else if (graphable && df_direct[cur] >= 1) {
-            DCD_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            const dcd_status sc = df_body(cur, cnt, has1, has2);
-            cudaGraph_t graph = nullptr;
-            const cudaError_t ec = cudaStreamEndCapture(st, &graph);
-            const bool ok = sc == DCD_OK && ec == cudaSuccess && graph != nullptr &&
-                            cudaGraphInstantiate(&graph_df[cur], graph, 0) == cudaSuccess;
-            if (ok) stats.gpu_launches_per_step = count_kernel_nodes(graph);
-            if (graph) cudaGraphDestroy(graph);
-            if (!ok) {
-                cudaGetLastError();
-                graph_df[cur] = nullptr;
-                graph_failed = true;
-                dcd_status r = df_body(cur, cnt, has1, has2);
-                if (r != DCD_OK) return r;
-            } else {
-                DCD_TRY(cudaGraphLaunch(graph_df[cur], st));
-            }
-        } else {
-            dcd_status r = df_body(cur, cnt, has1, has2);
-            if (r != DCD_OK) return r;
-            if (graphable) ++df_direct[cur];
-        }
-        df_cur = nxt;
+        dcd_status r = DCD_OK;
+        *ran = 1;
+        if (has1 && has2)  // the steady state
+            r = replay_steps(cur, 3, std::min<int64_t>(avail, (o.max_iters - done) / o.s - 2),
+                             [&](int q) { return df_body(q, o.s, true, true); }, ran);
+        else
+            r = df_body(cur, cnt, has1, has2);
+        if (r != DCD_OK) return r;
+        const int last = (cur + (int)(*ran - 1)) % 3;  // the set of the last step run
+        df_cur = (last + 1) % 3;
         df_chain = has1;
         df_prod = has2 ? o.s : 0;
         la_cnt = has1 ? o.s : 0;  // the products of the next step are in place
-        use_bufs(cur);  // the set just used is free (for a gradient recomputation)
+        use_bufs(last);  // the set just used is free (for a gradient recomputation)
         col_w_hi = std::max<int64_t>(col_w_hi, sb);  // any set's coefficients may fill sb entries
         return DCD_OK;
     }
@@ -1618,7 +1626,7 @@ struct Solver {
     }
 
     // one full step through the deferred bodies
-    dcd_status dfs_step(int64_t cnt)
+    dcd_status dfs_step(int64_t cnt, int64_t avail, int64_t *ran)
     {
         const int cur = df_cur, nxt = (cur + 1) % 3, nn = (cur + 2) % 3;
         const int64_t rem1 = o.max_iters - done - cnt, rem2 = rem1 - o.s;
@@ -1643,38 +1651,21 @@ struct Solver {
             }
             df_chain = true;
         }
-        const bool graphable = !graph_failed && has1 && has2;  // the steady state replays three graphs
-        if (graphable && graph_df[cur]) {
-            DCD_TRY(cudaGraphLaunch(graph_df[cur], st));
-        } else if (graphable && df_direct[cur] >= 1) {
-            DCD_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            const dcd_status sc = dfs_body(cur, cnt, has1, has2);
-            cudaGraph_t graph = nullptr;
-            const cudaError_t ec = cudaStreamEndCapture(st, &graph);
-            const bool ok = sc == DCD_OK && ec == cudaSuccess && graph != nullptr &&
-                            cudaGraphInstantiate(&graph_df[cur], graph, 0) == cudaSuccess;
-            if (ok) stats.gpu_launches_per_step = count_kernel_nodes(graph);
-            if (graph) cudaGraphDestroy(graph);
-            if (!ok) {
-                cudaGetLastError();
-                graph_df[cur] = nullptr;
-                graph_failed = true;
-                dcd_status r = dfs_body(cur, cnt, has1, has2);
-                if (r != DCD_OK) return r;
-            } else {
-                DCD_TRY(cudaGraphLaunch(graph_df[cur], st));
-            }
-        } else {
-            dcd_status r = dfs_body(cur, cnt, has1, has2);
-            if (r != DCD_OK) return r;
-            if (graphable) ++df_direct[cur];
-        }
-        df_cur = nxt;
+        dcd_status r = DCD_OK;
+        *ran = 1;
+        if (has1 && has2)  // the steady state
+            r = replay_steps(cur, 3, std::min<int64_t>(avail, (o.max_iters - done) / o.s - 2),
+                             [&](int q) { return dfs_body(q, o.s, true, true); }, ran);
+        else
+            r = dfs_body(cur, cnt, has1, has2);
+        if (r != DCD_OK) return r;
+        const int last = (cur + (int)(*ran - 1)) % 3;  // the set of the last step run
+        df_cur = (last + 1) % 3;
         df_chain = has1;
         df_prod = has2 ? o.s : 0;
         la_cnt = has1 ? o.s : 0;  // the products of the next step are in place
-        la_par = nxt < 2 ? nxt : 0;
-        use_bufs(cur);  // the set just used is free (for a gradient recomputation)
+        la_par = df_cur < 2 ? df_cur : 0;
+        use_bufs(last);  // the set just used is free (for a gradient recomputation)
         col_w_hi = std::max<int64_t>(col_w_hi, sb);  // any set's coefficients may fill sb entries
         return DCD_OK;
     }
@@ -1752,7 +1743,7 @@ struct Solver {
         return DCD_OK;
     }
 
-    dcd_status lag_step(int64_t cnt)
+    dcd_status lag_step(int64_t cnt, int64_t avail, int64_t *ran)
     {
         if (la_cnt != cnt) {  // nothing pending: this step's products first, on st
             DCD_TRY(cudaMemcpyAsync(ctr_la + la_par, ctr, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
@@ -1760,73 +1751,42 @@ struct Solver {
             if (r != DCD_OK) return r;
             la_cnt = cnt;
         }
-        const int p = la_par;
-        const int64_t next = (o.max_iters - done - cnt) >= o.s ? o.s : 0;  // only full steps are prepared ahead
-        if (next && cnt == o.s && !graph_failed) {
-            if (graph_la[p]) {
-                DCD_TRY(cudaGraphLaunch(graph_la[p], st));
-            } else if (la_direct[p] >= 1) {
-                DCD_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-                const dcd_status sc = lag_body(p, cnt, next);
-                cudaGraph_t graph = nullptr;
-                const cudaError_t ec = cudaStreamEndCapture(st, &graph);
-                const bool ok = sc == DCD_OK && ec == cudaSuccess && graph != nullptr &&
-                                cudaGraphInstantiate(&graph_la[p], graph, 0) == cudaSuccess;
-                if (ok) stats.gpu_launches_per_step = count_kernel_nodes(graph);
-                if (graph) cudaGraphDestroy(graph);
-                if (!ok) {
-                    cudaGetLastError();
-                    graph_la[p] = nullptr;
-                    graph_failed = true;
-                    dcd_status r = lag_body(p, cnt, next);
-                    if (r != DCD_OK) return r;
-                } else {
-                    DCD_TRY(cudaGraphLaunch(graph_la[p], st));
-                }
-            } else {
-                dcd_status r = lag_body(p, cnt, next);
-                if (r != DCD_OK) return r;
-                ++la_direct[p];
-            }
-        } else {
-            dcd_status r = lag_body(p, cnt, next);
-            if (r != DCD_OK) return r;
-        }
+        const int64_t left = o.max_iters - done;
+        const int64_t next = left - cnt >= o.s ? o.s : 0;  // only full steps are prepared ahead
+        dcd_status r = DCD_OK;
+        *ran = 1;
+        if (next && cnt == o.s)
+            r = replay_steps(la_par, 2, std::min<int64_t>(avail, left / o.s - 1),
+                             [&](int p) { return lag_body(p, o.s, o.s); }, ran);
+        else
+            r = lag_body(la_par, cnt, next);
+        if (r != DCD_OK) return r;
+        const int p = (la_par + (int)(*ran - 1)) & 1;  // the set of the last step run
         la_par = 1 - p;
         la_cnt = next;
-        use_bufs(p);  // the set just used is free (for a gradient recomputation)
+        use_bufs(p);  // free (for a gradient recomputation) while the other holds products
         return DCD_OK;
     }
 
-    dcd_status outer_step(int64_t cnt, EventTimer &tm)
+    // one outer step of cnt inner iterations, or more full ones where they are replayed from a graph (at
+    // most avail; *ran receives how many)
+    dcd_status outer_step(int64_t cnt, EventTimer &tm, int64_t avail, int64_t *ran)
     {
-        if (dfs && !tm.on && cnt == o.s) {
-            dcd_status r = dfs_step(cnt);
-            if (r != DCD_OK) return r;
-            done += cnt;
-            ++steps;
-            return DCD_OK;
-        }
-        if (lag && !tm.on) {
-            dcd_status r = lag_step(cnt);
-            if (r != DCD_OK) return r;
-            done += cnt;
-            ++steps;
-            return DCD_OK;
-        }
-        if (df && !tm.on && cnt == o.s) {
-            dcd_status r = df_step(cnt);
-            if (r != DCD_OK) return r;
-            done += cnt;
-            ++steps;
-            return DCD_OK;
-        }
-        if (la && !df && !tm.on && recur_cluster_size((int)cnt, o.b, 2) > 0) {
-            dcd_status r = la_step(cnt);
-            if (r != DCD_OK) return r;
-            done += cnt;
-            ++steps;
-            return DCD_OK;
+        *ran = 1;
+        if (!tm.on) {
+            dcd_status r = DCD_OK;
+            bool taken = true;
+            if (dfs && cnt == o.s) r = dfs_step(cnt, avail, ran);
+            else if (lag) r = lag_step(cnt, avail, ran);
+            else if (df && cnt == o.s) r = df_step(cnt, avail, ran);
+            else if (la && !df && recur_cluster_size((int)cnt, o.b, 2) > 0) r = la_step(cnt, avail, ran);
+            else taken = false;
+            if (taken) {
+                if (r != DCD_OK) return r;
+                done += cnt * *ran;
+                steps += *ran;
+                return DCD_OK;
+            }
         }
         if (la_cnt) return DCD_EINTERNAL;  // prepared products would be skipped
         const bool graphable = !tm.on && !(o.flags & DCD_FLAG_NO_GRAPH) && cnt == o.s && st != nullptr &&
@@ -1978,13 +1938,17 @@ struct Solver {
         cudaEventCreate(&e1);
         cudaEventRecord(e0, st);
         const int check_every = o.check_every > 0 ? o.check_every : 0;
-        for (int64_t k = 0; !finished() && (max_steps < 0 || k < max_steps); ++k) {
+        for (int64_t k = 0, ran = 0; !finished() && (max_steps < 0 || k < max_steps); k += ran) {
             const int64_t cnt = std::min<int64_t>(o.s, o.max_iters - done);
-            s0 = outer_step(cnt, tm);
+            int64_t avail = max_steps < 0 ? INT64_MAX : max_steps - k;
+            if (check_every && o.tol > 0) avail = std::min<int64_t>(avail, check_every - steps % check_every);
+            s0 = outer_step(cnt, tm, std::min(avail, (o.max_iters - done + o.s - 1) / o.s), &ran);
             if (s0 != DCD_OK) break;
+            idle = false;
             if (check_every && o.tol > 0 && steps % check_every == 0 && done < o.max_iters) {
                 tm.start();
                 s0 = check_converged();
+                idle = true;
                 tm.stop(stats.ms_check);
                 tm.flush();
                 if (s0 != DCD_OK) break;
@@ -2008,6 +1972,7 @@ struct Solver {
             metric = primal = dual = NAN;
         }
         dcd_status se = check_device_error();
+        idle = true;
         if (s0 == DCD_OK) s0 = se;
         if (s0 == DCD_OK) s0 = publish();
         cudaEventRecord(e1, st);
@@ -2052,9 +2017,10 @@ struct Solver {
         if (s0 == DCD_OK) {
             EventTimer off;
             off.init(false, st);
-            for (; !finished() && k < max_steps; ++k) {
-                s0 = outer_step(std::min<int64_t>(o.s, o.max_iters - done), off);
+            for (int64_t ran = 0; !finished() && k < max_steps; k += ran) {
+                s0 = outer_step(std::min<int64_t>(o.s, o.max_iters - done), off, max_steps - k, &ran);
                 if (s0 != DCD_OK) break;
+                idle = false;
             }
         }
         stats.iters_done = done;
