@@ -138,7 +138,10 @@ typedef enum {
                                    samples (an s b x s b product) and the update's: the same sums up to
                                    their association, so the bits differ from the in-order steps by
                                    rounding only.  With this flag the steps give the bits of the one-stream
-                                   steps */
+                                   steps.  (K-SVM on a small dense FP64 problem runs many steps per launch
+                                   on one resident grid, on any stream, unless this flag, DCD_FLAG_NO_GRAPH
+                                   or the phase timers are set or a tolerance is checked more often than
+                                   every 16 steps; the sums are associated differently there too) */
 #define DCD_FLAG_REFRESH 0x10     /* with tol > 0: when the metric of the cached gradient first meets tol,
                                      recompute the gradient from alpha by full kernel passes (tensor-core
                                      modes: DCD_PREC_REFRESH; FP64 mode: FP64) and accept convergence only
@@ -233,8 +236,9 @@ dcd_status dcd_plan_destroy(dcd_plan *plan);
  * 0 steps) reports any device-side error, publishes and fills the
  * statistics.  *enqueued (may be NULL) receives the number of steps
  * enqueued, fewer than asked once the budget H is exhausted.  Full outer
- * steps are replayed from a CUDA graph unless DCD_FLAG_NO_GRAPH is set or
- * the plan's stream is the legacy default stream.  Returns DCD_EINVAL for a
+ * steps are replayed from CUDA graphs (several steps in one where that many
+ * are enqueued) unless DCD_FLAG_NO_GRAPH is set or the plan's stream is the
+ * legacy default stream.  Returns DCD_EINVAL for a
  * NULL plan or outer_steps < 0, DCD_ECUDA if a launch fails.
  */
 dcd_status dcd_plan_enqueue(dcd_plan *plan, int64_t outer_steps, int64_t *enqueued);

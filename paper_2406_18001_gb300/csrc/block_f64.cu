@@ -33,6 +33,7 @@
 // Measured (K-RR, m = 6000, n = 512, sb = 256): block 4753 -> 92 us, Gram 4722 -> 34 us;
 // the solve's alpha after 64 block updates is 3.3e-15 from 64-bit arithmetic (direct block 7.2e-15).
 #include "dcd_internal.cuh"
+#include "f64_math.cuh"
 #include "tc_ptx.cuh"
 
 namespace dcd {
@@ -94,25 +95,6 @@ __device__ __forceinline__ double int_to_double(long long i)
     return __longlong_as_double(0x4338000000000000LL + i) - 6755399441055744.0;
 }
 
-// e^x for -700 < x <= 0 by table and polynomial (Tang, ACM TOMS 15, 1989): x = k ln2 / 64 + r,
-// |r| <= ln2 / 128, e^x = 2^(k / 64) e^r with 2^(j / 64) from the table tab[j] and e^r - 1 by its
-// Taylor polynomial of degree 5 (truncation below 4e-17).  Ten FP64 operations; within about one ulp.
-__device__ __forceinline__ double exp_tab(double x, const double *tab)
-{
-    const double t = fma(x, 92.332482616893656877, 6755399441055744.0);  // 64 / ln 2
-    const int k = __double2loint(t);
-    const double kd = t - 6755399441055744.0;
-    double r = fma(kd, -0x1.62e42fee00000p-7, x);  // ln 2 / 64: 33 leading bits, exact with |k| < 2^17
-    r = fma(kd, -0x1.a39ef35793c76p-39, r);
-    double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-    p = fma(p, r, 1.0 / 6.0);
-    p = fma(p, r, 0.5);
-    p = fma(p, r * r, r);
-    const double c = tab[k & 63];
-    const double v = fma(c, p, c);
-    return __hiloint2double(__double2hiint(v) + ((k >> 6) << 20), __double2loint(v));
-}
-
 template <int KIND>
 __global__ void __launch_bounds__(F64S_THREADS, 1)
     block_f64s_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, F64Args a)
@@ -145,8 +127,7 @@ __global__ void __launch_bounds__(F64S_THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (KIND == DCD_RBF && threadIdx.x >= 64 && threadIdx.x < 128)
-        tab[threadIdx.x - 64] = exp2((double)(threadIdx.x - 64) * (1.0 / 64.0));
+    if (KIND == DCD_RBF && threadIdx.x >= 64 && threadIdx.x < 128) tab[threadIdx.x - 64] = exp_tab_entry(threadIdx.x - 64);
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_holder)),
                      "r"(512u)
@@ -371,7 +352,7 @@ __global__ void __launch_bounds__(F64S_THREADS, 1)
 // exponent and gamma times its squared norm (compensated sum: TwoProd and TwoSum).  The scaled
 // value is rounded once to a 56-bit integer whose signed base-128 digits are the slices.
 // stat[0]: set when a value is not finite or an exponent leaves [-400, 400]; stat[1]: the largest
-// gamma |a|^2 (bit pattern of a non-negative double).
+// gamma |a|^2 (bit pattern of a non-negative double).  dst (and ex) null: norms only.
 __global__ void pack_f64s_kernel(const double *__restrict__ A, int64_t lda, int64_t m, int64_t n, double gamma,
                                  __nv_bfloat162 *dst, int64_t n_pad, int32_t *ex, double *h, unsigned long long *stat)
 {
@@ -403,12 +384,12 @@ __global__ void pack_f64s_kernel(const double *__restrict__ A, int64_t lda, int6
     bad |= e > 400 || e < -400;
     const double nrm = gamma * (s + c);
     if (lane == 0) {
-        ex[r] = e;
+        if (ex) ex[r] = e;
         h[r] = nrm;
         if (bad) atomicMax(stat, 1ull);
         else atomicMax(stat + 1, (unsigned long long)__double_as_longlong(fabs(nrm)));
     }
-    if (bad) return;
+    if (bad || !dst) return;
     const double sc = __hiloint2double((1023 + 55 - e) << 20, 0);  // 2^(55 - e)
     __nv_bfloat162 *d = dst + r * (NSL / 2) * n_pad;
     for (int64_t k = 2 * lane; k < n_pad; k += 64) {
@@ -450,7 +431,7 @@ int64_t f64s_tiles(int64_t m) { return (m + FM - 1) / FM; }
 cudaError_t launch_pack_f64s(const double *A, int64_t lda, int64_t m, int64_t n, const KernelParams &kp, void *packed,
                              int32_t *ex, double *h, unsigned long long *stat, cudaStream_t st)
 {
-    if (m <= 0 || n <= 0 || n > F64S_N_MAX) return cudaErrorInvalidValue;
+    if (m <= 0 || n <= 0 || (packed && n > F64S_N_MAX)) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(stat, 0, 2 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     pack_f64s_kernel<<<(unsigned)((m * 32 + 255) / 256), 256, 0, st>>>(

@@ -116,7 +116,8 @@ struct F64Sliced {
 int64_t f64s_row_bytes(int64_t n);
 size_t f64s_part_bytes(int64_t m, int64_t ncols);
 int64_t f64s_tiles(int64_t m);
-// stat: two words (zeroed here): whether a value rules the form out, and the largest gamma |a|^2
+// stat: two words (zeroed here): whether a value rules the form out, and the largest gamma |a|^2.
+// packed and ex null: the norms alone.
 cudaError_t launch_pack_f64s(const double *A, int64_t lda, int64_t m, int64_t n, const KernelParams &kp, void *packed,
                              int32_t *ex, double *h, unsigned long long *stat, cudaStream_t st);
 // rows, cols: packed rows (all of f.packed, or gathered ones with the data rows they hold in
@@ -126,6 +127,20 @@ cudaError_t launch_block_f64s(const F64Sliced &f, const void *rows, int64_t nrow
                               const void *cols, int64_t ncols, const int32_t *col_id, const KernelParams &kp,
                               const double *w, const double *rs, double *g, double *out, int64_t ldo, int *err,
                               cudaStream_t st);
+// Resident K-SVM steps of a small dense FP64 problem (svm_grid.cu): many outer steps per launch on one
+// co-resident grid.  ctas = 0: the shape does not fit.
+struct SvmGrid {
+    int ctas = 0, R = 0, ks = 0;  // CTAs, rows each, lanes per kernel value
+    size_t smem = 0;
+};
+SvmGrid svm_grid_plan(int64_t m, int64_t n, int s);
+size_t svm_grid_scratch_bytes(int s);
+// `steps` full steps of s coordinates from stream position *ctr (advanced): alpha and g updated in
+// place.  h: gamma |a|^2 per row (launch_pack_f64s), or null for squared distances from differences.
+cudaError_t launch_svm_grid(const SvmGrid &gp, const double *A, int64_t lda, int64_t m, int64_t n,
+                            const KernelParams &kp, const double *h, const double *y, double *alpha, double *g,
+                            uint64_t seed, uint64_t *ctr, int steps, int s, double omega, double nu, void *scratch,
+                            int *err, cudaStream_t st);
 // 2-D tensor map over a row-major bf16 matrix of nrows x cols elements, box of box_rows x 64,
 // 128-byte swizzle, out-of-range rows read as zero (block_tc.cu)
 bool make_map_bf16_2d(CUtensorMap *map, const void *base, int64_t cols, int64_t nrows, int box_rows);

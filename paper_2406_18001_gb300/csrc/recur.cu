@@ -12,6 +12,7 @@
 //                       G_jt = Kss_jt / lambda + m [S_j = S_t]   (Algorithm 4)
 // All arithmetic here is FP64.
 #include "dcd_internal.cuh"
+#include "dcd_chain.cuh"
 #include "ptx.cuh"
 
 #include <algorithm>
@@ -948,30 +949,6 @@ cudaError_t refined_bdcd_b(const KT *Kss, int64_t ldk, const int32_t *S, int nbl
 // before them are done.  One warp in lockstep over all coordinates took 1.2 k cycles per
 // coordinate.  Measured per step: s = 64 (split bf16, m = 2000, n = 64) 38 -> 10.7 us over a whole
 // solve; s = 8 (FP64) 7.6 -> 2.7; s = 32 on CSR data from alpha = 0, every step nonzero, 26 -> 18.
-constexpr int DCD_FAST_MAX = 128;
-constexpr int DCD_FAST_K = DCD_FAST_MAX / 32;
-
-__device__ __forceinline__ int ld_acquire_shared(const int *p)
-{
-    int v;
-    asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(ptx::su32(p)) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_release_shared(int *p, int v)
-{
-    asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(ptx::su32(p)), "r"(v) : "memory");
-}
-
-// clip(x, 0, nu) by the bit patterns (nub: those of nu, +infinity for no upper bound); a NaN gives 0,
-// as fmin(fmax(x, 0), nu) does
-__device__ __forceinline__ double clip_bits(double x, long long nub)
-{
-    const long long b = __double_as_longlong(x);
-    if (b <= 0 || b > 0x7ff0000000000000LL) return 0.0;
-    return __longlong_as_double(b > nub ? nub : b);
-}
-
 // pend (optional): alpha and g at the step's coordinates are pend[0][t] + pend[1][t] and
 // pend[2][t] + pend[3][t] (a snapshot and the parts not yet in it) instead of alpha[S[t]], g[S[t]]
 template <typename KT>
@@ -1043,56 +1020,7 @@ __global__ void __launch_bounds__(DCD_THREADS) recur_dcd_fast_kernel(const KT *K
         rho += a1;
         gj += g1;
     }
-    const int tc = mine ? t : cnt - 1;  // a valid column for lanes past the end
-    auto apply = [&](int j, double tj) {
-        gj = fma(C[j * ldc + tc], tj, gj);
-        const uint32_t m = rep[j * DCD_FAST_K + warp];
-        if (m) rho += (m >> lane) & 1u ? tj : 0.0;  // repeats are rare (warp-uniform)
-    };
-    int n = 0;  // published steps applied (or, in the chain below, published)
-    if (warp > 0) {
-        const long long t0 = clock64();
-        for (;;) {
-            const int dn = ld_acquire_shared(pub + 1);
-            const int np = ld_acquire_shared(pub);
-            for (; n < np; ++n) apply(list_j[n], list_t[n]);
-            if (dn >= warp) break;
-            if (clock64() - t0 > 4200000000LL) {  // about 2 s
-                set_error(err, DEV_TIMEOUT);
-                break;
-            }
-        }
-        __syncwarp();
-    }
-    const bool more = 32 * (warp + 1) < cnt;
-    const long long nub = __double_as_longlong(nu);
-    double th = 0.0;
-    uint32_t left = __ballot_sync(0xffffffffu, mine);  // coordinates not yet decided
-    const bool solvable = (__double_as_longlong(ie) << 1) != 0;
-    for (;;) {
-        const double c1 = clip_bits(rho - gj, nub), c2 = clip_bits(fma(-gj, ie, rho), nub);
-        // the projected gradient clip(rho - g) - rho is nonzero iff the clip moved rho
-        const long long b1 = __double_as_longlong(c1), b0 = __double_as_longlong(rho);
-        const bool moved = b1 != b0 && ((b1 | b0) << 1) != 0;  // +0 and -0 are the same value
-        const double st = moved && solvable ? c2 - rho : 0.0;
-        const uint32_t nz = __ballot_sync(0xffffffffu, (__double_as_longlong(st) << 1) != 0) & left;
-        if (!nz) break;
-        const int l = __ffs(nz) - 1, j = 32 * warp + l;
-        const double tj = __shfl_sync(0xffffffffu, st, l);
-        if (lane == l) {
-            th = tj;
-            if (more) {
-                list_j[n] = j;
-                list_t[n] = tj;
-                st_release_shared(pub, n + 1);
-            }
-        }
-        ++n;
-        left &= ~((2u << l) - 1u);
-        apply(j, tj);
-    }
-    __syncwarp();
-    if (more && lane == 0) st_release_shared(pub + 1, warp + 1);
+    const double th = dcd_chain_group(C, ldc, rep, list_t, list_j, pub, cnt, warp, lane, rho, gj, ie, nu, err);
     if (mine) {
         delta[t] = th;
         // y_t th

@@ -258,6 +258,11 @@ struct Solver {
     bool f64s = false;
     F64Sliced fs;
     void *ws_f64s = nullptr;
+    // K-SVM on a small dense FP64 problem: many steps per launch on one resident grid (svm_grid.cu)
+    SvmGrid grid;
+    void *grid_ws = nullptr;
+    double *grid_h = nullptr;
+    unsigned long long *grid_stat = nullptr;
     // CSR data matrix: the CUDA-core SpMM block (FP32, or FP64 in the FP64 mode)
     bool csr = false;
     CsrOperand ca;
@@ -387,7 +392,13 @@ struct Solver {
         // the look-ahead of the other steps (K-SVM, dense or CSR; K-RR in FP64, on CSR or with a
         // chain longer than one cluster): the next step's sample, column map or gathers and Gram
         // on a second stream beside the recurrence and block
-        const bool lag_pos = !t_no_lookahead && !la_pos && !literal &&
+        // (not with steps asked for in order or directly, or checked so often that a launch would hold
+        // only a few; from the line of the slice form on, that form's block is the faster one)
+        if (problem == 0 && !csr && !tc && !literal && !f64s_worth() &&
+            !(o.flags & (DCD_FLAG_NO_GRAPH | DCD_FLAG_NO_DEFER | DCD_FLAG_PHASE_TIMERS)) &&
+            (o.tol <= 0.0 || o.check_every <= 0 || o.check_every >= 16))
+            grid = svm_grid_plan(m, n, (int)o.s);
+        const bool lag_pos = !t_no_lookahead && !la_pos && !literal && !grid.ctas &&
                              !(o.flags & (DCD_FLAG_NO_GRAPH | DCD_FLAG_PHASE_TIMERS)) && st != nullptr &&
                              st != cudaStreamLegacy && st != cudaStreamPerThread;
         const bool set2 = la_pos || lag_pos;  // a second set of step buffers
@@ -446,6 +457,9 @@ struct Solver {
             double *w64i[3];
             for (int q = 0; q < 3; ++q)
                 w64i[q] = (double *)ar.take(fwd64 && (q == 0 || (q == 1 && set2)) ? sizeof(double) * sb * o.b : 0);
+            grid_ws = ar.take(grid.ctas ? svm_grid_scratch_bytes((int)o.s) : 0);
+            grid_h = (double *)ar.take(grid.ctas ? sizeof(double) * m : 0);
+            grid_stat = (unsigned long long *)ar.take(grid.ctas ? 2 * sizeof(unsigned long long) : 0);
             uint64_t *cr = (uint64_t *)ar.take(sizeof(uint64_t));
             // the second set of step buffers and the look-ahead counter
             int32_t *sidx_b = (int32_t *)ar.take(set2 ? sizeof(int32_t) * col_pad : 0);
@@ -747,6 +761,17 @@ struct Solver {
             op.a64 = (const double *)vals;
             op.lda = A->ld;
         }
+        if (grid.ctas && kp.kind == DCD_RBF) {  // norms for the expansion, where it is as exact as the differences
+            DCD_TRY(launch_pack_f64s(op.a64, op.lda, m, n, kp, nullptr, nullptr, grid_h, grid_stat, st));
+            unsigned long long hs[2] = {1, 0};
+            DCD_TRY(cudaMemcpyAsync(hs, grid_stat, sizeof(hs), cudaMemcpyDeviceToHost, st));
+            DCD_TRY(cudaStreamSynchronize(st));
+            double hmax;
+            memcpy(&hmax, &hs[1], sizeof(hmax));
+            if (hs[0] || !(hmax <= F64S_HMAX)) grid_h = nullptr;
+        } else {
+            grid_h = nullptr;
+        }
         if (!csr && !tc && !literal) {
             const dcd_status fst = setup_f64s(set3 ? 3 : set2 ? 2 : 1);
             if (fst != DCD_OK) return fst;
@@ -791,10 +816,15 @@ struct Solver {
     // 74 / 52, 6000 x 512 x 32 511 / 93: from 6 M; wider ones, in tiles of 64 rows, 2000 x 64 x 64
     // (8.2 M) 351 / 71, 6000 x 512 x 256 9510 / 148: from 1 M.  No memory for the slices (16 bytes
     // a value): the direct form.
-    dcd_status setup_f64s(int sets)
+    bool f64s_worth() const
     {
         const double work = (double)m * (double)sb * (double)n;
-        if (n > F64S_N_MAX || work < (sb > 32 ? 1e6 : 6e6) || !tc_available()) return DCD_OK;
+        return n <= F64S_N_MAX && work >= (sb > 32 ? 1e6 : 6e6) && tc_available();
+    }
+
+    dcd_status setup_f64s(int sets)
+    {
+        if (!f64s_worth()) return DCD_OK;
         const size_t rb = (size_t)f64s_row_bytes(n);
         Arena ar;
         for (int pass = 0; pass < 2; ++pass) {
@@ -1776,7 +1806,13 @@ struct Solver {
         if (!tm.on) {
             dcd_status r = DCD_OK;
             bool taken = true;
-            if (dfs && cnt == o.s) r = dfs_step(cnt, avail, ran);
+            if (grid.ctas && cnt == o.s) {
+                // a launch of a few tens of milliseconds at most
+                *ran = std::min<int64_t>({avail, (o.max_iters - done) / o.s, (int64_t)4096});
+                stats.gpu_launches_per_step = 1;
+                r = cuda_status(launch_svm_grid(grid, op.a64, op.lda, m, n, kp, grid_h, y, alpha, g, o.seed, ctr,
+                                                (int)*ran, (int)o.s, omega, nu, grid_ws, err, st));
+            } else if (dfs && cnt == o.s) r = dfs_step(cnt, avail, ran);
             else if (lag) r = lag_step(cnt, avail, ran);
             else if (df && cnt == o.s) r = df_step(cnt, avail, ran);
             else if (la && !df && recur_cluster_size((int)cnt, o.b, 2) > 0) r = la_step(cnt, avail, ran);
