@@ -390,12 +390,29 @@ constexpr int CSC_SCATTER_THREADS = 256;
 
 constexpr int CSC_SHORT_ROW = 8;   // a row with more entries in a tile makes the warp sort the tile jointly
 
+constexpr int CSC_CNT_STRIDE = 8;  // a counter per 32-byte sector: its atomics wait on no neighbour's
+
+// The apply's scratch of a warp: the sorted keys and products share the full pass's hit list (an
+// overflowed tile's only), beside the counters of the counting sort.
 template <typename T>
 struct alignas(16) CscWarpSmem {
-    int64_t skey[CSC_TILE_CAP], rkey[CSC_TILE_CAP];
-    T sprod[CSC_TILE_CAP], rprod[CSC_TILE_CAP];
-    int32_t rcnt[32], roff[32];
+    WarpSmem<T> ws;  // hoff: sorted keys; hcol: ranked keys; hprod: their products; hj: ranked products (FP32)
+    int32_t rcnt[32];
+    T rprod64[sizeof(T) == 8 ? CSC_TILE_CAP : 1];
+    __device__ uint32_t *skey() { return (uint32_t *)ws.hoff; }
+    __device__ uint32_t *rkey() { return (uint32_t *)ws.hcol; }
+    __device__ T *sprod() { return ws.hprod; }
+    __device__ T *rprod() { return sizeof(T) == 4 ? (T *)ws.hj : rprod64; }
+    __device__ int32_t *roff() { return ws.rp; }
 };
+static_assert(CSC_TILE_CAP <= CSR_HL, "the sorted bucket shares the hit list");
+
+// CtaSmem without its bitmap
+template <typename T>
+__host__ __device__ constexpr size_t csc_cta_bytes()
+{
+    return (offsetof(CtaSmem<T>, bits) + 15) / 16 * 16;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(CSC_SCATTER_THREADS)
@@ -443,84 +460,83 @@ __global__ void __launch_bounds__(CSC_SCATTER_THREADS)
             q[u] = qq;
             k[u] = x < total ? cstart[qq] + (x - pre[qq]) : -1;
         }
+        uint32_t el[CSC_U];  // every load in flight before the counters' round trips
+        T cv[CSC_U];
 #pragma unroll
-        for (int u = 0; u < CSC_U; ++u) row[u] = k[u] >= 0 ? C.row[k[u]] : -1;
+        for (int u = 0; u < CSC_U; ++u) {
+            row[u] = k[u] >= 0 ? C.row[k[u]] : -1;
+            el[u] = k[u] >= 0 ? C.elem[k[u]] : 0;
+            cv[u] = k[u] >= 0 ? cval[k[u]] : (T)0;
+        }
 #pragma unroll
-        for (int u = 0; u < CSC_U; ++u) pos[u] = row[u] >= 0 ? atomicAdd(W.tile_cnt + (row[u] >> 5), 1) : CSC_TILE_CAP;
+        for (int u = 0; u < CSC_U; ++u) 
+            pos[u] = row[u] >= 0 ? atomicAdd(W.tile_cnt + (int64_t)(row[u] >> 5) * CSC_CNT_STRIDE, 1) : CSC_TILE_CAP;
 #pragma unroll
         for (int u = 0; u < CSC_U; ++u)
             if (pos[u] < CSC_TILE_CAP) {
                 const int64_t at = (int64_t)(row[u] >> 5) * CSC_TILE_CAP + pos[u];
-                W.key[at] = (C.elem[k[u]] << 10) | ((int64_t)(row[u] & 31) << 5) | j;
-                prod[at] = mul_rn(cval[k[u]], aval[q[u]]);  // the full pass's product, rounded in T
+                W.key[at] = (el[u] << 10) | ((uint32_t)(row[u] & 31) << 5) | (uint32_t)j;
+                prod[at] = mul_rn(cv[u], aval[q[u]]);  // the full pass's product, rounded in T
             }
     }
 }
 
+// Latency- and instruction-bound (loads, a small sort and a few FMAs a tile), so what counts is how
+// many warps are resident: 32-bit keys and the scratch shared with the full pass's leave FP32 four
+// CTAs per SM, where 64-bit keys, scratch of their own and a tile loaded ahead left two.  At three
+// (80 registers) nothing spills: m = 200000, 50 nonzeros a row, s = 32 takes 19 us beside the chain of
+// the step, at four CTAs of 64 registers (spilled) 22.
 template <typename T, int KIND>
-__global__ void __launch_bounds__(CSR_AW * 32, 2)
+__global__ void __launch_bounds__(CSR_AW * 32, sizeof(T) == 4 ? 3 : 2)
     csc_apply_kernel(CsrOperand A, CsrColMap M, CscStep W, int64_t nrows, const int32_t *S, int j0, int jc,
                      KernelParams kp, const float *w32, const double *w64, const double *rs, double *g)
 {
     extern __shared__ __align__(16) unsigned char csr_sm[];
-    CtaSmem<T> &cs = *(CtaSmem<T> *)csr_sm;
+    CtaSmem<T> &cs = *(CtaSmem<T> *)csr_sm;  // without its bitmap
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpSmem<T> &ws = ((WarpSmem<T> *)(csr_sm + sizeof(CtaSmem<T>)))[warp];
-    CscWarpSmem<T> &xs =
-        ((CscWarpSmem<T> *)(csr_sm + sizeof(CtaSmem<T>) + sizeof(WarpSmem<T>) * CSR_AW))[warp];
+    CscWarpSmem<T> &xs = ((CscWarpSmem<T> *)(csr_sm + csc_cta_bytes<T>()))[warp];
+    WarpSmem<T> &ws = xs.ws;
     const T *vals = (const T *)(sizeof(T) == 8 ? (const void *)A.vals64 : (const void *)A.vals32);
     const T *prod = (const T *)W.prod;
-    // the bitmap stays in global memory: only tiles that overflowed their bucket test it
-    csr_cta_setup<T, KIND, false>(cs, ws, A, M, S, j0, jc, kp, w32, w64);
     const int64_t ntiles = (nrows + 31) / 32;
     const int64_t tstride = (int64_t)gridDim.x * CSR_AW;
     constexpr int PER = CSC_TILE_CAP / 32;
-    // a tile's counter, row offsets and whole bucket (entries past the counter are stale and
-    // masked later); the next tile's are loaded while this one is processed
-    int nt_n = 0;
-    int64_t rpv_n = 0, rend_n = 0;
-    int64_t kk_n[PER];
-    T pp_n[PER];
+    // a tile's counter and whole bucket (entries past the counter are stale and masked)
+    int nt = 0;
+    uint32_t kk[PER];
+    T pp[PER];
     auto load_tile = [&](int64_t tl) {
         if (tl >= ntiles) return;
-        const int64_t t0 = tl * 32;
-        const int nr = (int)min((int64_t)32, nrows - t0);
-        nt_n = W.tile_cnt[tl];
-        rpv_n = lane < nr ? A.row_ptr[t0 + lane] : 0;
-        rend_n = A.row_ptr[t0 + nr];
+        nt = W.tile_cnt[tl * CSC_CNT_STRIDE];
 #pragma unroll
         for (int u = 0; u < PER; ++u) {
-            kk_n[u] = W.key[tl * CSC_TILE_CAP + lane + 32 * u];
-            pp_n[u] = prod[tl * CSC_TILE_CAP + lane + 32 * u];
+            kk[u] = W.key[tl * CSC_TILE_CAP + lane + 32 * u];
+            pp[u] = prod[tl * CSC_TILE_CAP + lane + 32 * u];
         }
     };
     load_tile((int64_t)blockIdx.x * CSR_AW + warp);
-    for (int64_t tile = (int64_t)blockIdx.x * CSR_AW + warp; tile < ntiles; tile += tstride) {
+    // the bitmap stays in global memory: only tiles that overflowed their bucket test it
+    csr_cta_setup<T, KIND, false>(cs, ws, A, M, S, j0, jc, kp, w32, w64);
+    for (int64_t tile = (int64_t)blockIdx.x * CSR_AW + warp; tile < ntiles;) {
         const int64_t t0 = tile * 32;
         const int nr = (int)min((int64_t)32, nrows - t0);
-        const int nt = nt_n;
-        const int64_t rpv = rpv_n, rend = rend_n;
-        int64_t kk[PER];
-        T pp[PER];
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            kk[u] = lane + 32 * u < nt ? kk_n[u] : -1;
-            pp[u] = pp_n[u];
-        }
-        load_tile(tile + tstride);
-        const int64_t e0 = __shfl_sync(0xffffffffu, rpv, 0);
         uint32_t touched = 0;
         if (nt > CSC_TILE_CAP) {  // the bucket overflowed: the full pass over this tile
-            if (lane < nr) ws.rp[lane] = (int32_t)(rpv - e0);
+            const int64_t e0 = A.row_ptr[t0], rend = A.row_ptr[t0 + nr];
+            if (lane < nr) ws.rp[lane] = (int32_t)(A.row_ptr[t0 + lane] - e0);
             if (lane == 0) ws.rp[nr] = (int32_t)(rend - e0);
             csr_tile_stream<T, false>(A, M, ws, M.bits, vals, e0, (int)(rend - e0), j0, jc, lane, nr, touched);
         } else if (nt > 0) {
             // counting sort by row (the row's index within the tile is bits 5..9 of the key)
+            uint32_t *skey = xs.skey();
+            T *sprod = xs.sprod();
+            int32_t *roff = xs.roff();
             xs.rcnt[lane] = 0;
             __syncwarp();
+            int at[PER];  // the entry's place among its row's
 #pragma unroll
             for (int u = 0; u < PER; ++u)
-                if (kk[u] >= 0) atomicAdd(&xs.rcnt[(int)(kk[u] >> 5) & 31], 1);
+                if (lane + 32 * u < nt) at[u] = atomicAdd(&xs.rcnt[(kk[u] >> 5) & 31], 1);
             __syncwarp();
             const int rc = xs.rcnt[lane];
             int incl = rc;
@@ -529,47 +545,47 @@ __global__ void __launch_bounds__(CSR_AW * 32, 2)
                 const int v = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += v;
             }
-            xs.roff[lane] = incl - rc;
-            xs.rcnt[lane] = 0;
+            roff[lane] = incl - rc;
             __syncwarp();
 #pragma unroll
             for (int u = 0; u < PER; ++u)
-                if (kk[u] >= 0) {
-                    const int rl = (int)(kk[u] >> 5) & 31;
-                    const int at = xs.roff[rl] + atomicAdd(&xs.rcnt[rl], 1);
-                    xs.skey[at] = kk[u];
-                    xs.sprod[at] = pp[u];
+                if (lane + 32 * u < nt) {
+                    const int q = roff[(kk[u] >> 5) & 31] + at[u];
+                    skey[q] = kk[u];
+                    sprod[q] = pp[u];
                 }
             __syncwarp();
             const int b0 = incl - rc, b1 = incl;
-            const int64_t *sk = xs.skey;
-            const T *sp = xs.sprod;
+            const uint32_t *sk = skey;
+            const T *sp = sprod;
             if (__reduce_max_sync(0xffffffffu, (unsigned)rc) > (unsigned)CSC_SHORT_ROW) {
                 // rank every key of the tile (keys are unique; the rank order groups the rows in
                 // the order of the counting sort, so the row segments stay where they are)
+                uint32_t *rkey = xs.rkey();
+                T *rprod = xs.rprod();
 #pragma unroll
                 for (int u = 0; u < PER; ++u)
-                    if (kk[u] >= 0) {
+                    if (lane + 32 * u < nt) {
                         int r = 0;
-                        for (int y = 0; y < nt; ++y) r += xs.skey[y] < kk[u] ? 1 : 0;
-                        xs.rkey[r] = kk[u];
-                        xs.rprod[r] = pp[u];
+                        for (int y = 0; y < nt; ++y) r += skey[y] < kk[u] ? 1 : 0;
+                        rkey[r] = kk[u];
+                        rprod[r] = pp[u];
                     }
                 __syncwarp();
-                sk = xs.rkey;
-                sp = xs.rprod;
+                sk = rkey;
+                sp = rprod;
             } else {
                 for (int h = b0 + 1; h < b1; ++h) {  // lane r: its row's few entries by key
-                    const int64_t kv = xs.skey[h];
-                    const T pv = xs.sprod[h];
+                    const uint32_t kv = skey[h];
+                    const T pv = sprod[h];
                     int q = h - 1;
-                    while (q >= b0 && xs.skey[q] > kv) {
-                        xs.skey[q + 1] = xs.skey[q];
-                        xs.sprod[q + 1] = xs.sprod[q];
+                    while (q >= b0 && skey[q] > kv) {
+                        skey[q + 1] = skey[q];
+                        sprod[q + 1] = sprod[q];
                         --q;
                     }
-                    xs.skey[q + 1] = kv;
-                    xs.sprod[q + 1] = pv;
+                    skey[q + 1] = kv;
+                    sprod[q + 1] = pv;
                 }
             }
             for (int h = b0; h < b1; ++h) {  // the products per j in element order
@@ -579,80 +595,108 @@ __global__ void __launch_bounds__(CSR_AW * 32, 2)
             }
             __syncwarp();
         }
+        const int64_t done = tile;
+        tile += tstride;
+        load_tile(tile);
         csr_row_finish<T, KIND>(ws, cs, A, kp, t0, lane, nr, touched, rs, g);
-        if (lane == 0) W.tile_cnt[tile] = 0;  // the counter returns to zero for the next chunk
+        if (lane == 0) W.tile_cnt[done * CSC_CNT_STRIDE] = 0;  // back to zero for the next chunk
     }
 }
 
 // Store (the sampled Gram and the component block): one warp per listed row
-// (rows == nullptr: row r), columns S[j0 .. j0 + jc).  The lanes resolve a
-// group of 32 nonzeros' hits in parallel, then the hits are added one at a
-// time in element order (a slot with several entries spreads its distinct j
-// over the lanes), so every partial dot is summed in a fixed order -- the
-// products and order of the apply kernel.
-template <typename T>
+// (rows == nullptr: row r), columns S[j0 .. j0 + jc).  The lanes resolve the
+// hits of two groups of 32 nonzeros in parallel, then the hits are added one
+// at a time in element order, each by the lane that owns its column (column j
+// in register j / 32 of lane j % 32), so every partial dot is summed in a
+// fixed order -- the products and order of the apply kernel.  Latency-bound:
+// a row of the Gram meets all its own columns, and adding those through one
+// lane and shared memory, a group at a time, took 10.7 us at 32 rows of 50
+// (now 10, and 5 for the rows between two steps).
+constexpr int CSR_GU = 2;  // groups of nonzeros resolved at once
+
+template <typename T, int NJ>
 __global__ void __launch_bounds__(CSR_WARPS * 32)
     csr_gram_kernel(CsrOperand A, CsrColMap M, const int32_t *rows, int64_t nrows, const int32_t *S, int j0, int jc,
                     KernelParams kp, float *out32, double *out64, int64_t ldo)
 {
-    __shared__ T acc[CSR_WARPS][CSR_GJ];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const T *vals = (const T *)(sizeof(T) == 8 ? (const void *)A.vals64 : (const void *)A.vals32);
     const T *norm = (const T *)(sizeof(T) == 8 ? (const void *)A.norm64 : (const void *)A.norm32);
-    for (int64_t k = (int64_t)blockIdx.x * CSR_WARPS + warp; k < nrows; k += (int64_t)gridDim.x * CSR_WARPS) {
-        for (int j = lane; j < jc; j += 32) acc[warp][j] = (T)0;
-        __syncwarp();
+    for (int64_t k = (int64_t)blockIdx.x * nw + warp; k < nrows; k += (int64_t)gridDim.x * nw) {
+        T acc[NJ];
+#pragma unroll
+        for (int u = 0; u < NJ; ++u) acc[u] = (T)0;
+        // the hit (j, product) added by the lane that owns column j
+        auto add = [&](int j, T p) {
+#pragma unroll
+            for (int u = 0; u < NJ; ++u)
+                if (j == 32 * u + lane) acc[u] += p;
+        };
         const int64_t r = rows ? (int64_t)rows[k] : k;
         const int64_t e0 = A.row_ptr[r], e1 = A.row_ptr[r + 1];
-        for (int64_t eb = e0; eb < e1; eb += 32) {
+        for (int64_t eb = e0; eb < e1; eb += 32 * CSR_GU) {
+            int jj[CSR_GU];   // column, or -2 - slot (over two entries), or -1
+            int j2[CSR_GU];   // the column of a slot's second entry, or -1
+            T prod[CSR_GU], prod2[CSR_GU];
+            unsigned mk[CSR_GU];
             // the lanes resolve their hits in parallel: value, slot, and for a slot with one entry
             // (nearly all) its column and the product
-            const int64_t e = eb + lane;
-            const int32_t c = e < e1 ? __ldg(A.col_idx + e) : -1;
-            const bool hit = c >= 0 && col_hit(M.bits, c);
-            int jj = -1;
-            T prod = (T)0;
-            if (hit) {
-                const T v = vals[e];
-                const int slot = col_slot(M.bits, M.wprefix, c);
-                const int q0 = M.slot_off[slot], q1 = M.slot_off[slot + 1];
-                if (q1 - q0 == 1) {
-                    const int j = M.ent_j[q0] - j0;
-                    jj = j >= 0 && j < jc ? j : -1;
-                    prod = mul_rn(v, (T)M.ent_v[q0]);
-                } else {
-                    jj = -2 - slot;
-                    prod = v;
-                }
-            }
-            // then add them in element order
-            unsigned mk = __ballot_sync(0xffffffffu, hit);
-            while (mk) {
-                const int src = __ffs(mk) - 1;
-                mk &= mk - 1;
-                const int js = __shfl_sync(0xffffffffu, jj, src);
-                const T ps = __shfl_sync(0xffffffffu, prod, src);
-                if (js >= 0) {
-                    if (lane == 0) acc[warp][js] += ps;
-                } else if (js <= -2) {  // several sampled rows hold this column: distinct j, one per lane
-                    const int sl = -2 - js;
-                    for (int q = M.slot_off[sl] + lane; q < M.slot_off[sl + 1]; q += 32) {
-                        const int j = M.ent_j[q] - j0;
-                        if (j >= 0 && j < jc) acc[warp][j] += mul_rn(ps, (T)M.ent_v[q]);
+#pragma unroll
+            for (int u = 0; u < CSR_GU; ++u) {
+                const int64_t e = eb + 32 * u + lane;
+                const int32_t c = e < e1 ? __ldg(A.col_idx + e) : -1;
+                const bool hit = c >= 0 && col_hit(M.bits, c);
+                jj[u] = j2[u] = -1;
+                prod[u] = prod2[u] = (T)0;
+                if (hit) {
+                    const T v = vals[e];
+                    const int slot = col_slot(M.bits, M.wprefix, c);
+                    const int q0 = M.slot_off[slot], q1 = M.slot_off[slot + 1];
+                    if (q1 - q0 <= 2) {  // (a column that two sampled rows hold is not rare)
+                        const int j = M.ent_j[q0] - j0, k2 = M.ent_j[q1 - 1] - j0;
+                        jj[u] = j >= 0 && j < jc ? j : -1;
+                        j2[u] = q1 - q0 == 2 && k2 >= 0 && k2 < jc ? k2 : -1;
+                        prod[u] = mul_rn(v, (T)M.ent_v[q0]);
+                        prod2[u] = mul_rn(v, (T)M.ent_v[q1 - 1]);
+                    } else {
+                        jj[u] = -2 - slot;
+                        prod[u] = v;
                     }
                 }
-                __syncwarp();
+                mk[u] = __ballot_sync(0xffffffffu, jj[u] != -1 || j2[u] != -1);
             }
+            // then they are added in element order
+#pragma unroll
+            for (int u = 0; u < CSR_GU; ++u)
+                while (mk[u]) {
+                    const int src = __ffs(mk[u]) - 1;
+                    mk[u] &= mk[u] - 1;
+                    const int js = __shfl_sync(0xffffffffu, jj[u], src);
+                    const T ps = __shfl_sync(0xffffffffu, prod[u], src);
+                    if (js >= -1) {
+                        const int js2 = __shfl_sync(0xffffffffu, j2[u], src);
+                        add(js, ps);
+                        if (js2 >= 0) add(js2, __shfl_sync(0xffffffffu, prod2[u], src));
+                    } else {  // more sampled rows hold this column: distinct columns j
+                        const int sl = -2 - js;
+                        for (int q = M.slot_off[sl]; q < M.slot_off[sl + 1]; ++q) {
+                            const int j = M.ent_j[q] - j0;
+                            if (j >= 0 && j < jc) add(j, mul_rn(ps, (T)M.ent_v[q]));
+                        }
+                    }
+                }
         }
         const T na = kp.kind == DCD_RBF ? norm[r] : (T)0;
-        for (int j = lane; j < jc; j += 32) {
+#pragma unroll
+        for (int u = 0; u < NJ; ++u) {
+            const int j = 32 * u + lane;
+            if (j >= jc) continue;
             const int32_t sj = S[j0 + j];
             const T nb = kp.kind == DCD_RBF ? norm[sj] : (T)0;
-            const T kv = kfun_t<T>(kp, acc[warp][j], na, nb, sj == r);
+            const T kv = kfun_t<T>(kp, acc[u], na, nb, sj == r);
             if (sizeof(T) == 8) out64[k * ldo + j0 + j] = (double)kv;
             else out32[k * ldo + j0 + j] = (float)kv;
         }
-        __syncwarp();
     }
 }
 
@@ -803,6 +847,126 @@ __global__ void __launch_bounds__(MAP_THREADS) csr_colmap_kernel(CsrOperand A, c
 
 // squared row norms (FP32 and FP64), the longest row, and a validity check
 // of the CSR arrays (bad counts the offending rows and entries)
+
+// The same map with every entry in registers: the sampled rows' nonzeros as one flat range of at most
+// MAP_E a thread (position j = x / maxrow, nonzero q = x % maxrow), read once, all loads of a level in
+// flight together; the counts per slot in shared memory, whose atomics give each entry its place.
+// Latency-bound (four dependent loads: sample, row, column, its CSC range): the general kernel, which
+// walks the rows again for each pass and counts in memory, took 20 us at 32 rows of 50, n = 50000
+// (this one 9.5).
+constexpr int MAP_E = 4;
+
+__global__ void __launch_bounds__(MAP_THREADS) csr_colmap_small_kernel(CsrOperand A, const int32_t *S, int cnt,
+                                                                       int maxrow, CsrColMap M, int *err)
+{
+    extern __shared__ uint32_t map_sm[];
+    __shared__ int wsum[MAP_THREADS / 32];
+    __shared__ int tot_slots, tot_ent;
+    uint32_t *bits = map_sm;
+    int32_t *wprefix = (int32_t *)(map_sm + M.nw);
+    int32_t *counts = wprefix + M.nw;  // MAP_E * MAP_THREADS
+    const int tid = threadIdx.x;
+    const int total = cnt * maxrow;
+    int j[MAP_E], c[MAP_E];
+    int64_t e[MAP_E];
+    double v[MAP_E];
+#pragma unroll
+    for (int i = 0; i < MAP_E; ++i) {
+        const int x = tid + i * MAP_THREADS;
+        j[i] = x < total ? x / maxrow : -1;
+        e[i] = -1;
+        c[i] = -1;
+        if (j[i] < 0) continue;
+        const int q = x - j[i] * maxrow;
+        const int64_t r = S[j[i]];
+        if (r < 0 || r >= A.m) {
+            if (q == 0) set_error(err, DEV_BAD_INDEX);
+            continue;
+        }
+        const int64_t e0 = A.row_ptr[r], e1 = A.row_ptr[r + 1];
+        if (e0 + q < e1) e[i] = e0 + q;
+    }
+#pragma unroll
+    for (int i = 0; i < MAP_E; ++i) {
+        v[i] = 0.0;
+        if (e[i] < 0) continue;
+        c[i] = A.col_idx[e[i]];
+        v[i] = A.vals64 ? A.vals64[e[i]] : (double)A.vals32[e[i]];
+    }
+    for (int w = tid; w < M.nw; w += MAP_THREADS) bits[w] = 0u;
+    for (int w = tid; w < MAP_E * MAP_THREADS; w += MAP_THREADS) counts[w] = 0;
+    __syncthreads();
+    // 1. mark the columns; the transposed apply's pair table meanwhile: per sampled position and nonzero
+    // slot, the column's CSC range and the value
+#pragma unroll
+    for (int i = 0; i < MAP_E; ++i)
+        if (c[i] >= 0) atomicOr(&bits[c[i] >> 5], 1u << (c[i] & 31));
+    if (M.plen && M.pmax) {
+        int64_t c0[MAP_E], c1[MAP_E];
+#pragma unroll
+        for (int i = 0; i < MAP_E; ++i) {
+            c0[i] = c[i] >= 0 ? M.csc_col_ptr[c[i]] : 0;
+            c1[i] = c[i] >= 0 ? M.csc_col_ptr[c[i] + 1] : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < MAP_E; ++i)
+            if (j[i] >= 0) {
+                const int64_t at = (int64_t)j[i] * M.pmax + (tid + i * MAP_THREADS - j[i] * maxrow);
+                M.pstart[at] = c0[i];
+                M.plen[at] = (int32_t)(c1[i] - c0[i]);
+                M.pval[at] = v[i];
+            }
+    }
+    __syncthreads();
+    // 2. exclusive popcount prefix over the words (contiguous chunk per thread)
+    const int per = (M.nw + MAP_THREADS - 1) / MAP_THREADS;
+    const int w0 = min(M.nw, tid * per), w1 = min(M.nw, w0 + per);
+    int s = 0;
+    for (int w = w0; w < w1; ++w) s += __popc(bits[w]);
+    int run = cta_excl_scan(s, wsum, &tot_slots);
+    for (int w = w0; w < w1; ++w) {
+        wprefix[w] = run;
+        run += __popc(bits[w]);
+    }
+    __syncthreads();
+    const int nslots = tot_slots;  // at most the entries
+    // 3. each entry's slot and its place in it
+    int slot[MAP_E], ord[MAP_E];
+#pragma unroll
+    for (int i = 0; i < MAP_E; ++i)
+        if (c[i] >= 0) {
+            slot[i] = wprefix[c[i] >> 5] + __popc(bits[c[i] >> 5] & ((1u << (c[i] & 31)) - 1u));
+            ord[i] = atomicAdd(&counts[slot[i]], 1);
+        }
+    for (int w = tid; w < M.nw; w += MAP_THREADS) {
+        M.bits[w] = bits[w];
+        M.wprefix[w] = wprefix[w];
+    }
+    __syncthreads();
+    // 4. slot offsets: exclusive scan of the counts (contiguous chunk per thread)
+    const int sper = (nslots + MAP_THREADS - 1) / MAP_THREADS;
+    const int s0 = min(nslots, tid * sper), s1 = min(nslots, s0 + sper);
+    int cs = 0;
+    for (int q = s0; q < s1; ++q) cs += counts[q];
+    int run2 = cta_excl_scan(cs, wsum, &tot_ent);
+    for (int q = s0; q < s1; ++q) {
+        const int k = counts[q];
+        M.slot_off[q] = run2;
+        counts[q] = run2;
+        run2 += k;
+    }
+    if (tid == 0) M.slot_off[nslots] = tot_ent;
+    __syncthreads();
+    // 5. the entries
+#pragma unroll
+    for (int i = 0; i < MAP_E; ++i)
+        if (c[i] >= 0) {
+            const int pos = counts[slot[i]] + ord[i];
+            M.ent_j[pos] = j[i];
+            M.ent_v[pos] = v[i];
+        }
+}
+
 __global__ void csr_prep_kernel(CsrOperand A, int *bad, int *maxlen)
 {
     const int lane = threadIdx.x & 31;
@@ -884,12 +1048,14 @@ cudaError_t launch_csr_gram(const CsrOperand &A, const CsrColMap &M, const int32
                             const int32_t *S, int64_t ncols, const KernelParams &kp, float *out32, double *out64,
                             int64_t ldo, cudaStream_t st)
 {
-    int64_t grid = (nrows + CSR_WARPS - 1) / CSR_WARPS;
+    // few rows: a warp per CTA, each on an SM of its own
+    const int warps = nrows <= sm_count() ? 1 : CSR_WARPS;
+    int64_t grid = (nrows + warps - 1) / warps;
     if (grid > sm_count() * 8) grid = sm_count() * 8;
     for (int64_t j0 = 0; j0 < ncols; j0 += CSR_GJ) {
         const int jc = (int)min((int64_t)CSR_GJ, ncols - j0);
-        csr_gram_kernel<T><<<(unsigned)grid, CSR_WARPS * 32, 0, st>>>(A, M, rows, nrows, S, (int)j0, jc, kp, out32,
-                                                                       out64, ldo);
+        auto kfn = jc <= 32 ? csr_gram_kernel<T, 1> : jc <= 128 ? csr_gram_kernel<T, 4> : csr_gram_kernel<T, CSR_GJ / 32>;
+        kfn<<<(unsigned)grid, warps * 32, 0, st>>>(A, M, rows, nrows, S, (int)j0, jc, kp, out32, out64, ldo);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -957,18 +1123,19 @@ __global__ void __launch_bounds__(1024) excl_scan_kernel(const int32_t *cnt, int
 }
 
 template <typename T>
-__global__ void csc_fill_kernel(CsrOperand A, const int64_t *col_ptr, int32_t *cur, int32_t *row, int64_t *elem,
+__global__ void csc_fill_kernel(CsrOperand A, const int64_t *col_ptr, int32_t *cur, int32_t *row, uint32_t *elem,
                                 T *val)
 {
     const int lane = threadIdx.x & 31;
     const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (r >= A.m) return;
     const T *vals = (const T *)(sizeof(T) == 8 ? (const void *)A.vals64 : (const void *)A.vals32);
+    const int64_t t0 = A.row_ptr[r & ~(int64_t)31];  // the tile's first nonzero
     for (int64_t e = A.row_ptr[r] + lane; e < A.row_ptr[r + 1]; e += 32) {
         const int32_t c = A.col_idx[e];
         const int64_t pos = col_ptr[c] + atomicAdd(cur + c, 1);
         row[pos] = (int32_t)r;
-        elem[pos] = e;
+        elem[pos] = (uint32_t)(e - t0);
         val[pos] = vals[e];
     }
 }
@@ -988,7 +1155,7 @@ cudaError_t launch_csc_apply_k(const CsrOperand &A, const CsrColMap &M, const Cs
                                const double *w64, const double *rs, double *g, bool first_scattered, cudaStream_t st)
 {
     auto kfn = csc_apply_kernel<T, KIND>;
-    const size_t smem = sizeof(CtaSmem<T>) + (sizeof(WarpSmem<T>) + sizeof(CscWarpSmem<T>)) * CSR_AW;
+    const size_t smem = csc_cta_bytes<T>() + sizeof(CscWarpSmem<T>) * CSR_AW;
     static int per_sm = 0;  // resident CTAs per SM, queried once per instantiation (before any capture)
     if (!per_sm) {
         cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1062,9 +1229,25 @@ cudaError_t launch_csr_prep(const CsrOperand &A, int *bad, int *maxlen, cudaStre
 }
 
 cudaError_t launch_csr_colmap(const CsrOperand &A, const int32_t *S, int64_t cnt, const CsrColMap &M, int *err,
-                              cudaStream_t st)
+                              cudaStream_t st, int maxrow)
 {
     if (cnt <= 0) return cudaSuccess;
+    // (rows of about one length: a flat range of maxrow slots a row wastes little; the pair table, where
+    // there is one, has as many)
+    if (maxrow > 0 && cnt * maxrow <= MAP_E * MAP_THREADS && M.nw <= MAP_SMEM_WORDS && cnt * maxrow <= M.cap &&
+        (!M.plen || M.pmax == 0 || M.pmax == maxrow)) {
+        const size_t smem = (size_t)M.nw * 8 + sizeof(int32_t) * MAP_E * MAP_THREADS;
+        static bool attr = false;
+        if (!attr) {
+            const cudaError_t e =
+                cudaFuncSetAttribute(csr_colmap_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     MAP_SMEM_WORDS * 8 + (int)sizeof(int32_t) * MAP_E * MAP_THREADS);
+            if (e != cudaSuccess) return e;
+            attr = true;
+        }
+        csr_colmap_small_kernel<<<1, MAP_THREADS, smem, st>>>(A, S, (int)cnt, maxrow, M, err);
+        return cudaGetLastError();
+    }
     if (M.nw <= MAP_SMEM_WORDS) {
         const size_t smem = (size_t)M.nw * 8;
         static bool attr = false;
@@ -1109,7 +1292,7 @@ size_t take_bytes(char *&p, size_t bytes)
 
 size_t csc_bytes(int64_t n, int64_t nnz, bool fp64)
 {
-    return (size_t)(n + 1) * 8 + (size_t)n * 4 + (size_t)nnz * (4 + 8 + (fp64 ? 8 : 4)) + 256 * 5;
+    return (size_t)(n + 1) * 8 + (size_t)n * 4 + (size_t)nnz * (4 + 4 + (fp64 ? 8 : 4)) + 256 * 5;
 }
 
 cudaError_t launch_csc_build(const CsrOperand &A, bool fp64, void *base, CscOperand *C, int *maxcol_dev,
@@ -1122,8 +1305,8 @@ cudaError_t launch_csc_build(const CsrOperand &A, bool fp64, void *base, CscOper
     take_bytes(p, (size_t)A.n * 4);
     int32_t *row = (int32_t *)p;
     take_bytes(p, (size_t)A.nnz * 4);
-    int64_t *elem = (int64_t *)p;
-    take_bytes(p, (size_t)A.nnz * 8);
+    uint32_t *elem = (uint32_t *)p;
+    take_bytes(p, (size_t)A.nnz * 4);
     void *val = p;
     C->col_ptr = col_ptr;
     C->row = row;
@@ -1149,8 +1332,8 @@ cudaError_t launch_csc_build(const CsrOperand &A, bool fp64, void *base, CscOper
 size_t csc_step_bytes(int64_t m, int64_t cnt, int maxrow, bool fp64)
 {
     const int64_t ntiles = (m + 31) / 32, pairs = cnt * (int64_t)std::max(maxrow, 1);
-    return (size_t)ntiles * 4 + (size_t)ntiles * CSC_TILE_CAP * (8 + (fp64 ? 8 : 4)) + (size_t)pairs * (8 + 4 + 8) +
-           256 * 6;
+    return (size_t)ntiles * 4 * CSC_CNT_STRIDE + (size_t)ntiles * CSC_TILE_CAP * (4 + (fp64 ? 8 : 4)) +
+           (size_t)pairs * (8 + 4 + 8) + 256 * 6;
 }
 
 CscStep csc_step_carve(void *base, int64_t m, int64_t cnt, int maxrow, const CscOperand &C, CsrColMap *M)
@@ -1159,9 +1342,9 @@ CscStep csc_step_carve(void *base, int64_t m, int64_t cnt, int maxrow, const Csc
     char *p = (char *)base;
     CscStep W;
     W.tile_cnt = (int32_t *)p;
-    take_bytes(p, (size_t)ntiles * 4);
-    W.key = (int64_t *)p;
-    take_bytes(p, (size_t)ntiles * CSC_TILE_CAP * 8);
+    take_bytes(p, (size_t)ntiles * 4 * CSC_CNT_STRIDE);
+    W.key = (uint32_t *)p;
+    take_bytes(p, (size_t)ntiles * CSC_TILE_CAP * 4);
     M->pstart = (int64_t *)p;
     take_bytes(p, (size_t)pairs * 8);
     M->pval = (double *)p;

@@ -376,22 +376,25 @@ struct CsrColMap {
 size_t csr_colmap_bytes(int64_t n, int64_t cap);
 CsrColMap csr_colmap_carve(void *base, int64_t n, int64_t cap);
 cudaError_t launch_csr_prep(const CsrOperand &A, int *bad, int *maxlen, cudaStream_t st);
+// (maxrow: the longest row of A where the caller knows it, else 0)
 cudaError_t launch_csr_colmap(const CsrOperand &A, const int32_t *S, int64_t cnt, const CsrColMap &M, int *err,
-                              cudaStream_t st);
+                              cudaStream_t st, int maxrow = 0);
 // Transposed copy of a CSR operand: per column its entries' rows, CSR element
 // indices and values (in the block's precision); and the per-step scratch of
 // the apply through it: per 32-row tile a counter (zero between uses) and a
-// bucket of incidence keys and products.
+// bucket of incidence keys and products.  (No row longer than CSC_ROW_MAX: the offsets of a tile fit
+// the keys.)
+constexpr int CSC_ROW_MAX = (1 << 22) / 32 - 1;
 struct CscOperand {
     const int64_t *col_ptr = nullptr;
     const int32_t *row = nullptr;
-    const int64_t *elem = nullptr;
+    const uint32_t *elem = nullptr;  // offset from the first nonzero of the row's 32-row tile, < 2^22
     const void *val = nullptr;
     int64_t n = 0;
 };
 struct CscStep {
     int32_t *tile_cnt = nullptr;
-    int64_t *key = nullptr;
+    uint32_t *key = nullptr;  // element offset, row in tile (5 bits), sampled position (5 bits)
     void *prod = nullptr;
 };
 size_t csc_bytes(int64_t n, int64_t nnz, bool fp64);

@@ -116,7 +116,7 @@ dcd_status csc_choose(const CsrOperand &ca, bool fp64, int64_t cnt, int maxrow, 
     *use = false;
     const int64_t jc = std::min<int64_t>(cnt, 32);
     const int64_t m = ca.m, n = ca.n;
-    if (ca.nnz <= 0 || m <= 0 || jc <= 0) return DCD_OK;
+    if (ca.nnz <= 0 || m <= 0 || jc <= 0 || maxrow > CSC_ROW_MAX) return DCD_OK;
     DCD_TRY(malloc_async(ws_csc, csc_bytes(n, ca.nnz, fp64), st));
     DCD_TRY(launch_csc_build(ca, fp64, *ws_csc, C, maxcol_dev, st));
     std::vector<int64_t> cp((size_t)n + 1);
@@ -275,6 +275,11 @@ struct Solver {
     CscOperand cscop;
     CscStep cstep;
     void *ws_csc = nullptr, *ws_cstep = nullptr;
+    // the deferred step's buckets of each set, filled a step ahead (none: each step fills its own)
+    CscStep cstep_set[3];
+    void *ws_cstep2 = nullptr;
+    bool scatter_ahead = false;
+    int csr_scattered = -1;  // the set whose buckets hold its first chunk
     int csr_maxrow = 0;
     // the first chunk's scatter runs on csr_st beside the Gram and the recurrence
     cudaStream_t csr_st = nullptr;
@@ -326,6 +331,7 @@ struct Solver {
         if (csr_join) cudaEventDestroy(csr_join);
         if (ws_csc) cudaFreeAsync(ws_csc, st);
         if (ws_cstep) cudaFreeAsync(ws_cstep, st);
+        if (ws_cstep2) cudaFreeAsync(ws_cstep2, st);
         if (ws_f64s) cudaFreeAsync(ws_f64s, st);
         if (ws) cudaFreeAsync(ws, st);
     }
@@ -714,6 +720,24 @@ struct Solver {
                 c2.csc_col_ptr = cm.csc_col_ptr;
                 cm_set[q] = c2;
             }
+            if (dfs && use_csc) {
+                const size_t bb = (csc_step_bytes(m, sb, csr_maxrow, !tc) + 255) / 256 * 256;
+                const cudaError_t e = malloc_async(&ws_cstep2, 2 * bb, st);
+                if (e == cudaSuccess) {
+                    DCD_TRY(cudaMemsetAsync(ws_cstep2, 0, 2 * bb, st));
+                    CsrColMap unused;
+                    cstep_set[0] = cstep;
+                    for (int q = 1; q < 3; ++q)
+                        cstep_set[q] =
+                            csc_step_carve((char *)ws_cstep2 + (q - 1) * bb, m, sb, csr_maxrow, cscop, &unused);
+                    scatter_ahead = true;
+                } else if (e == cudaErrorMemoryAllocation) {
+                    cudaGetLastError();
+                    ws_cstep2 = nullptr;
+                } else {
+                    return cuda_status(e);
+                }
+            }
         } else if (tc) {
             op.n_pad = n_pad;
             op.kind = pack_kind(o.prec);
@@ -948,7 +972,7 @@ struct Solver {
     // gather A_S for the tensor-core path (of the step operand, or of x)
     cudaError_t gather(int64_t ncols)
     {
-        if (csr) return launch_csr_colmap(ca, S, ncols, cm, err, st);
+        if (csr) return launch_csr_colmap(ca, S, ncols, cm, err, st, csr_maxrow);
         if (f64s) return launch_gather_rows(fs.packed, f64s_row_bytes(n), S, ncols, m, As, err, st);
         return gather_op(ncols, op, As, col_h);
     }
@@ -1072,12 +1096,14 @@ struct Solver {
         return e;
     }
 
-    cudaError_t csr_apply(int64_t ncols, const double *rs)
+    // (scattered: the first chunk's scatter is done)
+    cudaError_t csr_apply(int64_t ncols, const double *rs, bool scattered = false)
     {
         if (use_csc) {
-            const bool first = csr_forked;
+            const bool first = csr_forked || scattered;
+            const bool join = csr_forked;
             csr_forked = false;
-            if (first) {
+            if (join) {
                 const cudaError_t e = cudaStreamWaitEvent(st, csr_join, 0);
                 if (e != cudaSuccess) return e;
             }
@@ -1256,6 +1282,7 @@ struct Solver {
             col_w = sbuf[p].col_w;
         }
         if (lag && csr) cm = cm_set[p];
+        if (scatter_ahead) cstep = cstep_set[p];
         if (ref_shared) {
             Asr = As;
             col_hr = col_h;
@@ -1613,17 +1640,18 @@ struct Solver {
     {
         const int nxt = (cur + 1) % 3, nn = (cur + 2) % 3;
         const bool scatter = csr && use_csc;
+        // what needs only the index stream and the products before it forks off at the start
+        if (has2) DCD_TRY(cudaEventRecord(la_fork, st));
+        if (scatter && !scatter_ahead) DCD_TRY(cudaEventRecord(csr_fork, st));
         if (has1) {
             DCD_TRY(launch_dcd_snapshot(sbuf[nxt].S, o.s, m, alpha, g, dfs_v[nxt][0], dfs_v[nxt][2], st));
             DCD_TRY(cudaEventRecord(df_fork, st));
-        }
-        if (scatter) DCD_TRY(cudaEventRecord(csr_fork, st));
-        if (has1) {  // the recurrence first, so that it is the first of the step's kernels to take an SM
+            // the recurrence first, so that it is the first of the step's kernels to take an SM
             DCD_TRY(cudaStreamWaitEvent(st3, df_fork, 0));
             DCD_TRY(dfs_chain_of(nxt, o.s, true, st3));
         }
         if (has2) {
-            DCD_TRY(cudaStreamWaitEvent(st2, df_fork, 0));
+            DCD_TRY(cudaStreamWaitEvent(st2, la_fork, 0));
             dcd_status r = lag_side(nn, o.s, st2, (nn + 1) % 3, df_rows);
             if (r != DCD_OK) return r;
             DCD_TRY(cudaEventRecord(la_join, st2));
@@ -1636,7 +1664,7 @@ struct Solver {
         if (has1) DCD_TRY(cudaEventRecord(df_side, st3));
         use_bufs(cur);
         const int64_t ncols = cnt * o.b;
-        if (scatter) {  // this step's first scatter through the transposed copy, beside the block's start
+        if (scatter && !scatter_ahead) {  // this step's first scatter, beside the block's start
             DCD_TRY(cudaStreamWaitEvent(csr_st, csr_fork, 0));
             DCD_TRY(launch_csr_csc_scatter_first(cm, cscop, cstep, !tc, csr_maxrow, ncols, csr_st));
             DCD_TRY(cudaEventRecord(csr_join, csr_st));
@@ -1644,12 +1672,21 @@ struct Solver {
         }
         const double *rs = y;
         if (csr)
-            DCD_TRY(csr_apply(ncols, rs));
+            DCD_TRY(csr_apply(ncols, rs, scatter_ahead));
         else if (tc)
             DCD_TRY(block_tc_apply(ncols, rs));  // (every set's coefficients past sb stay zero)
         else
             DCD_TRY(block_f64_apply(ncols, rs));
+        if (scatter_ahead && has1) {
+            // the next step's first scatter through the transposed copy into its set's buckets, beside this
+            // whole step (its column map is a step old); behind the snapshot and captured last, as the
+            // dispatch of its many CTAs holds up what is launched after them
+            DCD_TRY(cudaStreamWaitEvent(csr_st, df_fork, 0));
+            DCD_TRY(launch_csr_csc_scatter_first(cm_set[nxt], cscop, cstep_set[nxt], !tc, csr_maxrow, o.s, csr_st));
+            DCD_TRY(cudaEventRecord(csr_join, csr_st));
+        }
         DCD_TRY(launch_update(S, delta, ncols, diag, alpha, g, ctr, (uint64_t)cnt, m, err, st));
+        if (scatter_ahead && has1) DCD_TRY(cudaStreamWaitEvent(st, csr_join, 0));
         if (has2) DCD_TRY(cudaStreamWaitEvent(st, la_join, 0));
         if (has1) DCD_TRY(cudaStreamWaitEvent(st, df_side, 0));
         return DCD_OK;
@@ -1681,6 +1718,10 @@ struct Solver {
             }
             df_chain = true;
         }
+        if (scatter_ahead && csr_scattered != cur) {
+            DCD_TRY(launch_csr_csc_scatter_first(cm_set[cur], cscop, cstep_set[cur], !tc, csr_maxrow, cnt, st));
+            csr_scattered = cur;
+        }
         dcd_status r = DCD_OK;
         *ran = 1;
         if (has1 && has2)  // the steady state
@@ -1691,6 +1732,7 @@ struct Solver {
         if (r != DCD_OK) return r;
         const int last = (cur + (int)(*ran - 1)) % 3;  // the set of the last step run
         df_cur = (last + 1) % 3;
+        csr_scattered = has1 ? df_cur : -1;
         df_chain = has1;
         df_prod = has2 ? o.s : 0;
         la_cnt = has1 ? o.s : 0;  // the products of the next step are in place
