@@ -75,7 +75,6 @@ dcd_status csc_choose(const CsrOperand &ca, bool fp64, int64_t cnt, int maxrow, 
 constexpr int64_t SB_MAX = 8192;   // s*b per outer step
 constexpr int B_MAX = 128;         // block size
 constexpr int DF_XPAIRS = 16;      // CTA pairs (at most) of the deferred gradient's cross product
-constexpr int DF_GRAM_CTAS = 24;   // CTAs (at most) of the Gram computed beside the deferred step's block
 
 // Set while the batched driver and the autotuner build their plans: those
 // capture many plans' steps into one graph and run without the look-ahead.
@@ -648,13 +647,9 @@ struct Solver {
             DCD_TRY(cudaEventCreateWithFlags(&df_rows, cudaEventDisableTiming));
             DCD_TRY(cudaEventCreateWithFlags(&df_gram, cudaEventDisableTiming));
             DCD_TRY(cudaStreamCreateWithFlags(&st3, cudaStreamNonBlocking));
-            // the block leaves SMs for the recurrence ahead (one cluster) and the next step's Gram (an
-            // item a CTA; its chunks are 256 columns at most)
+            // the block leaves SMs for the recurrence ahead (one cluster) and the next step's Gram
             const int P = recur_cluster_size((int)o.s, o.b, 2);
-            int gi = tc_store_items(sb, sb, 64, true);
-            for (int w = 128; gi > DF_GRAM_CTAS && w <= 256; w *= 2) gi = tc_store_items(sb, sb, w, true);
-            df_gram_ctas = std::min(gi, DF_GRAM_CTAS);
-            df_pairs = std::max(split_pairs - (P + 1) / 2 - (df_gram_ctas + 1) / 2, 1);
+            df_split(split_pairs - (P + 1) / 2, (int)((sb + 255) / 256));
             int p_least = 0, p_greatest = 0;
             DCD_TRY(cudaDeviceGetStreamPriorityRange(&p_least, &p_greatest));
             df_prio = p_greatest;
@@ -1419,6 +1414,35 @@ struct Solver {
     int df_pairs = 0;          // CTA pairs of the block
     int df_gram_ctas = 0;      // CTAs of the Gram beside it
     int df_prio = 0;           // launch priority of the recurrence and the block
+
+    // The SMs that the block (`avail` CTA pairs without the recurrence's cluster) leaves to the Gram of
+    // the step after next.  A step lasts as long as the longer of two paths: the block, whole rounds of
+    // (256-row tile, 256-column chunk) units over its pairs, then the update; and the sampled rows, their
+    // Gram, the panels' preparation and the cross product.  So both are estimated (us, from timelines)
+    // for a Gram of at most 24, 16 and 8 CTAs, an item of 128 rows and 64 to 256 columns at a time, and
+    // the shorter step taken.  Measured, 8 steps of m = 50000, n = 512, 1024 coordinates: fp16 541 with
+    // 24 CTAs and 608 with 8; split bf16, where a round of the block takes twice as long, 965 and 931; at
+    // m = 20000, 704 coordinates, TF32x3 679 with 24, 634 with 12, 670 with 8.
+    void df_split(int avail, int chunks)
+    {
+        const int kind = pack_kind(o.prec);
+        const double passes = kind == PACK_TF32X3 ? 6 : kind == PACK_BF16X3 ? 3 : kind == PACK_TF32 ? 2 :
+                              kind == PACK_FP8 ? 0.5 : 1;                   // tensor time of a product, bf16 = 1
+        const double mma = 256.0 * 256.0 * 2.0 * (double)n * passes / 27.6e6;   // a unit on one pair
+        const double unit = std::max(mma, 3.5), units = (double)((m + 255) / 256) * chunks;
+        double best = 0;
+        for (int most : {24, 16, 8}) {
+            int w = 64, items = tc_store_items(sb, sb, w, true);
+            while (items > most && w < 256) items = tc_store_items(sb, sb, w *= 2, true);
+            const int ctas = std::min(items, most), pairs = std::max(avail - (ctas + 1) / 2, 1);
+            const double gram = std::ceil((double)items / ctas) * (4 + 1.15 * mma * w / 256);
+            const double t = std::max(std::ceil(units / pairs) * unit + 18, 58 + gram);
+            if (best > 0 && t >= best) continue;
+            best = t;
+            df_gram_ctas = ctas;
+            df_pairs = pairs;
+        }
+    }
 
     // the recurrence of the step in set q on stream s: right-hand side -(g[S] + x), x the part that
     // step `prev`'s set holds (-1: none, -g[S]); no fused update
