@@ -10,16 +10,19 @@ namespace dcd {
 constexpr int DCD_FAST_MAX = 128;
 constexpr int DCD_FAST_K = DCD_FAST_MAX / 32;
 
-__device__ __forceinline__ int ld_acquire_shared(const int *p)
+// a step that is not decided yet: a signalling NaN, which no FP64 operation returns
+constexpr long long CHAIN_OPEN = 0x7ff4000000000000LL;
+
+__device__ __forceinline__ double chain_ld(const double *p)
 {
-    int v;
-    asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(ptx::su32(p)) : "memory");
+    double v;
+    asm volatile("ld.volatile.shared.f64 %0, [%1];" : "=d"(v) : "r"(ptx::su32(p)) : "memory");
     return v;
 }
 
-__device__ __forceinline__ void st_release_shared(int *p, int v)
+__device__ __forceinline__ void chain_st(double *p, double v)
 {
-    asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(ptx::su32(p)), "r"(v) : "memory");
+    asm volatile("st.volatile.shared.f64 [%0], %1;" ::"r"(ptx::su32(p)), "d"(v) : "memory");
 }
 
 // clip(x, 0, nu) by the bit patterns (nub: those of nu, +infinity for no upper bound); a NaN gives 0,
@@ -31,67 +34,110 @@ __device__ __forceinline__ double clip_bits(double x, long long nub)
     return __longlong_as_double(b > nub ? nub : b);
 }
 
-// Warp `warp`'s 32 coordinates t = 32 warp + lane of a chain of cnt <= DCD_FAST_MAX: returns the lane's
-// step.  C[j ldc + t]: the coupling of t to the step of j < t (zero for t <= j); rep[j DCD_FAST_K +
-// q]: bit l set where coordinate 32 q + l > j holds j's row; list_t, list_j (cnt entries) and pub (two
-// words, zero at the start): the published steps; rho, gj, ie: alpha_t, g_t, 1 / eta_t (0: no step).
-__device__ __forceinline__ double dcd_chain_group(const double *C, int ldc, const uint32_t *rep, double *list_t,
-                                                  int *list_j, int *pub, int cnt, int warp, int lane, double rho,
-                                                  double gj, double ie, double nu, int *err)
+// The chain of one group.  SCALED (each eta in [2^-20, 2^300], a usual nu): the lane keeps u = eta_t
+// alpha_t - g_t, so a round on the critical path is one FMA into u, the clip of u to [0, eta nu] by
+// integer compares, a ballot (the step is nonzero iff the clip differs from eta alpha_t) and, beside
+// the ballot, one FMA to the step clip(u) / eta - alpha: 0.15 us a round.
+// Otherwise the candidate steps are formed as Algorithm 2 writes them, with three more FP64
+// instructions a round: rho - g, rho - g / eta, and the difference to rho (0.38 us).
+template <bool SCALED>
+__device__ __forceinline__ double dcd_chain_run(const double *C, int ldc, const uint32_t *rep, double *slot, int cnt,
+                                                int warp, int lane, double rho, double gj, double eta, double ie,
+                                                double nu, int *err)
 {
     const int t = 32 * warp + lane;
     const bool mine = t < cnt;
     const int tc = mine ? t : cnt - 1;  // a valid column for lanes past the end
-    auto apply = [&](int j, double tj) {
-        gj = fma(C[j * ldc + tc], tj, gj);
-        const uint32_t m = rep[j * DCD_FAST_K + warp];
-        if (m) rho += (m >> lane) & 1u ? tj : 0.0;  // repeats are rare (warp-uniform)
+    double re = rho * eta, x = SCALED ? fma(rho, eta, -gj) : gj;
+    auto repeat = [&](double tj) {  // an earlier coordinate with this one's index moved
+        rho += tj;
+        if (SCALED) {
+            re = rho * eta;
+            x = fma(eta, tj, x);
+        }
     };
-    int n = 0;  // published steps applied (or, in the chain below, published)
-    if (warp > 0) {
+    if (warp > 0) {  // the earlier groups' steps, as they are published, in order
         const long long t0 = clock64();
-        for (;;) {
-            const int dn = ld_acquire_shared(pub + 1);
-            const int np = ld_acquire_shared(pub);
-            for (; n < np; ++n) apply(list_j[n], list_t[n]);
-            if (dn >= warp) break;
-            if (clock64() - t0 > 4200000000LL) {  // about 2 s
-                set_error(err, DEV_TIMEOUT);
-                break;
+        int spins = 0;
+        for (int g = 0; g < warp; ++g) {
+            const uint32_t row = rep[(32 * g + lane) * DCD_FAST_K + warp];
+            const bool any = __any_sync(0xffffffffu, row != 0);
+            for (uint32_t seen = 0; seen != 0xffffffffu;) {
+                const double v = chain_ld(slot + 32 * g + lane);
+                const uint32_t open = __ballot_sync(0xffffffffu, __double_as_longlong(v) == CHAIN_OPEN);
+                const uint32_t ready = (open & (0u - open)) - 1u;  // those below the first open one
+                if (ready == seen) {
+                    if ((++spins & 255) == 0 && __any_sync(0xffffffffu, clock64() - t0 > 4200000000LL)) {  // about 2 s
+                        if (lane == 0) set_error(err, DEV_TIMEOUT);
+                        return 0.0;
+                    }
+                    continue;
+                }
+                uint32_t nz = __ballot_sync(0xffffffffu, (__double_as_longlong(v) << 1) != 0) & ready & ~seen;
+                seen = ready;
+                while (nz) {
+                    const int l = __ffs(nz) - 1;
+                    nz &= nz - 1;
+                    const double tj = __shfl_sync(0xffffffffu, v, l), c = C[(32 * g + l) * ldc + tc];
+                    x = fma(SCALED ? -c : c, tj, x);
+                    if (any && (__shfl_sync(0xffffffffu, row, l) >> lane) & 1u) repeat(tj);
+                }
             }
         }
-        __syncwarp();
     }
     const bool more = 32 * (warp + 1) < cnt;
-    const long long nub = __double_as_longlong(nu);
+    const uint32_t own = mine ? rep[t * DCD_FAST_K + warp] : 0u;  // row t's repeats within the group
+    const bool any = __any_sync(0xffffffffu, own != 0);
+    const long long nub = __double_as_longlong(SCALED ? nu * eta : nu);
     double th = 0.0;
-    uint32_t left = __ballot_sync(0xffffffffu, mine);  // coordinates not yet decided
-    const bool solvable = (__double_as_longlong(ie) << 1) != 0;
+    uint32_t left = __ballot_sync(0xffffffffu, mine && ie > 0.0);  // coordinates not yet decided
+    int told = 0;                                                  // coordinates published
     for (;;) {
-        const double c1 = clip_bits(rho - gj, nub), c2 = clip_bits(fma(-gj, ie, rho), nub);
-        // the projected gradient clip(rho - g) - rho is nonzero iff the clip moved rho
-        const long long b1 = __double_as_longlong(c1), b0 = __double_as_longlong(rho);
-        const bool moved = b1 != b0 && ((b1 | b0) << 1) != 0;  // +0 and -0 are the same value
-        const double st = moved && solvable ? c2 - rho : 0.0;
-        const uint32_t nz = __ballot_sync(0xffffffffu, (__double_as_longlong(st) << 1) != 0) & left;
+        double st;
+        bool moved;
+        if (SCALED) {
+            const long long b = __double_as_longlong(x);
+            const bool lo = (uint32_t)__double2hiint(x) > 0x7ff00000u;  // negative, or a NaN
+            const bool hi = b >= nub;
+            moved = (lo ? 0LL : hi ? nub : b) != __double_as_longlong(re);
+            st = fma(lo ? 0.0 : hi ? nu : x, hi ? 1.0 : ie, -rho);
+        } else {
+            const double c1 = clip_bits(rho - x, nub), c2 = clip_bits(fma(-x, ie, rho), nub);
+            // the projected gradient clip(rho - g) - rho is nonzero iff the clip moved rho
+            st = __double_as_longlong(c1) != __double_as_longlong(rho) ? c2 - rho : 0.0;
+            moved = (__double_as_longlong(st) << 1) != 0;
+        }
+        const uint32_t nz = __ballot_sync(0xffffffffu, moved) & left;
         if (!nz) break;
         const int l = __ffs(nz) - 1, j = 32 * warp + l;
-        const double tj = __shfl_sync(0xffffffffu, st, l);
-        if (lane == l) {
-            th = tj;
-            if (more) {
-                list_j[n] = j;
-                list_t[n] = tj;
-                st_release_shared(pub, n + 1);
-            }
-        }
-        ++n;
+        const double tj = __shfl_sync(0xffffffffu, st, l), c = C[j * ldc + tc];
+        x = fma(SCALED ? -c : c, tj, x);
         left &= ~((2u << l) - 1u);
-        apply(j, tj);
+        th = lane == l ? tj : th;
+        if (more && lane >= told && lane <= l) chain_st(slot + t, lane == l ? tj : 0.0);
+        told = l + 1;
+        if (any && (__shfl_sync(0xffffffffu, own, l) >> lane) & 1u) repeat(tj);  // repeats are rare
     }
-    __syncwarp();
-    if (more && lane == 0) st_release_shared(pub + 1, warp + 1);
+    if (more && lane >= told) chain_st(slot + t, 0.0);
     return th;
+}
+
+// Warp `warp`'s 32 coordinates t = 32 warp + lane of a chain of cnt <= DCD_FAST_MAX: returns the lane's
+// step.  C[j ldc + t]: the coupling of t to the step of j < t (any number for t <= j in the same 32);
+// rep[j DCD_FAST_K + q]: bit l set where coordinate 32 q + l > j holds j's row; slot (cnt entries,
+// CHAIN_OPEN at the start): the steps published to the later groups; rho, gj, eta, ie: alpha_t, g_t,
+// eta_t, 1 / eta_t (0: no step).
+__device__ __forceinline__ double dcd_chain_group(const double *C, int ldc, const uint32_t *rep, double *slot, int cnt,
+                                                  int warp, int lane, double rho, double gj, double eta, double ie,
+                                                  double nu, int *err)
+{
+    const int e = __double2hiint(eta) >> 20, en = __double2hiint(nu) >> 20;  // biased exponents
+    const bool scaled = (ie == 0.0 || (e >= 1023 - 20 && e <= 1023 + 300)) &&
+                        (nu == __longlong_as_double(0x7ff0000000000000LL) || (en >= 1023 - 300 && en <= 1023 + 300));
+    rho += 0.0;  // -0 to +0: the comparisons are of bits
+    if (__all_sync(0xffffffffu, scaled))
+        return dcd_chain_run<true>(C, ldc, rep, slot, cnt, warp, lane, rho, gj, eta, ie, nu, err);
+    return dcd_chain_run<false>(C, ldc, rep, slot, cnt, warp, lane, rho, gj, eta, ie, nu, err);
 }
 
 }  // namespace dcd

@@ -33,6 +33,7 @@ __device__ __forceinline__ double kval(const KT *K, int64_t ld, int64_t r, int64
 // sequential chain, each lane owning the future coordinates t = lane mod 32
 // and folding every new theta_j into their pending corrections.
 constexpr int DCD_THREADS = 256;
+constexpr int FAST_THREADS = 512;  // the recurrence of at most 128 coordinates: four warps run it, all form its couplings
 constexpr int DCD_SMEM_GRAM_MAX = 128;   // cnt <= 128: Gram staged in shared memory
 constexpr size_t DCD_SMEM_LIMIT = 224 * 1024;
 
@@ -938,21 +939,21 @@ cudaError_t refined_bdcd_b(const KT *Kss, int64_t ldk, const int32_t *S, int nbl
 // runs the coordinates 32 k .. 32 k + 31 with lane l holding alpha_t, g_t and 1/eta_t of t = 32 k + l
 // in registers.
 //
-// What bounds it is the latency of dependent FP64 instructions in one warp (about 64 cycles each,
-// and some 80 of throughput per scheduler), so a round is cut to four: every lane forms its
-// coordinate's candidate step (Algorithm 2, the arithmetic of recur_dcd_kernel: rho - g and
-// rho - g / eta, clipped by integer comparisons of the bit patterns, less rho), a ballot finds the
-// next coordinate whose step is not zero -- those before it take a zero step, which changes
-// nothing -- and one FMA moves its step into every later gradient.  A round is one nonzero step, so
-// coordinates at a bound cost nothing.  The later groups' warps, each on its own scheduler, apply
-// the steps as they are published (shared memory, release / acquire) and take over when the groups
-// before them are done.  One warp in lockstep over all coordinates took 1.2 k cycles per
-// coordinate.  Measured per step: s = 64 (split bf16, m = 2000, n = 64) 38 -> 10.7 us over a whole
-// solve; s = 8 (FP64) 7.6 -> 2.7; s = 32 on CSR data from alpha = 0, every step nonzero, 26 -> 18.
+// What bounds it is the latency of dependent FP64 instructions in one warp (64 cycles each, and as
+// much of throughput per scheduler), so a round is cut to two (dcd_chain.cuh): every lane holds its
+// coordinate's candidate, a ballot finds the next coordinate whose step is not zero -- those before it
+// take a zero step, which changes nothing -- and one FMA moves its step into every later coordinate's.
+// A round is one nonzero step, so coordinates at a bound cost nothing.  The later groups' warps, each
+// on its own scheduler, apply the steps as they are published (a word of shared memory a step, no
+// fence: the value itself says that it is there) and take over when the groups before them are done.
+// One warp in lockstep over all coordinates took 1.2 k cycles per coordinate; rounds that form rho - g
+// and rho - g / eta anew, with steps published by release / acquire, 780, now 300.  Measured, every step
+// nonzero, FP64: 32 coordinates 14.7 -> 8.2 us, 64 28.9 -> 15.5, 128 61.7 -> 33, of which 3.5 are the
+// launch, the first loads and 1 / eta.
 // pend (optional): alpha and g at the step's coordinates are pend[0][t] + pend[1][t] and
 // pend[2][t] + pend[3][t] (a snapshot and the parts not yet in it) instead of alpha[S[t]], g[S[t]]
 template <typename KT>
-__global__ void __launch_bounds__(DCD_THREADS) recur_dcd_fast_kernel(const KT *Kss, int64_t ldk, const int32_t *S,
+__global__ void __launch_bounds__(FAST_THREADS) recur_dcd_fast_kernel(const KT *Kss, int64_t ldk, const int32_t *S,
                                                                      int cnt, const double *y, const double *alpha,
                                                                      const double *g, double omega, double nu,
                                                                      double *delta, double *w64, float *w32,
@@ -961,19 +962,32 @@ __global__ void __launch_bounds__(DCD_THREADS) recur_dcd_fast_kernel(const KT *K
     extern __shared__ double fsm[];
     const int ldc = cnt | 1;                            // odd: no bank conflicts down a column
     double *C = fsm;                                    // C[j * ldc + t]
-    double *list_t = C + (size_t)cnt * ldc;             // the nonzero steps so far, and their coordinates
-    int *list_j = (int *)(list_t + cnt);
-    int32_t *sI = list_j + cnt;
+    double *slot = C + (size_t)cnt * ldc;               // the steps, as they are decided
+    int32_t *sI = (int32_t *)(slot + cnt);
     uint32_t *sy = (uint32_t *)(sI + cnt);              // sign bit of y
     uint32_t *rep = sy + cnt;                           // rep[j * 4 + q]: later t = 32 q + bit with S_t = S_j
-    int *pub = (int *)(rep + DCD_FAST_K * cnt);         // steps published, groups done
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = threadIdx.x;  // warps 0..3: this thread's coordinate, if t < cnt
     const bool mine = t < cnt;
-    double a0 = 0.0, a1 = 0.0, g0 = 0.0, g1 = 0.0;
+    // C and the repeat masks: a warp per row t and 32 columns j, several in flight (the loads, which
+    // need nothing of S, ahead of the wait for it)
+    constexpr int U = 4;
+    const int nq = (cnt + 31) / 32, np = cnt * nq;
+    double v[U];
+    auto load = [&](double (&w)[U], int p0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int p = p0 + u * (FAST_THREADS / 32), r = p / nq, j = 32 * (p - r * nq) + lane;
+            w[u] = p < np && j < r ? kval(Kss, ldk, r, j) : 0.0;
+        }
+    };
+    load(v, warp);
+    double a0 = 0.0, a1 = 0.0, g0 = 0.0, g1 = 0.0, eta = 0.0, ie = 0.0;
     if (mine) {
         const int32_t i = S[t];
+        eta = kval(Kss, ldk, t, t);
         sI[t] = i;
+        slot[t] = __longlong_as_double(CHAIN_OPEN);
         sy[t] = (uint32_t)__double2hiint(y[i]) & 0x80000000u;
         if (pend.alpha_snap) {
             a0 = pend.alpha_snap[t];
@@ -985,33 +999,30 @@ __global__ void __launch_bounds__(DCD_THREADS) recur_dcd_fast_kernel(const KT *K
             g0 = g[i];
         }
     }
-    if (threadIdx.x == 0) pub[0] = pub[1] = 0;
     __syncthreads();
-    double ie = 0.0;
-    if (mine) {
-        const double eta = kval(Kss, ldk, t, t) + omega;  // G_k = V^T U_k + omega I, y_t^2 = 1
-        ie = eta > 0.0 ? 1.0 / eta : 0.0;
-    }
-    // C and the repeat masks, a warp per row t (lanes: columns j)
-    for (int r = warp; r < cnt; r += DCD_THREADS / 32) {
-        const int32_t ir = sI[r];
-        const uint32_t yr = sy[r];
-        for (int q = 0; 32 * q < cnt; ++q) {
-            const int j = 32 * q + lane;
+    for (int p0 = warp; p0 < np; p0 += U * (FAST_THREADS / 32)) {
+        double w[U];
+        load(w, p0 + U * (FAST_THREADS / 32));
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int p = p0 + u * (FAST_THREADS / 32), r = p / nq, q = p - r * nq, j = 32 * q + lane;
+            if (p >= np) break;  // warp-uniform
             const bool in = j < cnt;
-            const bool same = in && sI[in ? j : 0] == ir;
-            if (in) {
-                double v = 0.0;
-                if (r > j) {
-                    v = kval(Kss, ldk, r, j);
-                    v = __hiloint2double((int)((uint32_t)__double2hiint(v) ^ yr ^ sy[j]), __double2loint(v));
-                    if (same) v += omega;
-                }
-                C[j * ldc + r] = v;
+            const bool same = in && sI[in ? j : 0] == sI[r];
+            if (in && 32 * q <= r) {
+                double c = __hiloint2double((int)((uint32_t)__double2hiint(v[u]) ^ sy[r] ^ sy[j]), __double2loint(v[u]));
+                if (same) c += omega;
+                C[j * ldc + r] = c;
             }
             const uint32_t mask = __ballot_sync(0xffffffffu, same && j > r);  // positions after r with r's index
             if (lane == 0) rep[r * DCD_FAST_K + q] = mask;
         }
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = w[u];
+    }
+    if (mine) {
+        eta += omega;  // G_k = V^T U_k + omega I, y_t^2 = 1
+        ie = eta > 0.0 ? 1.0 / eta : 0.0;
     }
     __syncthreads();
     if (32 * warp >= cnt) return;
@@ -1020,7 +1031,7 @@ __global__ void __launch_bounds__(DCD_THREADS) recur_dcd_fast_kernel(const KT *K
         rho += a1;
         gj += g1;
     }
-    const double th = dcd_chain_group(C, ldc, rep, list_t, list_j, pub, cnt, warp, lane, rho, gj, ie, nu, err);
+    const double th = dcd_chain_group(C, ldc, rep, slot, cnt, warp, lane, rho, gj, eta, ie, nu, err);
     if (mine) {
         delta[t] = th;
         // y_t th
@@ -1039,7 +1050,7 @@ cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const in
     const DcdPending pd = pend ? *pend : DcdPending{};
     if (pend && cnt > DCD_FAST_MAX) return cudaErrorInvalidValue;
     if (cnt <= DCD_FAST_MAX) {
-        const size_t fsm = sizeof(double) * (size_t)(cnt * (cnt | 1) + cnt) + sizeof(int32_t) * ((3 + DCD_FAST_K) * cnt + 2);
+        const size_t fsm = sizeof(double) * (size_t)(cnt * (cnt | 1) + cnt) + sizeof(int32_t) * (2 + DCD_FAST_K) * cnt;
         static bool fattr[2] = {false, false};
         if (kss_f64) {
             if (!fattr[1]) {
@@ -1048,7 +1059,7 @@ cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const in
                 if (e != cudaSuccess) return e;
                 fattr[1] = true;
             }
-            recur_dcd_fast_kernel<double><<<1, DCD_THREADS, fsm, st>>>((const double *)Kss, ldk, S, (int)cnt, y, alpha,
+            recur_dcd_fast_kernel<double><<<1, FAST_THREADS, fsm, st>>>((const double *)Kss, ldk, S, (int)cnt, y, alpha,
                                                                        g, omega, nu, delta, w64, w32, pd, err);
         } else {
             if (!fattr[0]) {
@@ -1057,7 +1068,7 @@ cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const in
                 if (e != cudaSuccess) return e;
                 fattr[0] = true;
             }
-            recur_dcd_fast_kernel<float><<<1, DCD_THREADS, fsm, st>>>((const float *)Kss, ldk, S, (int)cnt, y, alpha,
+            recur_dcd_fast_kernel<float><<<1, FAST_THREADS, fsm, st>>>((const float *)Kss, ldk, S, (int)cnt, y, alpha,
                                                                       g, omega, nu, delta, w64, w32, pd, err);
         }
         return cudaGetLastError();

@@ -54,13 +54,13 @@ struct GridArgs {
     int steps, s, R, ks, nls;  // rows per CTA, lanes per entry, row stride in shared memory
     double omega, nu;
     double *xbuf;   // [2][s][2]: g and alpha at the step's coordinates
-    double *kss;    // [4][s * s + s] by step (a CTA may be two steps ahead of another's reads): K(S_t, S_j) for j < t at [j * s + t], then 1 / eta_t
+    double *kss;    // [4][s * s + 2 s] by step (a CTA may be two steps ahead of another's reads): K(S_t, S_j) for j < t at [j * s + t], then 1 / eta_t, eta_t
     unsigned *bar;  // arrivals, zero at the start
     int *err;
 };
 
 struct GridLayout {
-    size_t own, as, kb, gs, al, hr, hs, C, lt, th, w, tab, ints, total;
+    size_t own, as, kb, gs, al, hr, hs, C, slot, th, w, tab, ints, total;
 };
 
 __host__ __device__ inline GridLayout grid_layout(int n, int s, int R, int nls)
@@ -80,12 +80,12 @@ __host__ __device__ inline GridLayout grid_layout(int n, int s, int R, int nls)
     L.hr = take(R);
     L.hs = take(2 * (size_t)s);
     L.C = take((size_t)s * (s | 1));
-    L.lt = take(s);
+    L.slot = take(s);
     L.th = take(s);
     L.w = take(s);
     L.tab = take(64);
-    L.ints = c;  // S 2 s; sign of y: at S 2 s, own rows R; list_j s; rep 4 s; pub 2
-    L.total = 8 * c + 4 * ((size_t)(2 + 2 + 1 + DCD_FAST_K) * s + R + 2);
+    L.ints = c;  // S 2 s; sign of y: at S 2 s, own rows R; rep 4 s
+    L.total = 8 * c + 4 * ((size_t)(2 + 2 + DCD_FAST_K) * s + R);
     return L;
 }
 
@@ -148,14 +148,12 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
     const int s = a.s, R = a.R, n = a.n, nls = a.nls, ldc = s | 1;
     const GridLayout L = grid_layout(n, s, R, nls);
     double *own = gsm + L.own, *As = gsm + L.as, *kb = gsm + L.kb, *gs = gsm + L.gs, *al = gsm + L.al,
-           *hr = gsm + L.hr, *hS = gsm + L.hs, *C = gsm + L.C, *list_t = gsm + L.lt, *th_s = gsm + L.th, *w_s = gsm + L.w,
+           *hr = gsm + L.hr, *hS = gsm + L.hs, *C = gsm + L.C, *slot = gsm + L.slot, *th_s = gsm + L.th, *w_s = gsm + L.w,
            *tab = gsm + L.tab;
     int32_t *SS = (int32_t *)(gsm + L.ints);             // S of a step, by its parity
     uint32_t *sy = (uint32_t *)(SS + 2 * s);             // sign bits of y at S, by parity
     uint32_t *yr = sy + 2 * s;                           // sign bits of the own rows' y
-    int *list_j = (int *)(yr + R);
-    uint32_t *rep = (uint32_t *)(list_j + s);
-    int *pub = (int *)(rep + DCD_FAST_K * s);
+    uint32_t *rep = yr + R;
     __shared__ int stop_s;                               // the grid barrier's wait ran out
     const int cta = blockIdx.x, G = gridDim.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int r0 = cta * R, rows = max(min(R, a.m - r0), 0);
@@ -195,7 +193,7 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
             for (int e = bt; e < s * n; e += GB) Aq[e] = a.A[(int64_t)Sq[e / n] * a.lda + e % n];
             nb_sync<GB>(NB_BLOCK);
             // this CTA's entries of the step's Gram: pairs j <= t, a warp each
-            double *kss = a.kss + (size_t)(q & 3) * (s * s + s);
+            double *kss = a.kss + (size_t)(q & 3) * (s * s + 2 * s);
             for (int e = cta + G * bw; e < s * (s + 1) / 2; e += G * GB_WARPS) {
                 int t = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
                 while (t * (t + 1) / 2 > e) --t;
@@ -211,6 +209,7 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
                     } else {
                         const double eta = kv + a.omega;  // G_k = V^T U_k + omega I, y_t^2 = 1
                         kss[s * s + t] = eta > 0.0 ? 1.0 / eta : 0.0;
+                        kss[s * s + s + t] = eta;
                     }
                 }
             }
@@ -276,15 +275,16 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
         const int p = k & 1;
         const int32_t *S = SS + p * s;
         const uint32_t *yk = sy + p * s;
-        const double *kss = a.kss + (size_t)(k & 3) * (s * s + s);
-        double rho = 0.0, gj = 0.0, ie = 0.0;
+        const double *kss = a.kss + (size_t)(k & 3) * (s * s + 2 * s);
+        double rho = 0.0, gj = 0.0, ie = 0.0, eta = 0.0;
         if (tid < s) {
             const double *x = a.xbuf + ((size_t)p * s + tid) * 2;
             gj = __ldcg(x);
             rho = __ldcg(x + 1);
             ie = __ldcg(kss + s * s + tid);
+            eta = __ldcg(kss + s * s + s + tid);
+            slot[tid] = __longlong_as_double(CHAIN_OPEN);
         }
-        if (tid == 0) pub[0] = pub[1] = 0;
         for (int j = warp; j < s; j += GM_WARPS)
             for (int q = 0; q < ng; ++q) {
                 const int t = 32 * q + lane;
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
             }
         nb_sync<GM>(NB_MAIN);
         if (warp < ng) {
-            const double th = dcd_chain_group(C, ldc, rep, list_t, list_j, pub, s, warp, lane, rho, gj, ie, a.nu, a.err);
+            const double th = dcd_chain_group(C, ldc, rep, slot, s, warp, lane, rho, gj, eta, ie, a.nu, a.err);
             if (tid < s) {
                 th_s[tid] = th;
                 w_s[tid] = __hiloint2double((int)((uint32_t)__double2hiint(th) ^ yk[tid]), __double2loint(th));
@@ -388,7 +388,7 @@ SvmGrid svm_grid_plan(int64_t m, int64_t n, int s)
     return g;
 }
 
-size_t svm_grid_scratch_bytes(int s) { return sizeof(double) * (4 * (size_t)s + 4 * ((size_t)s * s + s)) + 256; }
+size_t svm_grid_scratch_bytes(int s) { return sizeof(double) * (4 * (size_t)s + 4 * ((size_t)s * s + 2 * s)) + 256; }
 
 cudaError_t launch_svm_grid(const SvmGrid &gp, const double *A, int64_t lda, int64_t m, int64_t n,
                             const KernelParams &kp, const double *h, const double *y, double *alpha, double *g,
