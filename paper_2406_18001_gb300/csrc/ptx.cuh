@@ -122,6 +122,28 @@ __device__ __forceinline__ void st_async_v4(uint32_t raddr, float4 v, uint32_t r
                  : "memory");
 }
 
+// Bulk copy from this CTA's shared memory into another CTA's, counted as complete_tx on that CTA's
+// mbarrier (dst and rbar from mapa; 16-byte aligned, bytes a multiple of 16).  A writer of src
+// passes fence_proxy_async first.
+__device__ __forceinline__ void bulk_s2cluster(uint32_t dst, const void *src, uint32_t bytes, uint32_t rbar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "r"(su32(src)), "r"(bytes), "r"(rbar)
+                 : "memory");
+}
+
+__device__ __forceinline__ void fence_proxy_async()
+{
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// 16-byte asynchronous copy global -> shared by this thread, and the wait for all of its own
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(dst)), "l"((uint64_t)src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

@@ -23,19 +23,30 @@
 // L2 at only ~40-60 B/clock, so the super-blocks are dealt to the P CTAs of a
 // cluster, two per CTA, folded (CTA c owns J = c and 2P-1-c, which balances
 // the triangle); each CTA copies its rows' Gram panels (Bs x Bs, row-major)
-// once by 2-D TMA.  Per own super-block a CTA runs two warps:
+// once by 2-D TMA.  Per own super-block a CTA runs three warps:
 //   round-0 warp: applies Delta0_T as it arrives (T < J), forms Delta0_J
-//                 and sends it to every CTA (st.async, completing the
-//                 receiver's per-step mbarrier); it accumulates the
-//                 double-single residual of its rows panel by panel while it
-//                 waits, so rho_J is ready just after Delta0_J;
+//                 and sends it to every CTA, completing the receiver's
+//                 per-step mbarrier;
+//   residual warp: accumulates the double-single residual of the rows
+//                 panel by panel as the Delta0_T arrive, Delta0_J last,
+//                 which gives rho_J;
 //   round-1 warp: applies Delta1_T as it arrives and once rho_J is ready
 //                 forms Delta1_J, sends it and writes Delta = Delta0 + Delta1.
 // The refinement chain thus runs a little behind the first one instead of
-// after it.  Panel rows are read as float4 chunks in a lane-rotated order
-// (conflict-free).  Every wait is bounded; on expiry the kernel records
-// DEV_TIMEOUT, skips its remaining waits and still lets every store
-// addressed to it land (bounded) before it leaves.
+// after it.
+//
+// What bounds it is the latency of one step of the chain: Delta_{J-1} arrives,
+// one 32 x 32 product, Delta_J leaves.  So the panel rows (and those of
+// L_JJ^-1 and L_JJ^-1 L_{J,J-1}) are in registers before the wait, the
+// residual is no work of the chain's warps, and a send goes to the two CTAs
+// that need it next as 16-byte remote stores and to the others as one bulk
+// copy each.  With 128 remote stores a send (1.8-3 k cycles to issue, in rank
+// order), the residual in the chain's warp (8-14 k cycles between Delta0_J and
+// rho_J) and the panels, inverses and masks copied through registers before
+// the start (17 k cycles) 1024 coordinates took 43 us; now 22.  Panel rows are
+// read as float4 chunks in a lane-rotated order (conflict-free).  Every wait is
+// bounded; on expiry the kernel records DEV_TIMEOUT, skips its remaining waits
+// and still lets every store addressed to it land (bounded) before it leaves.
 #include "dcd_internal.cuh"
 #include "ptx.cuh"
 
@@ -45,7 +56,9 @@
 namespace dcd {
 namespace {
 
-constexpr int CL_THREADS = 128;  // warps: slot 0 round 0, slot 1 round 0, slot 0 round 1, slot 1 round 1
+// warps (slot = warp & 1): 0-1 round 0, 2-3 round 1, 6-7 residual (on the schedulers of round 1, which
+// waits for it); 4-5 only help with the set-up
+constexpr int CL_THREADS = 256;
 constexpr int CL_SLOTS = 2;      // own super-blocks per CTA
 constexpr int CL_PMAX = 16;      // CTAs per cluster (non-portable size)
 constexpr int CL_NSUP_MAX = 2 * CL_PMAX;
@@ -140,30 +153,40 @@ __device__ __forceinline__ void ds_prod(float &hi, float &lo, float kv, float dv
     ds_add(hi, lo, pp, fmaf(kv, dv, -pp));
 }
 
-// Row `lane` of a panel (ncol columns, a multiple of 4) times v, FP32: float4
-// chunks visited from chunk `lane` onwards (mod ncol / 4), so the lanes of a
-// quarter-warp read distinct banks.
-__device__ __forceinline__ float panel_dot(const float *pr, const float *v, int lane, int ncol)
-{
-    const int nc = ncol >> 2;
-    const int m0 = nc == 8 ? (lane & 7) : lane % nc;
-    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        if (j < nc) {
-            int m = m0 + j;
-            m -= m >= nc ? nc : 0;
-            const float4 a = *(const float4 *)(pr + 4 * m), x = *(const float4 *)(v + 4 * m);
-            s0 = fmaf(a.x, x.x, s0);
-            s1 = fmaf(a.y, x.y, s1);
-            s2 = fmaf(a.z, x.z, s2);
-            s3 = fmaf(a.w, x.w, s3);
-        }
+// Row `lane` of a panel of BS columns (20, 24, 28 or 32) in registers, as float4 chunks from chunk
+// `lane` onwards (mod BS / 4), so the lanes of a quarter-warp read distinct banks, of the row and of
+// the vector alike.
+template <int BS> struct PanelRow {
+    static constexpr int NC = BS / 4;
+    float4 a[NC];
+    __device__ __forceinline__ static int chunk(int lane, int j)
+    {
+        const int m = lane % NC + j;
+        return m >= NC ? m - NC : m;
     }
-    return (s0 + s1) + (s2 + s3);
-}
+    __device__ __forceinline__ void load(const float *pr, int lane)
+    {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) a[j] = *(const float4 *)(pr + 4 * chunk(lane, j));
+    }
+    // FUSED: by FMAs; else every product rounded by itself, the sums that panel_dot_ds has in its high parts
+    template <bool FUSED> __device__ __forceinline__ float dot(const float *v, int lane) const
+    {
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            const float4 x = *(const float4 *)(v + 4 * chunk(lane, j));
+            s0 = FUSED ? fmaf(a[j].x, x.x, s0) : __fadd_rn(s0, __fmul_rn(a[j].x, x.x));
+            s1 = FUSED ? fmaf(a[j].y, x.y, s1) : __fadd_rn(s1, __fmul_rn(a[j].y, x.y));
+            s2 = FUSED ? fmaf(a[j].z, x.z, s2) : __fadd_rn(s2, __fmul_rn(a[j].z, x.z));
+            s3 = FUSED ? fmaf(a[j].w, x.w, s3) : __fadd_rn(s3, __fmul_rn(a[j].w, x.w));
+        }
+        return (s0 + s1) + (s2 + s3);
+    }
+};
 
-// The same dot product as a double-single pair, each product exact (TwoProd).
+// The same dot product over the row's first ncol columns (a multiple of 4) as a double-single pair,
+// each product exact (TwoProd).
 __device__ __forceinline__ void panel_dot_ds(const float *pr, const float *v, int lane, int ncol, float &hi, float &lo)
 {
     const int nc = ncol >> 2;
@@ -199,22 +222,14 @@ __device__ __forceinline__ float mask_sum(uint32_t mask, const float *v)
     return s;
 }
 
-__device__ __forceinline__ bool wait_local(uint64_t *bar, volatile int *abort_flag, int *err)
+// Warp-uniform.  REMOTE: bytes from other CTAs complete the barrier.
+template <bool REMOTE>
+__device__ __forceinline__ bool wait_bar(uint64_t *bar, volatile int *abort_flag, int *err)
 {
-    const bool ok = !*abort_flag && ptx::mbar_wait_bounded(bar, 0, CL_WAIT_NS);
-    if (!__all_sync(0xffffffffu, ok)) {
-        if ((threadIdx.x & 31) == 0 && !*abort_flag) {
-            *abort_flag = 1;
-            set_error(err, DEV_TIMEOUT);
-        }
-        return false;
-    }
-    return true;
-}
-
-__device__ __forceinline__ bool wait_remote(uint64_t *bar, volatile int *abort_flag, int *err)
-{
-    const bool ok = !*abort_flag && ptx::mbar_wait_cluster_bounded(bar, 0, CL_WAIT_NS);
+    bool ok = REMOTE ? ptx::mbar_test_cluster(bar, 0) : ptx::mbar_test(bar, 0);
+    if (__all_sync(0xffffffffu, ok)) return true;
+    ok = !*abort_flag && (REMOTE ? ptx::mbar_wait_cluster_bounded(bar, 0, CL_WAIT_NS)
+                                 : ptx::mbar_wait_bounded(bar, 0, CL_WAIT_NS));
     if (!__all_sync(0xffffffffu, ok)) {
         if ((threadIdx.x & 31) == 0 && !*abort_flag) {
             *abort_flag = 1;
@@ -348,6 +363,142 @@ __global__ void __launch_bounds__(PREP_THREADS)
 }
 
 // ---------------------------------------------------------------------------
+struct ClWarp {            // what a warp of own super-block J works with
+    int P, c, J, slot, sb, nsup, b, rows, lane;
+    int prow;              // the lane's row of a panel (lanes past Bs: a valid one)
+    float inv_lam, mf;
+    double lambda, mdiag;
+    float *recv;           // [round][sb]: Delta_round as received
+    const float *pan;      // panels T = 0 .. J, pstride floats apart
+    size_t pstride;
+    const float *xs, *ns;  // L_JJ^-1 and L_JJ^-1 L_{J,J-1}, 32 x 32 row-major
+    const uint32_t *dm;    // repeat masks [T][lane]
+    uint32_t nz;           // bit T: dm[T] is not all zero
+    double rhs;
+    double *rho;           // [32]
+    uint64_t *bars, *dbar, *pbar, *rbar;
+    volatile int *abort_flag;
+    int *err;
+};
+
+// The residual rho_J = rhs - L_{J, T<=J} Delta0 (double-single products; FP64 repeat term).
+template <int BS>
+__device__ void cl_residual(const ClWarp &w)
+{
+    constexpr int NC = BS / 4;
+    const int lane = w.lane;
+    float hi = 0.f, lo = 0.f;
+    bool alive = w.J == 0 || wait_bar<false>(w.pbar, w.abort_flag, w.err);
+    for (int T = 0; T < w.J && alive; ++T) {
+        PanelRow<BS> p;
+        p.load(w.pan + (size_t)T * w.pstride + w.prow * BS, lane);
+        if (!wait_bar<true>(&w.bars[T], w.abort_flag, w.err)) {
+            alive = false;
+            break;
+        }
+        const float *v = w.recv + T * BS;
+        float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f, h2 = 0.f, l2 = 0.f, h3 = 0.f, l3 = 0.f;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            const float4 x = *(const float4 *)(v + 4 * PanelRow<BS>::chunk(lane, j));
+            ds_prod(h0, l0, p.a[j].x, x.x);
+            ds_prod(h1, l1, p.a[j].y, x.y);
+            ds_prod(h2, l2, p.a[j].z, x.z);
+            ds_prod(h3, l3, p.a[j].w, x.w);
+        }
+        ds_add(h0, l0, h1, l1);
+        ds_add(h2, l2, h3, l3);
+        ds_add(h0, l0, h2, l2);
+        ds_add(hi, lo, h0, l0);
+    }
+    alive = alive && wait_bar<false>(w.dbar, w.abort_flag, w.err);
+    alive = alive && wait_bar<true>(&w.bars[w.J], w.abort_flag, w.err);
+    if (alive && lane < w.rows) {
+        const float *own = w.recv + w.J * BS;
+        float h, l;  // the diagonal panel: the blocks up to this row's block
+        panel_dot_ds(w.pan + (size_t)w.J * w.pstride + lane * BS, own, lane, (lane / w.b + 1) * w.b, h, l);
+        ds_add(hi, lo, h, l);
+        double dmv = (double)own[lane];
+        for (uint32_t nz = w.nz; nz; nz &= nz - 1) {  // repeats are rare
+            const int T = __ffs(nz) - 1;
+            uint32_t mask = w.dm[T * 32 + lane];
+            while (mask) {
+                dmv += (double)w.recv[T * BS + __ffs(mask) - 1];
+                mask &= mask - 1;
+            }
+        }
+        w.rho[lane] = w.rhs - (((double)hi + (double)lo) / w.lambda + w.mdiag * dmv);
+    }
+    __syncwarp();
+    if (lane == 0) ptx::mbar_arrive(w.rbar);  // always: the round-1 warp gives up if this one did
+}
+
+// The chain of round r.  All updates but the one from J-1 give r'_J; Delta_J = X_J r'_J - N_J
+// Delta_{J-1} with N_J = X_J L_{J,J-1}, X_J r'_J formed while Delta_{J-1} is on its way.
+// Returns whether Delta_J (d) was formed and sent.
+template <int BS>
+__device__ bool cl_chain(const ClWarp &w, int r, float *ds, float *rb, float &d)
+{
+    constexpr int Bs = BS;
+    const int lane = w.lane, J = w.J;
+    float *rv = w.recv + (size_t)r * w.sb;
+    uint64_t *bars = w.bars + r * w.nsup;
+    // the CTAs in the order in which they need Delta_J: owners of J + 1, J + 2, ...
+    auto dest = [&](int k) {
+        int q = w.slot == 1 ? w.c - 1 - k : w.c == w.P - 1 ? w.c - k : w.c + 1 + k;
+        q += q < 0 ? w.P : 0;
+        return q >= w.P ? q - w.P : q;
+    };
+    // lanes 0 .. 15: 16 bytes each to the first two; lanes 16 + k: a bulk copy to number 2 + k
+    const int nd = lane < 16 ? lane >> 3 : lane - 14, part = lane & 7;
+    const bool to = nd < w.P, sends = to && lane < 16 && 4 * part < w.rows, bulk = to && lane >= 16;
+    const uint32_t rank = (uint32_t)dest(to ? nd : 0);
+    const uint32_t raddr = ptx::mapa(ptx::su32(rv + J * Bs + (lane < 16 ? 4 * part : 0)), rank);
+    const uint32_t rbar = ptx::mapa(ptx::su32(&bars[J]), rank);
+
+    float rr = r == 0 ? (float)w.rhs : 0.f;  // round 0: the right-hand side minus updates; round 1: sum of updates
+    bool alive = J == 0 || wait_bar<false>(w.pbar, w.abort_flag, w.err);
+    PanelRow<BS> pr;
+    PanelRow<32> xr;
+    PanelRow<BS> nr;
+    xr.load(w.xs + lane * 32, lane);
+    if (J > 0) nr.load(w.ns + lane * 32, lane);
+    for (int T = 0; T + 1 < J && alive; ++T) {
+        pr.load(w.pan + (size_t)T * w.pstride + w.prow * Bs, lane);
+        if (!wait_bar<true>(&bars[T], w.abort_flag, w.err)) {
+            alive = false;
+            break;
+        }
+        const float *dt = rv + T * Bs;
+        const float sd = (w.nz >> T) & 1u ? mask_sum(lane < w.rows ? w.dm[T * 32 + lane] : 0u, dt) : 0.f;
+        if (r == 0) rr -= pr.template dot<false>(dt, lane) * w.inv_lam + w.mf * sd;
+        else rr += pr.template dot<true>(dt, lane) * w.inv_lam + w.mf * sd;
+    }
+    if (r == 1 && alive) {
+        alive = wait_bar<false>(w.rbar, w.abort_flag, w.err);
+        if (alive && lane < w.rows) rr = (float)w.rho[lane] - rr;
+    }
+    d = 0.f;
+    if (alive) {
+        rb[lane] = lane < w.rows ? rr : 0.f;
+        __syncwarp();
+        d = xr.template dot<true>(rb, lane);
+    }
+    if (alive && J > 0) {
+        alive = wait_bar<true>(&bars[J - 1], w.abort_flag, w.err);
+        if (alive) d -= nr.template dot<true>(rv + (J - 1) * Bs, lane);
+    }
+    if (!alive) return false;
+    ds[lane] = lane < w.rows ? d : 0.f;
+    __syncwarp();
+    if (sends) ptx::st_async_v4(raddr, *(const float4 *)(ds + 4 * part), rbar);
+    ptx::fence_proxy_async();
+    __syncwarp();
+    if (bulk) ptx::bulk_s2cluster(raddr, ds, (uint32_t)(w.rows * 4), rbar);
+    return true;
+}
+
+template <int BS>
 __global__ void __launch_bounds__(CL_THREADS, 1)
     bdcd_cluster_kernel(const __grid_constant__ CUtensorMap kmap, const int32_t *S, const float *X,
                         const float *Ng, const uint32_t *Mg, const int32_t *nextg, int nblk, int b, double lambda,
@@ -358,7 +509,8 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
     const int P = (int)gridDim.x;  // the grid is one cluster
     const int c = (int)ptx::cluster_ctarank();
     const ClGeom G = cl_geom(nblk, b);
-    const int Bs = G.Bs, nsup = G.nsup, sb = nblk * b;
+    constexpr int Bs = BS;
+    const int nsup = G.nsup, sb = nblk * b;
     const ClLayout L = cl_layout(nblk, b, P, c);
     float *recv = (float *)(sm + L.recv);          // [round][sb]: Delta_round as received
     float *xsa = (float *)(sm + L.xs);             // [slot][32][32]: L_JJ^-1, row-major
@@ -372,6 +524,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
     const uint32_t goff = ptx::su32(sm + L.gdata);
     unsigned char *gd = sm + L.gdata + ((128u - (goff & 127u)) & 127u);
     __shared__ int abort_flag_s;
+    __shared__ double rhs_pre[CL_SLOTS * 32];
     volatile int *abort_flag = &abort_flag_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int slot = warp & 1, role = warp >> 1;
@@ -380,192 +533,134 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
     // this cluster leaves free) may start its set-up and tensor-core products once every CTA has
     // signalled; it waits for this grid to finish before it reads the coefficients or the
     // gradient.  The CTA owning super-block trig_sup signals when its round-0 Delta is out (the
-    // kernels forked beside the chain have the other SMs until then); every other CTA at once.
+    // kernels forked beside the chain have the other SMs until then); every other CTA at once, or,
+    // with a part of the gradient not yet in g (x), when it has read its right-hand side: such a
+    // dependent may write g once every CTA has signalled.
     const bool trig_own = trig_sup >= 0 && (trig_sup == cl_own(0, c, P) || (nown > 1 && trig_sup == cl_own(1, c, P)));
-    // -(g_S + the part of the gradient not yet in g) is read before this CTA signals: a dependent may
-    // write g once every CTA has
-    __shared__ double rhs_pre[CL_SLOTS * 32];
-    if (x.x) {
-        for (int e = tid; e < nown * 32; e += CL_THREADS) {
-            const int k = e >> 5, i = e & 31, J = cl_own(k, c, P);
-            if (i >= cl_rows(J, Bs, sb)) continue;
-            const int p = J * Bs + i;
-            const int32_t row = S[p];
-            int q = x.link[p];
-            double v = 0.0;
-            for (int h = 0; h < x.nx; ++h) v += x.x[(int64_t)h * x.ldx + p];
-            if (q >= 0) {  // rare: the previous step's positions that hold this row, in order
-                double sum = 0.0;
-                for (; q >= 0; q = x.next[q]) sum += x.delta[q];
-                v += mdiag * sum;
-            }
-            rhs_pre[e] = -(g[row] + v);
-        }
-        __syncthreads();
-    }
-    if (tid == 0 && !trig_own) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const float inv_lam = (float)(1.0 / lambda);
-    const float mf = (float)mdiag;
 
-    // ---- set-up: barriers, Gram panels, inverses, repeat masks ----
-    if (tid == 0) {
-        for (int i = 0; i < 2 * nsup + NLOCAL; ++i) ptx::mbar_init(&bars[i], 1);
+    if (tid == 0 && !x.x && !trig_own) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    // ---- set-up: barriers and Gram panels (warp 0), right-hand sides (warps 1, 2), inverses and
+    // repeat masks (the others, by asynchronous copies) ----
+    if (warp == 0) {
+        for (int i = lane; i < 2 * nsup + NLOCAL; i += 32)
+            ptx::mbar_init(&bars[i], 1);
+        if (lane == 0) abort_flag_s = 0;
         ptx::mbar_init_fence();
-        abort_flag_s = 0;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        for (int r = 0; r < rounds; ++r)
-            for (int J = 0; J < nsup; ++J) ptx::mbar_expect_tx(&bars[r * nsup + J], (uint32_t)(cl_rows(J, Bs, sb) * 4));
-        // the panels the chain needs (T < J) first, the diagonal ones (residual only) last
+        __syncwarp();
+        for (int i = lane; i < rounds * nsup; i += 32) {
+            const int r = i >= nsup ? 1 : 0, J = i - r * nsup;
+            ptx::mbar_expect_tx(&bars[i], (uint32_t)(cl_rows(J, Bs, sb) * 4));
+        }
+        if (lane < nown) {
+            const int J = cl_own(lane, c, P);
+            if (J > 0) ptx::mbar_expect_tx(&lb[3 * lane + 1], (uint32_t)(J * Bs * Bs * 4));
+            ptx::mbar_expect_tx(&lb[3 * lane + 0], (uint32_t)(Bs * Bs * 4));
+        }
+        __syncwarp();
         size_t base = 0;
-        for (int k = 0; k < nown; ++k) {
+        for (int k = 0; k < nown; ++k) {  // panel T of own super-block k
             const int J = cl_own(k, c, P);
-            if (J > 0) {
-                ptx::mbar_expect_tx(&lb[3 * k + 1], (uint32_t)(J * Bs * Bs * 4));
-                for (int T = 0; T < J; ++T)
-                    ptx::tma_load_2d(gd + (base + T) * L.ps, &kmap, &lb[3 * k + 1], T * Bs, J * Bs);
+            if (lane <= J)
+                ptx::tma_load_2d(gd + (base + lane) * L.ps, &kmap, &lb[3 * k + (lane == J ? 0 : 1)], lane * Bs, J * Bs);
+            base += (size_t)J + 1;
+        }
+    } else if (warp <= CL_SLOTS) {
+        const int k = warp - 1, J = k < nown ? cl_own(k, c, P) : 0, p = J * Bs + lane;
+        if (k < nown && lane < cl_rows(J, Bs, sb)) {
+            double v = 0.0;
+            if (rhs_in) {
+                v = rhs_in[p];
+            } else {
+                const int32_t row = S[p];
+                if (x.x) {  // with the part of the gradient not yet in g
+                    int q = x.link[p];
+                    for (int h = 0; h < x.nx; ++h) v += x.x[(int64_t)h * x.ldx + p];
+                    if (q >= 0) {  // rare: the previous step's positions that hold this row, in order
+                        double sum = 0.0;
+                        for (; q >= 0; q = x.next[q]) sum += x.delta[q];
+                        v += mdiag * sum;
+                    }
+                }
+                v = -(g[row] + v);
             }
-            base += (size_t)J + 1;
+            rhs_pre[k * 32 + lane] = v;
         }
-        base = 0;
+        if (x.x) {
+            asm volatile("barrier.cta.sync 1, %0;" ::"n"(32 * CL_SLOTS) : "memory");
+            if (warp == 1 && lane == 0 && !trig_own) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        }
+    } else {
+        constexpr int NT = CL_THREADS - 32 * (1 + CL_SLOTS);
+        const int t = tid - 32 * (1 + CL_SLOTS);
         for (int k = 0; k < nown; ++k) {
             const int J = cl_own(k, c, P);
-            ptx::mbar_expect_tx(&lb[3 * k + 0], (uint32_t)(Bs * Bs * 4));
-            ptx::tma_load_2d(gd + (base + J) * L.ps, &kmap, &lb[3 * k + 0], J * Bs, J * Bs);
-            base += (size_t)J + 1;
+            for (int e = t; e < 256; e += NT) {
+                ptx::cp_async16(xsa + k * 1024 + 4 * e, X + (size_t)J * 1024 + 4 * e);
+                if (J > 0) ptx::cp_async16(nsa + k * 1024 + 4 * e, Ng + (size_t)J * 1024 + 4 * e);
+            }
+            for (int e = t; e < (J + 1) * 8; e += NT)
+                ptx::cp_async16(dmask + k * CL_NSUP_MAX * 32 + 4 * e, Mg + (size_t)J * CL_NSUP_MAX * 32 + 4 * e);
         }
-    }
-    for (int k = 0; k < nown; ++k) {
-        const int J = cl_own(k, c, P);
-        const float4 *xg = (const float4 *)(X + (size_t)J * 1024), *ng = (const float4 *)(Ng + (size_t)J * 1024);
-        float4 *xd = (float4 *)(xsa + k * 1024), *nd = (float4 *)(nsa + k * 1024);
-        for (int e = tid; e < 256; e += CL_THREADS) {
-            xd[e] = xg[e];
-            if (J > 0) nd[e] = ng[e];
-        }
-        for (int e = tid; e < (J + 1) * 32; e += CL_THREADS)
-            dmask[k * CL_NSUP_MAX * 32 + e] = Mg[(size_t)J * CL_NSUP_MAX * 32 + e];
+        ptx::cp_async_wait_all();
     }
     __syncthreads();
-    ptx::cluster_sync();  // every CTA's barriers exist and expect their bytes before any remote store
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
     const int J = slot < nown ? cl_own(slot, c, P) : -1;
-    if (J >= 0 && role < rounds) {
-        const int rows = cl_rows(J, Bs, sb);
-        const int row = J * Bs + lane;  // this lane's position in S (used for lane < rows)
-        const float *pan = (const float *)(gd + (slot == 0 ? 0 : (size_t)cl_own(0, c, P) + 1) * L.ps);
-        const size_t pstride = L.ps / 4;
-        const float *xs = xsa + slot * 1024, *ns = nsa + slot * 1024;
-        const uint32_t *dm = dmask + slot * CL_NSUP_MAX * 32;
-        uint64_t *dbar = &lb[3 * slot + 0], *pbar = &lb[3 * slot + 1], *rbar = &lb[3 * slot + 2];
-        const int r = role;  // the round this warp runs
-        float *rv = recv + (size_t)r * sb;
-        float *ds = dsend + (r * CL_SLOTS + slot) * 32;
-        float *rb = rbufa + (r * CL_SLOTS + slot) * 32;
-        // remote addresses of this warp's sends (Delta_J, rows/4 float4 parts, to every CTA)
-        const int nparts = rows / 4, nsend = P * nparts;
-        uint32_t raddr[4], rbarr[4];
-        int soff[4];
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int i = lane + 32 * t;
-            const int dest = i < nsend ? i / nparts : 0, pt = i < nsend ? i - dest * nparts : 0;
-            raddr[t] = ptx::mapa(ptx::su32(rv + J * Bs + 4 * pt), (uint32_t)dest);
-            rbarr[t] = ptx::mapa(ptx::su32(&bars[r * nsup + J]), (uint32_t)dest);
-            soff[t] = 4 * pt;
+    ClWarp w;
+    w.P = P;
+    w.c = c;
+    w.J = J;
+    w.slot = slot;
+    w.sb = sb;
+    w.nsup = nsup;
+    w.b = b;
+    w.rows = J >= 0 ? cl_rows(J, Bs, sb) : 0;
+    w.lane = lane;
+    w.prow = lane < Bs ? lane : Bs - 1;
+    w.inv_lam = (float)(1.0 / lambda);
+    w.mf = (float)mdiag;
+    w.lambda = lambda;
+    w.mdiag = mdiag;
+    w.recv = recv;
+    w.pan = (const float *)(gd + (slot == 0 ? 0 : (size_t)cl_own(0, c, P) + 1) * L.ps);
+    w.pstride = L.ps / 4;
+    w.xs = xsa + slot * 1024;
+    w.ns = nsa + slot * 1024;
+    w.dm = dmask + slot * CL_NSUP_MAX * 32;
+    w.rhs = lane < w.rows ? rhs_pre[slot * 32 + lane] : 0.0;
+    w.rho = rhoa + slot * 32;
+    w.bars = bars;
+    w.dbar = &lb[3 * slot + 0];
+    w.pbar = &lb[3 * slot + 1];
+    w.rbar = &lb[3 * slot + 2];
+    w.abort_flag = abort_flag;
+    w.err = err;
+    uint32_t seen = 0;  // lane T: the masks of panel T together
+    if (lane <= J)
+        for (int q = 0; q < 8; ++q) {
+            const uint4 v = *(const uint4 *)(w.dm + lane * 32 + 4 * ((lane + q) & 7));
+            seen |= v.x | v.y | v.z | v.w;
         }
+    w.nz = __ballot_sync(0xffffffffu, seen != 0);
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every CTA's barriers expect their bytes
 
-        // ---- the chain of round r ----
-        // r'_J: all updates but the one from J-1, which N_J = X_J L_{J,J-1} applies after the product:
-        // Delta_J = X_J r'_J - N_J Delta_{J-1}.  X_J r'_J is formed while Delta_{J-1} is on its way.
-        // the right-hand side: -g_S; or given (rhs_in); or with a part of the gradient not yet in g
-        // added first (x; read at the start)
-        const double rhs = lane >= rows ? 0.0
-                           : x.x        ? rhs_pre[slot * 32 + lane]
-                           : rhs_in     ? rhs_in[row]
-                                        : -g[S[row]];
-        float rr = r == 0 ? (float)rhs : 0.f;  // round 0: -g_S minus updates; round 1: sum of updates
-        float hi = 0.f, lo = 0.f;              // round 0: double-single sum of L_{row, T<J} Delta0_T
-        bool alive = J == 0 || wait_local(pbar, abort_flag, err);
-        for (int T = 0; T + 1 < J && alive; ++T) {
-            if (!wait_remote(&bars[r * nsup + T], abort_flag, err)) {
-                alive = false;
-                break;
-            }
-            if (lane < rows) {
-                const float *pr = pan + (size_t)T * pstride + lane * Bs;
-                const float *dt = rv + T * Bs;
-                const uint32_t mk = dm[T * 32 + lane];
-                const float sd = mk ? mask_sum(mk, dt) : 0.f;
-                if (r == 0) {  // exact sum, also for the residual
-                    float h, l;
-                    panel_dot_ds(pr, dt, lane, Bs, h, l);
-                    ds_add(hi, lo, h, l);
-                    rr -= h * inv_lam + mf * sd;
-                } else {
-                    rr += panel_dot(pr, dt, lane, Bs) * inv_lam + mf * sd;
-                }
-            }
-        }
-        if (r == 1 && alive) {
-            alive = wait_local(rbar, abort_flag, err);  // rho_J from the round-0 warp
-            rr = lane < rows ? (float)rhoa[slot * 32 + lane] - rr : 0.f;
-        }
-        float d = 0.f;
-        if (alive) {
-            rb[lane] = lane < rows ? rr : 0.f;
-            __syncwarp();
-            d = panel_dot(xs + lane * 32, rb, lane, 32);  // X_J r'_J (X row `lane` in rotated float4 chunks)
-        }
-        if (alive && J > 0) {
-            if (wait_remote(&bars[r * nsup + J - 1], abort_flag, err))
-                d -= panel_dot(ns + lane * 32, rv + (J - 1) * Bs, lane, Bs);
-            else
-                alive = false;
-        }
-        if (alive) {
-            // Delta_J to every CTA of the cluster (this one included)
-            ds[lane] = lane < rows ? d : 0.f;
-            __syncwarp();
-#pragma unroll
-            for (int t = 0; t < 4; ++t)
-                if (lane + 32 * t < nsend) ptx::st_async_v4(raddr[t], *(const float4 *)(ds + soff[t]), rbarr[t]);
-            if (r == 0 && rounds > 1) {
-                // residual rho_J = -g_J - L_{J, T<=J} Delta0 (double-single products; FP64 repeat term)
-                const bool okd = wait_local(dbar, abort_flag, err);
-                if (okd && lane < rows) {
-                    if (J > 0) {
-                        float h, l;
-                        panel_dot_ds(pan + (size_t)(J - 1) * pstride + lane * Bs, rv + (J - 1) * Bs, lane, Bs, h, l);
-                        ds_add(hi, lo, h, l);
-                    }
-                    float h, l;  // the diagonal panel: the blocks up to this row's block
-                    panel_dot_ds(pan + (size_t)J * pstride + lane * Bs, ds, lane, (lane / b + 1) * b, h, l);
-                    ds_add(hi, lo, h, l);
-                    double dmv = (double)ds[lane];
-                    for (int T = 0; T <= J; ++T) {
-                        uint32_t mask = dm[T * 32 + lane];
-                        const float *v = T < J ? rv + T * Bs : ds;
-                        while (mask) {
-                            dmv += (double)v[__ffs(mask) - 1];
-                            mask &= mask - 1;
-                        }
-                    }
-                    rhoa[slot * 32 + lane] = rhs - (((double)hi + (double)lo) / lambda + mdiag * dmv);
-                }
-            } else if (lane < rows) {
-                // Delta = sum over rounds
-                const double dd = (rounds > 1 ? (double)dsend[(0 * CL_SLOTS + slot) * 32 + lane] : 0.0) + (double)d;
-                delta[row] = dd;
-                if (w64) w64[row] = dd / lambda;
-                if (w32) w32[row] = (float)(dd / lambda);
-            }
-        }
+    if (J >= 0 && role == 3 && rounds > 1) cl_residual<BS>(w);
+    if (J >= 0 && role < rounds) {
+        const int r = role;  // the round this warp runs
+        float d;
+        const bool sent = cl_chain<BS>(w, r, dsend + (r * CL_SLOTS + slot) * 32, rbufa + (r * CL_SLOTS + slot) * 32, d);
         if (r == 0 && J == trig_sup && lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        if (r == 0 && rounds > 1) {  // always release the round-1 warp (it gives up if this one did)
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(rbar);
+        // Delta = the sum over the rounds
+        const bool have = sent && (r == 0 || wait_bar<true>(&bars[J], abort_flag, err));
+        if (have && r == rounds - 1 && lane < w.rows) {
+            const int row = J * Bs + lane;
+            const double dd = (r == 1 ? (double)recv[row] : 0.0) + (double)d, dw = dd / lambda;
+            delta[row] = dd;
+            if (w64) w64[row] = dw;
+            if (w32) w32[row] = (float)dw;
         }
     }
     // every Delta addressed to this CTA, and every panel copy, lands before it leaves
@@ -612,9 +707,16 @@ __global__ void __launch_bounds__(CL_THREADS, 1)
     ptx::cluster_sync();  // no CTA leaves while another may still address it
 }
 
-bool cluster_fits(int P, size_t smem)
+// super-blocks have 20, 24, 28 or 32 rows (b a multiple of 4, at most 32)
+auto cluster_kernel(int bs)
 {
-    auto kfn = bdcd_cluster_kernel;
+    return bs == 32 ? bdcd_cluster_kernel<32> : bs == 28 ? bdcd_cluster_kernel<28> : bs == 24 ? bdcd_cluster_kernel<24>
+                                                                                             : bdcd_cluster_kernel<20>;
+}
+
+bool cluster_fits(int P, size_t smem, int bs)
+{
+    auto kfn = cluster_kernel(bs);
     if (cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_MAX) != cudaSuccess)
         return false;
     if (cudaFuncSetAttribute(kfn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
@@ -667,7 +769,7 @@ int recur_cluster_size(int nblk, int b, int rounds)
     if (it != cache.end()) return it->second;
     const int P = cluster_ctas(G.nsup);
     const size_t smem = cluster_smem(nblk, b, P);
-    const bool ok = smem <= CL_SMEM_MAX && cluster_fits(P, smem);
+    const bool ok = smem <= CL_SMEM_MAX && cluster_fits(P, smem, G.Bs);
     cache[key] = ok ? P : 0;
     return ok ? P : 0;
 }
@@ -718,8 +820,9 @@ cudaError_t launch_recur_cluster_chain(const float *Kss, int64_t ldk, const int3
     int32_t *next = (int32_t *)(M + (size_t)G.nsup * CL_NSUP_MAX * 32);
     CUtensorMap kmap;
     if (!make_map_f32_2d(&kmap, Kss, sb, sb, ldk, G.Bs, G.Bs)) return cudaErrorInvalidValue;
-    auto kfn = bdcd_cluster_kernel;
-    static bool attr = false;
+    auto kfn = cluster_kernel(G.Bs);
+    static bool attrs[4] = {false, false, false, false};
+    bool &attr = attrs[(32 - G.Bs) / 4];
     cudaError_t e;
     if (!attr) {
         e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CL_SMEM_MAX);

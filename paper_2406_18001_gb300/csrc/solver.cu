@@ -74,7 +74,10 @@ dcd_status csc_choose(const CsrOperand &ca, bool fp64, int64_t cnt, int maxrow, 
 
 constexpr int64_t SB_MAX = 8192;   // s*b per outer step
 constexpr int B_MAX = 128;         // block size
-constexpr int DF_XPAIRS = 16;      // CTA pairs (at most) of the deferred gradient's cross product
+// CTA pairs (at most) of the deferred gradient's cross product: those that fit the SMs that the
+// recurrence before it leaves.  (16 took the SMs that the panels' preparation needs: it ran 43 us
+// beside them, not 17, and a step of m = 50000, 1024 coordinates 70, not 67.)
+constexpr int DF_XPAIRS = 8;
 
 // Set while the batched driver and the autotuner build their plans: those
 // capture many plans' steps into one graph and run without the look-ahead.
