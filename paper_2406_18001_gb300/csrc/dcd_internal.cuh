@@ -301,20 +301,18 @@ cudaError_t launch_f64_to_f32(const double *src, int64_t count, float *dst, cuda
 cudaError_t launch_row_terms_fp8(const void *packed, int64_t n_pad, int64_t m, const KernelParams &kp, float *h,
                                  cudaStream_t st, const float *rscale);
 // with the rows, optionally the per-row values f0 (and f1) of the same
-// indices: d0[j] = f0[idx[j]] (0 for an index outside [0, m))
+// indices: d0[j] = f0[idx[j]] (0 for an index outside [0, m)); and, with link (the deferred gradient,
+// solver.cu), link[j] = the first q < cprev with prev[q] == idx[j], or -1 (prev 16-byte aligned)
 cudaError_t launch_gather_rows(const void *src, int64_t row_bytes, const int32_t *idx, int64_t count, int64_t m,
                                void *dst, int *err, cudaStream_t st, const float *f0 = nullptr, float *d0 = nullptr,
                                const float *f1 = nullptr, float *d1 = nullptr, const float *f2 = nullptr,
-                               float *d2 = nullptr);
+                               float *d2 = nullptr, const int32_t *prev = nullptr, int64_t cprev = 0,
+                               int32_t *link = nullptr);
 cudaError_t launch_fill_f64(double *p, double v, int64_t count, cudaStream_t st);
 // out[i] = start + i, i < count (shard.cu)
 cudaError_t launch_iota(int32_t *out, int64_t count, int64_t start, cudaStream_t st);
 cudaError_t launch_init_grad(int problem, const double *y, const double *alpha, double diag, int64_t m, double *g,
                              cudaStream_t st);
-// the deferred gradient (solver.cu): link[p] = the first position q of the previous step with Sprev[q]
-// == S[p], or -1.  cprev <= 8192.
-cudaError_t launch_defer_links(const int32_t *S, int64_t cnt, const int32_t *Sprev, int64_t cprev, int32_t *link,
-                               cudaStream_t st);
 // the deferred K-SVM step (sample_update.cu): alpha and g at S (before they change), and the
 // pending parts of the next step's alpha and g from this step's Kx = K(A_S, A_Sc) (row-major,
 // leading dimension ldx), theta and w = y theta

@@ -331,41 +331,72 @@ cudaError_t launch_row_terms_fp8(const void *packed, int64_t n_pad, int64_t m, c
 // dst row j = src row idx[j] (whole packed rows, 16-byte vectors; row_bytes
 // is a multiple of 128), and d0[j] = f0[idx[j]], d1[j] = f1[idx[j]] where
 // given.  Indices outside [0, m) give a zero row (and zero values) and set
-// DEV_BAD_INDEX.
-__global__ void gather_rows_kernel(const uint4 *src, int64_t row_vec, const int32_t *idx, int64_t count, int64_t m,
-                                   uint4 *dst, int *err, const float *f0, float *d0, const float *f1, float *d1,
-                                   const float *f2, float *d2)
+// DEV_BAD_INDEX.  With link: link[j] = the first position q of the previous
+// step with prev[q] == idx[j], or -1 (where the update's part of the gradient
+// at a row that the next step samples is found).
+// A warp per row, its loads in flight together: latency-bound, the index, then the row.  The links are a
+// scan of prev by the same warp (int4 loads, L2 hits) while the row is on its way: a kernel of its own
+// took 6 us, which the CTAs of the Gram waited for (their SMs), after 5 us of a gather element by element.
+constexpr int GATHER_WARPS = 8;
+
+__global__ void __launch_bounds__(GATHER_WARPS * 32)
+    gather_rows_kernel(const uint4 *src, int64_t row_vec, const int32_t *idx, int64_t count, int64_t m, uint4 *dst,
+                       int *err, const float *f0, float *d0, const float *f1, float *d1, const float *f2, float *d2,
+                       const int32_t *prev, int cprev, int32_t *link)
 {
-    const int64_t total = count * row_vec;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = e / row_vec, c = e - j * row_vec;
-        const int64_t r = idx[j];
+    const int lane = threadIdx.x & 31;
+    for (int64_t j = (int64_t)blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5); j < count;
+         j += (int64_t)gridDim.x * GATHER_WARPS) {
+        const int32_t r = idx[j];
         const bool bad = r < 0 || r >= m;
-        if (bad) {
-            if (c == 0) set_error(err, DEV_BAD_INDEX);
-            dst[e] = make_uint4(0, 0, 0, 0);
-        } else {
-            dst[e] = src[r * row_vec + c];
+        if (bad && lane == 0) set_error(err, DEV_BAD_INDEX);
+        const uint4 *s = src + (bad ? 0 : r) * row_vec;
+        uint4 *d = dst + j * row_vec;
+        for (int64_t c0 = 0; c0 < row_vec; c0 += 128) {
+            uint4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t c = c0 + 32 * u + lane;
+                if (c < row_vec) v[u] = bad ? make_uint4(0, 0, 0, 0) : s[c];
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t c = c0 + 32 * u + lane;
+                if (c < row_vec) d[c] = v[u];
+            }
         }
-        if (c == 0) {
-            if (d0) d0[j] = bad ? 0.f : f0[r];
-            if (d1) d1[j] = bad ? 0.f : f1[r];
-            if (d2) d2[j] = bad ? 0.f : f2[r];
+        if (lane == 0 && d0) d0[j] = bad ? 0.f : f0[r];
+        if (lane == 1 && d1) d1[j] = bad ? 0.f : f1[r];
+        if (lane == 2 && d2) d2[j] = bad ? 0.f : f2[r];
+        if (link) {
+            int first = INT32_MAX;
+            const int4 *p4 = (const int4 *)prev;
+#pragma unroll 8
+            for (int q = lane; q < cprev / 4; q += 32) {
+                const int4 v = p4[q];
+                const int at = v.x == r ? 0 : v.y == r ? 1 : v.z == r ? 2 : v.w == r ? 3 : -1;
+                if (at >= 0) first = min(first, 4 * q + at);
+            }
+            for (int q = (cprev & ~3) + lane; q < cprev; q += 32)
+                if (prev[q] == r) first = min(first, q);
+            first = __reduce_min_sync(0xffffffffu, first);
+            if (lane == 0) link[j] = first == INT32_MAX ? -1 : first;
         }
     }
 }
 
 cudaError_t launch_gather_rows(const void *src, int64_t row_bytes, const int32_t *idx, int64_t count, int64_t m,
                                void *dst, int *err, cudaStream_t st, const float *f0, float *d0, const float *f1,
-                               float *d1, const float *f2, float *d2)
+                               float *d1, const float *f2, float *d2, const int32_t *prev, int64_t cprev, int32_t *link)
 {
     if (count <= 0) return cudaSuccess;
     if ((d0 && !f0) || (d1 && !f1) || (d2 && !f2)) return cudaErrorInvalidValue;
-    const int64_t row_vec = row_bytes / 16;
-    int64_t blocks = (count * row_vec + 255) / 256;
-    if (blocks > 152 * 16) blocks = 152 * 16;
-    gather_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>((const uint4 *)src, row_vec, idx, count, m, (uint4 *)dst,
-                                                         err, f0, d0, f1, d1, f2, d2);
+    if (link && (!prev || cprev > INT32_MAX || ((uintptr_t)prev & 15) != 0)) return cudaErrorInvalidValue;
+    int64_t blocks = (count + GATHER_WARPS - 1) / GATHER_WARPS;
+    if (blocks > 152 * 8) blocks = 152 * 8;
+    gather_rows_kernel<<<(unsigned)blocks, GATHER_WARPS * 32, 0, st>>>((const uint4 *)src, row_bytes / 16, idx, count, m,
+                                                                       (uint4 *)dst, err, f0, d0, f1, d1, f2, d2, prev,
+                                                                       (int)cprev, link);
     return cudaGetLastError();
 }
 
@@ -590,42 +621,6 @@ cudaError_t launch_dcd_pending(const int32_t *S, int64_t cnt, const double *y, c
     else
         dcd_pending_kernel<float><<<blocks, 128, 0, st>>>(S, (int)cnt, y, (const float *)Kx, ldx, Sc, theta, w,
                                                           (int)cc, diag, alpha_add, g_add);
-    return cudaGetLastError();
-}
-
-// link[p] = the first position q of the previous step with Sprev[q] == S[p], or -1: where the
-// update's part of the gradient at a row the next step samples is found.  One warp per position p,
-// Sprev staged in shared memory, 32 positions q per ballot.  It needs the samples only, so it runs
-// beside the recurrence; the recurrence after it adds the sums (the sums formed here, after the
-// recurrence they come from, were 5 us of the loop of steps).
-constexpr int REP_WARPS = 8;
-
-__global__ void __launch_bounds__(REP_WARPS * 32)
-    defer_links_kernel(const int32_t *S, int64_t cnt, const int32_t *Sprev, int cprev, int32_t *link)
-{
-    extern __shared__ int32_t sp[];  // as much as the step needs, so that the CTAs fit beside the block's
-    for (int q = threadIdx.x; q < cprev; q += blockDim.x) sp[q] = Sprev[q];
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int64_t p = (int64_t)blockIdx.x * REP_WARPS + (threadIdx.x >> 5);
-    if (p >= cnt) return;  // warp-uniform
-    const int32_t key = S[p];
-    int first = -1;
-    for (int q0 = 0; q0 < cprev && first < 0; q0 += 32) {
-        const int q = q0 + lane;
-        const unsigned hit = __ballot_sync(0xffffffffu, q < cprev && sp[q] == key);
-        if (hit) first = q0 + __ffs(hit) - 1;
-    }
-    if (lane == 0) link[p] = first;
-}
-
-cudaError_t launch_defer_links(const int32_t *S, int64_t cnt, const int32_t *Sprev, int64_t cprev, int32_t *link,
-                               cudaStream_t st)
-{
-    if (cnt <= 0) return cudaSuccess;
-    if (cprev > UPD_MAX) return cudaErrorInvalidValue;
-    defer_links_kernel<<<(unsigned)((cnt + REP_WARPS - 1) / REP_WARPS), REP_WARPS * 32, sizeof(int32_t) * cprev, st>>>(
-        S, cnt, Sprev, (int)cprev, link);
     return cudaGetLastError();
 }
 

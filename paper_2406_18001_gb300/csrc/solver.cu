@@ -1289,13 +1289,14 @@ struct Solver {
 
     // step products of a step of cnt blocks into buffer set q, on stream s2: the sample and the
     // gathers (la_rows), then the Gram and the prep (la_gram)
-    dcd_status la_side(int q, int64_t cnt, cudaStream_t s2, int qnext = -1, int max_ctas = 0)
+    dcd_status la_side(int q, int64_t cnt, cudaStream_t s2, int qnext = -1, int max_ctas = 0, int prev = -1)
     {
-        dcd_status r = la_rows(q, cnt, s2, qnext);
+        dcd_status r = la_rows(q, cnt, s2, qnext, prev);
         return r != DCD_OK ? r : la_gram(q, cnt, s2, max_ctas);
     }
 
-    dcd_status la_rows(int q, int64_t cnt, cudaStream_t s2, int qnext = -1)
+    // prev (deferred steps, both full): also where the rows are in the step before, in that set
+    dcd_status la_rows(int q, int64_t cnt, cudaStream_t s2, int qnext = -1, int prev = -1)
     {
         const StepBufs &Bq = sbuf[q];
         const int64_t ncols = cnt * o.b;
@@ -1304,7 +1305,8 @@ struct Solver {
         DCD_TRY(launch_sample(problem, o.seed, ctr_la + q, 0, m, o.b, cnt, Bq.S, err, s2, ctr_la + qnext));
         const bool f8 = op.kind == PACK_FP8 || op.kind == PACK_FP16;  // per-row scales gathered too
         DCD_TRY(launch_gather_rows(op.packed, packed_row_bytes(op.kind, op.n_pad), Bq.S, ncols, m, Bq.As, err, s2,
-                                   op.row_h, Bq.col_h, f8 ? op.row_s : nullptr, f8 ? Bq.col_s : nullptr));
+                                   op.row_h, Bq.col_h, f8 ? op.row_s : nullptr, f8 ? Bq.col_s : nullptr, nullptr, nullptr,
+                                   prev >= 0 ? sbuf[prev].S : nullptr, ncols, prev >= 0 ? df_link[q] : nullptr));
         return DCD_OK;
     }
 
@@ -1469,13 +1471,6 @@ struct Solver {
         return DCD_OK;
     }
 
-    // where the rows of the step in set r (full) are in the step before, in set c
-    dcd_status df_links_of(int r, int c, cudaStream_t s)
-    {
-        const int64_t nc = o.s * o.b;
-        return cuda_status(launch_defer_links(sbuf[r].S, nc, sbuf[c].S, nc, df_link[r], s));
-    }
-
     // x of the step in set r (full) from the step in set c (full, its recurrence done), on stream s:
     // a part per 256 columns, every (256-row tile, part) on a CTA pair of its own; the recurrence adds
     // the parts and the update's (the links).  (Two column halves on four pairs each took 15 us, and
@@ -1511,12 +1506,10 @@ struct Solver {
         }
         if (has2) {
             DCD_TRY(cudaStreamWaitEvent(st2, df_fork, 0));
-            dcd_status r = la_rows(nn, o.s, st2, (nn + 1) % 3);
+            dcd_status r = la_rows(nn, o.s, st2, (nn + 1) % 3, nxt);
             if (r != DCD_OK) return r;
             DCD_TRY(cudaEventRecord(df_rows, st2));
             DCD_TRY(cudaStreamWaitEvent(st3, df_rows, 0));
-            r = df_links_of(nn, nxt, st3);
-            if (r != DCD_OK) return r;
             r = la_gram(nn, o.s, st2, df_gram_ctas);
             if (r != DCD_OK) return r;
             DCD_TRY(cudaEventRecord(df_gram, st2));
@@ -1578,12 +1571,11 @@ struct Solver {
             if (r != DCD_OK) return r;
             if (has1) {  // step k+1's products and x
                 if (df_prod != o.s) {
-                    r = la_side(nxt, o.s, st, nn);
+                    r = la_side(nxt, o.s, st, nn, 0, cur);
                     if (r != DCD_OK) return r;
                     df_prod = o.s;
                 }
-                r = df_links_of(nxt, cur, st);
-                if (r == DCD_OK) r = df_cross(nxt, cur, st);
+                r = df_cross(nxt, cur, st);
                 if (r != DCD_OK) return r;
             }
             df_chain = true;
