@@ -80,7 +80,7 @@ __device__ __forceinline__ double kfun_f64(const KernelParams &kp, double v)
 dcd_status validate_kernel(const dcd_kernel *k);
 dcd_status validate_dense(const dcd_matrix *A);
 
-// Every device allocation of the library (selftest.cu): cudaMallocAsync, or a
+// Every device allocation of the library (selftest.cu), from its own memory pool: freed with cudaFreeAsync; or a
 // failure injected by dcd_inject_alloc_failures.
 cudaError_t malloc_async(void **p, size_t bytes, cudaStream_t st);
 

@@ -15,11 +15,45 @@
 #include "ptx.cuh"
 
 #include <atomic>
+#include <mutex>
 
 namespace dcd {
 namespace {
 
 std::atomic<int> g_fail_allocs{0};
+
+// The library's own memory pool on the current device (nullptr: none could be made; a stream-ordered
+// pool, so safe from several threads and streams).  It keeps at most POOL_KEEP of freed memory mapped:
+// the default pool returns all of it to the driver at every synchronisation, and mapping it again took
+// 50 to 170 us of an allocation after one (a sweep of 32 plans: 19.7 -> 15.9 ms).  What it keeps goes
+// back when an allocation of the library's fails, and with the process.
+constexpr int POOL_DEVICES = 64;
+constexpr uint64_t POOL_KEEP = 512ull << 20;
+
+cudaMemPool_t device_pool()
+{
+    static std::mutex mu;
+    static cudaMemPool_t pools[POOL_DEVICES] = {};
+    static bool made[POOL_DEVICES] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= POOL_DEVICES) return nullptr;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!made[dev]) {
+        made[dev] = true;
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        uint64_t keep = POOL_KEEP;
+        if (cudaMemPoolCreate(&pools[dev], &props) != cudaSuccess) {
+            cudaGetLastError();
+            pools[dev] = nullptr;
+        } else if (cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();  // it keeps nothing, as the default pool
+        }
+    }
+    return pools[dev];
+}
 
 __global__ void bounded_wait_selftest_kernel(unsigned long long limit_ns, int *err, int *waited)
 {
@@ -44,7 +78,15 @@ cudaError_t malloc_async(void **p, size_t bytes, cudaStream_t st)
             return cudaErrorMemoryAllocation;
         }
     }
-    return cudaMallocAsync(p, bytes, st);
+    const cudaMemPool_t pool = device_pool();
+    if (!pool) return cudaMallocAsync(p, bytes, st);
+    cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    if (e == cudaErrorMemoryAllocation) {  // what the pool keeps may be in the way
+        cudaGetLastError();
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    }
+    return e;
 }
 
 }  // namespace dcd
