@@ -31,7 +31,8 @@
 // Warp roles in both:
 //   warp 0      TMA producer: 128-byte-swizzled k-blocks of A and B into a
 //               shared-memory ring (mbarrier complete_tx)
-//   warp 1      TMEM allocator and MMA issuer (one thread); accumulators are
+//   warp 1      TMEM allocator and MMA issuer (one elected lane of a warp
+//               whose loops are uniform, tc_ptx.cuh); accumulators are
 //               double-buffered (2 x BN columns) so the epilogue of one
 //               N-chunk overlaps the MMAs of the next
 //   warps 2..9  epilogue: tcgen05.ld 32 lanes x 32 columns per load, one

@@ -1215,13 +1215,15 @@ struct Solver {
     bool ref_shared = false;  // the recomputed gradient uses the step operand's buffers
 
     // ---- replayed steps of the look-ahead bodies ----
-    // Graphs of 1, 3, 7 and 15 consecutive steady bodies, by the buffer set they start with; body(q) enqueues one on set q, the next on set q + 1 mod nsets.  Between two
-    // launches the GPU stands still for 5-7 us, within a graph a body follows in about one, so the
-    // longest graph that fits the steps to run is taken -- but one body where the stream is idle, as its
-    // kernels are submitted soonest and the long graph's while it runs (K-SVM FP64 at m = 2000, s = 8:
-    // 18.2 -> 15.0 us a step; K-RR fp16 at m = 50000, s = 64: GRAPH_KRR).  A graph is captured once every set has run a body
-    // directly (attributes and occupancy queries are then cached) and, the long ones, once the plan's
-    // steps so far and at hand pay for the capture (about 25 us a body against 5 us a step saved).
+    // Graphs of 1, 3, 7 and 15 consecutive steady bodies, by the buffer set they start with; body(q)
+    // enqueues one on set q, the next on set q + 1 mod nsets.  Between two launches the GPU stands still
+    // for 5-7 us, within a graph a body follows in about one, so the longest graph that fits the steps to
+    // run is taken -- but one body where the stream is idle, as its kernels are submitted soonest and the
+    // long graph's while it runs (K-SVM FP64 at m = 2000, s = 8: 18.2 -> 15.0 us a step; K-RR fp16 at
+    // m = 50000, s = 64: 8 steps 583 -> 547, and 636 with the long graph first).  A graph is captured once
+    // every set has run a body directly (attributes and occupancy queries are then cached) and, the long
+    // ones, once the plan's steps so far and at hand pay for the capture (about 25 us a body against 5 us
+    // a step saved).
     static constexpr int GRAPH_LENS = 4;
     cudaGraphExec_t graph_steps[GRAPH_LENS][3] = {};
     int body_direct[3] = {0, 0, 0};

@@ -9,17 +9,28 @@
 // CTA runs the recurrence on them for itself and updates its own rows.  Two groups of warps run beside
 // each other in a CTA:
 //   main (4 warps)     step k: read the exchange and the couplings, the chain (dcd_chain.cuh), g_i +=
-//                      y_i sum_j K(a_i, a_Sj) w_j and alpha on the own rows, publish, grid barrier;
-//   block (12 warps)   ahead of it, as it needs the index stream only: the rows of step q, this CTA's
-//                      share of its Gram (to memory, read by all a step later) and the own rows' kernel
-//                      values against them, KS lanes an entry, into one of two buffers.
-// So the FP64 pipe's work (m s (n + 14) operations a step) runs beside the latencies (barrier, L2
-// read, chain).  Kernel values: dot products, the RBF from the expansion with compensated norms where
+//                      y_i sum_j K(a_i, a_Sj) w_j and alpha on the own rows, publish;
+//   block (12 warps)   ahead of it, as it needs the index stream only: four warps fetch the rows of step
+//                      q + 1 by asynchronous copies and form this CTA's share of step q's Gram (to
+//                      memory, read by all a step later); beside them eight form the own rows' kernel
+//                      values against step q's rows, KS lanes an entry, into one of two buffers.
+// So the FP64 pipe's work (m s (n + 14) operations a step) runs beside the latencies (L2 round trips,
+// chain).  Kernel values: dot products, the RBF from the expansion with compensated norms where
 // gamma |a|^2 <= F64S_HMAX for every row, else from coordinate differences; K = 1 on a row's own
 // sample.
 //
-// Measured (FP64, hinge): m = 2000, n = 64, s = 8: 15.3 us a step as long graphs -> 5.6; m = 300,
-// n = 16, s = 1 on the default stream: 27 -> 4.1.
+// The exchange is no grid barrier.  A published value is its own signal: the four slots x(k) of xbuf
+// take turns, X_OPEN stands in an entry that is not there yet, and the readers poll the entries.  The
+// rest is ordered by one counter: a CTA arrives in step k, between its chain and its update, when it has
+// read x(k), emptied its share of x(k + 2)'s slot and finished its share of step k + 1's Gram, and
+// it begins step k + 1 when all have arrived -- by then mostly long past.  So the couplings may be
+// read in step k + 1 (all shares are there), x(k + 2) may be written at its end (all entries are open)
+// and the slot of x(k - 2) may be emptied in step k (all have read it).  Barriers with a fence on
+// both sides took 4.4 k of a step's 11 k cycles at m = 2000, s = 8.
+//
+// Measured (FP64, hinge): m = 2000, n = 64, s = 8: 15.3 us a step as long graphs, 5.8 with a grid
+// barrier a step, 4.7 now (the FP64 pipe of the own rows' values 3.4 of it); m = 300, n = 16, s = 1 on
+// the default stream: 27, 4.1, 3.3 (1 of it host work).
 #include "dcd_chain.cuh"
 #include "dcd_internal.cuh"
 #include "f64_math.cuh"
@@ -34,12 +45,16 @@ namespace {
 constexpr int GM_WARPS = 4, GB_WARPS = 12;  // main and block warps
 constexpr int GM = 32 * GM_WARPS, GB = 32 * GB_WARPS;
 constexpr int GRID_THREADS = GM + GB;
+constexpr int GX_WARPS = 4, GX = 32 * GX_WARPS, GY = GB - GX;  // block warps of samples and Gram; threads of the own rows' values
+constexpr int GRAM_THREADS = GB + 32;  // at NB_GRAM: the block and the main warp that counts arrivals
 constexpr size_t GRID_SMEM_MAX = 200 * 1024;
-constexpr long long GRID_WAIT_CYCLES = 4200000000LL;  // about 2 s: bound on a wait at the grid barrier
+constexpr int GU = GM - 32;  // threads that update; the last main warp counts arrivals meanwhile
+constexpr long long GRID_WAIT_CYCLES = 4200000000LL;  // about 2 s: bound on a wait for other CTAs
+constexpr long long X_OPEN = -1;  // the bits of an entry that is not published
 // kernel-value forms
 constexpr int GK_LINEAR = 0, GK_POLY = 1, GK_RBF = 2, GK_RBF_DIRECT = 3;
 // named barriers (0 is __syncthreads)
-constexpr int NB_MAIN = 1, NB_BLOCK = 2, NB_FULL = 3, NB_FREE = 5, NB_GRAM = 7;  // the last three + parity
+constexpr int NB_MAIN = 1, NB_BLOCK = 2, NB_FULL = 3, NB_FREE = 5, NB_GRAM = 7, NB_UPD = 9, NB_X = 10;  // FULL, FREE, GRAM: + parity
 
 struct GridArgs {
     const double *A;
@@ -53,14 +68,14 @@ struct GridArgs {
     uint64_t *ctr;
     int steps, s, R, ks, nls;  // rows per CTA, lanes per entry, row stride in shared memory
     double omega, nu;
-    double *xbuf;   // [2][s][2]: g and alpha at the step's coordinates
+    double *xbuf;   // [4][s][2]: g and alpha at the step's coordinates
     double *kss;    // [4][s * s + 2 s] by step (a CTA may be two steps ahead of another's reads): K(S_t, S_j) for j < t at [j * s + t], then 1 / eta_t, eta_t
     unsigned *bar;  // arrivals, zero at the start
     int *err;
 };
 
 struct GridLayout {
-    size_t own, as, kb, gs, al, hr, hs, C, slot, th, w, tab, ints, total;
+    size_t own, as, kb, gs, al, hr, hs, yv, C, slot, th, w, tab, ints, total;
 };
 
 __host__ __device__ inline GridLayout grid_layout(int n, int s, int R, int nls)
@@ -79,13 +94,14 @@ __host__ __device__ inline GridLayout grid_layout(int n, int s, int R, int nls)
     L.al = take(R);
     L.hr = take(R);
     L.hs = take(2 * (size_t)s);
+    L.yv = take(4 * (size_t)s);
     L.C = take((size_t)s * (s | 1));
     L.slot = take(s);
     L.th = take(s);
     L.w = take(s);
     L.tab = take(64);
-    L.ints = c;  // S 2 s; sign of y: at S 2 s, own rows R; rep 4 s
-    L.total = 8 * c + 4 * ((size_t)(2 + 2 + DCD_FAST_K) * s + R);
+    L.ints = c;  // S 4 s; sign bits of the own rows' y R; rep 4 s
+    L.total = 8 * c + 4 * ((size_t)(4 + DCD_FAST_K) * s + R);
     return L;
 }
 
@@ -141,6 +157,18 @@ __device__ __forceinline__ double k_value(double v, double hi, double hj, bool o
     return exp_tab(x, tab);
 }
 
+__device__ __forceinline__ double x_ld(const double *p)
+{
+    double v;
+    asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void x_st(double *p, double v)
+{
+    asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
+}
+
 template <int FORM>
 __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
 {
@@ -148,11 +176,10 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
     const int s = a.s, R = a.R, n = a.n, nls = a.nls, ldc = s | 1;
     const GridLayout L = grid_layout(n, s, R, nls);
     double *own = gsm + L.own, *As = gsm + L.as, *kb = gsm + L.kb, *gs = gsm + L.gs, *al = gsm + L.al,
-           *hr = gsm + L.hr, *hS = gsm + L.hs, *C = gsm + L.C, *slot = gsm + L.slot, *th_s = gsm + L.th, *w_s = gsm + L.w,
+           *hr = gsm + L.hr, *hS = gsm + L.hs, *yv = gsm + L.yv, *C = gsm + L.C, *slot = gsm + L.slot, *th_s = gsm + L.th, *w_s = gsm + L.w,
            *tab = gsm + L.tab;
-    int32_t *SS = (int32_t *)(gsm + L.ints);             // S of a step, by its parity
-    uint32_t *sy = (uint32_t *)(SS + 2 * s);             // sign bits of y at S, by parity
-    uint32_t *yr = sy + 2 * s;                           // sign bits of the own rows' y
+    int32_t *SS = (int32_t *)(gsm + L.ints);             // S of a step, by step mod 4
+    uint32_t *yr = (uint32_t *)(SS + 4 * s);             // sign bits of the own rows' y
     uint32_t *rep = yr + R;
     __shared__ int stop_s;                               // the grid barrier's wait ran out
     const int cta = blockIdx.x, G = gridDim.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -176,25 +203,42 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
     if (warp >= GM_WARPS) {
         // ----------------------------------------------------------- block --
         const int bt = tid - GM, bw = warp - GM_WARPS, ks = a.ks;
+        // the sample of step q with its labels and RBF terms; its rows (asynchronous; S is there)
+        auto sample = [&](int q) {
+            for (int j = bt; j < s; j += GX) {
+                const int32_t i = index_of(q, j);
+                SS[(q & 3) * s + j] = i;
+                ptx::cp_async8(yv + (q & 3) * s + j, a.y + i);
+                if (FORM == GK_RBF) ptx::cp_async8(hS + (q & 1) * s + j, a.h + i);
+            }
+        };
+        auto gather = [&](int q) {
+            double *Aq = As + (size_t)(q & 1) * s * n;
+            const int32_t *Sq = SS + (q & 3) * s;
+            for (int j = bw; j < s; j += GX_WARPS) {
+                const double *row = a.A + (int64_t)Sq[j] * a.lda;
+                for (int c = lane; c < n; c += 32) ptx::cp_async8(Aq + (size_t)j * n + c, row + c);
+            }
+        };
+        const bool is_x = bw < GX_WARPS;
+        if (is_x) {
+            sample(0);
+            nb_sync<GX>(NB_X);
+            gather(0);
+            ptx::cp_async_wait_all();
+        }
+        nb_sync<GB>(NB_BLOCK);
         for (int q = 0; q < a.steps; ++q) {
             const int p = q & 1;
             double *Aq = As + (size_t)p * s * n, *kq = kb + (size_t)p * s * R;
-            int32_t *Sq = SS + p * s;
+            const int32_t *Sq = SS + (q & 3) * s;
             double *hq = hS + p * s;
             if (q >= 2) nb_sync<GRID_THREADS>(NB_FREE + p);  // main is done with step q - 2's buffer
             if (*(volatile int *)&stop_s) break;
-            for (int j = bt; j < s; j += GB) {
-                const int32_t i = index_of(q, j);
-                Sq[j] = i;
-                sy[p * s + j] = (uint32_t)__double2hiint(a.y[i]) & 0x80000000u;
-                hq[j] = FORM == GK_RBF ? a.h[i] : 0.0;
-            }
-            nb_sync<GB>(NB_BLOCK);
-            for (int e = bt; e < s * n; e += GB) Aq[e] = a.A[(int64_t)Sq[e / n] * a.lda + e % n];
-            nb_sync<GB>(NB_BLOCK);
             // this CTA's entries of the step's Gram: pairs j <= t, a warp each
             double *kss = a.kss + (size_t)(q & 3) * (s * s + 2 * s);
-            for (int e = cta + G * bw; e < s * (s + 1) / 2; e += G * GB_WARPS) {
+            if (!is_x) nb_arrive<GRAM_THREADS>(NB_GRAM + p);
+            for (int e = cta + G * bw; is_x && e < s * (s + 1) / 2; e += G * GX_WARPS) {
                 int t = (int)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
                 while (t * (t + 1) / 2 > e) --t;
                 while ((t + 1) * (t + 2) / 2 <= e) ++t;
@@ -213,12 +257,19 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
                     }
                 }
             }
-            __threadfence();
-            nb_arrive<GRID_THREADS>(NB_GRAM + p);
+            if (is_x) {
+                __threadfence();
+                nb_arrive<GRAM_THREADS>(NB_GRAM + p);
+                if (q + 1 < a.steps) {  // after the Gram, which the other CTAs wait for
+                    sample(q + 1);
+                    nb_sync<GX>(NB_X);
+                    gather(q + 1);
+                }
+            }
             // the own rows' kernel values against the step's: entry (j, r), ks lanes each
             const int items = s * R * ks;
-            for (int e0 = 0; e0 < items; e0 += GB) {
-                const int e = e0 + bt, l = e & (ks - 1), en = e / ks, j = en / R, r = en - j * R;
+            for (int e0 = 0; !is_x && e0 < items; e0 += GY) {
+                const int e = e0 + bt - GX, l = e & (ks - 1), en = e / ks, j = en / R, r = en - j * R;
                 const bool in = e < items && r < rows;
                 double v = in ? dot_part<FORM>(own + (size_t)r * nls, Aq + (size_t)j * n, n, l, ks) : 0.0;
                 for (int o = ks >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -228,119 +279,170 @@ __global__ void __launch_bounds__(GRID_THREADS, 1) svm_grid_kernel(GridArgs a)
                 }
             }
             nb_arrive<GRID_THREADS>(NB_FULL + p);
+            if (is_x) ptx::cp_async_wait_all();  // step q + 1's rows
+            nb_sync<GB>(NB_BLOCK);
         }
         return;
     }
 
     // ---------------------------------------------------------------- main --
     const int ng = (s + 31) / 32;
+    auto give_up = [&] {
+        set_error(a.err, DEV_TIMEOUT);
+        stop_s = 1;
+    };
     auto publish = [&](int k) {  // the own rows' alpha and g at step k's coordinates
-        const int p = k & 1;
-        for (int j = tid; j < s; j += GM) {
-            const int32_t i = SS[p * s + j];
+        for (int j = tid; j < s; j += GU) {
+            const int32_t i = SS[(k & 3) * s + j];
             if (i >= r0 && i < r0 + rows) {
-                double *x = a.xbuf + ((size_t)p * s + j) * 2;
-                x[0] = gs[i - r0];
-                x[1] = al[i - r0];
+                double *x = a.xbuf + ((size_t)(k & 3) * s + j) * 2;
+                const double v[2] = {gs[i - r0], al[i - r0]};
+                for (int u = 0; u < 2; ++u)  // a NaN that looks like an open entry: another one
+                    x_st(x + u, __double_as_longlong(v[u]) == X_OPEN ? __longlong_as_double(X_OPEN - 1) : v[u]);
             }
         }
     };
-    auto grid_barrier = [&](int k) -> bool {  // every CTA is past its publish(k)
-        nb_sync<GM>(NB_MAIN);
-        if (tid == 0) {
-            __threadfence();
-            const unsigned want = (unsigned)G * (unsigned)(k + 1);
-            atomicAdd(a.bar, 1u);
-            const long long c0 = clock64();
+    // one thread: this CTA's arrival number k (from 0), and the wait until every CTA has made it
+    auto arrive = [&](int k) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(a.bar), "r"(1u) : "memory");
+        const unsigned want = (unsigned)G * (unsigned)(k + 1);
+        const long long c0 = clock64();
+        for (;;) {
             unsigned v;
-            for (;;) {
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.bar) : "memory");
-                if ((int)(v - want) >= 0) break;
-                if (clock64() - c0 > GRID_WAIT_CYCLES) {
-                    set_error(a.err, DEV_TIMEOUT);
-                    stop_s = 1;
-                    break;
-                }
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.bar) : "memory");
+            if ((int)(v - want) >= 0) break;
+            if (clock64() - c0 > GRID_WAIT_CYCLES) {
+                give_up();
+                break;
             }
-            __threadfence();
         }
-        nb_sync<GM>(NB_MAIN);
-        return !*(volatile int *)&stop_s;
     };
-    nb_sync<GRID_THREADS>(NB_GRAM);
-    publish(0);
-    bool ok = grid_barrier(0);
+    // lanes per row of the update
+    int nls2 = 0;  // their log2
+    while (nls2 < 5 && (2 << nls2) <= s && (2 << nls2) * R <= GU) ++nls2;
+    const int nl = 1 << nls2;
+    if (warp == GM_WARPS - 1) nb_sync<GRAM_THREADS>(NB_GRAM);
+    nb_sync<GM>(NB_MAIN);
+    if (warp == GM_WARPS - 1) {
+        if (lane == 0) arrive(0);
+        __syncwarp();
+    } else {
+        publish(0);
+    }
+    bool ok = true;
     int k = 0;
-    for (; ok && k < a.steps; ++k) {
+    for (; k < a.steps; ++k) {
         const int p = k & 1;
-        const int32_t *S = SS + p * s;
-        const uint32_t *yk = sy + p * s;
+        const int32_t *S = SS + (k & 3) * s;
+        const double *yk = yv + (k & 3) * s;
+        auto ysign = [&](int t) { return (uint32_t)__double2hiint(yk[t]) & 0x80000000u; };
         const double *kss = a.kss + (size_t)(k & 3) * (s * s + 2 * s);
         double rho = 0.0, gj = 0.0, ie = 0.0, eta = 0.0;
         if (tid < s) {
-            const double *x = a.xbuf + ((size_t)p * s + tid) * 2;
-            gj = __ldcg(x);
-            rho = __ldcg(x + 1);
+            const double *x = a.xbuf + ((size_t)(k & 3) * s + tid) * 2;
+            const long long c0 = clock64();
+            for (;;) {
+                gj = x_ld(x);
+                rho = x_ld(x + 1);
+                if (__double_as_longlong(gj) != X_OPEN && __double_as_longlong(rho) != X_OPEN) break;
+                if (clock64() - c0 > GRID_WAIT_CYCLES) {
+                    give_up();
+                    break;
+                }
+            }
+        }
+        nb_sync<GM>(NB_MAIN);
+        if (*(volatile int *)&stop_s) {  // the same in every main thread: it changes between barriers only
+            ok = false;
+            break;
+        }
+        if (k + 2 < a.steps)
+            for (int j = cta + G * tid; j < s; j += G * GM) {
+                double *x = a.xbuf + ((size_t)((k + 2) & 3) * s + j) * 2;
+                x_st(x, __longlong_as_double(X_OPEN));
+                x_st(x + 1, __longlong_as_double(X_OPEN));
+            }
+        if (tid < s) {
             ie = __ldcg(kss + s * s + tid);
             eta = __ldcg(kss + s * s + s + tid);
             slot[tid] = __longlong_as_double(CHAIN_OPEN);
         }
-        for (int j = warp; j < s; j += GM_WARPS)
-            for (int q = 0; q < ng; ++q) {
-                const int t = 32 * q + lane;
-                const bool later = t < s && t > j;
-                const bool same = later && S[later ? t : 0] == S[j];
-                double v = later ? __ldcg(kss + j * s + t) : 0.0;
-                v = __hiloint2double((int)((uint32_t)__double2hiint(v) ^ (later ? yk[t] ^ yk[j] : 0u)), __double2loint(v));
-                if (same) v += a.omega;
-                if (t < s) C[j * ldc + t] = v;
-                const uint32_t mask = __ballot_sync(0xffffffffu, same);
-                if (lane == 0) rep[j * DCD_FAST_K + q] = mask;
+        constexpr int U = 4;  // rows' couplings in flight
+        for (int q = 0; q < ng; ++q) {
+            const int t = 32 * q + lane;
+            const uint32_t yt = t < s ? ysign(t) : 0u;
+            const int32_t St = t < s ? S[t] : -1;
+            for (int j0 = warp; j0 < s; j0 += GM_WARPS * U) {
+                double v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int j = j0 + GM_WARPS * u;
+                    v[u] = j < s && t < s && t > j ? __ldcg(kss + j * s + t) : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int j = j0 + GM_WARPS * u;
+                    if (j >= s) break;  // warp-uniform
+                    const bool later = t < s && t > j, same = later && St == S[j];
+                    double c = __hiloint2double((int)((uint32_t)__double2hiint(v[u]) ^ (later ? yt ^ ysign(j) : 0u)),
+                                                __double2loint(v[u]));
+                    if (same) c += a.omega;
+                    if (t < s) C[j * ldc + t] = c;
+                    const uint32_t mask = __ballot_sync(0xffffffffu, same);
+                    if (lane == 0) rep[j * DCD_FAST_K + q] = mask;
+                }
             }
+        }
         nb_sync<GM>(NB_MAIN);
         if (warp < ng) {
             const double th = dcd_chain_group(C, ldc, rep, slot, s, warp, lane, rho, gj, eta, ie, a.nu, a.err);
             if (tid < s) {
                 th_s[tid] = th;
-                w_s[tid] = __hiloint2double((int)((uint32_t)__double2hiint(th) ^ yk[tid]), __double2loint(th));
+                w_s[tid] = __hiloint2double((int)((uint32_t)__double2hiint(th) ^ ysign(tid)), __double2loint(th));
             }
         }
         nb_sync<GM>(NB_MAIN);
         nb_sync<GRID_THREADS>(NB_FULL + p);  // the own rows' kernel values are there
-        const double *kq = kb + (size_t)p * s * R;
-        for (int r = tid; r < rows; r += GM) {
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0, sum = 0.0;
-            bool mine = false;
-            int j = 0;
-            for (; j + 3 < s; j += 4) {
-                s0 = fma(kq[j * R + r], w_s[j], s0);
-                s1 = fma(kq[(j + 1) * R + r], w_s[j + 1], s1);
-                s2 = fma(kq[(j + 2) * R + r], w_s[j + 2], s2);
-                s3 = fma(kq[(j + 3) * R + r], w_s[j + 3], s3);
-                mine |= S[j] == r0 + r || S[j + 1] == r0 + r || S[j + 2] == r0 + r || S[j + 3] == r0 + r;
+        if (warp == GM_WARPS - 1) {
+            if (k + 1 < a.steps) {
+                nb_sync<GRAM_THREADS>(NB_GRAM + (p ^ 1));
+                if (lane == 0) arrive(k + 1);
             }
-            for (; j < s; ++j) {
-                s0 = fma(kq[j * R + r], w_s[j], s0);
-                mine |= S[j] == r0 + r;
+            __syncwarp();
+        } else {
+            const double *kq = kb + (size_t)p * s * R;
+            for (int e0 = 32 * warp; e0 < R * nl; e0 += GU) {  // nl lanes per own row
+                const int r = (e0 + lane) >> nls2, l = (e0 + lane) & (nl - 1);
+                const bool in = r < rows;
+                double v = 0.0, own = 0.0;
+                bool hit = false;
+                for (int j = l; j < s; j += nl) {
+                    if (in) v = fma(kq[j * R + r], w_s[j], v);
+                    if (in && S[j] == r0 + r) {
+                        own += th_s[j];
+                        hit = true;
+                    }
+                }
+                for (int o = nl >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (__any_sync(0xffffffffu, hit))
+                    for (int o = nl >> 1; o > 0; o >>= 1) {
+                        own += __shfl_xor_sync(0xffffffffu, own, o);
+                        hit |= __shfl_xor_sync(0xffffffffu, (int)hit, o) != 0;
+                    }
+                if (in && l == 0) {
+                    v = __hiloint2double((int)((uint32_t)__double2hiint(v) ^ yr[r]), __double2loint(v));  // y_r
+                    double gn = gs[r] + v;
+                    if (hit) {  // this row's own steps
+                        al[r] += own;
+                        gn += a.omega * own;
+                    }
+                    gs[r] = gn;
+                }
             }
-            double v = (s0 + s1) + (s2 + s3);
-            v = __hiloint2double((int)((uint32_t)__double2hiint(v) ^ yr[r]), __double2loint(v));  // y_r
-            double gn = gs[r] + v;
-            if (mine) {  // this row's own steps, in position order
-                for (j = 0; j < s; ++j)
-                    if (S[j] == r0 + r) sum += th_s[j];
-                al[r] += sum;
-                gn += a.omega * sum;
-            }
-            gs[r] = gn;
+            nb_sync<GU>(NB_UPD);
+            if (k + 1 < a.steps) publish(k + 1);
         }
         if (k + 2 < a.steps) nb_arrive<GRID_THREADS>(NB_FREE + p);
-        if (k + 1 < a.steps) {
-            nb_sync<GM>(NB_MAIN);
-            nb_sync<GRID_THREADS>(NB_GRAM + (p ^ 1));
-            publish(k + 1);
-            ok = grid_barrier(k + 1);
-        }
     }
     nb_sync<GM>(NB_MAIN);
     for (int r = tid; r < rows; r += GM) {
@@ -380,7 +482,7 @@ SvmGrid svm_grid_plan(int64_t m, int64_t n, int s)
     const size_t smem = grid_layout((int)n, s, R, nls).total;
     if (smem > GRID_SMEM_MAX) return g;
     int ks = 1;
-    while (ks < 8 && 2 * ks * R * s <= GB && 8 * ks <= n) ks *= 2;
+    while (ks < 8 && 2 * ks * R * s <= GY && 8 * ks <= n) ks *= 2;
     g.R = R;
     g.ks = ks;
     g.ctas = (int)((m + R - 1) / R);
@@ -388,7 +490,7 @@ SvmGrid svm_grid_plan(int64_t m, int64_t n, int s)
     return g;
 }
 
-size_t svm_grid_scratch_bytes(int s) { return sizeof(double) * (4 * (size_t)s + 4 * ((size_t)s * s + 2 * s)) + 256; }
+size_t svm_grid_scratch_bytes(int s) { return sizeof(double) * (8 * (size_t)s + 4 * ((size_t)s * s + 2 * s)) + 256; }
 
 cudaError_t launch_svm_grid(const SvmGrid &gp, const double *A, int64_t lda, int64_t m, int64_t n,
                             const KernelParams &kp, const double *h, const double *y, double *alpha, double *g,
@@ -417,9 +519,10 @@ cudaError_t launch_svm_grid(const SvmGrid &gp, const double *A, int64_t lda, int
     a.nu = nu;
     a.bar = (unsigned *)scratch;
     a.xbuf = (double *)((char *)scratch + 256);
-    a.kss = a.xbuf + 4 * (size_t)s;
+    a.kss = a.xbuf + 8 * (size_t)s;
     a.err = err;
     cudaError_t e = cudaMemsetAsync(a.bar, 0, sizeof(unsigned), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.xbuf, 0xff, sizeof(double) * 8 * (size_t)s, st);  // X_OPEN
     if (e != cudaSuccess) return e;
     if (kp.kind == DCD_LINEAR) return launch_form<GK_LINEAR>(a, gp.ctas, gp.smem, st);
     if (kp.kind == DCD_POLY) return launch_form<GK_POLY>(a, gp.ctas, gp.smem, st);
