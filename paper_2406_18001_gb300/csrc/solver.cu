@@ -1220,8 +1220,8 @@ struct Solver {
     // for 5-7 us, within a graph a body follows in about one, so the longest graph that fits the steps to
     // run is taken -- but one body where the stream is idle, as its kernels are submitted soonest and the
     // long graph's while it runs (K-SVM FP64 at m = 2000, s = 8: 18.2 -> 15.0 us a step; K-RR fp16 at
-    // m = 50000, s = 64: 8 steps 583 -> 547, and 636 with the long graph first).  A graph is captured once
-    // every set has run a body directly (attributes and occupancy queries are then cached) and, the long
+    // m = 50000, s = 64, 8 steps from an idle stream: 636 us with the long graph first, 547 with one body
+    // before it).  A graph is captured once every set has run a body directly (attributes and occupancy queries are then cached) and, the long
     // ones, once the plan's steps so far and at hand pay for the capture (about 25 us a body against 5 us
     // a step saved).
     static constexpr int GRAPH_LENS = 4;
