@@ -30,7 +30,7 @@
 //
 // Measured (FP64, hinge): m = 2000, n = 64, s = 8: 15.3 us a step as long graphs, 5.8 with a grid
 // barrier a step, 4.7 now (the FP64 pipe of the own rows' values 3.4 of it); m = 300, n = 16, s = 1 on
-// the default stream: 27, 4.1, 3.3 (1 of it host work).
+// the default stream: 27, 4.5, 3.6 (1 of it host work).
 #include "dcd_chain.cuh"
 #include "dcd_internal.cuh"
 #include "f64_math.cuh"

@@ -76,7 +76,7 @@ __device__ __noinline__ void mbar_drain(uint64_t *bar, uint32_t parity)
 // addresses), one elected lane issuing the copies and MMAs; a wait's common case is one inlined
 // test, the descriptors step by addition.  Issued by a single lane of a diverged warp, a k-block
 // took some 780 cycles beside the epilogue warps against the 512 its MMAs need (fp16 and FP8
-// alike); now 300-480.  FP8 apply at m = 400000, n = 2048, 4096 columns: 2212 -> 1780 us.
+// alike); now 300-480.  FP8 apply at m = 400000, n = 2048, 4096 columns: 2217 -> 1771 us.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort_flag, int *err)
 {
     if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
