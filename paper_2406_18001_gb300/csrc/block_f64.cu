@@ -10,8 +10,16 @@
 // g = p + q.  Every sum is an exact integer: at most (g + 1) n 2^12 <= 2^24 for n <= 512.  The
 // epilogue joins the eight in integer arithmetic and FP64, so that
 //     a_i.a_j = 2^(e_i + e_j - 61) (I_hi 2^28 + I_lo),  I_hi, I_lo exact 64-bit integers,
-// is rounded once; what is left out (p + q >= 8, the ninth slice) is below the rounding of an
-// FP64 sum of n products.  The RBF exponent comes from the expansion gamma |a_i|^2 + gamma |a_j|^2
+// is rounded once.  What is left out (p + q >= 8, the ninth slice) is at most 9 2^-56 2^(e_i + e_j) a
+// feature that is nonzero in both rows, about a tenth of that on average and of either sign: relative to
+// the rows' largest magnitudes, not to sum_k |a_ik a_jk| as the rounding of an FP64 sum is.  The two are
+// alike while the features that make up a product are not all tiny beside others; where a large feature
+// of one row meets a zero of the other they are not (features of 1 beside one of 1e9: 1e-7 relative).  So
+// the linear and polynomial kernels take the form only if every row of the matrix has its magnitude
+// spread over its features, or if the four last slices are zero in all of them (whole numbers up to
+// 2^27, bits: nothing is left out); see f64s_row_flags.  Where the first holds, sum_k |a_ik a_jk| >= n
+// 2^-11 2^(e_i + e_j) for every two rows, and the part left out stays below 2^-45 / sqrt(n) of it (n
+// roundings of like size, of either sign).  The RBF exponent comes from the expansion gamma |a_i|^2 + gamma |a_j|^2
 // - 2 gamma a_i.a_j with norms from compensated FP64 sums: its absolute error is some 2^-53
 // gamma (|a_i|^2 + |a_j|^2), so the form is used where gamma |a|^2 <= F64S_HMAX for every row
 // (pack_f64s reports the largest) and the direct differences serve elsewhere.
@@ -348,11 +356,31 @@ __global__ void __launch_bounds__(F64S_THREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
 }
 
+// What one value v != 0 of a row with max |a| in [2^(e-1), 2^e) adds to the row's rule: min(|v| 2^-e, 2^-4)
+// in units of 2^-25 (x = v 2^(55-e) rounded), and whether v is no multiple of 2^(e-27) (its last four
+// slices are not all zero).
+// A row's magnitude is spread over its features if the mean of min(|a_k| 2^-e, 2^-4) is at least 9/16 of
+// 2^-4.  With t the truncated values of one such row and u those of another, sum t u >= 2^-4 (sum t + sum
+// u) - n 2^-8 >= n 2^-11.  Normal, uniform and +-1 features pass from some 16 features on (a normal row's
+// mean is 0.9 of 2^-4, 0.8 where its largest value is beyond 4 sigma; 9/16 is 7 and 4 deviations below
+// at n = 30).
+__device__ __forceinline__ void f64s_row_flags(double v, long long x, int e, long long &mid, bool &lng)
+{
+    const long long ax = x < 0 ? -x : x;
+    mid += (ax < (1LL << 51) ? ax : 1LL << 51) >> 30;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int be = (int)(b >> 52) & 2047;
+    const unsigned long long mant = (b & 0xfffffffffffffULL) | (be ? 1ULL << 52 : 0ULL);
+    if (mant) lng |= (be ? be : 1) - 1075 + __ffsll((long long)mant) - 1 < e - 27;
+}
+
 // The eight slices of each row of a dense FP64 matrix (a warp per row, two features per lane), its
 // exponent and gamma times its squared norm (compensated sum: TwoProd and TwoSum).  The scaled
 // value is rounded once to a 56-bit integer whose signed base-128 digits are the slices.
-// stat[0]: set when a value is not finite or an exponent leaves [-400, 400]; stat[1]: the largest
-// gamma |a|^2 (bit pattern of a non-negative double).  dst (and ex) null: norms only.
+// stat[0]: F64S_BAD when a value is not finite or an exponent leaves [-400, 400], F64S_UNEVEN when a row's
+// magnitude is not spread over its features, F64S_LONG when a row has a value in its last four slices (a
+// row of zeros sets neither); stat[1]: the largest gamma |a|^2 (bit pattern of a non-negative double).
+// dst (and ex) null: norms only.
 __global__ void pack_f64s_kernel(const double *__restrict__ A, int64_t lda, int64_t m, int64_t n, double gamma,
                                  __nv_bfloat162 *dst, int64_t n_pad, int32_t *ex, double *h, unsigned long long *stat)
 {
@@ -386,14 +414,19 @@ __global__ void pack_f64s_kernel(const double *__restrict__ A, int64_t lda, int6
     if (lane == 0) {
         if (ex) ex[r] = e;
         h[r] = nrm;
-        if (bad) atomicMax(stat, 1ull);
+        if (bad) atomicOr(stat, F64S_BAD);
         else atomicMax(stat + 1, (unsigned long long)__double_as_longlong(fabs(nrm)));
     }
     if (bad || !dst) return;
     const double sc = __hiloint2double((1023 + 55 - e) << 20, 0);  // 2^(55 - e)
     __nv_bfloat162 *d = dst + r * (NSL / 2) * n_pad;
+    long long mid = 0;
+    bool lng = false;
     for (int64_t k = 2 * lane; k < n_pad; k += 64) {
-        long long x0 = k < n ? __double2ll_rn(ar[k] * sc) : 0, x1 = k + 1 < n ? __double2ll_rn(ar[k + 1] * sc) : 0;
+        const double v0 = k < n ? ar[k] : 0.0, v1 = k + 1 < n ? ar[k + 1] : 0.0;
+        long long x0 = __double2ll_rn(v0 * sc), x1 = __double2ll_rn(v1 * sc);
+        f64s_row_flags(v0, x0, e, mid, lng);
+        f64s_row_flags(v1, x1, e, mid, lng);
 #pragma unroll
         for (int p = NSL - 1; p >= 1; --p) {
             const int d0 = (int)((x0 + 64) & 127) - 64, d1 = (int)((x1 + 64) & 127) - 64;
@@ -402,6 +435,12 @@ __global__ void pack_f64s_kernel(const double *__restrict__ A, int64_t lda, int6
             d[(p * n_pad + k) >> 1] = __floats2bfloat162_rn((float)d0, (float)d1);
         }
         d[k >> 1] = __floats2bfloat162_rn((float)(int)x0, (float)(int)x1);
+    }
+    for (int o = 16; o > 0; o >>= 1) mid += __shfl_xor_sync(0xffffffffu, mid, o);
+    lng = __any_sync(0xffffffffu, lng);
+    if (lane == 0 && mx > 0.0) {
+        const unsigned long long f = (mid < n * (9LL << 17) ? F64S_UNEVEN : 0) | (lng ? F64S_LONG : 0);
+        if ((*(volatile unsigned long long *)stat & f) != f) atomicOr(stat, f);  // the first few rows only
     }
 }
 

@@ -830,8 +830,9 @@ struct Solver {
     }
 
     // The FP64 form's block through exact slices (block_f64.cu) where it is the faster one and as
-    // exact: n within the exact sums, every value finite with a moderate exponent, and for the RBF
-    // gamma |a|^2 <= F64S_HMAX (the expansion's error).  The line is on the products m sb n of the
+    // exact: n within the exact sums, every value finite with a moderate exponent, for the RBF
+    // gamma |a|^2 <= F64S_HMAX (the expansion's error), and for the other kernels rows whose magnitude is
+    // spread over their features, or short values (what the form leaves out, block_f64.cu).  The line is on the products m sb n of the
     // block, by measured time of sample + Gram + block a step (direct / slices, us): blocks of at
     // most 32 columns, whose direct form is spread over every SM, 2000 x 64 x 16 (2.0 M) 36 / 56,
     // 6000 x 64 x 8 (3.1 M) 39 / 44, 2000 x 200 x 8 (3.2 M) 58 / 53, 6000 x 200 x 8 (9.6 M)
@@ -877,7 +878,9 @@ struct Solver {
             DCD_TRY(cudaStreamSynchronize(st));
             double hmax;
             memcpy(&hmax, &hs[1], sizeof(hmax));
-            if (hs[0] || !(hmax <= F64S_HMAX)) {
+            // linear, polynomial: a dot product that is small beside the rows' largest magnitudes counts
+            const bool uneven = kp.kind != DCD_RBF && (hs[0] & F64S_UNEVEN) && (hs[0] & F64S_LONG);
+            if ((hs[0] & F64S_BAD) || uneven || !(hmax <= F64S_HMAX)) {
                 DCD_TRY(cudaFreeAsync(ws_f64s, st));
                 ws_f64s = nullptr;
                 return DCD_OK;
