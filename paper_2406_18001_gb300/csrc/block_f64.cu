@@ -22,7 +22,11 @@
 // roundings of like size, of either sign).  The RBF exponent comes from the expansion gamma |a_i|^2 + gamma |a_j|^2
 // - 2 gamma a_i.a_j with norms from compensated FP64 sums: its absolute error is some 2^-53
 // gamma (|a_i|^2 + |a_j|^2), so the form is used where gamma |a|^2 <= F64S_HMAX for every row
-// (pack_f64s reports the largest) and the direct differences serve elsewhere.
+// (pack_f64s reports the largest) and the direct differences serve elsewhere.  What the slices leave out
+// of 2 gamma a_i.a_j, about 2 gamma sqrt(n) 2^-56 2^(e_i + e_j), is less than that for rows whose
+// magnitude is spread over their features; where one feature holds it and n is large it is more (one
+// feature of 2.05, 511 of 1e-3, gamma |a|^2 = 7.9: 4.3e-14 in a kernel value), so gamma 4^e sqrt(n) / 2
+// has the same limit: at most four times 2^-53 is left out.
 //
 // What bounds it: the FP64 pipe, with 16 operations an entry instead of 2 n: two integer-to-double
 // differences, a sum of the terms and two FMAs for the exponent, ten for exp, one for the
@@ -379,8 +383,8 @@ __device__ __forceinline__ void f64s_row_flags(double v, long long x, int e, lon
 // value is rounded once to a 56-bit integer whose signed base-128 digits are the slices.
 // stat[0]: F64S_BAD when a value is not finite or an exponent leaves [-400, 400], F64S_UNEVEN when a row's
 // magnitude is not spread over its features, F64S_LONG when a row has a value in its last four slices (a
-// row of zeros sets neither); stat[1]: the largest gamma |a|^2 (bit pattern of a non-negative double).
-// dst (and ex) null: norms only.
+// row of zeros sets neither); stat[1]: the largest gamma |a|^2 and, with the slices, gamma 4^e sqrt(n) / 2
+// (bit pattern of a non-negative double).  dst (and ex) null: norms only.
 __global__ void pack_f64s_kernel(const double *__restrict__ A, int64_t lda, int64_t m, int64_t n, double gamma,
                                  __nv_bfloat162 *dst, int64_t n_pad, int32_t *ex, double *h, unsigned long long *stat)
 {
@@ -415,7 +419,10 @@ __global__ void pack_f64s_kernel(const double *__restrict__ A, int64_t lda, int6
         if (ex) ex[r] = e;
         h[r] = nrm;
         if (bad) atomicOr(stat, F64S_BAD);
-        else atomicMax(stat + 1, (unsigned long long)__double_as_longlong(fabs(nrm)));
+        else {
+            const double cut = dst && mx > 0.0 ? ldexp(0.5 * gamma * sqrt((double)n), 2 * e) : 0.0;
+            atomicMax(stat + 1, (unsigned long long)__double_as_longlong(fmax(fabs(nrm), cut)));
+        }
     }
     if (bad || !dst) return;
     const double sc = __hiloint2double((1023 + 55 - e) << 20, 0);  // 2^(55 - e)

@@ -116,8 +116,9 @@ struct F64Sliced {
 int64_t f64s_row_bytes(int64_t n);
 size_t f64s_part_bytes(int64_t m, int64_t ncols);
 int64_t f64s_tiles(int64_t m);
-// stat: two words (zeroed here): F64S_* flags, and the largest gamma |a|^2.  packed and ex null: the
-// norms alone.
+// stat: two words (zeroed here): F64S_* flags, and what F64S_HMAX limits: the largest gamma |a|^2, and with
+// the slices gamma 4^e sqrt(n) / 2 (2^e: the power of two above the row's largest magnitude).  packed and
+// ex null: the norms alone.
 constexpr unsigned long long F64S_BAD = 1;     // a value rules the form out
 constexpr unsigned long long F64S_UNEVEN = 2;  // a row's magnitude is not spread over its features
 constexpr unsigned long long F64S_LONG = 4;    // a row's last four slices are not all zero

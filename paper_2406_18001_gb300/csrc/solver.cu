@@ -831,7 +831,7 @@ struct Solver {
 
     // The FP64 form's block through exact slices (block_f64.cu) where it is the faster one and as
     // exact: n within the exact sums, every value finite with a moderate exponent, for the RBF
-    // gamma |a|^2 <= F64S_HMAX (the expansion's error), and for the other kernels rows whose magnitude is
+    // gamma |a|^2 and gamma 4^e sqrt(n) / 2 <= F64S_HMAX (the expansion's and the slices' errors), and for the other kernels rows whose magnitude is
     // spread over their features, or short values (what the form leaves out, block_f64.cu).  The line is on the products m sb n of the
     // block, by measured time of sample + Gram + block a step (direct / slices, us): blocks of at
     // most 32 columns, whose direct form is spread over every SM, 2000 x 64 x 16 (2.0 M) 36 / 56,
