@@ -58,7 +58,7 @@ constexpr int NSL = 8;             // slices
 constexpr int A_SLICE = FM * 128;  // a k-block (64 features) of one row slice: 16 KB
 constexpr int B_SLICE = FN * 128;  // of one column slice: 4 KB
 constexpr int B_STK = NSL * B_SLICE;
-constexpr int COL_WORDS = 16 * 5;  // staged column terms of an epilogue warp: w, h (FP64), exponent
+constexpr int COL_WORDS = 16 * 6;  // staged column terms of an epilogue warp: w, h (FP64), exponent, data row
 constexpr int F64S_SMEM = 1024 + NSL * A_SLICE + 2 * B_STK + 256 + 64 * 8 + 8 * 2 * COL_WORDS * 4;
 constexpr int F64S_THREADS = 320;
 constexpr int F64S_COLS = 1024;    // columns per launch (bounds the scratch of the row sums)
@@ -244,13 +244,16 @@ __global__ void __launch_bounds__(F64S_THREADS, 1)
         double *ct = colterms + (warp - 2) * COL_WORDS;  // two buffers of COL_WORDS / 2 doubles
         // the unit's column and row terms, loaded one unit ahead
         double n_w = 0.0, n_h = 0.0, r_h = 0.0;
-        int n_e = 0, r_e = 0;
+        int n_e = 0, r_e = 0, n_id = -1, r_id = -2;  // no column and no row are no sample's own pair
         auto load_terms = [&](int u) {
             const int64_t c = (int64_t)(u % a.nchunks) * FN + half * 16 + (lane & 15);
             n_w = n_h = r_h = 0.0;
             n_e = r_e = 0;
+            n_id = -1;
+            r_id = -2;
             if (c < a.ncols) {
                 const int64_t id = a.col_id ? a.col_id[c] : c;
+                n_id = (int)id;
                 if (id >= 0 && id < a.m) {
                     n_e = a.ex[id];
                     if (KIND == DCD_RBF) n_h = a.h[id];
@@ -260,6 +263,7 @@ __global__ void __launch_bounds__(F64S_THREADS, 1)
             const int64_t r = (int64_t)(u / a.nchunks) * FM + quarter * 32 + lane;
             if (r < a.nrows) {
                 const int64_t id = a.row_id ? a.row_id[r] : r;
+                r_id = (int)id;
                 if (id >= 0 && id < a.m) {
                     r_e = a.ex[id];
                     if (KIND == DCD_RBF) r_h = a.h[id];
@@ -276,9 +280,10 @@ __global__ void __launch_bounds__(F64S_THREADS, 1)
                 cb[lane] = n_w;
                 cb[16 + lane] = n_h;
                 ((int *)(cb + 32))[lane] = n_e;
+                ((int *)(cb + 40))[lane] = n_id;
             }
             const double hr = r_h;
-            const int er = r_e - 61;
+            const int er = r_e - 61, rid = r_id;
             if (u + (int)gridDim.x < nunits) load_terms(u + gridDim.x);
             __syncwarp();
             if (!mbar_wait_warp(&tfull[buf], aph, abort_flag, a.err)) break;
@@ -309,7 +314,8 @@ __global__ void __launch_bounds__(F64S_THREADS, 1)
                     double kv;
                     if (KIND == DCD_RBF) {
                         double x = fma(rf, ds, -(hr + cb[16 + j]));
-                        x = __double2hiint(x) < 0 ? x : 0.0;  // -gamma d^2 <= 0
+                        // -gamma d^2 <= 0, and 0 of a row against itself
+                        x = __double2hiint(x) < 0 && ((const int *)(cb + 40))[j] != rid ? x : 0.0;
                         kv = exp_tab(x, tab);
                     } else {
                         const double dot = scale2(ds, er);
