@@ -95,6 +95,7 @@ __device__ __forceinline__ void tmem_wait8(uint32_t (&r)[8])
 }
 
 // v 2^k for a normal or zero v whose result is normal (an integer add to the exponent field)
+// (|k| <= 461 here: a value of 2^-500 or more stays normal)
 __device__ __forceinline__ double scale2(double v, int k)
 {
     const int hi = __double2hiint(v);

@@ -839,9 +839,12 @@ struct Solver {
     // 74 / 52, 6000 x 512 x 32 511 / 93: from 6 M; wider ones, in tiles of 64 rows, 2000 x 64 x 64
     // (8.2 M) 351 / 71, 6000 x 512 x 256 9510 / 148: from 1 M.  No memory for the slices (16 bytes
     // a value): the direct form.
+    // (An RBF gamma below 2^-500 leaves the range in which the slices' epilogue scales by exponent arithmetic:
+    // the direct form.)
     bool f64s_worth() const
     {
         const double work = (double)m * (double)sb * (double)n;
+        if (kp.kind == DCD_RBF && !(kp.gamma >= 0x1p-500)) return false;
         return n <= F64S_N_MAX && work >= (sb > 32 ? 1e6 : 6e6) && tc_available();
     }
 
