@@ -432,11 +432,12 @@ cudaError_t launch_csr_block(const CsrOperand &A, const CsrColMap &M, bool fp64,
 struct DcdPending {
     const double *alpha_snap = nullptr, *alpha_add = nullptr, *g_snap = nullptr, *g_add = nullptr;
 };
-// (pend: the chain reads alpha and g from it; only for cnt <= 128, else cudaErrorInvalidValue)
+// (pend: the chain reads alpha and g from it; only for cnt <= 128, else cudaErrorInvalidValue.
+// weights: y may hold any numbers; else +-1)
 cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const int32_t *S, int64_t cnt,
                              const double *y, const double *alpha, const double *g, double omega, double nu,
                              double *delta, double *w64, float *w32, int *err, cudaStream_t st,
-                             const DcdPending *pend = nullptr);
+                             const DcdPending *pend = nullptr, bool weights = false);
 size_t recur_bdcd_scratch_bytes(int64_t nblk, int b);
 // true when launch_recur_bdcd with these arguments reads only the lower
 // triangle (with the diagonal blocks) of an FP32 Gram

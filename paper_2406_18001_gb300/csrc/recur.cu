@@ -950,9 +950,11 @@ cudaError_t refined_bdcd_b(const KT *Kss, int64_t ldk, const int32_t *S, int nbl
 // and rho - g / eta anew, with steps published by release / acquire, 780, now 300.  Measured, every step
 // nonzero, FP64: 32 coordinates 14.7 -> 8.2 us, 64 28.9 -> 15.5, 128 61.7 -> 33, of which 3.5 are the
 // launch, the first loads and 1 / eta.
+// Labels (+-1) enter by their sign bits.  WEIGHTS: any y, which only the entry point of the recurrence
+// takes; other weights enter by two FP64 products a coupling.
 // pend (optional): alpha and g at the step's coordinates are pend[0][t] + pend[1][t] and
 // pend[2][t] + pend[3][t] (a snapshot and the parts not yet in it) instead of alpha[S[t]], g[S[t]]
-template <typename KT>
+template <typename KT, bool WEIGHTS>
 __global__ void __launch_bounds__(FAST_THREADS) recur_dcd_fast_kernel(const KT *Kss, int64_t ldk, const int32_t *S,
                                                                      int cnt, const double *y, const double *alpha,
                                                                      const double *g, double omega, double nu,
@@ -963,7 +965,8 @@ __global__ void __launch_bounds__(FAST_THREADS) recur_dcd_fast_kernel(const KT *
     const int ldc = cnt | 1;                            // odd: no bank conflicts down a column
     double *C = fsm;                                    // C[j * ldc + t]
     double *slot = C + (size_t)cnt * ldc;               // the steps, as they are decided
-    int32_t *sI = (int32_t *)(slot + cnt);
+    double *yS = slot + cnt;
+    int32_t *sI = (int32_t *)(yS + cnt);
     uint32_t *sy = (uint32_t *)(sI + cnt);              // sign bit of y
     uint32_t *rep = sy + cnt;                           // rep[j * 4 + q]: later t = 32 q + bit with S_t = S_j
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -982,13 +985,15 @@ __global__ void __launch_bounds__(FAST_THREADS) recur_dcd_fast_kernel(const KT *
         }
     };
     load(v, warp);
-    double a0 = 0.0, a1 = 0.0, g0 = 0.0, g1 = 0.0, eta = 0.0, ie = 0.0;
+    double a0 = 0.0, a1 = 0.0, g0 = 0.0, g1 = 0.0, eta = 0.0, ie = 0.0, yt = 1.0;
     if (mine) {
         const int32_t i = S[t];
         eta = kval(Kss, ldk, t, t);
         sI[t] = i;
         slot[t] = __longlong_as_double(CHAIN_OPEN);
-        sy[t] = (uint32_t)__double2hiint(y[i]) & 0x80000000u;
+        yt = y[i];
+        sy[t] = (uint32_t)__double2hiint(yt) & 0x80000000u;
+        if (WEIGHTS) yS[t] = yt;
         if (pend.alpha_snap) {
             a0 = pend.alpha_snap[t];
             a1 = pend.alpha_add[t];
@@ -999,7 +1004,9 @@ __global__ void __launch_bounds__(FAST_THREADS) recur_dcd_fast_kernel(const KT *
             g0 = g[i];
         }
     }
-    __syncthreads();
+    bool labels = true;
+    if (WEIGHTS) labels = __syncthreads_and((__double_as_longlong(yt) & 0x7fffffffffffffffLL) == 0x3ff0000000000000LL);
+    else __syncthreads();
     for (int p0 = warp; p0 < np; p0 += U * (FAST_THREADS / 32)) {
         double w[U];
         load(w, p0 + U * (FAST_THREADS / 32));
@@ -1010,7 +1017,9 @@ __global__ void __launch_bounds__(FAST_THREADS) recur_dcd_fast_kernel(const KT *
             const bool in = j < cnt;
             const bool same = in && sI[in ? j : 0] == sI[r];
             if (in && 32 * q <= r) {
-                double c = __hiloint2double((int)((uint32_t)__double2hiint(v[u]) ^ sy[r] ^ sy[j]), __double2loint(v[u]));
+                double c = labels ? __hiloint2double((int)((uint32_t)__double2hiint(v[u]) ^ sy[r] ^ sy[j]),
+                                                     __double2loint(v[u]))
+                                  : yS[r] * yS[j] * v[u];
                 if (same) c += omega;
                 C[j * ldc + r] = c;
             }
@@ -1034,8 +1043,8 @@ __global__ void __launch_bounds__(FAST_THREADS) recur_dcd_fast_kernel(const KT *
     const double th = dcd_chain_group(C, ldc, rep, slot, cnt, warp, lane, rho, gj, eta, ie, nu, err);
     if (mine) {
         delta[t] = th;
-        // y_t th
-        const double wv = __hiloint2double((int)((uint32_t)__double2hiint(th) ^ sy[t]), __double2loint(th));
+        const double wv = labels ? __hiloint2double((int)((uint32_t)__double2hiint(th) ^ sy[t]), __double2loint(th))
+                                 : yt * th;
         if (w64) w64[t] = wv;
         if (w32) w32[t] = (float)wv;
     }
@@ -1044,34 +1053,31 @@ __global__ void __launch_bounds__(FAST_THREADS) recur_dcd_fast_kernel(const KT *
 cudaError_t launch_recur_dcd(const void *Kss, int kss_f64, int64_t ldk, const int32_t *S, int64_t cnt,
                              const double *y, const double *alpha, const double *g, double omega, double nu,
                              double *delta, double *w64, float *w32, int *err, cudaStream_t st,
-                             const DcdPending *pend)
+                             const DcdPending *pend, bool weights)
 {
     if (cnt <= 0) return cudaSuccess;
     const DcdPending pd = pend ? *pend : DcdPending{};
     if (pend && cnt > DCD_FAST_MAX) return cudaErrorInvalidValue;
     if (cnt <= DCD_FAST_MAX) {
-        const size_t fsm = sizeof(double) * (size_t)(cnt * (cnt | 1) + cnt) + sizeof(int32_t) * (2 + DCD_FAST_K) * cnt;
-        static bool fattr[2] = {false, false};
-        if (kss_f64) {
-            if (!fattr[1]) {
-                cudaError_t e = cudaFuncSetAttribute(recur_dcd_fast_kernel<double>,
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DCD_SMEM_LIMIT);
+        auto run = [&](auto kfn, auto K, bool &attr) -> cudaError_t {
+            if (!attr) {
+                const cudaError_t e =
+                    cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DCD_SMEM_LIMIT);
                 if (e != cudaSuccess) return e;
-                fattr[1] = true;
+                attr = true;
             }
-            recur_dcd_fast_kernel<double><<<1, FAST_THREADS, fsm, st>>>((const double *)Kss, ldk, S, (int)cnt, y, alpha,
-                                                                       g, omega, nu, delta, w64, w32, pd, err);
-        } else {
-            if (!fattr[0]) {
-                cudaError_t e = cudaFuncSetAttribute(recur_dcd_fast_kernel<float>,
-                                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DCD_SMEM_LIMIT);
-                if (e != cudaSuccess) return e;
-                fattr[0] = true;
-            }
-            recur_dcd_fast_kernel<float><<<1, FAST_THREADS, fsm, st>>>((const float *)Kss, ldk, S, (int)cnt, y, alpha,
-                                                                      g, omega, nu, delta, w64, w32, pd, err);
-        }
-        return cudaGetLastError();
+            const size_t fsm =
+                sizeof(double) * (size_t)(cnt * (cnt | 1) + 2 * cnt) + sizeof(int32_t) * (2 + DCD_FAST_K) * cnt;
+            kfn<<<1, FAST_THREADS, fsm, st>>>(K, ldk, S, (int)cnt, y, alpha, g, omega, nu, delta, w64, w32, pd, err);
+            return cudaGetLastError();
+        };
+        static bool fattr[4] = {false, false, false, false};
+        bool &fa = fattr[2 * (kss_f64 != 0) + weights];
+        if (kss_f64)
+            return run(weights ? recur_dcd_fast_kernel<double, true> : recur_dcd_fast_kernel<double, false>,
+                       (const double *)Kss, fa);
+        return run(weights ? recur_dcd_fast_kernel<float, true> : recur_dcd_fast_kernel<float, false>,
+                   (const float *)Kss, fa);
     }
     size_t sm = sizeof(double) * 7 * cnt + sizeof(int32_t) * ((cnt + 1) & ~1);
     if (cnt <= DCD_SMEM_GRAM_MAX) sm += sizeof(double) * cnt * cnt;

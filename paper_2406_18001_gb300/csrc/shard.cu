@@ -288,6 +288,7 @@ extern "C" dcd_status dcd_dcd_recurrence(const void *Kss, int32_t kss_f64, int64
     first_pos_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(S, cnt, Sc);
     SH_TRY(cudaGetLastError());
     const double omega = loss == 2 ? 1.0 / (2.0 * C) : 0.0, nu = loss == 2 ? INFINITY : C;
-    SH_TRY(launch_recur_dcd(Kss, kss_f64, ldk, Sc, cnt, y_S, alpha_S, g_S, omega, nu, theta, w, nullptr, err, st));
+    SH_TRY(launch_recur_dcd(Kss, kss_f64, ldk, Sc, cnt, y_S, alpha_S, g_S, omega, nu, theta, w, nullptr, err, st, nullptr,
+                            true));
     return finish(err, st);
 }
