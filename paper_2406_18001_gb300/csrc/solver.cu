@@ -1878,9 +1878,18 @@ struct Solver {
             if (grid.ctas && cnt == o.s) {
                 // a launch of a few tens of milliseconds at most
                 *ran = std::min<int64_t>({avail, (o.max_iters - done) / o.s, (int64_t)4096});
-                stats.gpu_launches_per_step = 1;
-                r = cuda_status(launch_svm_grid(grid, op.a64, op.lda, m, n, kp, grid_h, y, alpha, g, o.seed, ctr,
-                                                (int)*ran, (int)o.s, omega, nu, grid_ws, err, st));
+                const cudaError_t e = launch_svm_grid(grid, op.a64, op.lda, m, n, kp, grid_h, y, alpha, g, o.seed, ctr,
+                                                      (int)*ran, (int)o.s, omega, nu, grid_ws, err, st);
+                if (e == cudaErrorCooperativeLaunchTooLarge) {
+                    // the stream has part of the SMs only (a green context): steps of separate kernels
+                    cudaGetLastError();
+                    grid.ctas = 0;
+                    *ran = 1;
+                    taken = false;
+                } else {
+                    r = cuda_status(e);
+                    stats.gpu_launches_per_step = 1;
+                }
             } else if (dfs && cnt == o.s) r = dfs_step(cnt, avail, ran);
             else if (lag) r = lag_step(cnt, avail, ran);
             else if (df && cnt == o.s) r = df_step(cnt, avail, ran);
