@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(CSR_AW * 32, 3)
 //            with their prefix sums, then the CTA's threads sweep the group's
 //            incidences as one flat range (CSC_U independent loads and
 //            atomics per thread in flight) and append key = (e << 10) | (i mod
-//            32) << 5 | j and the product a_ie * a_{S_j},c to the bucket of
+//            32) << 5 | j (e counted from the tile's first nonzero) and the product a_ie * a_{S_j},c to the bucket of
 //            the incidence's 32-row tile (a fixed capacity per tile; a counter
 //            per tile, in arbitrary order);
 //   apply    a warp per tile (the next tile's bucket loaded while this one
@@ -381,10 +381,11 @@ __global__ void __launch_bounds__(CSR_AW * 32, 3)
 //            the warp ranks every key of the tile jointly -- so the products
 //            for each j come in element order, the order of the full pass,
 //            and forms the row's sum exactly as the full pass does.  A tile
-//            whose bucket overflowed runs the full pass over its rows.
+//            whose bucket overflowed, or that met an element 2^22 or more into
+//            it (rows of more than 131072 nonzeros), runs the full pass over its
+//            rows.
 // The result is bit-identical to the full pass.
 constexpr int CSC_TILE_CAP = 128;  // incidences per 32-row tile (bucket size, sorted in shared memory)
-constexpr int CSC_G = 4;           // sampled-row nonzeros per scatter CTA
 constexpr int CSC_U = 4;           // incidences per scatter thread in flight
 constexpr int CSC_SCATTER_THREADS = 256;
 
@@ -469,8 +470,13 @@ __global__ void __launch_bounds__(CSC_SCATTER_THREADS)
             cv[u] = k[u] >= 0 ? cval[k[u]] : (T)0;
         }
 #pragma unroll
-        for (int u = 0; u < CSC_U; ++u) 
-            pos[u] = row[u] >= 0 ? atomicAdd(W.tile_cnt + (int64_t)(row[u] >> 5) * CSC_CNT_STRIDE, 1) : CSC_TILE_CAP;
+        for (int u = 0; u < CSC_U; ++u) {
+            pos[u] = CSC_TILE_CAP;
+            if (row[u] < 0) continue;
+            int32_t *cnt = W.tile_cnt + (int64_t)(row[u] >> 5) * CSC_CNT_STRIDE;
+            if (el[u] != CSC_FAR) pos[u] = atomicAdd(cnt, 1);
+            else atomicOr(cnt, 1 << 30);  // as an overflow (fewer than 2^30 incidences are counted beside it)
+        }
 #pragma unroll
         for (int u = 0; u < CSC_U; ++u)
             if (pos[u] < CSC_TILE_CAP) {
@@ -1135,7 +1141,7 @@ __global__ void csc_fill_kernel(CsrOperand A, const int64_t *col_ptr, int32_t *c
         const int32_t c = A.col_idx[e];
         const int64_t pos = col_ptr[c] + atomicAdd(cur + c, 1);
         row[pos] = (int32_t)r;
-        elem[pos] = (uint32_t)(e - t0);
+        elem[pos] = (uint32_t)min(e - t0, (int64_t)CSC_FAR);
         val[pos] = vals[e];
     }
 }

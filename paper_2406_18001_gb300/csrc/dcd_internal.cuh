@@ -384,13 +384,15 @@ cudaError_t launch_csr_colmap(const CsrOperand &A, const int32_t *S, int64_t cnt
 // Transposed copy of a CSR operand: per column its entries' rows, CSR element
 // indices and values (in the block's precision); and the per-step scratch of
 // the apply through it: per 32-row tile a counter (zero between uses) and a
-// bucket of incidence keys and products.  (No row longer than CSC_ROW_MAX: the offsets of a tile fit
-// the keys.)
-constexpr int CSC_ROW_MAX = (1 << 22) / 32 - 1;
+// bucket of incidence keys and products.  An element too far into its tile
+// for a key (CSC_FAR) sends the tile to the full pass.
+constexpr int CSC_G = 4;                      // sampled-row nonzeros per scatter CTA
+constexpr int CSC_ROW_MAX = 65535 * CSC_G;    // longest row: the scatter's grid
+constexpr uint32_t CSC_FAR = 1u << 22;
 struct CscOperand {
     const int64_t *col_ptr = nullptr;
     const int32_t *row = nullptr;
-    const uint32_t *elem = nullptr;  // offset from the first nonzero of the row's 32-row tile, < 2^22
+    const uint32_t *elem = nullptr;  // offset from the first nonzero of the row's 32-row tile, or CSC_FAR
     const void *val = nullptr;
     int64_t n = 0;
 };
