@@ -16,7 +16,7 @@
  *    out) are recorded in a device error word and turned into a status.
  *  - The library allocates its scratch memory on `stream`, from a
  *    stream-ordered memory pool of its own, and frees it before returning.
- *    The pool keeps at most 512 MB of freed memory per device for later
+ *    The pool keeps at most 512 MB of freed memory per CUDA context for later
  *    calls.
  *  - All indices are 0-based.  Dense matrices are row-major with leading
  *    dimension ld >= n (elements).  CSR uses int64 row_ptr[m+1] and int32

@@ -14,6 +14,8 @@
 #include "dcd_internal.cuh"
 #include "ptx.cuh"
 
+#include <cuda.h>
+
 #include <atomic>
 #include <mutex>
 
@@ -22,37 +24,66 @@ namespace {
 
 std::atomic<int> g_fail_allocs{0};
 
-// The library's own memory pool on the current device (nullptr: none could be made; a stream-ordered
+// The number of the current context (one is made where none is current, or the one that was has been
+// reset), never used twice in a process; 0: it cannot be had.
+unsigned long long context_id(int dev)
+{
+    typedef CUresult(CUDAAPI * GetId)(CUcontext, unsigned long long *);
+    static const GetId get = [] {
+        cudaDriverEntryPointQueryResult q;
+        void *p = nullptr;
+        return cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+                       q == cudaDriverEntryPointSuccess
+                   ? (GetId)p
+                   : nullptr;
+    }();
+    unsigned long long id = 0;
+    if (!get) return 0;
+    if (get(nullptr, &id) == CUDA_SUCCESS) return id;
+    if (cudaSetDevice(dev) != cudaSuccess || get(nullptr, &id) != CUDA_SUCCESS) return 0;
+    return id;
+}
+
+// The library's own memory pool in the current context (nullptr: none could be made; a stream-ordered
 // pool, so safe from several threads and streams).  It keeps at most POOL_KEEP of freed memory mapped:
 // the default pool returns all of it to the driver at every synchronisation, and mapping it again took
 // 50 to 170 us of an allocation after one (a sweep of 32 plans: 19.7 -> 15.9 ms).  What it keeps goes
-// back when an allocation of the library's fails, and with the process.
-constexpr int POOL_DEVICES = 64;
+// back when an allocation of the library's fails, and with the process.  A pool dies with its context
+// (cudaDeviceReset), so pools go by the context's number.
+constexpr size_t POOL_CONTEXTS = 64;
 constexpr uint64_t POOL_KEEP = 512ull << 20;
 
-cudaMemPool_t device_pool()
+cudaMemPool_t context_pool()
 {
+    struct Entry {
+        unsigned long long id;
+        cudaMemPool_t pool;
+    };
     static std::mutex mu;
-    static cudaMemPool_t pools[POOL_DEVICES] = {};
-    static bool made[POOL_DEVICES] = {};
+    static Entry pools[POOL_CONTEXTS];
+    static size_t count = 0;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= POOL_DEVICES) return nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    const unsigned long long id = context_id(dev);
+    if (!id) return nullptr;
     std::lock_guard<std::mutex> lock(mu);
-    if (!made[dev]) {
-        made[dev] = true;
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        uint64_t keep = POOL_KEEP;
-        if (cudaMemPoolCreate(&pools[dev], &props) != cudaSuccess) {
-            cudaGetLastError();
-            pools[dev] = nullptr;
-        } else if (cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-            cudaGetLastError();  // it keeps nothing, as the default pool
-        }
+    for (size_t i = 0; i < count; ++i)
+        if (pools[i].id == id) return pools[i].pool;
+    if (count == POOL_CONTEXTS) return nullptr;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t keep = POOL_KEEP;
+    cudaMemPool_t pool = nullptr;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        cudaGetLastError();
+        pool = nullptr;
+    } else if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();  // it keeps nothing, as the default pool
     }
-    return pools[dev];
+    pools[count++] = {id, pool};
+    return pool;
 }
 
 __global__ void bounded_wait_selftest_kernel(unsigned long long limit_ns, int *err, int *waited)
@@ -78,7 +109,7 @@ cudaError_t malloc_async(void **p, size_t bytes, cudaStream_t st)
             return cudaErrorMemoryAllocation;
         }
     }
-    const cudaMemPool_t pool = device_pool();
+    const cudaMemPool_t pool = context_pool();
     if (!pool) return cudaMallocAsync(p, bytes, st);
     cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
     if (e == cudaErrorMemoryAllocation) {  // what the pool keeps may be in the way
