@@ -168,7 +168,8 @@ typedef struct {
     int64_t iters_done;       /* inner iterations performed */
     int64_t outer_steps;      /* outer s-steps performed */
     int32_t converged;        /* 1 if the tolerance was met */
-    int32_t gpu_launches_per_step; /* kernels one outer step launches */
+    int32_t gpu_launches_per_step; /* kernels one outer step launches; 1 where one kernel runs many (a K-SVM
+                                      problem on the resident grid: those of a call, up to 4096) */
     double final_metric;      /* relative gap (K-SVM) or relative residual (K-RR); NaN after a
                                  dcd_plan_run that neither reached a check point nor the budget end */
     double primal, dual;      /* K-SVM: P and D at the final alpha (from the cached gradient) */

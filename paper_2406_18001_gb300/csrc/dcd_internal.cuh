@@ -135,6 +135,7 @@ cudaError_t launch_block_f64s(const F64Sliced &f, const void *rows, int64_t nrow
 // co-resident grid.  ctas = 0: the shape does not fit.
 struct SvmGrid {
     int ctas = 0, R = 0, ks = 0;  // CTAs, rows each, lanes per kernel value
+    int64_t steps = 0;            // outer steps a launch takes at most
     size_t smem = 0;
 };
 SvmGrid svm_grid_plan(int64_t m, int64_t n, int s);

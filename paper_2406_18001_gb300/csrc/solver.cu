@@ -1876,8 +1876,7 @@ struct Solver {
             dcd_status r = DCD_OK;
             bool taken = true;
             if (grid.ctas && cnt == o.s) {
-                // a launch of a few tens of milliseconds at most
-                *ran = std::min<int64_t>({avail, (o.max_iters - done) / o.s, (int64_t)4096});
+                *ran = std::min<int64_t>({avail, (o.max_iters - done) / o.s, grid.steps});
                 const cudaError_t e = launch_svm_grid(grid, op.a64, op.lda, m, n, kp, grid_h, y, alpha, g, o.seed, ctr,
                                                       (int)*ran, (int)o.s, omega, nu, grid_ws, err, st);
                 if (e == cudaErrorCooperativeLaunchTooLarge) {

@@ -487,6 +487,12 @@ SvmGrid svm_grid_plan(int64_t m, int64_t n, int s)
     g.ks = ks;
     g.ctas = (int)((m + R - 1) / R);
     g.smem = smem;
+    // A launch of some 60 ms at most, so that what is queued behind it gets its turn: a step takes less than
+    // 4 us, 0.4 us a coordinate of the chain, and m s (2 n + 40) FP64 operations (distances from
+    // differences) at the pipe's 0.46 M a us.  m = 3500, n = 600, s = 8: 725 steps a launch, 22 ms, 46 with
+    // distances from differences (4096 took 126 and 262); m = 2000, n = 64, s = 8: 4096 steps, 18 and 26 ms.
+    const double us = 4.0 + 0.4 * s + (double)m * s * (2.0 * (double)n + 40.0) / 0.46e6;
+    g.steps = std::min<int64_t>(std::max<int64_t>((int64_t)(60000.0 / us), 1), 4096);
     return g;
 }
 
