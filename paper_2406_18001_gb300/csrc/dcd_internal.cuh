@@ -500,7 +500,7 @@ cudaError_t launch_recur_bdcd(const void *Kss, int kss_f64, int64_t ldk, const i
                               double *delta, double *w64, float *w32, FusedUpdate *upd, int *err, cudaStream_t st,
                               const double *W64 = nullptr);
 // The FP64 form's block forward substitution (up to 1024 rows, b <= 32): whether launch_recur_bdcd
-// takes it for an FP64 Gram, and the inverses of the diagonal blocks (nblk b x b) it reads, which a
+// takes it for an FP64 Gram, and the inverses of the diagonal blocks (nblk b x b, and nblk marks) it reads, which a
 // caller may form ahead and pass as W64 (else formed in the scratch).
 bool recur_bdcd_forward64(int64_t nblk, int b);
 cudaError_t launch_bdcd_inverse64(const double *Kss, int64_t ldk, int64_t nblk, int b, double lambda, double mdiag,

@@ -630,11 +630,18 @@ __global__ void __launch_bounds__(256) bdcd_residual_kernel(const KT *Kss, int64
 // each waited on the single CTA's chain: sb = 256, b = 16: 215 us of recurrence a step -> 45 us
 // (the inverses, 16 us, beside the block before).  Beyond FWD64_SB rows the square overtakes the
 // refined chain.
+//
+// The product with an inverse has a Cholesky solve's error but not its residual, which grows with
+// cond(G_jj)^2: up to 10 times a Cholesky solve's at a condition number of 1e2 - 1e3, 800 at 1e7, 1e4 at 1e10
+// (random blocks of 2 to 32 rows; near-duplicate rows and a small lambda have such).  So the kernel that
+// forms an inverse marks a block where |G|_inf |W|_inf is above FWD64_COND, and for those the forward kernel
+// adds W (r - G_jj Delta_j), which brings the residual to a Cholesky solve's at every condition number tried.
 constexpr int FWD64_SB = 1024;
 constexpr int INV64_NT = 256;
+constexpr float FWD64_COND = 128.f;
 
 // W_j by Gauss-Jordan on [G_jj | I], only the columns that can change at pivot k touched; the owner of
-// the next pivot forms its reciprocal.  W: nblk blocks of b x b, row-major.
+// the next pivot forms its reciprocal.  W: nblk blocks of b x b, row-major, then a mark per block (0 or 1).
 template <typename KT>
 __global__ void __launch_bounds__(INV64_NT) bdcd_inverse64_kernel(const KT *Kss, int64_t ldk, int b, double lambda,
                                                                   double mdiag, double *W, int *err)
@@ -679,6 +686,19 @@ __global__ void __launch_bounds__(INV64_NT) bdcd_inverse64_kernel(const KT *Kss,
     }
     double *w = W + o * b;
     for (int e = tid; e < b * b; e += INV64_NT) w[e] = a[cur][e / b][b + e % b];
+    if (tid < 32) {  // largest row sums of |G| and |W|, to FP32
+        const float il = (float)(1.0 / lambda), md = (float)mdiag;
+        float gs = 0.f, ws = 0.f;
+        for (int q = 0; tid < b && q < b; ++q) {
+            gs += fabsf((float)kval(Kss, ldk, o + q, o + tid) * il + (tid == q ? md : 0.f));
+            ws += fabsf((float)a[cur][tid][b + q]);
+        }
+        const bool over = !(gs < 3e38f) || !(ws < 3e38f);
+        gs = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(gs)));
+        ws = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(ws)));
+        const bool mark = __any_sync(0xffffffffu, over) || !(gs * ws <= FWD64_COND);
+        if (tid == 0) W[(int64_t)gridDim.x * b * b + j] = mark ? 1.0 : 0.0;
+    }
 }
 
 template <typename KT, int BT, int FWD64_NT>
@@ -687,7 +707,7 @@ __global__ void __launch_bounds__(FWD64_NT) bdcd_forward64_kernel(const KT *Kss,
                                                                   const double *g, const double *W, double *delta,
                                                                   double *w64, float *w32)
 {
-    __shared__ double r[FWD64_SB], ds[BT];
+    __shared__ double r[FWD64_SB], ds[BT], rs[BT];
     __shared__ int32_t sI[FWD64_SB];
     const int sb = nblk * b, tid = threadIdx.x, lane = tid & 31;
     const double inv_lam = 1.0 / lambda;
@@ -699,8 +719,9 @@ __global__ void __launch_bounds__(FWD64_NT) bdcd_forward64_kernel(const KT *Kss,
     // warp 0: its block's inverse, LPR lanes a row (lane: row lane / LPR, every LPR-th column)
     constexpr int LPR = BT <= 8 ? 4 : BT <= 16 ? 2 : 1, QL = BT / LPR;
     const int wp = lane / LPR, wq = lane % LPR;
-    double wv[QL];
+    double wv[QL], marked = 0.0;
     auto load_w = [&](int j) {
+        marked = W[(int64_t)nblk * b * b + j];
 #pragma unroll
         for (int i = 0; i < QL; ++i) {
             const int q = wq + LPR * i;
@@ -743,6 +764,24 @@ __global__ void __launch_bounds__(FWD64_NT) bdcd_forward64_kernel(const KT *Kss,
             double d = d0 + d1;
 #pragma unroll
             for (int o = LPR / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (__double2hiint(marked)) {  // d += W (r - G_jj d); warp-uniform (an integer test: no FP64 latency)
+                if (wp < b && wq == 0) ds[wp] = d;
+                __syncwarp();
+                double e = 0.0;
+                for (int q = wq; wp < b && q < b; q += LPR)
+                    e = fma(kval(Kss, ldk, (int64_t)tb + q, tb + wp), ds[q], e);
+                for (int o = LPR / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+                if (wp < b && wq == 0) rs[wp] = r[tb + wp] - (e * inv_lam + mdiag * d);
+                __syncwarp();
+                e = 0.0;
+#pragma unroll
+                for (int i = 0; i < QL; ++i) {
+                    const int q = wq + LPR * i;
+                    if (q < b) e = fma(wv[i], rs[q], e);
+                }
+                for (int o = LPR / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+                d += e;
+            }
             if (wp < b && wq == 0) {
                 ds[wp] = d;
                 delta[tb + wp] = d;
@@ -1152,7 +1191,7 @@ cudaError_t launch_recur_bdcd(const void *Kss, int kss_f64, int64_t ldk, const i
     if (nblk <= 0) return cudaSuccess;
     if (kss_f64 && recur_bdcd_forward64(nblk, b)) {
         const double *K = (const double *)Kss;
-        if (!W64) {  // nblk b (b + 1) doubles of scratch hold the inverses
+        if (!W64) {  // nblk b (b + 1) doubles of scratch hold the inverses and the marks
             const cudaError_t e = launch_bdcd_inverse64(K, ldk, nblk, b, lambda, mdiag, (double *)scratch, err, st);
             if (e != cudaSuccess) return e;
             W64 = (const double *)scratch;

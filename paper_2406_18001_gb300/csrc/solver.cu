@@ -464,7 +464,7 @@ struct Solver {
             const bool fwd64 = problem == 1 && !tc && recur_bdcd_forward64(o.s, o.b);
             double *w64i[3];
             for (int q = 0; q < 3; ++q)
-                w64i[q] = (double *)ar.take(fwd64 && (q == 0 || (q == 1 && set2)) ? sizeof(double) * sb * o.b : 0);
+                w64i[q] = (double *)ar.take(fwd64 && (q == 0 || (q == 1 && set2)) ? sizeof(double) * (sb * o.b + o.s) : 0);
             grid_ws = ar.take(grid.ctas ? svm_grid_scratch_bytes((int)o.s) : 0);
             grid_h = (double *)ar.take(grid.ctas ? sizeof(double) * m : 0);
             grid_stat = (unsigned long long *)ar.take(grid.ctas ? 2 * sizeof(unsigned long long) : 0);
