@@ -16,6 +16,7 @@
 #include "ptx.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace dcd {
 
@@ -708,6 +709,7 @@ __global__ void __launch_bounds__(FWD64_NT) bdcd_forward64_kernel(const KT *Kss,
                                                                   double *w64, float *w32)
 {
     __shared__ double r[FWD64_SB], ds[BT], rs[BT];
+    __shared__ bool mk[FWD64_SB];  // the blocks' marks
     __shared__ int32_t sI[FWD64_SB];
     const int sb = nblk * b, tid = threadIdx.x, lane = tid & 31;
     const double inv_lam = 1.0 / lambda;
@@ -719,9 +721,8 @@ __global__ void __launch_bounds__(FWD64_NT) bdcd_forward64_kernel(const KT *Kss,
     // warp 0: its block's inverse, LPR lanes a row (lane: row lane / LPR, every LPR-th column)
     constexpr int LPR = BT <= 8 ? 4 : BT <= 16 ? 2 : 1, QL = BT / LPR;
     const int wp = lane / LPR, wq = lane % LPR;
-    double wv[QL], marked = 0.0;
+    double wv[QL];
     auto load_w = [&](int j) {
-        marked = W[(int64_t)nblk * b * b + j];
 #pragma unroll
         for (int i = 0; i < QL; ++i) {
             const int q = wq + LPR * i;
@@ -750,54 +751,63 @@ __global__ void __launch_bounds__(FWD64_NT) bdcd_forward64_kernel(const KT *Kss,
         r[p] -= (s0 + s1) * inv_lam + (rep ? mdiag * dm : 0.0);
     };
     load_k(0, b + tid);
-    __syncthreads();
-    for (int j = 0; j < nblk; ++j) {
-        const int tb = j * b;
-        if (tid < 32) {
-            double d0 = 0.0, d1 = 0.0;
-#pragma unroll
-            for (int i = 0; i < QL; i += 2) {
-                const int q = wq + LPR * i;
-                if (q < b) d0 = fma(wv[i], r[tb + q], d0);
-                if (i + 1 < QL && q + LPR < b) d1 = fma(wv[i + 1], r[tb + q + LPR], d1);
-            }
-            double d = d0 + d1;
-#pragma unroll
-            for (int o = LPR / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            if (__double2hiint(marked)) {  // d += W (r - G_jj d); warp-uniform (an integer test: no FP64 latency)
-                if (wp < b && wq == 0) ds[wp] = d;
-                __syncwarp();
-                double e = 0.0;
-                for (int q = wq; wp < b && q < b; q += LPR)
-                    e = fma(kval(Kss, ldk, (int64_t)tb + q, tb + wp), ds[q], e);
-                for (int o = LPR / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-                if (wp < b && wq == 0) rs[wp] = r[tb + wp] - (e * inv_lam + mdiag * d);
-                __syncwarp();
-                e = 0.0;
-#pragma unroll
-                for (int i = 0; i < QL; ++i) {
-                    const int q = wq + LPR * i;
-                    if (q < b) e = fma(wv[i], rs[q], e);
-                }
-                for (int o = LPR / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-                d += e;
-            }
-            if (wp < b && wq == 0) {
-                ds[wp] = d;
-                delta[tb + wp] = d;
-            }
-            if (j + 1 < nblk) load_w(j + 1);
-        }
-        __syncthreads();
-        const int p0 = tb + b + tid;
-        if (p0 < sb) update(tb, p0);
-        for (int p = p0 + FWD64_NT; p < sb; p += FWD64_NT) {
-            load_k(j, p);
-            update(tb, p);
-        }
-        if (j + 1 < nblk) load_k(j + 1, p0 + b);
-        __syncthreads();
+    bool any = false;
+    for (int j = tid; j < nblk; j += FWD64_NT) {
+        mk[j] = __double2hiint(W[(int64_t)nblk * b * b + j]) != 0;
+        any |= mk[j];
     }
+    // (a loop for the steps without a mark, nearly all: a test a block in the chain took 1.6 us at sb = 256)
+    auto walk = [&](auto marks) {
+        for (int j = 0; j < nblk; ++j) {
+            const int tb = j * b;
+            if (tid < 32) {
+                double d0 = 0.0, d1 = 0.0;
+#pragma unroll
+                for (int i = 0; i < QL; i += 2) {
+                    const int q = wq + LPR * i;
+                    if (q < b) d0 = fma(wv[i], r[tb + q], d0);
+                    if (i + 1 < QL && q + LPR < b) d1 = fma(wv[i + 1], r[tb + q + LPR], d1);
+                }
+                double d = d0 + d1;
+#pragma unroll
+                for (int o = LPR / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+                if (decltype(marks)::value && mk[j]) {  // d += W (r - G_jj d)
+                    if (wp < b && wq == 0) ds[wp] = d;
+                    __syncwarp();
+                    double e = 0.0;
+                    for (int q = wq; wp < b && q < b; q += LPR)
+                        e = fma(kval(Kss, ldk, (int64_t)tb + q, tb + wp), ds[q], e);
+                    for (int o = LPR / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+                    if (wp < b && wq == 0) rs[wp] = r[tb + wp] - (e * inv_lam + mdiag * d);
+                    __syncwarp();
+                    e = 0.0;
+#pragma unroll
+                    for (int i = 0; i < QL; ++i) {
+                        const int q = wq + LPR * i;
+                        if (q < b) e = fma(wv[i], rs[q], e);
+                    }
+                    for (int o = LPR / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+                    d += e;
+                }
+                if (wp < b && wq == 0) {
+                    ds[wp] = d;
+                    delta[tb + wp] = d;
+                }
+                if (j + 1 < nblk) load_w(j + 1);
+            }
+            __syncthreads();
+            const int p0 = tb + b + tid;
+            if (p0 < sb) update(tb, p0);
+            for (int p = p0 + FWD64_NT; p < sb; p += FWD64_NT) {
+                load_k(j, p);
+                update(tb, p);
+            }
+            if (j + 1 < nblk) load_k(j + 1, p0 + b);
+            __syncthreads();
+        }
+    };
+    if (__syncthreads_or(any)) walk(std::true_type());
+    else walk(std::false_type());
     for (int p = tid; p < sb; p += FWD64_NT) {
         const double w = delta[p] / lambda;
         if (w64) w64[p] = w;
