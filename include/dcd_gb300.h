@@ -89,7 +89,20 @@ typedef struct {
  * the b x b solves and the alpha / gradient accumulation are FP64 in every
  * mode. */
 typedef enum {
-    DCD_PREC_FP64 = 0,   /* FP64 CUDA-core block, direct RBF distances */
+    DCD_PREC_FP64 = 0,   /* FP64 block.  Small blocks, n > 512, CSR and the component entry points: FP64
+                            CUDA cores, RBF distances from coordinate differences.  Larger dense
+                            blocks of a solve: rows cut into eight bf16 slices of a 56-bit integer
+                            relative to the row's largest entry, exact slice products on tcgen05,
+                            joined in FP64; the RBF exponent as gamma |a|^2 + gamma |b|^2 - 2 gamma
+                            a.b (absolute error a few 2^-53 of the two norm terms, which are at most
+                            8 each; exactly 0 of a row against itself, not of a row against an equal
+                            one), exp by table within about one ulp.  Data on which that would lose
+                            digits take the CUDA cores: gamma |a|^2 > 8 or a row whose largest entry
+                            holds its norm (RBF), rows that are not spread over their features and
+                            are no short numbers either (linear, polynomial; what the slices drop
+                            stays below 2^-45 / sqrt(n) of sum |a_k b_k|), exponents beyond +-400.
+                            Small K-SVM problems on the resident grid (DCD_FLAG_NO_DEFER) have FP64
+                            dot products, and the same RBF exponent where gamma |a|^2 <= 8 */
     DCD_PREC_TF32 = 1,   /* tcgen05 kind::tf32 block, FP32 accumulation */
     DCD_PREC_BF16 = 2,   /* tcgen05 kind::f16 (bf16) block, FP32 accumulation */
     DCD_PREC_FP8 = 3,    /* tcgen05 kind::f8f6f4 block on e4m3 codes with per-row scales (the
@@ -433,9 +446,13 @@ dcd_status dcd_quantize_e4m3(const dcd_matrix *A, uint8_t *q, int64_t ldq, float
  *   handled), g_S[p] = g[S[p]].  The Gram is Kss / lambda + mdiag * [S_p ==
  *   S_q] (mdiag = m).  Output: delta[p] (the change of alpha at position p)
  *   and, when w is non-NULL, w[p] = delta[p] / lambda (the coefficients of
- *   the kernel-block update).  FP64 arithmetic throughout; an FP64 Kss gets
- *   the adaptive refinement of the FP64 solve, an FP32 one a refined FP32
- *   factorisation.  A non-positive-definite diagonal block gives DCD_ENOTSPD.
+ *   the kernel-block update).  An FP64 Kss gets the recurrence of the FP64
+ *   solve: for b <= 32 and nblk*b <= 1024 an FP64 forward substitution with
+ *   the blocks' inverses, corrected by the residual where a block is
+ *   ill-conditioned; else FP32 chains refined by FP64 residuals, the rounds
+ *   decided on the device, with an FP64 factorisation as the fallback.  An
+ *   FP32 Kss gets a refined FP32 factorisation.  A non-positive-definite
+ *   diagonal block gives DCD_ENOTSPD.
  *
  * dcd_dcd_recurrence -- the K-SVM recurrence of Algorithm 2 on gathered
  *   values: Kss the sampled kernel block (raw kernel values), S the sampled

@@ -882,8 +882,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         // The column terms of a half's <= 4 groups (K-term, coefficient, scale, ids), shared by the
         // half's four warps and double-buffered.  Each warp loads its 32 of them (and its rows'
         // terms) into registers one unit ahead, so that no unit starts with a chain of L2 round
-        // trips, and the units are stepped without divisions: at n = 512 an epilogue unit took
-        // 7.0 k cycles, now 4.0-5.0 k beside the 4.1 k of its MMAs.
+        // trips, and the units are stepped without divisions: at n = 512 a unit took 7.0 k cycles,
+        // now 5.5 k beside the 4.1 k of its MMAs, whose warp waits 2.5 k of them for an accumulator
+        // still being read here and 0.75 k for operands.
         float *const cst0 = (float *)(smem + RING2_BYTES + 256 + XCH_BYTES) + half * 2 * CST_FLOATS;
         float *cst = cst0;
         const int ncols_h = (cg1 - cg0) * 32;  // columns of this half

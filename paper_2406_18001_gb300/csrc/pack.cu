@@ -5,9 +5,9 @@
 // see).  HBM-bound: each value is read once and each plane written once (a second read where every
 // row's scale hangs on the matrix's largest magnitude, fp16).  Loads go eight columns a lane ahead
 // of the conversions; lanes own columns lane, lane + 32, ... and sum them in that order.  Measured
-// at 50000 x 512 FP32 (102 MB): fp16 packed and its terms 52 us (227 when the largest
-// magnitude, the pack and the terms were kernels with scalar loads, one atomic per row and FP64
-// sums), sliced 20000 x 512 30 us (714).
+// at 50000 x 512 FP32 (102 MB): fp16 packed and its terms 34 us and the largest magnitude 18 (227
+// together when the magnitude, the pack and the terms were kernels with scalar loads, one atomic per row
+// and FP64 sums), sliced 20000 x 512 30 us (714).
 #include "dcd_internal.cuh"
 
 #include <cuda_fp16.h>

@@ -47,7 +47,8 @@ unsigned long long context_id(int dev)
 // The library's own memory pool in the current context (nullptr: none could be made; a stream-ordered
 // pool, so safe from several threads and streams).  It keeps at most POOL_KEEP of freed memory mapped:
 // the default pool returns all of it to the driver at every synchronisation, and mapping it again took
-// 50 to 170 us of an allocation after one (a sweep of 32 plans: 19.7 -> 15.9 ms).  What it keeps goes
+// 50 to 170 us of an allocation after one (a sweep of 32 plans: 19.7 -> 15.9 ms on one host, 22.0 -> 19.0
+// on another).  What it keeps goes
 // back when an allocation of the library's fails, and with the process.  A pool dies with its context
 // (cudaDeviceReset), so pools go by the context's number.
 constexpr size_t POOL_CONTEXTS = 64;

@@ -263,8 +263,8 @@ extern "C" dcd_status dcd_bdcd_recurrence(const void *Kss, int32_t kss_f64, int6
     SH_TRY(cudaMemsetAsync(err, 0, sizeof(int), st));
     first_pos_kernel<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(S, cnt, Sc);
     SH_TRY(cudaGetLastError());
-    // the refinement setting of the single-GPU step: adaptive FP64 refinement
-    // on an FP64 Gram, one refinement round on an FP32 one
+    // the setting of the single-GPU step: on an FP64 Gram the FP64 form (forward substitution, or adaptive
+    // refinement where it is large), one refinement round on an FP32 one
     SH_TRY(launch_recur_bdcd(Kss, kss_f64, ldk, Sc, nblk, b, lambda, mdiag, g_S, kss_f64 ? 2 : 1, base + off_l, delta,
                              w, nullptr, nullptr, err, st));
     return finish(err, st);

@@ -401,7 +401,8 @@ struct Solver {
         // chain longer than one cluster): the next step's sample, column map or gathers and Gram
         // on a second stream beside the recurrence and block
         // (not with steps asked for in order or directly, or checked so often that a launch would hold
-        // only a few; from the line of the slice form on, that form's block is the faster one)
+        // only a few: a line that could lie lower, at m = 2000, n = 64, s = 8 a step takes 6.8 us on the grid with a
+        // check every 16, 8.8 every 8 and 21.6 every 2, as separate kernels 19.1 every 8 and 30.1 every 2; from the line of the slice form on, that form's block is the faster one)
         if (problem == 0 && !csr && !tc && !literal && !f64s_worth() &&
             !(o.flags & (DCD_FLAG_NO_GRAPH | DCD_FLAG_NO_DEFER | DCD_FLAG_PHASE_TIMERS)) &&
             (o.tol <= 0.0 || o.check_every <= 0 || o.check_every >= 16))
@@ -1421,7 +1422,8 @@ struct Solver {
     bool df_chain = false;     // its recurrence outputs (and x of the step after it) are in place
     int64_t df_prod = 0;       // step size of the products in (df_cur + 1) % 3 (0: none)
     double *df_x[3] = {nullptr, nullptr, nullptr};  // per set: x of its step (a part per 256 columns)
-    cudaStream_t st3 = nullptr, st4 = nullptr;  // x of the step after next, beside its Gram and prep
+    // K-RR: x of the step after next, beside its Gram and prep; K-SVM: the recurrence, and on st4 the cross product
+    cudaStream_t st3 = nullptr, st4 = nullptr;
     cudaEvent_t df_fork = nullptr, df_chained = nullptr, df_rows = nullptr, df_gram = nullptr, df_side = nullptr;
     int32_t *df_link[3] = {nullptr, nullptr, nullptr};  // per set: where its rows are in the step before
     int df_pairs = 0;          // CTA pairs of the block
