@@ -635,11 +635,14 @@ __global__ void __launch_bounds__(256) bdcd_residual_kernel(const KT *Kss, int64
 // The product with an inverse has a Cholesky solve's error but not its residual, which grows with
 // cond(G_jj)^2: up to 10 times a Cholesky solve's at a condition number of 1e2 - 1e3, 800 at 1e7, 1e4 at 1e10
 // (random blocks of 2 to 32 rows; near-duplicate rows and a small lambda have such).  So the kernel that
-// forms an inverse marks a block where |G|_inf |W|_inf is above FWD64_COND, and for those the forward kernel
-// adds W (r - G_jj Delta_j), which brings the residual to a Cholesky solve's at every condition number tried.
+// forms an inverse marks a block where b max G_pp max W_pp, between the condition number over b and b times
+// it, is above FWD64_COND, and for those the forward kernel adds W (r - G_jj Delta_j), which brings the
+// residual to a Cholesky solve's at every condition number tried.  Unmarked blocks stay below 30 2^-53 of
+// |G| |Delta| (random blocks, three kernels); with kernels and widths in use the product is 10 to 150.  (Row
+// sums of |G| and |W| instead took the inverses' kernel 2 us more, which holds SMs that the block waits for.)
 constexpr int FWD64_SB = 1024;
 constexpr int INV64_NT = 256;
-constexpr float FWD64_COND = 128.f;
+constexpr float FWD64_COND = 256.f;
 
 // W_j by Gauss-Jordan on [G_jj | I], only the columns that can change at pivot k touched; the owner of
 // the next pivot forms its reciprocal.  W: nblk blocks of b x b, row-major, then a mark per block (0 or 1).
@@ -658,6 +661,7 @@ __global__ void __launch_bounds__(INV64_NT) bdcd_inverse64_kernel(const KT *Kss,
         if (p == 0 && q == 0) ip_s[0] = 1.0 / a[0][0][0];
     }
     __syncthreads();
+    float dg = tid < b ? (float)a[0][tid][tid] : 0.f;  // for the mark
     int cur = 0;
     bool bad = false;
     for (int k = 0; k < b; ++k) {
@@ -687,17 +691,12 @@ __global__ void __launch_bounds__(INV64_NT) bdcd_inverse64_kernel(const KT *Kss,
     }
     double *w = W + o * b;
     for (int e = tid; e < b * b; e += INV64_NT) w[e] = a[cur][e / b][b + e % b];
-    if (tid < 32) {  // largest row sums of |G| and |W|, to FP32
-        const float il = (float)(1.0 / lambda), md = (float)mdiag;
-        float gs = 0.f, ws = 0.f;
-        for (int q = 0; tid < b && q < b; ++q) {
-            gs += fabsf((float)kval(Kss, ldk, o + q, o + tid) * il + (tid == q ? md : 0.f));
-            ws += fabsf((float)a[cur][tid][b + q]);
-        }
-        const bool over = !(gs < 3e38f) || !(ws < 3e38f);
-        gs = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(gs)));
-        ws = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(ws)));
-        const bool mark = __any_sync(0xffffffffu, over) || !(gs * ws <= FWD64_COND);
+    if (tid < 32) {
+        float dw = tid < b ? (float)a[cur][tid][b + tid] : 0.f;
+        const bool over = !(dg < 3e38f) || !(dw < 3e38f);
+        dg = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(dg, 0.f))));
+        dw = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(dw, 0.f))));
+        const bool mark = __any_sync(0xffffffffu, over) || !((float)b * dg * dw <= FWD64_COND);
         if (tid == 0) W[(int64_t)gridDim.x * b * b + j] = mark ? 1.0 : 0.0;
     }
 }
