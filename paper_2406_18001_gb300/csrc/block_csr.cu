@@ -370,8 +370,9 @@ __global__ void __launch_bounds__(CSR_AW * 32, 3)
 //            with their prefix sums, then the CTA's threads sweep the group's
 //            incidences as one flat range (CSC_U independent loads and
 //            atomics per thread in flight) and append key = (e << 10) | (i mod
-//            32) << 5 | j (e counted from the tile's first nonzero) and the product a_ie * a_{S_j},c to the bucket of
-//            the incidence's 32-row tile (a fixed capacity per tile; a counter
+//            32) << 5 | j (e counted from the tile's first nonzero) and the
+//            product a_ie * a_{S_j},c to the bucket of the
+//            incidence's 32-row tile (a fixed capacity per tile; a counter
 //            per tile, in arbitrary order);
 //   apply    a warp per tile (the next tile's bucket loaded while this one
 //            is processed) counting-sorts its incidences by row (shared

@@ -11,22 +11,22 @@
 // epilogue joins the eight in integer arithmetic and FP64, so that
 //     a_i.a_j = 2^(e_i + e_j - 61) (I_hi 2^28 + I_lo),  I_hi, I_lo exact 64-bit integers,
 // is rounded once.  What is left out (p + q >= 8, the ninth slice) is at most 9 2^-56 2^(e_i + e_j) a
-// feature that is nonzero in both rows, about a tenth of that on average and of either sign: relative to
-// the rows' largest magnitudes, not to sum_k |a_ik a_jk| as the rounding of an FP64 sum is.  The two are
-// alike while the features that make up a product are not all tiny beside others; where a large feature
-// of one row meets a zero of the other they are not (features of 1 beside one of 1e9: 1e-7 relative).  So
-// the linear and polynomial kernels take the form only if every row of the matrix has its magnitude
-// spread over its features, or if the four last slices are zero in all of them (whole numbers up to
-// 2^27, bits: nothing is left out); see f64s_row_flags.  Where the first holds, sum_k |a_ik a_jk| >= n
-// 2^-11 2^(e_i + e_j) for every two rows, and the part left out stays below 2^-45 / sqrt(n) of it (n
-// roundings of like size, of either sign).  The RBF exponent comes from the expansion gamma |a_i|^2 + gamma |a_j|^2
-// - 2 gamma a_i.a_j with norms from compensated FP64 sums: its absolute error is some 2^-53
-// gamma (|a_i|^2 + |a_j|^2), so the form is used where gamma |a|^2 <= F64S_HMAX for every row
-// (pack_f64s reports the largest) and the direct differences serve elsewhere.  What the slices leave out
-// of 2 gamma a_i.a_j, about 2 gamma sqrt(n) 2^-56 2^(e_i + e_j), is less than that for rows whose
-// magnitude is spread over their features; where one feature holds it and n is large it is more (one
-// feature of 2.05, 511 of 1e-3, gamma |a|^2 = 7.9: 4.3e-14 in a kernel value), so gamma 4^e sqrt(n) / 2
-// has the same limit: at most four times 2^-53 is left out.
+// feature that is nonzero in both rows, about a tenth of that on average and of either sign: relative
+// to the rows' largest magnitudes, not to sum_k |a_ik a_jk| as the rounding of an FP64 sum is.  The two
+// are alike while the features that make up a product are not all tiny beside others; where a large
+// feature of one row meets a zero of the other they are not (features of 1 beside one of 1e9: 1e-7
+// relative).  So the linear and polynomial kernels take the form only if every row of the matrix has
+// its magnitude spread over its features, or if the four last slices are zero in all of them (whole
+// numbers up to 2^27, bits: nothing is left out); see f64s_row_flags.  Where the first holds,
+// sum_k |a_ik a_jk| >= n 2^-11 2^(e_i + e_j) for every two rows, and the part left out stays below
+// 2^-45 / sqrt(n) of it (n roundings of like size, of either sign).  The RBF exponent comes from the
+// expansion gamma |a_i|^2 + gamma |a_j|^2 - 2 gamma a_i.a_j with norms from compensated FP64 sums: its
+// absolute error is some 2^-53 gamma (|a_i|^2 + |a_j|^2), so the form is used where gamma |a|^2 <=
+// F64S_HMAX for every row (pack_f64s reports the largest) and the direct differences serve elsewhere.
+// What the slices leave out of 2 gamma a_i.a_j, about 2 gamma sqrt(n) 2^-56 2^(e_i + e_j), is less than
+// that for rows whose magnitude is spread over their features; where one feature holds it and n is
+// large it is more (one feature of 2.05, 511 of 1e-3, gamma |a|^2 = 7.9: 4.3e-14 in a kernel value), so
+// gamma 4^e sqrt(n) / 2 has the same limit: at most four times 2^-53 is left out.
 //
 // What bounds it: the FP64 pipe, with 16 operations an entry instead of 2 n: two integer-to-double
 // differences, a sum of the terms and two FMAs for the exponent, ten for exp, one for the

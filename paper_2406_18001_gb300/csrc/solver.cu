@@ -400,9 +400,10 @@ struct Solver {
         // the look-ahead of the other steps (K-SVM, dense or CSR; K-RR in FP64, on CSR or with a
         // chain longer than one cluster): the next step's sample, column map or gathers and Gram
         // on a second stream beside the recurrence and block
-        // (not with steps asked for in order or directly, or checked so often that a launch would hold
-        // only a few: a line that could lie lower, at m = 2000, n = 64, s = 8 a step takes 6.8 us on the grid with a
-        // check every 16, 8.8 every 8 and 21.6 every 2, as separate kernels 19.1 every 8 and 30.1 every 2; from the line of the slice form on, that form's block is the faster one)
+        // (not with steps asked for in order or directly, or checked so often that a launch would hold only
+        // a few: a line that could lie lower, at m = 2000, n = 64, s = 8 a step takes 6.8 us on the grid with a
+        // check every 16 steps, 8.8 every 8 and 21.6 every 2, as separate kernels 19.1 every 8 and 30.1 every
+        // 2; from the line of the slice form on, that form's block is the faster one)
         if (problem == 0 && !csr && !tc && !literal && !f64s_worth() &&
             !(o.flags & (DCD_FLAG_NO_GRAPH | DCD_FLAG_NO_DEFER | DCD_FLAG_PHASE_TIMERS)) &&
             (o.tol <= 0.0 || o.check_every <= 0 || o.check_every >= 16))
@@ -832,8 +833,9 @@ struct Solver {
 
     // The FP64 form's block through exact slices (block_f64.cu) where it is the faster one and as
     // exact: n within the exact sums, every value finite with a moderate exponent, for the RBF
-    // gamma |a|^2 and gamma 4^e sqrt(n) / 2 <= F64S_HMAX (the expansion's and the slices' errors), and for the other kernels rows whose magnitude is
-    // spread over their features, or short values (what the form leaves out, block_f64.cu).  The line is on the products m sb n of the
+    // gamma |a|^2 and gamma 4^e sqrt(n) / 2 <= F64S_HMAX (the expansion's and the slices' errors), and
+    // for the other kernels rows whose magnitude is spread over their features, or short values (what
+    // the form leaves out, block_f64.cu).  The line is on the products m sb n of the
     // block, by measured time of sample + Gram + block a step (direct / slices, us): blocks of at
     // most 32 columns, whose direct form is spread over every SM, 2000 x 64 x 16 (2.0 M) 36 / 56,
     // 6000 x 64 x 8 (3.1 M) 39 / 44, 2000 x 200 x 8 (3.2 M) 58 / 53, 6000 x 200 x 8 (9.6 M)
