@@ -118,7 +118,7 @@ struct TcArgs {
     int64_t ncols;
     int num_tiles, nchunks, kblocks, bn;
     int store;            // 1: store epilogue, 0: apply
-    int lower;            // store: skip the N-chunks above the diagonal
+    int lower;            // store: skip the N-chunks past lower - 1 columns above the diagonal (0: none)
     int items;            // apply: num_tiles; store: num_tiles * nchunks
     int degree;
     float two_gl;         // 2 * gamma * log2(e)
@@ -274,12 +274,16 @@ __device__ __forceinline__ void k_accurate(float dh, float dl, float hr, float h
 // store form: one item = one (row tile, N-chunk) pair; with `lower`, the
 // chunks that start past the tile's last row are empty items (every role
 // skips them alike)
-// N-chunks of row tile t that reach the lower triangle (the store form's lower option)
-__host__ __device__ __forceinline__ int lower_chunks(int t, int bn, int nchunks)
+// N-chunks of row tile t that start at or before column last row + lower - 1 (the store form's lower option)
+__host__ __device__ __forceinline__ int lower_chunks(int t, int bn, int nchunks, int lower)
 {
-    const int64_t n = ((int64_t)t * BM + BM - 1) / bn + 1;
+    const int64_t n = ((int64_t)t * BM + BM - 2 + lower) / bn + 1;
     return n < nchunks ? (int)n : nchunks;
 }
+
+// ... of the lower triangle with diagonal blocks of b rows: a block that lies across a tile's last row has
+// up to b - 1 columns past it
+inline int lower_of(int b) { return b <= 0 ? 0 : BM % b ? b : 1; }
 
 // The single-CTA kernel's work item: one (row tile, N-chunk); with lower, only the chunks that
 // reach the lower triangle are items, numbered tile by tile
@@ -287,8 +291,8 @@ __device__ __forceinline__ void item_range(const TcArgs &a, int item, int &tile,
 {
     if (a.lower) {
         int t = 0, rem = item;
-        for (int n = lower_chunks(0, a.bn, a.nchunks); rem >= n && t + 1 < a.num_tiles;
-             n = lower_chunks(++t, a.bn, a.nchunks))
+        for (int n = lower_chunks(0, a.bn, a.nchunks, a.lower); rem >= n && t + 1 < a.num_tiles;
+             n = lower_chunks(++t, a.bn, a.nchunks, a.lower))
             rem -= n;
         tile = t;
         c0 = rem;
@@ -1421,12 +1425,12 @@ cudaError_t launch_mode2(int npairs, const CUtensorMap &mA, const CUtensorMap &m
 
 }  // namespace
 
-int tc_store_items(int64_t nrows, int64_t ncols, int bn, bool lower)
+int tc_store_items(int64_t nrows, int64_t ncols, int bn, int lower_b)
 {
     const int tiles = (int)((nrows + BM - 1) / BM), chunks = (int)((ncols + bn - 1) / bn);
-    if (!lower) return tiles * chunks;
+    if (!lower_b) return tiles * chunks;
     int items = 0;
-    for (int t = 0; t < tiles; ++t) items += lower_chunks(t, bn, chunks);
+    for (int t = 0; t < tiles; ++t) items += lower_chunks(t, bn, chunks, lower_of(lower_b));
     return items;
 }
 
@@ -1470,7 +1474,7 @@ bool make_map_f32_2d(CUtensorMap *map, const float *base, int64_t cols, int64_t 
 
 cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const KernelParams &kp, const float *row_h,
                             const float *col_h, const float *col_w, const double *rs, double *g, float *out,
-                            int64_t ldo, int64_t nrows_out, int64_t ncols, int *err, cudaStream_t st, bool lower,
+                            int64_t ldo, int64_t nrows_out, int64_t ncols, int *err, cudaStream_t st, int lower_b,
                             const TcSplit *split, bool pdl, int max_pairs, const TcAccurate *acc, bool pdl_wait,
                             int prio, const TcCross *cross)
 {
@@ -1495,7 +1499,7 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
     // CTA one item
     if (out != nullptr) {
         const int bn0 = bn;
-        for (bn = bn0 < 64 ? bn0 : 64; max_pairs > 0 && bn < bn0 && tc_store_items(nrows_out, ncols, bn, lower) > max_pairs;)
+        for (bn = bn0 < 64 ? bn0 : 64; max_pairs > 0 && bn < bn0 && tc_store_items(nrows_out, ncols, bn, lower_b) > max_pairs;)
             bn = 2 * bn < bn0 ? 2 * bn : bn0;
     }
     // the apply form runs on CTA pairs (each CTA stages half of an N-chunk of B)
@@ -1520,8 +1524,8 @@ cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const Ke
     a.kblocks = (int)(Aop.n_pad / kb_elems);
     a.bn = bn;
     a.store = out != nullptr;
-    a.lower = a.store && lower;
-    a.items = a.store ? tc_store_items(nrows_out, ncols, bn, a.lower) : a.num_tiles;
+    a.lower = a.store ? lower_of(lower_b) : 0;
+    a.items = a.store ? tc_store_items(nrows_out, ncols, bn, lower_b) : a.num_tiles;
     a.degree = kp.degree;
     a.two_gl = (float)(2.0 * kp.gamma * 1.4426950408889634);
     a.coef0 = (float)kp.coef0;

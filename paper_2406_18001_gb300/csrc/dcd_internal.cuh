@@ -199,10 +199,10 @@ __host__ __device__ inline int64_t packed_row_bytes(int kind, int64_t n_pad)
                                                         : 2 * n_pad;
 }
 bool tc_available();
-// the store form's work items with N-chunks of bn columns (128-row tiles; lower: those that reach the diagonal)
-int tc_store_items(int64_t nrows, int64_t ncols, int bn, bool lower);
-// lower (store form only): write only the N-chunks that reach the diagonal
-// (column chunk start <= last row of the tile); the rest of out is left as is
+// the store form's work items with N-chunks of bn columns (128-row tiles; lower_b as below)
+int tc_store_items(int64_t nrows, int64_t ncols, int bn, int lower_b);
+// lower_b (store form only; 0: the whole): write only the N-chunks that reach the lower triangle with its
+// diagonal blocks of lower_b rows; the rest of out is left as is
 //
 // pdl (apply form): launch as a programmatic dependent of the kernel before
 // it on st; the products start at once, the epilogue waits for that kernel
@@ -254,7 +254,7 @@ struct TcAccurate {
 cudaError_t launch_block_tc(const TcOperand &Aop, const TcOperand &Bop, const KernelParams &kp,
                             const float *row_h, const float *col_h, const float *col_w, const double *rs,
                             double *g, float *out, int64_t ldo, int64_t nrows_out, int64_t ncols,
-                            int *err, cudaStream_t st, bool lower = false, const TcSplit *split = nullptr,
+                            int *err, cudaStream_t st, int lower_b = 0, const TcSplit *split = nullptr,
                             bool pdl = false, int max_pairs = 0, const TcAccurate *acc = nullptr,
                             bool pdl_wait = true, int prio = 0, const TcCross *cross = nullptr);
 // (pdl: launched as the programmatic dependent of the kernel before it in the stream, whose

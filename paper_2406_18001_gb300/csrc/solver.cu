@@ -997,11 +997,11 @@ struct Solver {
             return launch_csr_block(ca, cm, !tc, kp, S, ncols, S, ncols, nullptr, nullptr, nullptr, nullptr, Kss, ldk,
                                     st);
         if (tc) {
-            // the cluster and blocked recurrences read the lower triangle only
+            // the cluster and blocked recurrences read the lower triangle and the diagonal blocks only
             const bool lower = problem == 1 && recur_bdcd_lower_gram(ncols / o.b, o.b, 1, ldk);
             TcOperand B{As, ncols, op.n_pad, op.kind, col_s, S};
             return launch_block_tc(B, B, kp, col_h, col_h, nullptr, nullptr, nullptr, (float *)Kss, ldk, ncols, ncols,
-                                   err, st, lower);
+                                   err, st, lower ? o.b : 0);
         }
         if (f64s)
             return launch_block_f64s(fs, As, ncols, S, As, ncols, S, kp, nullptr, nullptr, nullptr, (double *)Kss, ldk,
@@ -1042,7 +1042,7 @@ struct Solver {
             acc.row_hl = row_hlr;
             acc.col_hl = col_hlr;
             return cuda_status(launch_block_tc(Aop, Bop, kp, opr.row_h, col_hr, col_w, rs, g, nullptr, 0, m, ncols,
-                                               err, st, false, &tsplit, false, 0, &acc));
+                                               err, st, 0, &tsplit, false, 0, &acc));
         }
         if (tc) {
             const Operand &x = ref ? opr : op;
@@ -1059,7 +1059,7 @@ struct Solver {
             TcOperand Bop{Asx, ncols, x.n_pad, x.kind, x.kind == PACK_FP8 || x.kind == PACK_FP16 ? col_s : nullptr,
                           S};
             return cuda_status(
-                launch_block_tc(Aop, Bop, kp, x.row_h, chx, col_w, rs, g, nullptr, 0, m, ncols, err, st, false, &tsplit));
+                launch_block_tc(Aop, Bop, kp, x.row_h, chx, col_w, rs, g, nullptr, 0, m, ncols, err, st, 0, &tsplit));
         }
         if (f64s) DCD_TRY(gather(ncols));
         return cuda_status(block_f64_apply(ncols, rs));
@@ -1124,7 +1124,7 @@ struct Solver {
     {
         TcOperand Aop{op.packed, m, op.n_pad, op.kind, op.row_s};
         TcOperand Bop{As, ncols, op.n_pad, op.kind, col_s, S};
-        return launch_block_tc(Aop, Bop, kp, op.row_h, col_h, col_w, rs, g, nullptr, 0, m, ncols, err, st, false,
+        return launch_block_tc(Aop, Bop, kp, op.row_h, col_h, col_w, rs, g, nullptr, 0, m, ncols, err, st, 0,
                                &tsplit);
     }
 
@@ -1327,7 +1327,7 @@ struct Solver {
         const int64_t ncols = cnt * o.b;
         TcOperand Bo{Bq.As, ncols, op.n_pad, op.kind, Bq.col_s, Bq.S};
         DCD_TRY(launch_block_tc(Bo, Bo, kp, Bq.col_h, Bq.col_h, nullptr, nullptr, nullptr, (float *)Bq.Kss, ldk, ncols,
-                                ncols, err, s2, true, nullptr, false, max_ctas));
+                                ncols, err, s2, o.b, nullptr, false, max_ctas));
         DCD_TRY(launch_recur_cluster_prep((const float *)Bq.Kss, ldk, Bq.S, (int)cnt, o.b, lambda, (double)m, Bq.Lbuf,
                                           err, s2));
         return DCD_OK;
@@ -1373,7 +1373,7 @@ struct Solver {
         sp.late_pairs = (P + 1) / 2;
         sp.late_units = 2;
         DCD_TRY(launch_block_tc(Aop, Bop, kp, op.row_h, Bp.col_h, col_w, nullptr, g, nullptr, 0, m, ncols, err, st,
-                                false, &sp, true));
+                                0, &sp, true));
         if (next) DCD_TRY(cudaStreamWaitEvent(st, la_join, 0));
         return DCD_OK;
     }
@@ -1449,8 +1449,8 @@ struct Solver {
         const double unit = std::max(mma, 3.5), units = (double)((m + 255) / 256) * chunks;
         double best = 0;
         for (int most : {24, 16, 8}) {
-            int w = 64, items = tc_store_items(sb, sb, w, true);
-            while (items > most && w < 256) items = tc_store_items(sb, sb, w *= 2, true);
+            int w = 64, items = tc_store_items(sb, sb, w, o.b);
+            while (items > most && w < 256) items = tc_store_items(sb, sb, w *= 2, o.b);
             const int ctas = std::min(items, most), pairs = std::max(avail - (ctas + 1) / 2, 1);
             const double gram = std::ceil((double)items / ctas) * (4 + 1.15 * mma * w / 256);
             const double t = std::max(std::ceil(units / pairs) * unit + 18, 58 + gram);
@@ -1500,7 +1500,7 @@ struct Solver {
         cr.row_link = df_link[r];
         cr.col_next = recur_cluster_next(Bc.Lbuf, (int)o.s, o.b);
         DCD_TRY(launch_block_tc(Ax, Bx, kp, Br.col_h, Bc.col_h, Bc.col_w, nullptr, nullptr, nullptr, 0, nc, nc, err, s,
-                                false, nullptr, false, DF_XPAIRS, nullptr, true, 0, &cr));
+                                0, nullptr, false, DF_XPAIRS, nullptr, true, 0, &cr));
         return DCD_OK;
     }
 
@@ -1556,7 +1556,7 @@ struct Solver {
         TcOperand Aop{op.packed, m, op.n_pad, op.kind, op.row_s};
         TcOperand Bop{Bc.As, ncols, op.n_pad, op.kind, Bc.col_s, Bc.S};
         DCD_TRY(launch_block_tc(Aop, Bop, kp, op.row_h, Bc.col_h, Bc.col_w, nullptr, g, nullptr, 0, m, ncols, err, st,
-                                false, &tsplit, has1, has1 ? df_pairs : 0, nullptr, false, df_prio));
+                                0, &tsplit, has1, has1 ? df_pairs : 0, nullptr, false, df_prio));
         DCD_TRY(launch_update(Bc.S, Bc.delta, ncols, diag, alpha, g, ctr, (uint64_t)cnt, m, err, st));
         if (has2) {
             DCD_TRY(cudaStreamWaitEvent(st, df_gram, 0));
@@ -2602,7 +2602,7 @@ dcd_status component_block(const dcd_matrix *A, const dcd_kernel *k, int32_t pre
     acc.row_hl = rl;
     acc.col_hl = cl;
     DCD_TRY(launch_block_tc(Aop, Bop, kp, rh, ch, w ? cw : nullptr, rs, g, (float *)out, ldo, nrows, ncols, err, st,
-                            false, &sp, false, 0, accurate ? &acc : nullptr));
+                            0, &sp, false, 0, accurate ? &acc : nullptr));
     return finish_component(err, st);
 }
 
